@@ -770,7 +770,7 @@ std::vector<int32_t> pair_lanes(bc_ctx *ctx, const Graph &g, const int32_t *d_sr
   for (int i = 0; i < count; ++i)
     if (flags[(size_t)i]) bigs.push_back(i);
   Workspace &ws = ctx->ws;
-  const bool deep = graph_depth_hint(ctx, g) > ctx->deep_levels;
+  const bool deep = lane_major(ctx, g);
   B.idx.ensure(64 * 4);
   for (size_t k0 = 0; k0 < bigs.size(); k0 += 64) {
     const int c = (int)std::min<size_t>(64, bigs.size() - k0);

@@ -518,15 +518,16 @@ static void launch_draw_sources(bc_ctx *ctx, uint64_t seed, uint64_t qid, uint64
 
 // Lanes whose path counts exceed 2^64-1 skip the integer backward pass and are
 // recomputed in the extended form (bc_ext.cu); the others are unaffected.
-// Deep graphs (the hub's eccentricity above ctx->deep_levels, e.g. grids) go
-// lane-major: level masks and 64-lane rows cost O(levels * n) there, while each
-// lane's own BFS costs O(n + nnz).
+// Graphs whose per-source state fits shared memory (solo_fits) and deep graphs
+// (the hub's eccentricity above ctx->deep_levels, e.g. grids) run one source
+// per CTA: on deep graphs level masks and 64-lane rows cost O(levels * n),
+// while each source's own BFS costs O(n + nnz).
 void run_source_batch(bc_ctx *ctx, const Graph &g, int count, const Sink &sink) {
   if (g.w) {  // edge lengths: the weighted engine at any width
     wlane_sink(ctx, g, ctx->ws.sources.as<int32_t>(), count, sink);
   } else if (batch_width(ctx) == 1) {
     plain_source(ctx, g, ctx->ws.sources.as<int32_t>(), sink, nullptr, nullptr);
-  } else if (graph_depth_hint(ctx, g) > ctx->deep_levels) {
+  } else if (lane_major(ctx, g)) {
     lane_sink(ctx, g, ctx->ws.sources.as<int32_t>(), count, sink);
   } else {
     const int maxl = batch_forward(ctx, g, count, false, OVF_EXTEND);
@@ -600,7 +601,7 @@ static void copy_scan_out(bc_ctx *ctx, int32_t T, const ScanState &st, double sc
 // BCG_KEY_LANDMARKS; 1 gives the hub distance alone, rescaled).
 struct KeyMeta {
   DevBuf key, order;
-  int32_t ecc = 0;  // largest finite distance from the hub
+  int32_t ecc = -1;  // largest finite distance from the hub (-1: not known yet)
 };
 static std::map<const int32_t *, KeyMeta> g_keys;
 static std::mutex g_keys_mu;
@@ -758,27 +759,48 @@ static KeyMeta &key_meta(bc_ctx *ctx, const Graph &g, bool need_order) {
   return km;
 }
 
-constexpr int WMAX = 1024;
+constexpr int WMAX = 1024;       // draws per window of the 64-lane engine
+constexpr int WMAX_SOLO = 4096;  // ... of the engines that run one source per CTA
 
-// Draws [i0, i0+W) of (seed, qid), grouped by source key: afterwards
-// ws.win = draws[W] | sorted sources[W] | sorted draw positions[W].
-static void draw_window(bc_ctx *ctx, const Graph &g, const KeyMeta &km, uint64_t seed, uint64_t qid, int64_t i0,
-                        int W) {
-  Workspace &ws = ctx->ws;
-  ws.win.ensure(3 * WMAX * 4);
-  int32_t *draws = ws.win.as<int32_t>();
-  launch_draw_sources(ctx, seed, qid, (uint64_t)i0, W, g.n, draws);
-  LaunchScope ls(ctx, F_DRAW);
-  k_sort_window<<<1, 1024, 0, ctx->stream>>>(W, draws, km.key.as<uint8_t>(), draws + WMAX, draws + 2 * WMAX);
+bool lane_major(bc_ctx *ctx, const Graph &g) {
+  return solo_fits(ctx, g) || graph_depth_hint(ctx, g) > ctx->deep_levels;  // (a fitting graph needs no depth here)
 }
 
-// Runs the window's sources in batches of the context's width; lane t of the
-// batch starting at position b is the window's sorted entry b + t.
-// Engines that run one source per persistent CTA (edge lengths; deep or
-// directed graphs) take a whole window in one launch, so every resident CTA
-// has a source; the 64-lane engine and the plain width take 64 or 1 at a time.
-static bool one_source_per_cta(bc_ctx *ctx, const Graph &g) {
-  return batch_width(ctx) != 1 && (g.w || graph_depth_hint(ctx, g) > ctx->deep_levels);
+// Engines that run one source per persistent CTA (edge lengths; deep graphs;
+// graphs whose state fits shared memory) take a whole window in one launch, so
+// every resident CTA has a source; the 64-lane engine and the plain width take
+// 64 or 1 at a time.
+bool one_source_per_cta(bc_ctx *ctx, const Graph &g) {
+  return batch_width(ctx) != 1 && (g.w || lane_major(ctx, g));
+}
+
+// The draws a window can hold and the size of the first one. Where a source
+// has a CTA of its own, fewer sources than CTAs leave SMs idle, so windows
+// start at one source per resident CTA (per SM on the weighted engine and on
+// deep graphs in global memory, where more sources at once compete for
+// bandwidth) instead of 64.
+static int window_max(bc_ctx *ctx, const Graph &g, int32_t T) {
+  return one_source_per_cta(ctx, g) && T <= 4096 ? WMAX_SOLO : WMAX;
+}
+static int window_first(bc_ctx *ctx, const Graph &g) {
+  if (!one_source_per_cta(ctx, g)) return 64;
+  return std::max(64, g.w ? 152 : solo_slots(ctx, g));
+}
+
+// Draws [i0, i0+W) of (seed, qid): ws.win = draws[W] and, for the 64-lane
+// engine, grouped by source key, sorted sources[W] at WMAX and sorted draw
+// positions[W] at 2 WMAX (where a source has a CTA of its own, which sources
+// run together does not matter, and no key is built).
+static void draw_window(bc_ctx *ctx, const Graph &g, uint64_t seed, uint64_t qid, int64_t i0, int W) {
+  Workspace &ws = ctx->ws;
+  ws.win.ensure(WMAX_SOLO * 4);
+  static_assert(WMAX_SOLO >= 3 * WMAX, "the window buffer holds the draws and their sorted form");
+  int32_t *draws = ws.win.as<int32_t>();
+  launch_draw_sources(ctx, seed, qid, (uint64_t)i0, W, g.n, draws);
+  if (one_source_per_cta(ctx, g)) return;
+  const KeyMeta &km = key_meta(ctx, g, false);
+  LaunchScope ls(ctx, F_DRAW);
+  k_sort_window<<<1, 1024, 0, ctx->stream>>>(W, draws, km.key.as<uint8_t>(), draws + WMAX, draws + 2 * WMAX);
 }
 
 static void run_sources_per_cta(bc_ctx *ctx, const Graph &g, const int32_t *d_sources, int count, const Sink &sink) {
@@ -788,23 +810,47 @@ static void run_sources_per_cta(bc_ctx *ctx, const Graph &g, const int32_t *d_so
     lane_sink(ctx, g, d_sources, count, sink);
 }
 
+// Runs the window's sources: one launch where a source has a CTA, else batches
+// of the context's width (lane t of the batch starting at position b is the
+// window's sorted entry b + t).
 static void run_window(bc_ctx *ctx, const Graph &g, int W, Sink sink) {
   Workspace &ws = ctx->ws;
   const int width = batch_width(ctx);
-  const int32_t *sorted_src = ws.win.as<int32_t>() + WMAX;
-  const int32_t *sorted_pos = ws.win.as<int32_t>() + 2 * WMAX;
-  if (one_source_per_cta(ctx, g)) {
-    Sink sk = sink;
-    if (sk.tslot) sk.lane_col = sorted_pos;
-    run_sources_per_cta(ctx, g, sorted_src, W, sk);
+  if (one_source_per_cta(ctx, g)) {  // column = draw position
+    run_sources_per_cta(ctx, g, ws.win.as<int32_t>(), W, sink);
     return;
   }
+  const int32_t *sorted_src = ws.win.as<int32_t>() + WMAX;
+  const int32_t *sorted_pos = ws.win.as<int32_t>() + 2 * WMAX;
   for (int b = 0; b < W; b += width) {
     const int count = std::min(width, W - b);
     BCG_CUDA(cudaMemcpyAsync(ws.sources.p, sorted_src + b, (size_t)count * 4, cudaMemcpyDeviceToDevice, ctx->stream));
     Sink sk = sink;
     if (sk.tslot) sk.lane_col = sorted_pos + b;
     run_source_batch(ctx, g, count, sk);
+  }
+}
+
+// The exact all-vertex sums of draws [i0, i0 + count) of (seed, qid) into
+// sink.acc. One launch where the state fits shared memory (the draws are made
+// in the kernel), else window by window.
+static void run_draws(bc_ctx *ctx, const Graph &g, uint64_t seed, uint64_t qid, int64_t i0, int64_t count,
+                      const Sink &sink) {
+  const bool solo = batch_width(ctx) != 1 && !g.w && lane_major(ctx, g);
+  const int64_t most = solo ? (int64_t)1 << 30 : window_max(ctx, g, 0);
+  for (int64_t a = 0; a < count; a += most) {
+    const int W = (int)std::min<int64_t>(most, count - a);
+    if (solo) {
+      SoloSources src{};
+      src.base = (uint64_t)(i0 + a);
+      src.seed = seed;
+      src.qid = qid;
+      src.draw = 1;
+      solo_sources(ctx, g, src, W, sink, SoloRows{});
+    } else {
+      draw_window(ctx, g, seed, qid, i0 + a, W);
+      run_window(ctx, g, W, sink);
+    }
   }
 }
 
@@ -817,26 +863,23 @@ static void do_exact_or_uniform(bc_ctx *ctx, const Graph &g, bool exact, int64_t
   Sink sink;
   sink.acc = ws.acc.as<Acc>();
   const int width = batch_width(ctx);
-  KeyMeta &km = key_meta(ctx, g, exact);
-  if (exact && one_source_per_cta(ctx, g)) {
-    // all n sources, up to a window's worth per launch
-    for (int64_t i0 = 0; i0 < (int64_t)g.n; i0 += WMAX) {
-      const int count = (int)std::min<int64_t>(WMAX, (int64_t)g.n - i0);
-      run_sources_per_cta(ctx, g, km.order.as<int32_t>() + i0, count, sink);
-    }
-  } else if (exact) {
+  if (!exact) {
+    run_draws(ctx, g, seed, qid, 0, k, sink);
+  } else if (one_source_per_cta(ctx, g) && !g.w) {
+    solo_sources(ctx, g, SoloSources{}, g.n, sink, SoloRows{});  // every vertex once
+  } else {
     // all n sources, grouped by key (the sum over sources is exact, so any order)
-    for (int64_t i0 = 0; i0 < (int64_t)g.n; i0 += width) {
-      const int count = (int)std::min<int64_t>(width, (int64_t)g.n - i0);
+    const KeyMeta &km = key_meta(ctx, g, true);
+    const int step = g.w && width != 1 ? WMAX_SOLO : width;
+    for (int64_t i0 = 0; i0 < (int64_t)g.n; i0 += step) {
+      const int count = (int)std::min<int64_t>(step, (int64_t)g.n - i0);
+      if (step > 64) {
+        run_sources_per_cta(ctx, g, km.order.as<int32_t>() + i0, count, sink);
+        continue;
+      }
       BCG_CUDA(cudaMemcpyAsync(ws.sources.p, km.order.as<int32_t>() + i0, (size_t)count * 4,
                                cudaMemcpyDeviceToDevice, ctx->stream));
       run_source_batch(ctx, g, count, sink);
-    }
-  } else {
-    for (int64_t i0 = 0; i0 < k; i0 += WMAX) {
-      const int W = (int)std::min<int64_t>(WMAX, k - i0);
-      draw_window(ctx, g, km, seed, qid, i0, W);
-      run_window(ctx, g, W, sink);
     }
   }
   ws.misc2.ensure(n * 8);
@@ -852,7 +895,18 @@ static void do_exact_or_uniform(bc_ctx *ctx, const Graph &g, bool exact, int64_t
 // The depth that decides between the level-mask engine and one source per
 // persistent CTA: the largest finite distance from the hub (along out-edges on
 // a directed graph; the level-mask engine pulls counts over the in-neighbour CSR).
-int graph_depth_hint(bc_ctx *ctx, const Graph &g) { return key_meta(ctx, g, false).ecc; }
+// Small graphs get it from one CTA's BFS; the others with their source key.
+int graph_depth_hint(bc_ctx *ctx, const Graph &g) {
+  if (!solo_fits(ctx, g)) return key_meta(ctx, g, false).ecc;
+  {
+    std::lock_guard<std::mutex> lk(g_keys_mu);
+    const KeyMeta &km = g_keys[g.rp];
+    if (km.ecc >= 0) return km.ecc;
+  }
+  const int ecc = solo_depth(ctx, g, g.hub);
+  std::lock_guard<std::mutex> lk(g_keys_mu);
+  return g_keys[g.rp].ecc = ecc;
+}
 
 void uniform_one(bc_ctx *ctx, const Graph &g, int64_t k, uint64_t seed, uint64_t qid, double *out) {
   do_exact_or_uniform(ctx, g, false, k, seed, qid, out);
@@ -861,8 +915,8 @@ void uniform_one(bc_ctx *ctx, const Graph &g, int64_t k, uint64_t seed, uint64_t
 // Bader's loop over windows of draws: each window's draws run grouped by source
 // key, their target dependencies land in draw order, and the stop scan walks
 // the window in draw order. The window grows with the number of draws already
-// made (64 .. 1024), so draws past the last stop are at most about half of
-// those made.
+// made (window_first .. window_max), so draws past the last stop are at most
+// about half of those made beyond the first window.
 static void do_adaptive_sources(bc_ctx *ctx, const Graph &g, const int32_t *targets, int32_t T, double c,
                                 int64_t cap, uint64_t seed, uint64_t qid, double *est, int64_t *k, double *S,
                                 int32_t *status) {
@@ -870,7 +924,8 @@ static void do_adaptive_sources(bc_ctx *ctx, const Graph &g, const int32_t *targ
   const size_t n = (size_t)g.n;
   cudaStream_t st = ctx->stream;
   ws.tslot.ensure(n * 4);
-  ws.tdelta.ensure((size_t)std::max(T, 1) * WMAX * 8);
+  const int wmax = window_max(ctx, g, T);
+  ws.tdelta.ensure((size_t)std::max(T, 1) * wmax * 8);
   {
     LaunchScope ls(ctx, F_MISC);
     k_fill_i32<<<(unsigned)((n + 255) / 256), 256, 0, st>>>((int64_t)n, -1, ws.tslot.as<int32_t>());
@@ -882,13 +937,13 @@ static void do_adaptive_sources(bc_ctx *ctx, const Graph &g, const int32_t *targ
     k_set_slots<<<(T + 127) / 128, 128, 0, st>>>(T, d_targets, ws.tslot.as<int32_t>());
   }
   ScanState ss = make_scan(ctx, T);
-  KeyMeta &km = key_meta(ctx, g, false);
   const double cn = c * (double)g.n;
+  const int64_t first = window_first(ctx, g);
   int32_t remaining = T;
   for (int64_t i0 = 0; i0 < cap && remaining > 0;) {
-    const int64_t want = std::max<int64_t>(64, i0 / 2);
-    const int W = (int)std::min<int64_t>(std::min<int64_t>(WMAX, want), cap - i0);
-    draw_window(ctx, g, km, seed, qid, i0, W);
+    const int64_t want = std::max<int64_t>(first, i0 / 2);
+    const int W = (int)std::min<int64_t>(std::min<int64_t>(wmax, want), cap - i0);
+    draw_window(ctx, g, seed, qid, i0, W);
     BCG_CUDA(cudaMemsetAsync(ws.tdelta.p, 0, (size_t)T * W * 8, st));
     Sink sink;
     sink.tslot = ws.tslot.as<int32_t>();
@@ -917,7 +972,8 @@ static void do_target_block(bc_ctx *ctx, const Graph &g, const int32_t *targets,
   const size_t n = (size_t)g.n;
   cudaStream_t st = ctx->stream;
   ws.tslot.ensure(n * 4);
-  ws.tdelta.ensure((size_t)std::max(T, 1) * WMAX * 8);
+  const int wmax = window_max(ctx, g, T);
+  ws.tdelta.ensure((size_t)std::max(T, 1) * wmax * 8);
   {
     LaunchScope ls(ctx, F_MISC);
     k_fill_i32<<<(unsigned)((n + 255) / 256), 256, 0, st>>>((int64_t)n, -1, ws.tslot.as<int32_t>());
@@ -928,11 +984,10 @@ static void do_target_block(bc_ctx *ctx, const Graph &g, const int32_t *targets,
     LaunchScope ls(ctx, F_MISC);
     k_set_slots<<<(T + 127) / 128, 128, 0, st>>>(T, d_targets, ws.tslot.as<int32_t>());
   }
-  KeyMeta &km = key_meta(ctx, g, false);
-  std::vector<double> h((size_t)T * WMAX);
-  for (int64_t a = 0; a < count; a += WMAX) {
-    const int W = (int)std::min<int64_t>(WMAX, count - a);
-    draw_window(ctx, g, km, seed, qid, i0 + a, W);
+  std::vector<double> h((size_t)T * wmax);
+  for (int64_t a = 0; a < count; a += wmax) {
+    const int W = (int)std::min<int64_t>(wmax, count - a);
+    draw_window(ctx, g, seed, qid, i0 + a, W);
     BCG_CUDA(cudaMemsetAsync(ws.tdelta.p, 0, (size_t)T * W * 8, st));
     Sink sink;
     sink.tslot = ws.tslot.as<int32_t>();
@@ -960,12 +1015,7 @@ static void do_uniform_partial(bc_ctx *ctx, const Graph &g, uint64_t seed, uint6
   BCG_CUDA(cudaMemsetAsync(ws.acc.p, 0, n * sizeof(Acc), ctx->stream));
   Sink sink;
   sink.acc = ws.acc.as<Acc>();
-  KeyMeta &km = key_meta(ctx, g, false);
-  for (int64_t a = 0; a < count; a += WMAX) {
-    const int W = (int)std::min<int64_t>(WMAX, count - a);
-    draw_window(ctx, g, km, seed, qid, i0 + a, W);
-    run_window(ctx, g, W, sink);
-  }
+  run_draws(ctx, g, seed, qid, i0, count, sink);
   check_err_bits(ctx);
   std::vector<Acc> h(n);
   BCG_CUDA(cudaMemcpyAsync(h.data(), ws.acc.p, n * sizeof(Acc), cudaMemcpyDeviceToHost, ctx->stream));
@@ -985,8 +1035,8 @@ void target_bfs(bc_ctx *ctx, const Graph &g, const int32_t *d_targets, int T, in
   Workspace &ws = ctx->ws;
   const size_t n = (size_t)g.n;
   tx.assign((size_t)Tp, 0);
-  if (T > 0 && graph_depth_hint(ctx, g) > ctx->deep_levels) {
-    // deep graph: one lane-major BFS per target
+  if (T > 0 && lane_major(ctx, g)) {
+    // one BFS per CTA and target
     if (!texp.p) texp.ensure(n * (size_t)Tp * 4);
     DevBuf dtx;
     dtx.ensure((size_t)Tp * 4);
@@ -1035,7 +1085,7 @@ uint64_t pair_batch(bc_ctx *ctx, const Graph &g, int count) {
   uint64_t ovf;
   if (batch_width(ctx) == 1) {
     ovf = plain_pair(ctx, g, ws.sources.as<int32_t>(), ws.targets.as<int32_t>()) ? 1ull : 0ull;
-  } else if (graph_depth_hint(ctx, g) > ctx->deep_levels) {
+  } else if (lane_major(ctx, g)) {
     ovf = lane_pairs(ctx, g, count);
   } else {
     batch_forward(ctx, g, count, true, OVF_EXTEND);
@@ -1272,6 +1322,55 @@ static void do_source_rows_weighted(bc_ctx *ctx, const Graph &g, const int32_t *
   for (DevBuf *b : {&dd, &ddist, &dsig, &dsm, &dse, &dtier}) b->release();
 }
 
+// The per-source rows where a source has a CTA of its own: as many sources per
+// launch as 256 MB of rows hold (at least 64). The rows live in the context's
+// workspace (device allocations cost more than the step on a small graph).
+static void do_source_rows_solo(bc_ctx *ctx, const Graph &g, const int32_t *sources, int32_t count,
+                                double *delta_out, int32_t *dist_out, uint64_t *sigma_out, double *sm_out,
+                                int32_t *se_out, int32_t *tier_out) {
+  Workspace &ws = ctx->ws;
+  const size_t n = (size_t)g.n;
+  cudaStream_t st = ctx->stream;
+  for (int32_t i = 0; i < count; ++i)
+    if (sources[i] < 0 || sources[i] >= g.n) fail(BC_E_INVALID, "source out of range");
+  const bool xf = sm_out || se_out;
+  const size_t per = n * (8 + (sigma_out ? 8 : 0) + (xf ? 12 : 0) + (dist_out ? 4 : 0));
+  const int chunk = (int)std::min<size_t>((size_t)count, std::max<size_t>(64, ((size_t)256 << 20) / per));
+  if (chunk < 1) return;
+  ws.rows.ensure(per * chunk + 8 * (size_t)chunk);
+  unsigned char *p = ws.rows.as<unsigned char>();
+  auto carve = [&](bool want, size_t bytes) -> void * {
+    if (!want) return nullptr;
+    void *q = p;
+    p += bytes;
+    return q;
+  };
+  SoloRows r;
+  r.delta = static_cast<double *>(carve(true, n * chunk * 8));
+  r.sig = static_cast<uint64_t *>(carve(sigma_out != nullptr, n * chunk * 8));
+  r.sm = static_cast<double *>(carve(xf, n * chunk * 8));
+  r.se = static_cast<int32_t *>(carve(xf, n * chunk * 4));
+  r.dist = static_cast<int32_t *>(carve(dist_out != nullptr, n * chunk * 4));
+  r.tier = static_cast<int32_t *>(carve(true, (size_t)chunk * 4));
+  int32_t *d_src = static_cast<int32_t *>(carve(true, (size_t)chunk * 4));
+  for (int32_t i0 = 0; i0 < count; i0 += chunk) {
+    const int cnt = std::min<int>(chunk, count - i0);
+    const size_t at = (size_t)i0 * n, m = n * cnt;
+    BCG_CUDA(cudaMemcpyAsync(d_src, sources + i0, (size_t)cnt * 4, cudaMemcpyHostToDevice, st));
+    SoloSources src{};
+    src.list = d_src;
+    solo_sources(ctx, g, src, cnt, Sink{}, r);
+    sync(ctx);
+    BCG_CUDA(cudaMemcpy(delta_out + at, r.delta, m * 8, cudaMemcpyDeviceToHost));
+    if (dist_out) BCG_CUDA(cudaMemcpy(dist_out + at, r.dist, m * 4, cudaMemcpyDeviceToHost));
+    if (sigma_out) BCG_CUDA(cudaMemcpy(sigma_out + at, r.sig, m * 8, cudaMemcpyDeviceToHost));
+    if (sm_out) BCG_CUDA(cudaMemcpy(sm_out + at, r.sm, m * 8, cudaMemcpyDeviceToHost));
+    if (se_out) BCG_CUDA(cudaMemcpy(se_out + at, r.se, m * 4, cudaMemcpyDeviceToHost));
+    if (tier_out) BCG_CUDA(cudaMemcpy(tier_out + i0, r.tier, (size_t)cnt * 4, cudaMemcpyDeviceToHost));
+  }
+  check_err_bits(ctx);
+}
+
 static void do_source_dependencies(bc_ctx *ctx, const Graph &g, const int32_t *sources, int32_t count,
                                    double *delta_out, int32_t *dist_out, uint64_t *sigma_out, double *sm_out,
                                    int32_t *se_out, int32_t *tier_out) {
@@ -1279,6 +1378,10 @@ static void do_source_dependencies(bc_ctx *ctx, const Graph &g, const int32_t *s
     // lengths: int64 distances (bc_source_dependencies_weighted gives them)
     if (dist_out) fail(BC_E_INVALID, "a weighted graph's distances need bc_source_dependencies_weighted");
     do_source_rows_weighted(ctx, g, sources, count, delta_out, nullptr, sigma_out, sm_out, se_out, tier_out);
+    return;
+  }
+  if (batch_width(ctx) != 1 && solo_fits(ctx, g)) {
+    do_source_rows_solo(ctx, g, sources, count, delta_out, dist_out, sigma_out, sm_out, se_out, tier_out);
     return;
   }
   Workspace &ws = ctx->ws;
@@ -1600,6 +1703,12 @@ bc_status bc_create(bc_ctx **out, int device, const bc_options *opt) {
     if (const char *sl = std::getenv("BCG_SEGMENT")) ctx->seg_len = std::atoi(sl);
     if (const char *bv = std::getenv("BCG_BWD_VARIANT")) ctx->bwd_variant = std::atoi(bv);
     if (const char *dl = std::getenv("BCG_DEEP_LEVELS")) ctx->deep_levels = std::atoi(dl);
+    if (const char *sn = std::getenv("BCG_SOLO_N")) ctx->solo_n = std::atoi(sn);
+    if (const char *sz = std::getenv("BCG_SOLO_NNZ")) ctx->solo_nnz = std::atoll(sz);
+    if (const char *so = std::getenv("BCG_SOLO_THREADS")) {
+      const int t = std::atoi(so);
+      ctx->solo_threads = (t == 256 || t == 1024) ? t : 0;
+    }
     if (const char *pm = std::getenv("BCG_PK_MAXL")) ctx->pk_maxl = std::atoi(pm);
     if (const char *pc = std::getenv("BCG_PK_MINCNT")) ctx->pk_mincnt = std::atoi(pc);
     if (const char *hl = std::getenv("BCG_HEAVY_LANE")) ctx->heavy_lane = std::atoi(hl);
@@ -1665,7 +1774,7 @@ void bc_destroy(bc_ctx *ctx) {
                       &ws.pair_sig, &ws.pair_exp, &ws.err, &ws.cnt, &ws.acc, &ws.tslot, &ws.tdelta, &ws.scan, &ws.misc, &ws.misc2,
                       &ws.delta_lm, &ws.p_dist, &ws.p_sigma, &ws.p_coef, &ws.p_queue, &ws.p_ctr,
                       &ws.x_dist, &ws.x_m, &ws.x_e, &ws.x_vis, &ws.x_nm, &ws.x_list, &ws.x_lmask, &ws.x_ctr,
-                      &ws.x_off})
+                      &ws.x_off, &ws.rows, &ws.win})
       b->release();
     if (ws.pinned) cudaFreeHost(ws.pinned);
     for (cudaEvent_t e : ctx->event_pool) cudaEventDestroy(e);

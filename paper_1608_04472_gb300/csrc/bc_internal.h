@@ -133,6 +133,7 @@ struct Workspace {
   DevBuf misc2;
   DevBuf delta_lm; // [n][64] f64
   DevBuf win;      // draw window: draws[W] | sorted sources[W] | sorted positions[W]
+  DevBuf rows;     // per-source output rows of one launch (one source per CTA)
   uint64_t last_ovf = 0ull;  // lanes of the last batched forward whose counts exceeded 2^64-1
   std::vector<uint8_t> hlev;  // per level of the last batched forward: a heavy vertex has lanes there
   // extended-form engine (bc_ext.cu): dist [n][64] i32, sigma/coef as
@@ -198,6 +199,11 @@ struct bc_ctx {
   // multi-graph split: hub eccentricity above which a graph goes to the
   // persistent kernel, and its CTAs per SM while the batched engine runs beside
   int32_t deep_levels = 32, multi_cap = 4;
+  // graphs of at most solo_n vertices and solo_nnz entries whose state fits
+  // shared memory run one source per CTA at any depth (BCG_SOLO_N, 0: only deep
+  // graphs do; BCG_SOLO_NNZ); solo_threads forces the CTA size (0: by rule)
+  int32_t solo_n = 65536, solo_threads = 0;
+  int64_t solo_nnz = 1000000;
   // pair lanes of Algorithm 1: 0 = bidirectional search, one pair per CTA
   // (bc_bidir.cu); 2 = the same search one pair per warp with hash-table
   // balls, pairs with large balls handed to one pair per CTA (measured slower,
@@ -309,12 +315,41 @@ void plain_distances(bc_ctx *ctx, const Graph &g, const int32_t *d_src, int32_t 
 void run_source_batch(bc_ctx *ctx, const Graph &g, int count, const Sink &sink);
 inline bool batch_width_is_plain(bc_ctx *ctx) { return ctx->batch_width == 1; }
 
-// ---- many graphs in one persistent launch (bc_multi.cu) ----
+// ---- one source per persistent CTA (bc_solo.cuh, bc_multi.cu) ----
+// Source t of a call: list[t]; without a list draw base + t of (seed, qid)
+// (draw = 1) or vertex base + t.
+struct SoloSources {
+  const int32_t *list = nullptr;
+  uint64_t base = 0;
+  uint64_t seed = 0, qid = 0;
+  int draw = 0;
+};
+// Per-source rows [count][n] (device; any may be null, sm and se go together):
+// delta, distances (-1 unreachable), counts (UINT64_MAX at reached vertices of
+// an extended sample), counts as mantissa and exponent, tier[count].
+struct SoloRows {
+  double *delta = nullptr;
+  int32_t *dist = nullptr;
+  uint64_t *sig = nullptr;
+  double *sm = nullptr;
+  int32_t *se = nullptr;
+  int32_t *tier = nullptr;
+};
+// Whether the graph's sources run one per CTA because their state fits shared
+// memory (deep graphs do as well: one_source_per_cta), and how many run at once.
+bool solo_fits(bc_ctx *ctx, const Graph &g);
+int solo_slots(bc_ctx *ctx, const Graph &g);
+// The largest finite distance from v by one CTA (any graph without lengths).
+int solo_depth(bc_ctx *ctx, const Graph &g, int32_t v);
+// (lane_major: at any width but 1, weighted graphs apart.)
+bool lane_major(bc_ctx *ctx, const Graph &g);
+bool one_source_per_cta(bc_ctx *ctx, const Graph &g);
+void solo_sources(bc_ctx *ctx, const Graph &g, const SoloSources &src, int count, const Sink &sink,
+                  const SoloRows &rows);
 void do_uniform_multi(bc_ctx *ctx, const std::vector<bc_graph> &handles, const std::vector<const Graph *> &gs,
                       const int64_t *k, const uint64_t *seed, const uint64_t *qid, double *est_out);
 void forget_multi_plan(bc_ctx *ctx);
-// One batch of sources on a deep graph, lane-major (persistent CTAs, one lane
-// at a time each, CTA barriers between levels), delivering to the sink.
+// Sources from a list, delivering to the sink.
 void lane_sink(bc_ctx *ctx, const Graph &g, const int32_t *d_sources, int count, const Sink &sink);
 void forget_lane_scratch(bc_ctx *ctx);
 // Pair sampling on a deep graph, lane-major: the targets' full BFS into the

@@ -1,51 +1,27 @@
-// bc_multi.cu -- uniform k-source estimates (n/k times the summed dependencies
-// of k drawn sources, the per-sample step of Sec. 3 without the adaptive stop)
-// for many graphs of uneven size and depth in one persistent launch.
+// bc_multi.cu -- one source per persistent CTA: the kernels and host side of
+// the engine in bc_solo.cuh, and uniform k-source estimates (n/k times the
+// summed dependencies of k drawn sources, the per-sample step of Sec. 3 without
+// the adaptive stop) for many graphs of uneven size and depth in one call.
 //
-// Work items are (graph, run of draws). Persistent CTAs take items from one
-// atomic counter, in decreasing order of estimated cost, and run each source of
-// an item on their own: a level-synchronous BFS with a queue (distances by
-// compare-and-swap, then path counts pulled from the previous level), the
-// dependency recursion of Theorem 1 in decreasing distance, and the exact
-// per-vertex sum of the item's dependencies. Levels are separated by CTA
-// barriers, not kernel launches, so graphs hundreds of levels deep (grids) cost
-// no launch or host round trip per level. A second kernel adds the items'
-// exact partial sums per vertex and rounds once; the two launches are replayed
-// from a captured CUDA graph.
-//
-// bc_uniform_sources_multi splits the graphs by depth (the hub's eccentricity):
-// deep ones go to this persistent kernel on a second stream, sized to leave
-// room on every SM, while shallow ones run concurrently on the 64-lane batched
-// engine, which amortises its traversal over 64 sources and wins there.
+// CTAs take sources (or, for many graphs, items (graph, run of draws) in
+// decreasing order of estimated cost) from one atomic counter and run each on
+// their own; levels are separated by CTA barriers, not kernel launches, so a
+// small graph costs no launches and a deep one (a grid) no host round trip per
+// level. All-vertex sums go to exact per-CTA (per-item) partials that a second
+// kernel adds per vertex; for many graphs the launches are replayed from a
+// captured CUDA graph.
 //
 // Arithmetic per source is the library's: exact uint64 counts and exact
-// successor sums (order-free); a source whose counts exceed 2^64-1 has its
-// counts re-pulled and its dependencies computed in the extended form
-// (bc_xf.cuh; sums in CSR order of the vertex). Vertices of degree above 32 are
-// handled by a whole warp.
+// successor sums (order-free); a source whose counts exceed 2^64-1 continues
+// in the extended form (bc_xf.cuh; sums in CSR order of the vertex).
 #include <algorithm>
 #include <cstring>
 #include <vector>
 
 #include "bc_internal.h"
-#include "bc_xf.cuh"
+#include "bc_solo.cuh"
 
 namespace bcg {
-
-constexpr int MT = 256;  // threads per CTA
-constexpr int MWARPS = MT / 32;
-constexpr int MHEAVY = 32;  // vertices above this degree are processed by a whole warp
-
-struct MGraph {
-  const int32_t *rp;     // out-neighbours: discovery, successors in the backward pass
-  const int32_t *col;
-  const int32_t *rp_in;  // in-neighbours: predecessors whose counts are pulled
-  const int32_t *col_in; // (the same arrays as rp/col for an undirected graph)
-  int32_t n;
-  int32_t pad;
-  int64_t k;
-  uint64_t seed, qid;
-};
 
 struct MItem {
   int32_t g;
@@ -54,274 +30,59 @@ struct MItem {
   int64_t part;    // first Acc of the item's partial sums
 };
 
-// Per-CTA scratch, each array nmax (+2) long.
-struct MScratch {
-  int32_t *dist, *queue, *lo, *sige, *coefe;
-  uint64_t *sig;  // tier 0 counts; extended-form mantissas (double bits)
-  double *coef;   // tier 0 coefficients; extended-form mantissas
-};
+extern __shared__ uint4 solo_shared[];
 
-__host__ __device__ inline size_t mscratch_stride(int32_t nmax) {
-  const size_t ints = ((size_t)5 * nmax + 2) * 4;
-  return ((ints + 255) / 256) * 256 + (size_t)nmax * 16;
-}
-
-__device__ inline MScratch mscratch_of(unsigned char *base, int32_t nmax) {
-  MScratch s;
-  s.dist = reinterpret_cast<int32_t *>(base);
-  s.queue = s.dist + nmax;
-  s.lo = s.queue + nmax;
-  s.sige = s.lo + nmax + 2;
-  s.coefe = s.sige + nmax;
-  const size_t ints = ((size_t)5 * nmax + 2) * 4;
-  s.sig = reinterpret_cast<uint64_t *>(base + ((ints + 255) / 256) * 256);
-  s.coef = reinterpret_cast<double *>(s.sig + nmax);
-  return s;
-}
-
-__device__ __forceinline__ Xf xf_at(const MScratch &S, bool coefs, int32_t v) {
-  return coefs ? Xf{S.coef[v], S.coefe[v]} : Xf{__longlong_as_double((long long)S.sig[v]), S.sige[v]};
-}
-
-// Sum over the CSR neighbours u of v with dist[u] == want, in CSR order, of the
-// extended counts (coefs = false) or coefficients (coefs = true). `coop`: the
-// whole warp works on v (every lane returns the sum); otherwise one thread.
-__device__ Xf xf_pull(const MScratch &S, const int32_t *__restrict__ col, int beg, int end, int32_t want,
-                      bool coefs, bool coop) {
-  Xf acc{0.0, 0};
-  if (!coop) {
-    for (int j = beg; j < end; ++j) {
-      const int32_t u = col[j];
-      if (S.dist[u] == want) acc = xf_add(acc, xf_at(S, coefs, u));
-    }
-    return acc;
-  }
-  const int lane = threadIdx.x & 31;
-  for (int base = beg; base < end; base += 32) {
-    const int j = base + lane;
-    bool ok = false;
-    Xf x{0.0, 0};
-    if (j < end) {
-      const int32_t u = col[j];
-      ok = S.dist[u] == want;
-      if (ok) x = xf_at(S, coefs, u);
-    }
-    const unsigned bal = __ballot_sync(FULL, ok);
-    for (unsigned b = bal; b; b &= b - 1u) {  // CSR order: lowest position first
-      const int k = __ffs(b) - 1;
-      acc = xf_add(acc, Xf{__shfl_sync(FULL, x.m, k), __shfl_sync(FULL, x.e, k)});
-    }
-  }
-  return acc;
-}
-
-// Runs fn(v, beg, end, coop) for the queue entries [b, e): light vertices one
-// per thread, heavy ones (degree > MHEAVY) by the whole warp.
-template <class F>
-__device__ __forceinline__ void for_level(const MScratch &S, const int32_t *__restrict__ rp, int b, int e, F fn) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int cb = b + warp * 32; cb < e; cb += MWARPS * 32) {
-    const int idx = cb + lane;
-    int32_t v = -1;
-    int beg = 0, end = 0;
-    if (idx < e) {
-      v = S.queue[idx];
-      beg = rp[v];
-      end = rp[v + 1];
-    }
-    const bool heavy = v >= 0 && end - beg > MHEAVY;
-    if (v >= 0 && !heavy) fn(v, beg, end, false);
-    for (unsigned hb = __ballot_sync(FULL, heavy); hb; hb &= hb - 1u) {
-      const int k = __ffs(hb) - 1;
-      fn(__shfl_sync(FULL, v, k), __shfl_sync(FULL, beg, k), __shfl_sync(FULL, end, k), true);
-    }
-  }
-}
-
-// Forward pass of one source on the whole CTA: distances, exact counts and the
-// level offsets; with dest >= 0 it stops once dest's level is settled. Returns
-// the deepest settled level; *s_ovf says whether a count of those levels
-// exceeded 2^64-1.
-__device__ int lane_forward(const MGraph &G, int32_t s, int32_t dest, const MScratch &S, int *s_tail, int *s_ovf) {
-  const int tid = threadIdx.x, lane = tid & 31;
-  const int32_t *__restrict__ rp = G.rp;
-  const int32_t *__restrict__ col = G.col;
-  for (int32_t v = tid; v < G.n; v += MT) S.dist[v] = -1;
-  __syncthreads();
-  if (tid == 0) {
-    S.dist[s] = 0;
-    S.sig[s] = 1ull;
-    S.queue[0] = s;
-    S.lo[0] = 0;
-    S.lo[1] = 1;
-    *s_tail = 1;
-    *s_ovf = 0;
-  }
-  __syncthreads();
-  int L = 0;
-  for (;;) {
-    const int b = S.lo[L], e = S.lo[L + 1];
-    // discovery of level L+1
-    for_level(S, rp, b, e, [&](int32_t v, int beg, int end, bool coop) {
-      const int step = coop ? 32 : 1;
-      for (int j = beg + (coop ? lane : 0); j < end; j += step) {
-        const int32_t w = col[j];
-        if (S.dist[w] == -1 && atomicCAS(&S.dist[w], -1, L + 1) == -1) S.queue[atomicAdd(s_tail, 1)] = w;
-      }
-      (void)v;
-    });
-    __syncthreads();
-    const int nt = *s_tail;
-    if (nt == e) break;  // no vertex at distance L+1
-    if (tid == 0) S.lo[L + 2] = nt;
-    // exact counts of level L+1, pulled from the in-neighbours at level L
-    // (order-free integer sums)
-    for_level(S, G.rp_in, e, nt, [&](int32_t w, int beg, int end, bool coop) {
-      uint64_t sum = 0ull;
-      bool ov = false;
-      const int step = coop ? 32 : 1;
-      for (int j = beg + (coop ? lane : 0); j < end; j += step) {
-        const int32_t u = G.col_in[j];
-        if (S.dist[u] == L) {
-          const uint64_t t = sum + S.sig[u];
-          ov |= t < sum;
-          sum = t;
-        }
-      }
-      if (coop) {
-        for (int off = 16; off > 0; off >>= 1) {
-          const uint64_t o = __shfl_xor_sync(FULL, sum, off);
-          const uint64_t t = sum + o;
-          ov |= t < sum;
-          sum = t;
-        }
-        ov = __any_sync(FULL, ov);
-      }
-      if (!coop || lane == 0) {
-        S.sig[w] = sum;
-        if (ov) *s_ovf = 1;
-      }
-    });
-    __syncthreads();
-    ++L;
-    if (dest >= 0 && S.dist[dest] >= 0) break;  // dest settled at level L
-  }
-  return L;
-}
-
-// The counts of levels 1..L again, in the extended form (pull order over the
-// in-neighbours).
-__device__ void lane_extend(const MGraph &G, int32_t s, const MScratch &S, int L) {
-  const int tid = threadIdx.x, lane = tid & 31;
-  const int32_t *__restrict__ rp = G.rp_in;
-  const int32_t *__restrict__ col = G.col_in;
-  if (tid == 0) {
-    S.sig[s] = (uint64_t)__double_as_longlong(1.0);
-    S.sige[s] = 0;
-  }
-  __syncthreads();
-  for (int d = 1; d <= L; ++d) {
-    for_level(S, rp, S.lo[d], S.lo[d + 1], [&](int32_t w, int beg, int end, bool coop) {
-      const Xf x = xf_pull(S, col, beg, end, d - 1, false, coop);
-      if (!coop || lane == 0) {
-        S.sig[w] = (uint64_t)__double_as_longlong(x.m);
-        S.sige[w] = x.e;
-      }
-    });
-    __syncthreads();
-  }
-}
-
-// One source on the whole CTA; every dependency delta_s(v) (v at distance >= 1)
-// is handed to deliver(v, delta) by one thread.
-template <class D>
-__device__ void multi_source(const MGraph &G, int32_t s, const MScratch &S, unsigned &err, int *s_tail, int *s_ovf,
-                             D deliver) {
-  const int lane = threadIdx.x & 31;
-  const int32_t *__restrict__ rp = G.rp;
-  const int32_t *__restrict__ col = G.col;
-  const int L = lane_forward(G, s, -1, S, s_tail, s_ovf);
-  const bool ext = *s_ovf != 0;
-  if (ext) lane_extend(G, s, S, L);
-  // Theorem 1 in decreasing distance
-  for (int d = L; d >= 1; --d) {
-    for_level(S, rp, S.lo[d], S.lo[d + 1], [&](int32_t v, int beg, int end, bool coop) {
-      double delta;
-      if (ext) {
-        const Xf sum = xf_pull(S, col, beg, end, d + 1, true, coop);
-        const Xf sg{__longlong_as_double((long long)S.sig[v]), S.sige[v]};
-        delta = xf_mul_to_double(sg, sum);
-        if (!coop || lane == 0) {
-          const Xf cf = xf_div(__dadd_rn(1.0, delta), sg);
-          S.coef[v] = cf.m;
-          S.coefe[v] = cf.e;
-        }
-      } else {
-        Acc a = acc_zero();
-        const int step = coop ? 32 : 1;
-        for (int j = beg + (coop ? lane : 0); j < end; j += step) {
-          const int32_t w = col[j];
-          if (S.dist[w] == d + 1) acc_add(a, S.coef[w], err);
-        }
-        if (coop) a = acc_warp_sum(a);
-        const uint64_t sg = S.sig[v];
-        delta = delta_rn_fp(sg, acc_round(a));
-        if (!coop || lane == 0) S.coef[v] = coef_of_fp(delta, sg);
-      }
-      if (!coop || lane == 0) deliver(v, delta);
-    });
-    __syncthreads();
-  }
-}
-
-__global__ void __launch_bounds__(MT)
-k_multi(const MGraph *__restrict__ graphs, const MItem *__restrict__ items, int nitems, unsigned *__restrict__ next,
-        unsigned char *__restrict__ scratch, size_t stride, int32_t nmax, Acc *__restrict__ partials,
-        unsigned *__restrict__ err) {
-  __shared__ int s_item, s_tail, s_ovf;
-  const MScratch S = mscratch_of(scratch + (size_t)blockIdx.x * stride, nmax);
-  unsigned e = 0u;
-  for (;;) {
-    if (threadIdx.x == 0) s_item = (int)atomicAdd(next, 1u);
-    __syncthreads();
-    const int it = s_item;
-    if (it >= nitems) break;
-    const MItem item = items[it];
-    const MGraph G = graphs[item.g];
-    Acc *part = partials + item.part;
-    for (int32_t v = threadIdx.x; v < G.n; v += MT) part[v] = acc_zero();
-    for (int64_t i = item.i0; i < item.i1; ++i)
-      multi_source(G, draw_source(G.seed, G.qid, (uint64_t)i, G.n), S, e, &s_tail, &s_ovf,
-                   [&](int32_t v, double delta) {
-                     Acc cur = part[v];
-                     acc_add(cur, delta, e);
-                     part[v] = cur;
-                   });
-    __syncthreads();  // s_item is rewritten only after every thread has used it
-  }
-  if (e) atomicOr(err, e);
-}
-
-// The lanes of one batch (sources[t], t < count) of a deep graph, lane-major:
-// persistent CTAs take lanes one at a time and deliver each dependency to the
-// batch's sink as the 64-lane engine would (target entries, per-lane rows);
-// all-vertex sums go to per-CTA exact partials, added into sink.acc after.
-__global__ void __launch_bounds__(MT)
-k_lane_sink(MGraph G, const int32_t *__restrict__ sources, int count, unsigned *__restrict__ next,
-            unsigned char *__restrict__ scratch, size_t stride, int32_t nmax, Acc *__restrict__ partials, Sink sink,
-            unsigned *__restrict__ err) {
-  __shared__ int s_item, s_tail, s_ovf;
-  const MScratch S = mscratch_of(scratch + (size_t)blockIdx.x * stride, nmax);
+// Sources [0, count) delivered to the sink (lane t = source t; all-vertex sums
+// to per-CTA partials) and, where asked, to per-source rows.
+template <int TIER, int T>
+__global__ void __launch_bounds__(T, 1024 / T)
+k_solo(MGraph G, SoloSources src, int count, unsigned *__restrict__ next, unsigned char *__restrict__ scratch,
+       size_t stride, Acc *__restrict__ partials, Sink sink, SoloRows rows, unsigned *__restrict__ err) {
+  __shared__ SoloCtl c;
+  const SoloMem<TIER> S =
+      solo_mem<TIER>(reinterpret_cast<unsigned char *>(solo_shared), scratch + (size_t)blockIdx.x * stride, G.n, G.nnz);
   Acc *part = partials ? partials + (size_t)blockIdx.x * G.n : nullptr;
   if (part)
-    for (int32_t v = threadIdx.x; v < G.n; v += MT) part[v] = acc_zero();
+    for (int32_t v = threadIdx.x; v < G.n; v += T) part[v] = acc_zero();
+  if (threadIdx.x == 0) c.nhuge[0] = c.nhuge[1] = c.nhuge[2] = c.grab[0] = c.grab[1] = 0;
+  int ph = 0;
   unsigned e = 0u;
   for (;;) {
-    if (threadIdx.x == 0) s_item = (int)atomicAdd(next, 1u);
+    if (threadIdx.x == 0) c.item = (int)atomicAdd(next, 1u);
     __syncthreads();
-    const int t = s_item;
+    const int t = c.item;
     if (t >= count) break;
-    multi_source(G, sources[t], S, e, &s_tail, &s_ovf, [&](int32_t v, double delta) {
+    const uint64_t i = src.base + (uint64_t)t;
+    const int32_t s = src.list ? src.list[t] : (src.draw ? draw_source(src.seed, src.qid, i, G.n) : (int32_t)i);
+    bool ext;
+    uint64_t maxc;
+    const int L = solo_forward<TIER, T>(G, s, -1, S, c, ph, &ext, &maxc);
+    if (rows.dist || rows.sig || rows.sm || rows.tier) {
+      // before Theorem 1: coefficients take the counts' place
+      const size_t row = (size_t)t * G.n;
+      for (int32_t v = threadIdx.x; v < G.n; v += T) {
+        const bool r = S.dist[v] != solo_unset<TIER>();
+        if (rows.dist) rows.dist[row + v] = r ? (int32_t)S.dist[v] : -1;
+        if (rows.sig) rows.sig[row + v] = r ? (ext ? ~0ull : S.get(v)) : 0ull;
+        if (rows.sm) {
+          Xf x{0.0, 0};
+          if (r) x = ext ? solo_xf<TIER>(S, v) : xf_of_u64(S.get(v));
+          rows.sm[row + v] = x.m;
+          rows.se[row + v] = x.e;
+        }
+        if (rows.delta) rows.delta[row + v] = 0.0;
+      }
+      if (TIER == 1 && L >= 65535 && rows.dist) {  // codes wrapped: distances from the level offsets
+        __syncthreads();
+        for (int l = 65535; l <= L; ++l)
+          for (int q = solo_lo<TIER>(S, c, l) + (int)threadIdx.x; q < solo_lo<TIER>(S, c, l + 1); q += T)
+            rows.dist[row + S.queue[q]] = l;
+      }
+      if (rows.tier && threadIdx.x == 0) rows.tier[t] = ext ? 1 : 0;
+      __syncthreads();
+    }
+    solo_backward<TIER, T>(G, L, ext, maxc, S, c, ph, e, [&](int32_t v, double delta) {
+      if (rows.delta) rows.delta[(size_t)t * G.n + v] = delta;
       if (sink.delta_lm) sink.delta_lm[(size_t)v * 64 + t] = delta;
       if (sink.tslot) sink_targets(sink, v, t, delta);
       if (part) {
@@ -335,71 +96,137 @@ k_lane_sink(MGraph G, const int32_t *__restrict__ sources, int count, unsigned *
   if (e) atomicOr(err, e);
 }
 
-// Pair sampling on a deep graph, lane-major. Targets: the full BFS of each
-// target into the [n][Tp] tables (counts in the extended form, with tx[j] = 1,
-// when the BFS overflows). Pair lanes: the BFS from sources[t] until dests[t]'s
-// level; sigma_st in the extended form (bit t of *pxmask) when a count up to
-// that level overflowed.
-__global__ void __launch_bounds__(MT)
-k_lane_targets(MGraph G, const int32_t *__restrict__ targets, int T, int Tp, unsigned *__restrict__ next,
-               unsigned char *__restrict__ scratch, size_t stride, int32_t nmax, int32_t *__restrict__ tdist,
-               uint64_t *__restrict__ tsig, int32_t *__restrict__ texp, int32_t *__restrict__ tx) {
-  __shared__ int s_item, s_tail, s_ovf;
-  const MScratch S = mscratch_of(scratch + (size_t)blockIdx.x * stride, nmax);
+// Items of many graphs (all within the launch's nmax).
+template <int TIER, int T>
+__global__ void __launch_bounds__(T, 1024 / T)
+k_multi(const MGraph *__restrict__ graphs, const MItem *__restrict__ items, int nitems, unsigned *__restrict__ next,
+        unsigned char *__restrict__ scratch, size_t stride, Acc *__restrict__ partials, unsigned *__restrict__ err) {
+  __shared__ SoloCtl c;
+  unsigned e = 0u;
+  if (threadIdx.x == 0) c.nhuge[0] = c.nhuge[1] = c.nhuge[2] = c.grab[0] = c.grab[1] = 0;
+  int ph = 0;
   for (;;) {
-    if (threadIdx.x == 0) s_item = (int)atomicAdd(next, 1u);
+    if (threadIdx.x == 0) c.item = (int)atomicAdd(next, 1u);
     __syncthreads();
-    const int j = s_item;
-    if (j >= T) break;
-    const int L = lane_forward(G, targets[j], -1, S, &s_tail, &s_ovf);
-    const bool ext = s_ovf != 0;
-    if (ext) lane_extend(G, targets[j], S, L);
-    for (int32_t v = threadIdx.x; v < G.n; v += MT) {
+    const int it = c.item;
+    if (it >= nitems) break;
+    const MItem item = items[it];
+    const MGraph G = graphs[item.g];
+    const SoloMem<TIER> S =
+        solo_mem<TIER>(reinterpret_cast<unsigned char *>(solo_shared), scratch + (size_t)blockIdx.x * stride, G.n, G.nnz);
+    Acc *part = partials + item.part;
+    for (int32_t v = threadIdx.x; v < G.n; v += T) part[v] = acc_zero();
+    for (int64_t i = item.i0; i < item.i1; ++i) {
+      bool ext;
+      uint64_t maxc;
+      const int L = solo_forward<TIER, T>(G, draw_source(G.seed, G.qid, (uint64_t)i, G.n), -1, S, c, ph, &ext, &maxc);
+      solo_backward<TIER, T>(G, L, ext, maxc, S, c, ph, e, [&](int32_t v, double delta) {
+        Acc cur = part[v];
+        acc_add(cur, delta, e);
+        part[v] = cur;
+      });
+    }
+    __syncthreads();  // c.item is rewritten only after every thread has used it
+  }
+  if (e) atomicOr(err, e);
+}
+
+// Pair sampling on a deep graph. Targets: the full BFS of each target into the
+// [n][Tp] tables (counts in the extended form, with tx[j] = 1, when the BFS
+// overflows), or its depth alone. Pair lanes: the BFS from sources[t] until dests[t]'s level;
+// sigma_st in the extended form (bit t of *pxmask) when a count up to that
+// level overflowed.
+template <int TIER, int T>
+__global__ void __launch_bounds__(T, 1024 / T)
+k_solo_targets(MGraph G, const int32_t *__restrict__ targets, int count, int Tp, unsigned *__restrict__ next,
+               unsigned char *__restrict__ scratch, size_t stride, int32_t *__restrict__ tdist,
+               uint64_t *__restrict__ tsig, int32_t *__restrict__ texp, int32_t *__restrict__ tx,
+               int32_t *__restrict__ depth) {
+  __shared__ SoloCtl c;
+  const SoloMem<TIER> S =
+      solo_mem<TIER>(reinterpret_cast<unsigned char *>(solo_shared), scratch + (size_t)blockIdx.x * stride, G.n, G.nnz);
+  if (threadIdx.x == 0) c.nhuge[0] = c.nhuge[1] = c.nhuge[2] = c.grab[0] = c.grab[1] = 0;
+  int ph = 0;
+  for (;;) {
+    if (threadIdx.x == 0) c.item = (int)atomicAdd(next, 1u);
+    __syncthreads();
+    const int j = c.item;
+    if (j >= count) break;
+    bool ext;
+    uint64_t maxc;
+    const int L = solo_forward<TIER, T>(G, targets[j], -1, S, c, ph, &ext, &maxc);
+    if (depth) {  // only the depth is wanted
+      if (threadIdx.x == 0) depth[j] = L;
+      continue;
+    }
+    for (int32_t v = threadIdx.x; v < G.n; v += T) {
       const size_t o = (size_t)v * Tp + j;
-      const int32_t d = S.dist[v];
-      tdist[o] = d;
-      tsig[o] = d >= 0 ? S.sig[v] : 0ull;
-      texp[o] = (ext && d >= 0) ? S.sige[v] : 0;
+      const bool r = S.dist[v] != solo_unset<TIER>();
+      tdist[o] = r ? (int32_t)S.dist[v] : -1;
+      tsig[o] = r ? S.get(v) : 0ull;
+      texp[o] = (ext && r) ? S.exp[v] : 0;
+    }
+    if (TIER == 1 && L >= 65535) {
+      __syncthreads();
+      for (int l = 65535; l <= L; ++l)
+        for (int q = solo_lo<TIER>(S, c, l) + (int)threadIdx.x; q < solo_lo<TIER>(S, c, l + 1); q += T)
+          tdist[(size_t)S.queue[q] * Tp + j] = l;
     }
     if (threadIdx.x == 0) tx[j] = ext ? 1 : 0;
     __syncthreads();
   }
 }
 
-__global__ void __launch_bounds__(MT)
-k_lane_pairs(MGraph G, const int32_t *__restrict__ sources, const int32_t *__restrict__ dests, int count,
-             unsigned *__restrict__ next, unsigned char *__restrict__ scratch, size_t stride, int32_t nmax,
+template <int TIER, int T>
+__global__ void __launch_bounds__(T, 1024 / T)
+k_solo_pairs(MGraph G, const int32_t *__restrict__ sources, const int32_t *__restrict__ dests, int count,
+             unsigned *__restrict__ next, unsigned char *__restrict__ scratch, size_t stride,
              int32_t *__restrict__ pair_d, uint64_t *__restrict__ pair_sig, int32_t *__restrict__ pair_exp,
              unsigned long long *__restrict__ pxmask) {
-  __shared__ int s_item, s_tail, s_ovf;
-  const MScratch S = mscratch_of(scratch + (size_t)blockIdx.x * stride, nmax);
+  __shared__ SoloCtl c;
+  const SoloMem<TIER> S =
+      solo_mem<TIER>(reinterpret_cast<unsigned char *>(solo_shared), scratch + (size_t)blockIdx.x * stride, G.n, G.nnz);
+  if (threadIdx.x == 0) c.nhuge[0] = c.nhuge[1] = c.nhuge[2] = c.grab[0] = c.grab[1] = 0;
+  int ph = 0;
   for (;;) {
-    if (threadIdx.x == 0) s_item = (int)atomicAdd(next, 1u);
+    if (threadIdx.x == 0) c.item = (int)atomicAdd(next, 1u);
     __syncthreads();
-    const int t = s_item;
+    const int t = c.item;
     if (t >= count) break;
     const int32_t dst = dests[t];
-    const int L = lane_forward(G, sources[t], dst, S, &s_tail, &s_ovf);
-    const bool reached = S.dist[dst] >= 0;
-    const bool ext = reached && s_ovf != 0;
-    if (ext) lane_extend(G, sources[t], S, L);
+    bool ext;
+    uint64_t maxc;
+    const int L = solo_forward<TIER, T>(G, sources[t], dst, S, c, ph, &ext, &maxc);
     if (threadIdx.x == 0) {
-      pair_d[t] = reached ? S.dist[dst] : -1;
-      pair_sig[t] = reached ? S.sig[dst] : 0ull;
-      pair_exp[t] = ext ? S.sige[dst] : 0;
-      if (ext) atomicOr(pxmask, 1ull << t);
+      const bool reached = S.dist[dst] != solo_unset<TIER>();
+      pair_d[t] = reached ? L : -1;  // the search ends with dst's level
+      pair_sig[t] = reached ? S.get(dst) : 0ull;
+      pair_exp[t] = (reached && ext) ? S.exp[dst] : 0;
+      if (reached && ext) atomicOr(pxmask, 1ull << t);
     }
     __syncthreads();
   }
 }
 
-// sink.acc[v] += the CTAs' partial sums (exact).
-__global__ void k_lane_acc(int32_t n, int nparts, const Acc *__restrict__ partials, Acc *__restrict__ acc) {
-  const int32_t v = blockIdx.x * blockDim.x + threadIdx.x;
-  if (v >= n) return;
-  Acc a = acc[v];
-  for (int c = 0; c < nparts; ++c) acc_add_acc(a, partials[(size_t)c * n + v]);
-  acc[v] = a;
+// acc[v] += the CTAs' partial sums (exact): a block takes 32 vertices, its 32
+// warps a 32nd of the parts each (one thread per vertex over all parts left
+// small graphs with few threads in flight).
+__global__ void __launch_bounds__(1024) k_solo_acc(int32_t n, int nparts, const Acc *__restrict__ partials,
+                                                   Acc *__restrict__ acc) {
+  __shared__ Acc sh[32][33];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int32_t v = blockIdx.x * 32 + lane;
+  Acc a = acc_zero();
+  if (v < n)
+    for (int p = warp; p < nparts; p += 32) acc_add_acc(a, partials[(size_t)p * n + v]);
+  sh[warp][lane] = a;
+  __syncthreads();
+  a = acc_warp_sum(sh[lane][warp]);  // warp w: vertex w of the block
+  const int32_t vw = blockIdx.x * 32 + warp;
+  if (lane == 0 && vw < n) {
+    acc_add_acc(a, acc[vw]);
+    acc[vw] = a;
+  }
 }
 
 // est[off_g + v] = (n * RN(sum of the items' exact partial sums)) / k
@@ -412,26 +239,143 @@ __global__ void k_multi_reduce(const MGraph *__restrict__ graphs, const int32_t 
   const int32_t v = blockIdx.x * blockDim.x + threadIdx.x;
   if (v >= G.n) return;
   Acc a = acc_zero();
+#pragma unroll 4
   for (int q = gio[g]; q < gio[g + 1]; ++q) acc_add_acc(a, partials[items[gitems[q]].part + v]);
   est[est_off[g] + v] = __ddiv_rn(__dmul_rn((double)G.n, acc_round(a)), (double)G.k);
 }
 
 // ------------------------------------------------------------------ host --
 
+// Shared memory a CTA can have for its state beside SoloCtl.
+constexpr size_t SOLO_SMEM_MAX = (size_t)227 * 1024 - sizeof(SoloCtl) - 64;
+
+struct SoloCfg {
+  int tier = 2, threads = 256, ncta = 1;
+  size_t smem = 0, stride = 0;
+};
+
+// The state tier a graph's sources run in. Tier 1's distance codes need an
+// undirected graph or n <= 65535 (bc_solo.cuh).
+static int solo_tier(const Graph &g) {
+  if (solo_smem(0, g.n) <= SOLO_SMEM_MAX) return 0;
+  if (solo_smem(1, g.n) <= SOLO_SMEM_MAX && (!g.directed || g.n <= 65535)) return 1;
+  return 2;
+}
+
+// Shallow graphs run one source per CTA up to 65,536 vertices and a million
+// entries. One source per CTA reads every row once per source, the 64-lane
+// engine shares its reads among 64 sources, so density and size favour the
+// latter. us a source, 1024 uniform draws, here / 64-lane engine: ER n = 2000
+// deg 8 0.27 / 6.9, n = 18,000 2.2 / 9.4, n = 50,000 6.6 / 11.0, n = 100,000
+// 29 / 17 (152 CTAs' counts no longer fit L2); BA n = 50,000 7.1 / 24, n =
+// 110,000 34 / 27; R-MAT s14 (nnz 426k) 3.4 / 8.5, s15 (883k) 6.6 / 9.1, s16
+// with 955k entries 7.7 / 8.3, with 1.82M 12.6 / 12.0.
+bool solo_fits(bc_ctx *ctx, const Graph &g) {
+  return !g.w && g.n <= ctx->solo_n && g.nnz <= ctx->solo_nnz && solo_tier(g) < 2;
+}
+
+static int solo_sms() {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return std::max(1, sms);
+}
+
+// fn(tier, threads) as compile-time constants.
+template <int A, int B> struct SoloForm {
+  static constexpr int tier = A, threads = B;
+};
+template <class F> static auto solo_form(const SoloCfg &c, F fn) {
+  if (c.tier == 0) return c.threads == 1024 ? fn(SoloForm<0, 1024>{}) : fn(SoloForm<0, 256>{});
+  if (c.tier == 1) return c.threads == 1024 ? fn(SoloForm<1, 1024>{}) : fn(SoloForm<1, 256>{});
+  return fn(SoloForm<2, 256>{});
+}
+
+template <class K> static int solo_resident(K kern, const SoloCfg &c) {
+  int per = 0;
+  if (c.smem) BCG_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c.smem));
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, c.threads, c.smem) != cudaSuccess || per < 1) {
+    cudaGetLastError();
+    per = 1;
+  }
+  return per;
+}
+
+// Launch settings for `count` sources of graphs of up to n vertices. Deep
+// graphs take CTAs of 256 threads: their levels are narrow, so more CTAs per SM
+// beat more threads per level (200x200 grid 14.2 us a source, 21.8 with 1024).
+// Shallow ones do so while at least three fit an SM's shared memory (ER n =
+// 5000 0.60 us a source, 0.69 with 1024; n = 10,000 1.97 and 1.08; n = 50,000
+// 16.6 and 6.6), unless there are too few sources to fill the SMs with small
+// CTAs.
+static SoloCfg solo_cfg(bc_ctx *ctx, int tier, int32_t n, int64_t nnz, int64_t count, bool deep) {
+  SoloCfg c;
+  c.tier = tier;
+  c.smem = solo_smem(tier, n);
+  c.stride = solo_stride(tier, n, nnz);
+  if (tier < 2 && !deep) {
+    const size_t cta = c.smem + sizeof(SoloCtl) + 1024;
+    const bool few = count <= solo_sms() && n >= 4096;
+    c.threads = (tier == 0 && 3 * cta <= (size_t)228 * 1024 && !few) ? 256 : 1024;
+  }
+  if (tier < 2 && ctx->solo_threads) c.threads = ctx->solo_threads;
+  return c;
+}
+static SoloCfg solo_cfg(bc_ctx *ctx, const Graph &g, int64_t count) {
+  return solo_cfg(ctx, solo_tier(g), g.n, g.nnz, count, graph_depth_hint(ctx, g) > ctx->deep_levels);
+}
+
+// Resident CTAs over all SMs (at most `cap` per SM when cap > 0, at most
+// `count`), within the scratch budget at `per` bytes each.
+template <class K> static void solo_ctas(SoloCfg &c, K kern, int64_t count, size_t per, int cap) {
+  int r = solo_resident(kern, c);
+  if (cap > 0) r = std::min(r, cap);
+  int64_t m = std::min<int64_t>(count, (int64_t)solo_sms() * r);
+  if ((size_t)m * per > ((size_t)1 << 30)) m = std::min<int64_t>(m, (int64_t)(cta_scratch_budget() / per));
+  c.ncta = (int)std::max<int64_t>(1, m);
+}
+
+static MGraph mgraph_of(const Graph &g) {
+  MGraph G{};
+  G.rp = g.rp;
+  G.col = g.col;
+  G.rp_in = g.rp_in;
+  G.col_in = g.col_in;
+  G.n = g.n;
+  G.nnz = g.nnz;
+  return G;
+}
+
+// ---- many graphs ----
+
+struct MultiGroup {
+  SoloCfg cfg;
+  int item0 = 0, nitems = 0;
+  size_t scratch = 0;  // byte offset of the group's CTAs in the plan's scratch
+};
+
 struct MultiPlan {
   std::vector<bc_graph> handles;
   int cap_per_sm = 0;
   std::vector<int64_t> k;
   std::vector<uint64_t> seed, qid;
-  int ncta = 0, nitems = 0, G = 0;
+  int nitems = 0, G = 0;
   int32_t nmax = 0;
   int64_t total_n = 0;
+  std::vector<MultiGroup> groups;
+  std::vector<cudaStream_t> streams;  // one per group after the first (fork and join)
+  std::vector<cudaEvent_t> events;
   DevBuf d_graphs, d_items, d_gio, d_gitems, d_estoff, d_next, partials, scratch, est;
   cudaGraphExec_t exec = nullptr;
   void release() {
     if (exec) cudaGraphExecDestroy(exec);
     exec = nullptr;
     nitems = 0;
+    for (cudaEvent_t e : events) cudaEventDestroy(e);
+    for (cudaStream_t s : streams) cudaStreamDestroy(s);
+    events.clear();
+    streams.clear();
+    groups.clear();
     for (DevBuf *b : {&d_graphs, &d_items, &d_gio, &d_gitems, &d_estoff, &d_next, &partials, &scratch, &est})
       b->release();
   }
@@ -457,89 +401,110 @@ bool multi_plan_uses_graph(bc_ctx *ctx, bc_graph g) {
   return false;
 }
 
-// Resident CTAs: every slot the SMs have, or at most `cap_per_sm` per SM when
-// other kernels run beside it.
-static int multi_ctas(int cap_per_sm) {
-  int dev = 0, sms = 0, per = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_multi, MT, 0) != cudaSuccess || per < 1) {
-    cudaGetLastError();
-    per = 1;
-  }
-  if (cap_per_sm > 0) per = std::min(per, cap_per_sm);
-  return std::max(1, sms) * per;
-}
-
+// Groups run beside one another (a group's CTAs start as the one before it
+// leaves the SMs), each on its own branch of the captured graph.
 static void enqueue_multi(bc_ctx *ctx, MultiPlan &P) {
   cudaStream_t st = ctx->stream;
-  cudaMemsetAsync(P.d_next.p, 0, 16, st);
-  k_multi<<<P.ncta, MT, 0, st>>>(P.d_graphs.as<MGraph>(), P.d_items.as<MItem>(), P.nitems, P.d_next.as<unsigned>(),
-                                 P.scratch.as<unsigned char>(), mscratch_stride(P.nmax), P.nmax, P.partials.as<Acc>(),
-                                 ctx->ws.err.as<unsigned>());
+  cudaMemsetAsync(P.d_next.p, 0, 16 * P.groups.size(), st);
+  if (P.groups.size() > 1) cudaEventRecord(P.events[0], st);
+  for (size_t i = 0; i < P.groups.size(); ++i) {
+    const MultiGroup &m = P.groups[i];
+    cudaStream_t gs = i == 0 ? st : P.streams[i - 1];
+    if (i > 0) cudaStreamWaitEvent(gs, P.events[0], 0);
+    solo_form(m.cfg, [&](auto f) {
+      k_multi<decltype(f)::tier, decltype(f)::threads><<<m.cfg.ncta, m.cfg.threads, m.cfg.smem, gs>>>(
+          P.d_graphs.as<MGraph>(), P.d_items.as<MItem>() + m.item0, m.nitems, P.d_next.as<unsigned>() + 4 * i,
+          P.scratch.as<unsigned char>() + m.scratch, m.cfg.stride, P.partials.as<Acc>(), ctx->ws.err.as<unsigned>());
+      return 0;
+    });
+    if (i > 0) {
+      cudaEventRecord(P.events[i], gs);
+      cudaStreamWaitEvent(st, P.events[i], 0);
+    }
+  }
   k_multi_reduce<<<dim3((unsigned)((P.nmax + 255) / 256), (unsigned)P.G), 256, 0, st>>>(
       P.d_graphs.as<MGraph>(), P.d_gio.as<int32_t>(), P.d_gitems.as<int32_t>(), P.d_items.as<MItem>(),
       P.partials.as<Acc>(), P.d_estoff.as<int64_t>(), P.est.as<double>());
 }
 
 // Items: each graph's draws are cut into runs of about equal cost (cost of a
-// source ~ n + nnz), at least 4 runs per CTA overall; runs are queued largest
-// first so the persistent CTAs finish close together.
+// source ~ n + nnz), at least 4 runs per CTA overall. Graphs whose state has
+// the same tier and CTA size form a group with its own launch; a group's runs
+// are queued largest first so its CTAs finish close together.
 static void build_plan(bc_ctx *ctx, MultiPlan &P, const std::vector<const Graph *> &gs) {
   const int G = (int)gs.size();
   P.G = G;
-  P.ncta = multi_ctas(P.cap_per_sm);
-  double total = 0.0;
   P.nmax = 1;
   P.total_n = 0;
+  std::map<std::pair<int, int>, std::vector<int>> by;  // (tier, threads) -> graphs
   for (int g = 0; g < G; ++g) {
-    total += (double)P.k[g] * (double)(gs[g]->n + gs[g]->nnz);
+    const int tier = solo_tier(*gs[g]);
+    by[{tier, solo_cfg(ctx, *gs[g], (int64_t)1 << 30).threads}].push_back(g);
     P.nmax = std::max(P.nmax, gs[g]->n);
     P.total_n += gs[g]->n;
   }
-  const double target = std::max(1.0, total / (4.0 * P.ncta));
   std::vector<MItem> items;
-  std::vector<double> cost;
-  for (int g = 0; g < G; ++g) {
-    const double c = (double)(gs[g]->n + gs[g]->nnz);
-    const int64_t chunk = std::max<int64_t>(1, std::min<int64_t>(P.k[g], (int64_t)(target / c)));
-    for (int64_t i0 = 0; i0 < P.k[g]; i0 += chunk) {
-      MItem it{};
-      it.g = g;
-      it.i0 = i0;
-      it.i1 = std::min(P.k[g], i0 + chunk);
-      items.push_back(it);
-      cost.push_back(c * (double)(it.i1 - it.i0));
-    }
-  }
-  std::vector<int> order(items.size());
-  for (size_t i = 0; i < order.size(); ++i) order[i] = (int)i;
-  std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return cost[a] > cost[b]; });
-  std::vector<MItem> sorted(items.size());
   int64_t part = 0;
-  for (size_t i = 0; i < order.size(); ++i) {
-    sorted[i] = items[order[i]];
-    sorted[i].part = part;
-    part += gs[sorted[i].g]->n;
+  size_t scratch = 0;
+  for (auto it = by.rbegin(); it != by.rend(); ++it) {  // the largest state first
+    MultiGroup m;
+    int32_t nmax = 1;
+    int64_t zmax = 0;
+    double total = 0.0;
+    for (int g : it->second) {
+      nmax = std::max(nmax, gs[g]->n);
+      zmax = std::max(zmax, gs[g]->nnz);
+      total += (double)P.k[g] * (double)(gs[g]->n + gs[g]->nnz);
+    }
+    m.cfg = solo_cfg(ctx, it->first.first, nmax, zmax, (int64_t)1 << 30, false);
+    m.cfg.threads = it->first.second;
+    solo_form(m.cfg, [&](auto f) {
+      solo_ctas(m.cfg, k_multi<decltype(f)::tier, decltype(f)::threads>, (int64_t)1 << 30, m.cfg.stride, P.cap_per_sm);
+      return 0;
+    });
+    const double target = std::max(1.0, total / (4.0 * m.cfg.ncta));
+    std::vector<MItem> mine;
+    std::vector<double> cost;
+    for (int g : it->second) {
+      const double c = (double)(gs[g]->n + gs[g]->nnz);
+      const int64_t chunk = std::max<int64_t>(1, std::min<int64_t>(P.k[g], (int64_t)(target / c)));
+      for (int64_t i0 = 0; i0 < P.k[g]; i0 += chunk) {
+        MItem x{};
+        x.g = g;
+        x.i0 = i0;
+        x.i1 = std::min(P.k[g], i0 + chunk);
+        mine.push_back(x);
+        cost.push_back(c * (double)(x.i1 - x.i0));
+      }
+    }
+    std::vector<int> order(mine.size());
+    for (size_t i = 0; i < order.size(); ++i) order[i] = (int)i;
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return cost[a] > cost[b]; });
+    m.item0 = (int)items.size();
+    m.nitems = (int)mine.size();
+    for (int i : order) {
+      items.push_back(mine[i]);
+      items.back().part = part;
+      part += gs[mine[i].g]->n;
+    }
+    m.cfg.ncta = std::min(m.cfg.ncta, m.nitems);
+    m.scratch = scratch;
+    scratch += m.cfg.stride * (size_t)m.cfg.ncta;
+    P.groups.push_back(m);
   }
-  P.nitems = (int)sorted.size();
-  std::vector<int32_t> gio(G + 1, 0), gitems(sorted.size());
-  for (const MItem &it : sorted) gio[it.g + 1]++;
+  P.nitems = (int)items.size();
+  std::vector<int32_t> gio(G + 1, 0), gitems(items.size());
+  for (const MItem &it : items) gio[it.g + 1]++;
   for (int g = 0; g < G; ++g) gio[g + 1] += gio[g];
   {
     std::vector<int32_t> fill(gio.begin(), gio.end() - 1);
-    for (size_t i = 0; i < sorted.size(); ++i) gitems[fill[sorted[i].g]++] = (int32_t)i;
+    for (size_t i = 0; i < items.size(); ++i) gitems[fill[items[i].g]++] = (int32_t)i;
   }
   std::vector<MGraph> mg(G);
   std::vector<int64_t> estoff(G);
   int64_t off = 0;
   for (int g = 0; g < G; ++g) {
-    mg[g].rp = gs[g]->rp;
-    mg[g].col = gs[g]->col;
-    mg[g].rp_in = gs[g]->rp_in;
-    mg[g].col_in = gs[g]->col_in;
-    mg[g].n = gs[g]->n;
-    mg[g].pad = 0;
+    mg[g] = mgraph_of(*gs[g]);
     mg[g].k = P.k[g];
     mg[g].seed = P.seed[g];
     mg[g].qid = P.qid[g];
@@ -548,20 +513,24 @@ static void build_plan(bc_ctx *ctx, MultiPlan &P, const std::vector<const Graph 
   }
   cudaStream_t st = ctx->stream;
   P.d_graphs.ensure(sizeof(MGraph) * G);
-  P.d_items.ensure(sizeof(MItem) * sorted.size());
+  P.d_items.ensure(sizeof(MItem) * items.size());
   P.d_gio.ensure(4 * (G + 1));
-  P.d_gitems.ensure(4 * std::max<size_t>(1, sorted.size()));
+  P.d_gitems.ensure(4 * std::max<size_t>(1, items.size()));
   P.d_estoff.ensure(8 * G);
-  P.d_next.ensure(16);
+  P.d_next.ensure(16 * P.groups.size());
   P.partials.ensure(sizeof(Acc) * (size_t)std::max<int64_t>(1, part));
-  P.scratch.ensure(mscratch_stride(P.nmax) * (size_t)P.ncta);
+  P.scratch.ensure(std::max<size_t>(scratch, 16));
   P.est.ensure(8 * (size_t)P.total_n);
   BCG_CUDA(cudaMemcpyAsync(P.d_graphs.p, mg.data(), sizeof(MGraph) * G, cudaMemcpyHostToDevice, st));
-  BCG_CUDA(cudaMemcpyAsync(P.d_items.p, sorted.data(), sizeof(MItem) * sorted.size(), cudaMemcpyHostToDevice, st));
+  BCG_CUDA(cudaMemcpyAsync(P.d_items.p, items.data(), sizeof(MItem) * items.size(), cudaMemcpyHostToDevice, st));
   BCG_CUDA(cudaMemcpyAsync(P.d_gio.p, gio.data(), 4 * (G + 1), cudaMemcpyHostToDevice, st));
-  BCG_CUDA(cudaMemcpyAsync(P.d_gitems.p, gitems.data(), 4 * sorted.size(), cudaMemcpyHostToDevice, st));
+  BCG_CUDA(cudaMemcpyAsync(P.d_gitems.p, gitems.data(), 4 * items.size(), cudaMemcpyHostToDevice, st));
   BCG_CUDA(cudaMemcpyAsync(P.d_estoff.p, estoff.data(), 8 * G, cudaMemcpyHostToDevice, st));
   BCG_CUDA(cudaStreamSynchronize(st));
+  P.events.assign(P.groups.size(), nullptr);
+  P.streams.assign(P.groups.size() - 1, nullptr);
+  for (cudaEvent_t &e : P.events) BCG_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+  for (cudaStream_t &s : P.streams) BCG_CUDA(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
   // the per-call launch sequence, captured once and replayed (a stream that
   // cannot be captured, such as the legacy default stream, launches directly)
   cudaGraph_t graph = nullptr;
@@ -580,18 +549,17 @@ static void build_plan(bc_ctx *ctx, MultiPlan &P, const std::vector<const Graph 
   cuda_check(ie, "cudaGraphInstantiate");
 }
 
-static int lane_ctas(int count, size_t per) {
-  return std::max(1, std::min({count, multi_ctas(0), (int)std::max<size_t>(1, cta_scratch_budget() / per)}));
-}
+// ---- one graph ----
 
-// Per-context scratch of the lane-major path (grown on demand).
+// Per-context scratch (grown on demand).
 struct LaneScratch {
   DevBuf scratch, partials, next;
 };
 static std::map<bc_ctx *, LaneScratch> g_lane;
+static std::mutex g_lane_mu;  // apart from g_plans_mu: a plan being built asks for a graph's depth
 
 void forget_lane_scratch(bc_ctx *ctx) {
-  std::lock_guard<std::mutex> lk(g_plans_mu);
+  std::lock_guard<std::mutex> lk(g_lane_mu);
   auto it = g_lane.find(ctx);
   if (it == g_lane.end()) return;
   it->second.scratch.release();
@@ -600,86 +568,110 @@ void forget_lane_scratch(bc_ctx *ctx) {
   g_lane.erase(it);
 }
 
-void lane_sink(bc_ctx *ctx, const Graph &g, const int32_t *d_sources, int count, const Sink &sink) {
-  if (count < 1) return;
-  std::unique_lock<std::mutex> lk(g_plans_mu);
+static LaneScratch &lane_scratch(bc_ctx *ctx) {
+  std::lock_guard<std::mutex> lk(g_lane_mu);
   LaneScratch &L = g_lane[ctx];
-  lk.unlock();
-  const size_t stride = mscratch_stride(g.n);
-  const size_t per = stride + (sink.acc ? sizeof(Acc) * (size_t)g.n : 0);
-  const int ncta = lane_ctas(count, per);  // resident CTAs, at most one per lane
-  L.scratch.ensure(stride * ncta);
-  if (sink.acc) L.partials.ensure(sizeof(Acc) * (size_t)g.n * ncta);
   L.next.ensure(16);
+  BCG_CUDA(cudaMemsetAsync(L.next.p, 0, 16, ctx->stream));
+  return L;
+}
+
+int solo_slots(bc_ctx *ctx, const Graph &g) {
+  SoloCfg c = solo_cfg(ctx, g, (int64_t)1 << 30);
+  solo_form(c, [&](auto f) {
+    solo_ctas(c, k_solo<decltype(f)::tier, decltype(f)::threads>, (int64_t)1 << 30, c.stride, 0);
+    return 0;
+  });
+  return c.ncta;
+}
+
+void solo_sources(bc_ctx *ctx, const Graph &g, const SoloSources &src, int count, const Sink &sink,
+                  const SoloRows &rows) {
+  if (count < 1) return;
+  SoloCfg c = solo_cfg(ctx, g, count);  // (may run a BFS of its own: before the counter is cleared)
+  LaneScratch &L = lane_scratch(ctx);
+  const size_t per = c.stride + (sink.acc ? sizeof(Acc) * (size_t)g.n : 0);
   cudaStream_t st = ctx->stream;
-  BCG_CUDA(cudaMemsetAsync(L.next.p, 0, 16, st));
-  MGraph G{};
-  G.rp = g.rp;
-  G.col = g.col;
-  G.rp_in = g.rp_in;
-  G.col_in = g.col_in;
-  G.n = g.n;
-  {
+  solo_form(c, [&](auto f) {
+    auto kern = k_solo<decltype(f)::tier, decltype(f)::threads>;
+    solo_ctas(c, kern, count, per, 0);
+    L.scratch.ensure(c.stride * c.ncta);
+    if (sink.acc) L.partials.ensure(sizeof(Acc) * (size_t)g.n * c.ncta);
     LaunchScope ls(ctx, F_XFWD);
-    k_lane_sink<<<ncta, MT, 0, st>>>(G, d_sources, count, L.next.as<unsigned>(), L.scratch.as<unsigned char>(), stride,
-                                     g.n, sink.acc ? L.partials.as<Acc>() : nullptr, sink, ctx->ws.err.as<unsigned>());
-  }
+    kern<<<c.ncta, c.threads, c.smem, st>>>(mgraph_of(g), src, count, L.next.as<unsigned>(),
+                                            L.scratch.as<unsigned char>(), c.stride,
+                                            sink.acc ? L.partials.as<Acc>() : nullptr, sink, rows,
+                                            ctx->ws.err.as<unsigned>());
+    return 0;
+  });
   if (sink.acc) {
     LaunchScope ls(ctx, F_XBWD);
-    k_lane_acc<<<(g.n + 255) / 256, 256, 0, st>>>(g.n, ncta, L.partials.as<Acc>(), sink.acc);
+    k_solo_acc<<<(g.n + 31) / 32, 1024, 0, st>>>(g.n, c.ncta, L.partials.as<Acc>(), sink.acc);
   }
   ctx->samples += count;
   ctx->batches += 1;
 }
 
+void lane_sink(bc_ctx *ctx, const Graph &g, const int32_t *d_sources, int count, const Sink &sink) {
+  SoloSources src{};
+  src.list = d_sources;
+  solo_sources(ctx, g, src, count, sink, SoloRows{});
+}
+
+int solo_depth(bc_ctx *ctx, const Graph &g, int32_t v) {
+  LaneScratch &L = lane_scratch(ctx);
+  SoloCfg c = solo_cfg(ctx, solo_tier(g), g.n, g.nnz, 1, false);
+  cudaStream_t st = ctx->stream;
+  int32_t *word = L.next.as<int32_t>() + 2;  // the counter is word 0
+  BCG_CUDA(cudaMemcpyAsync(word, &v, 4, cudaMemcpyHostToDevice, st));
+  solo_form(c, [&](auto f) {
+    auto kern = k_solo_targets<decltype(f)::tier, decltype(f)::threads>;
+    solo_ctas(c, kern, 1, c.stride, 0);
+    L.scratch.ensure(c.stride * c.ncta);
+    LaunchScope ls(ctx, F_MISC);
+    kern<<<1, c.threads, c.smem, st>>>(mgraph_of(g), word, 1, 1, L.next.as<unsigned>(), L.scratch.as<unsigned char>(),
+                                       c.stride, nullptr, nullptr, nullptr, nullptr, word + 1);
+    return 0;
+  });
+  int32_t *h = static_cast<int32_t *>(ctx->ws.pinned);
+  BCG_CUDA(cudaMemcpyAsync(h, word + 1, 4, cudaMemcpyDeviceToHost, st));
+  BCG_CUDA(cudaStreamSynchronize(st));
+  return *h;
+}
+
 void lane_targets(bc_ctx *ctx, const Graph &g, const int32_t *d_targets, int T, int Tp, int32_t *tdist,
                   uint64_t *tsig, int32_t *texp, int32_t *d_tx) {
   if (T < 1) return;
-  std::unique_lock<std::mutex> lk(g_plans_mu);
-  LaneScratch &L = g_lane[ctx];
-  lk.unlock();
-  const size_t stride = mscratch_stride(g.n);
-  const int ncta = lane_ctas(T, stride);
-  L.scratch.ensure(stride * ncta);
-  L.next.ensure(16);
-  cudaStream_t st = ctx->stream;
-  BCG_CUDA(cudaMemsetAsync(L.next.p, 0, 16, st));
-  MGraph G{};
-  G.rp = g.rp;
-  G.col = g.col;
-  G.rp_in = g.rp_in;
-  G.col_in = g.col_in;
-  G.n = g.n;
-  LaunchScope ls(ctx, F_XFWD);
-  k_lane_targets<<<ncta, MT, 0, st>>>(G, d_targets, T, Tp, L.next.as<unsigned>(), L.scratch.as<unsigned char>(), stride,
-                                      g.n, tdist, tsig, texp, d_tx);
+  SoloCfg c = solo_cfg(ctx, g, T);
+  LaneScratch &L = lane_scratch(ctx);
+  solo_form(c, [&](auto f) {
+    auto kern = k_solo_targets<decltype(f)::tier, decltype(f)::threads>;
+    solo_ctas(c, kern, T, c.stride, 0);
+    L.scratch.ensure(c.stride * c.ncta);
+    LaunchScope ls(ctx, F_XFWD);
+    kern<<<c.ncta, c.threads, c.smem, ctx->stream>>>(mgraph_of(g), d_targets, T, Tp, L.next.as<unsigned>(),
+                                                     L.scratch.as<unsigned char>(), c.stride, tdist, tsig, texp, d_tx, nullptr);
+    return 0;
+  });
 }
 
 uint64_t lane_pairs(bc_ctx *ctx, const Graph &g, int count) {
   if (count < 1) return 0ull;
-  std::unique_lock<std::mutex> lk(g_plans_mu);
-  LaneScratch &L = g_lane[ctx];
-  lk.unlock();
+  SoloCfg c = solo_cfg(ctx, g, count);
+  LaneScratch &L = lane_scratch(ctx);
   Workspace &ws = ctx->ws;
-  const size_t stride = mscratch_stride(g.n);
-  const int ncta = lane_ctas(count, stride);
-  L.scratch.ensure(stride * ncta);
-  L.next.ensure(16);
   cudaStream_t st = ctx->stream;
-  BCG_CUDA(cudaMemsetAsync(L.next.p, 0, 16, st));
-  MGraph G{};
-  G.rp = g.rp;
-  G.col = g.col;
-  G.rp_in = g.rp_in;
-  G.col_in = g.col_in;
-  G.n = g.n;
-  {
+  solo_form(c, [&](auto f) {
+    auto kern = k_solo_pairs<decltype(f)::tier, decltype(f)::threads>;
+    solo_ctas(c, kern, count, c.stride, 0);
+    L.scratch.ensure(c.stride * c.ncta);
     LaunchScope ls(ctx, F_PAIR);
-    k_lane_pairs<<<ncta, MT, 0, st>>>(G, ws.sources.as<int32_t>(), ws.targets.as<int32_t>(), count,
-                                      L.next.as<unsigned>(), L.scratch.as<unsigned char>(), stride, g.n,
-                                      ws.pair_d.as<int32_t>(), ws.pair_sig.as<uint64_t>(), ws.pair_exp.as<int32_t>(),
-                                      L.next.as<unsigned long long>() + 1);
-  }
+    kern<<<c.ncta, c.threads, c.smem, st>>>(mgraph_of(g), ws.sources.as<int32_t>(), ws.targets.as<int32_t>(), count,
+                                            L.next.as<unsigned>(), L.scratch.as<unsigned char>(), c.stride,
+                                            ws.pair_d.as<int32_t>(), ws.pair_sig.as<uint64_t>(),
+                                            ws.pair_exp.as<int32_t>(), L.next.as<unsigned long long>() + 1);
+    return 0;
+  });
   uint64_t *h = static_cast<uint64_t *>(ws.pinned);
   BCG_CUDA(cudaMemcpyAsync(h, L.next.as<unsigned long long>() + 1, 8, cudaMemcpyDeviceToHost, st));
   BCG_CUDA(cudaStreamSynchronize(st));
@@ -694,9 +686,10 @@ void do_uniform_multi(bc_ctx *ctx, const std::vector<bc_graph> &handles, const s
   std::vector<int64_t> off(G + 1, 0);
   for (int g = 0; g < G; ++g) off[g + 1] = off[g] + gs[g]->n;
   std::vector<int> deep, shallow;
-  // weighted graphs run per graph (the weighted engine); the persistent kernel takes unit lengths only
+  // deep graphs and ones whose state fits shared memory go to the persistent
+  // kernels; weighted graphs run per graph (the weighted engine)
   for (int g = 0; g < G; ++g)
-    (!gs[g]->w && graph_depth_hint(ctx, *gs[g]) > ctx->deep_levels ? deep : shallow).push_back(g);
+    (one_source_per_cta(ctx, *gs[g]) && !gs[g]->w ? deep : shallow).push_back(g);
   std::lock_guard<std::mutex> lk(g_plans_mu);
   MultiPlan &P = g_plans[ctx];
   cudaEvent_t done = nullptr;
@@ -749,7 +742,7 @@ void do_uniform_multi(bc_ctx *ctx, const std::vector<bc_graph> &handles, const s
     }
     BCG_CUDA(cudaGetLastError());
     BCG_CUDA(cudaEventRecord(done, ctx->stream2));
-    ctx->launches += 2;
+    ctx->launches += (int64_t)P.groups.size() + 1;
     ctx->batches += P.nitems;
     for (int g : deep) ctx->samples += k[g];
   }

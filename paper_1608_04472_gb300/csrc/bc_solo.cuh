@@ -1,0 +1,776 @@
+// bc_solo.cuh -- the per-sample Brandes step with one source per CTA (device
+// side; kernels and host in bc_multi.cu). Sec. 3 steps 1-2 for one source s:
+// a queue BFS (levels contiguous in the queue) whose single pass over a
+// level's out-edges finds the next level, pushes the path counts along the
+// shortest-path edges (exact integer sums in any order) and keeps one bit per
+// edge, set where the edge is on a shortest path; then Theorem 1 over the levels
+// in decreasing distance, which visits only the edges with a bit set. Levels
+// are separated by CTA barriers.
+//
+// What bounds it: instruction issue (an edge visit costs a column read, a look
+// at the neighbour's distance and its share of finding the row it belongs to)
+// and, on deep graphs, the latency of a level's chain of dependent loads. Two
+// passes over all edges forward and one backward, a row per group of threads,
+// took 190 instructions per edge visit on ER n = 2000 (issue 56 %, 0.50 us a
+// source); hence the single flattened pass and the edge bits. The state tiers:
+//   tier 0  distances, queue and counts in shared memory, 12 B per vertex
+//           (n up to ~18,500);
+//   tier 1  distances (2 B) in shared memory, queue and counts in global
+//           memory, where 152 CTAs' arrays mostly fit L2 (n up to ~113,000);
+//   tier 2  everything in global memory (any n).
+// Where each is taken, with the times: solo_fits (bc_multi.cu).
+#pragma once
+
+#include <type_traits>
+
+#include "bc_internal.h"
+#include "bc_xf.cuh"
+
+namespace bcg {
+
+struct MGraph {
+  const int32_t *rp;     // out-neighbours
+  const int32_t *col;
+  const int32_t *rp_in;  // in-neighbours (the same arrays for an undirected graph): counts in
+  const int32_t *col_in; // the extended form are summed over them in CSR order
+  int32_t n;
+  int32_t pad;
+  int64_t nnz;
+  int64_t k;
+  uint64_t seed, qid;
+};
+
+constexpr int SOLO_NEAR = 512;  // level offsets kept in shared memory (the rest in global)
+constexpr int SOLO_HUGE = 64;   // rows taken by the whole CTA per pass (more fall back to a warp)
+constexpr int SOLO_HUGE_DEG = 2048;
+constexpr int SOLO_U = 4;       // 32-edge windows a warp has in flight at once
+
+struct SoloCtl {
+  int item, tail;
+  int nhuge[3];                 // longest rows found by pass ph in slot ph % 3
+  int ovf;                      // a count of the last level left 64 bits
+  int l53;                      // first level with a count of 2^53 or more
+  int grab[2];                  // next list position of the running and of the next pass
+  unsigned long long maxc;      // largest count
+  int huge[SOLO_HUGE];          // queue positions
+  int near[SOLO_NEAR];
+  unsigned long long red[32][3];
+  uint8_t own[32][32];          // per warp: the threads that hold non-empty short rows
+};
+
+// The state of one source. Distances are codes: the level (tier 2), or the
+// level mod 65535 in 16 bits with 65535 for "not reached". On an undirected
+// graph neighbours differ by at most one level, so the code tells levels
+// apart at any depth; a directed graph takes the 16-bit form only while
+// n <= 65535. Edge bits: qmask[i] for the row of queue entry i (up to 32
+// entries); a longer row's words start at lmask[beg / 16] (rows above 32
+// entries never share a word there: they advance beg / 16 by at least
+// ceil(length / 32)).
+template <int TIER> struct SoloMem {
+  using D = typename std::conditional<TIER == 2, int32_t, uint16_t>::type;
+  using Q = typename std::conditional<TIER == 0, uint16_t, int32_t>::type;
+  D *dist;
+  Q *queue;
+  uint64_t *val;       // tiers 1, 2: counts, then coefficients (double bits; mantissas in the extended form)
+  uint32_t *lo, *hi;   // tier 0: the same in halves (shared memory adds 32 bits at once)
+  int32_t *exp;        // exponents of the extended form
+  int32_t *far;        // level offsets beyond SOLO_NEAR
+  uint32_t *qmask, *lmask;
+  __device__ __forceinline__ uint64_t get(int32_t v) const {
+    if constexpr (TIER == 0) return ((uint64_t)hi[v] << 32) | lo[v];
+    else return val[v];
+  }
+  __device__ __forceinline__ void set(int32_t v, uint64_t x) const {
+    if constexpr (TIER == 0) {
+      lo[v] = (uint32_t)x;
+      hi[v] = (uint32_t)(x >> 32);
+    } else {
+      val[v] = x;
+    }
+  }
+  // Adds x to v's count; true when the sum left 64 bits.
+  __device__ __forceinline__ bool add(int32_t v, uint64_t x) const {
+    if constexpr (TIER == 0) {
+      const uint32_t xl = (uint32_t)x, old = atomicAdd(&lo[v], xl);
+      const uint32_t carry = old + xl < xl ? 1u : 0u, h = (uint32_t)(x >> 32) + carry;
+      bool ov = h < carry;
+      if (h) ov |= atomicAdd(&hi[v], h) + h < h;
+      return ov;
+    } else {
+      return atomicAdd(reinterpret_cast<unsigned long long *>(val) + v, (unsigned long long)x) + x < x;
+    }
+  }
+};
+
+__host__ __device__ inline size_t solo_al(size_t x) { return (x + 255) / 256 * 256; }
+
+// Shared and global bytes of one CTA's state.
+__host__ __device__ inline size_t solo_smem(int tier, int32_t n) {
+  const size_t d = ((size_t)n * 2 + 15) / 16 * 16, w = ((size_t)n * 4 + 15) / 16 * 16;
+  return tier == 0 ? 2 * d + 2 * w : (tier == 1 ? d : 0);
+}
+__host__ __device__ inline size_t solo_stride(int tier, int32_t n, int64_t nnz) {
+  const size_t a4 = solo_al((size_t)n * 4 + 8);
+  return 3 * a4 + solo_al((size_t)(nnz / 16 + 2) * 4) + (tier >= 1 ? a4 + solo_al((size_t)n * 8) : 0) +
+         (tier == 2 ? a4 : 0);
+}
+
+template <int TIER>
+__device__ __forceinline__ SoloMem<TIER> solo_mem(unsigned char *sm, unsigned char *gm, int32_t n, int64_t nnz) {
+  SoloMem<TIER> S{};
+  const size_t a4 = solo_al((size_t)n * 4 + 8);
+  const size_t d = ((size_t)n * 2 + 15) / 16 * 16, w = ((size_t)n * 4 + 15) / 16 * 16;
+  S.exp = reinterpret_cast<int32_t *>(gm);
+  S.far = reinterpret_cast<int32_t *>(gm + a4);
+  S.qmask = reinterpret_cast<uint32_t *>(gm + 2 * a4);
+  S.lmask = reinterpret_cast<uint32_t *>(gm + 3 * a4);
+  gm += 3 * a4 + solo_al((size_t)(nnz / 16 + 2) * 4);
+  if constexpr (TIER == 0) {
+    S.dist = reinterpret_cast<uint16_t *>(sm);
+    S.queue = reinterpret_cast<uint16_t *>(sm + d);
+    S.lo = reinterpret_cast<uint32_t *>(sm + 2 * d);
+    S.hi = reinterpret_cast<uint32_t *>(sm + 2 * d + w);
+  } else {
+    S.queue = reinterpret_cast<int32_t *>(gm);
+    S.val = reinterpret_cast<uint64_t *>(gm + a4);
+    if constexpr (TIER == 1) S.dist = reinterpret_cast<uint16_t *>(sm);
+    else S.dist = reinterpret_cast<int32_t *>(gm + a4 + solo_al((size_t)n * 8));
+  }
+  return S;
+}
+
+template <int TIER> __device__ __forceinline__ typename SoloMem<TIER>::D solo_code(int level) {
+  if constexpr (TIER == 2) return level;
+  else return (uint16_t)(level < 65535 ? level : level % 65535);
+}
+template <int TIER> __device__ __forceinline__ typename SoloMem<TIER>::D solo_unset() {
+  if constexpr (TIER == 2) return -1;
+  else return (uint16_t)0xFFFFu;
+}
+
+// First thread to give w its level wins. 16-bit codes: an AND of the code into
+// the word's half turns "not reached" (all ones) into the code and leaves the
+// same code unchanged; the other half is ANDed with ones.
+template <int TIER> __device__ __forceinline__ bool solo_claim(const SoloMem<TIER> &S, int32_t w, int level) {
+  if constexpr (TIER == 2) {
+    return atomicCAS(&S.dist[w], -1, level) == -1;
+  } else {
+    const int sh = (w & 1) << 4;
+    const uint32_t keep = ~(0xFFFFu << sh) | ((uint32_t)solo_code<TIER>(level) << sh);
+    const uint32_t old = atomicAnd(reinterpret_cast<uint32_t *>(S.dist) + (w >> 1), keep);
+    return ((old >> sh) & 0xFFFFu) == 0xFFFFu;
+  }
+}
+
+template <int TIER> __device__ __forceinline__ int solo_lo(const SoloMem<TIER> &S, const SoloCtl &c, int l) {
+  return l < SOLO_NEAR ? c.near[l] : S.far[l];
+}
+
+// A pass over list positions [b, e) in runs of 32 from a shared counter (uneven
+// rows spread over the warps). Returns the warp's next run or e. ph counts the
+// passes, the same in every thread. A pass clears the next one's counters: that
+// pass's list position was last used one pass ago, its count of longest rows
+// was last read two passes ago, each before the barrier that ended the pass
+// before this one.
+__device__ __forceinline__ void solo_begin(SoloCtl &c, int ph) {
+  if (threadIdx.x == 0) {
+    c.grab[(ph + 1) & 1] = 0;
+    c.nhuge[(ph + 1) % 3] = 0;
+  }
+}
+__device__ __forceinline__ int solo_next(SoloCtl &c, int b, int e, int ph) {
+  int k = 0;
+  if ((threadIdx.x & 31) == 0) k = atomicAdd(&c.grab[ph & 1], 32);
+  return min(e, b + __shfl_sync(FULL, k, 0));
+}
+
+// U edge visits per thread (w[u] < 0: none): finds the vertices not reached so
+// far (they join `level` and the queue), adds sv[u] to the count of every
+// endpoint at `level`, and returns the warp's shortest-path bits in bal[u].
+template <int TIER, int U, bool COUNT>
+__device__ __forceinline__ void solo_visit(const SoloMem<TIER> &S, SoloCtl &c, int level, const int32_t (&w)[U],
+                                           const uint64_t (&sv)[U], unsigned (&bal)[U], const int32_t *rp) {
+  const int lane = threadIdx.x & 31;
+  const unsigned lt = (1u << lane) - 1u;
+  const typename SoloMem<TIER>::D code = solo_code<TIER>(level);
+  bool won[U], dag[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const typename SoloMem<TIER>::D d = w[u] >= 0 ? S.dist[w[u]] : (typename SoloMem<TIER>::D)0;
+    won[u] = w[u] >= 0 && d == solo_unset<TIER>();
+    dag[u] = won[u] || (w[u] >= 0 && d == code);
+  }
+#pragma unroll
+  for (int u = 0; u < U; ++u)
+    if (won[u]) won[u] = solo_claim<TIER>(S, w[u], level);
+  int total = 0, at[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const unsigned m = __ballot_sync(FULL, won[u]);
+    at[u] = total + __popc(m & lt);
+    total += __popc(m);
+    bal[u] = __ballot_sync(FULL, dag[u]);
+  }
+  if (total) {  // one queue reservation for the warp's finds
+    int base = 0;
+    if (lane == 0) base = atomicAdd(&c.tail, total);
+    base = __shfl_sync(FULL, base, 0);
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (won[u]) {
+        S.queue[base + at[u]] = (typename SoloMem<TIER>::Q)w[u];
+        asm volatile("prefetch.global.L1 [%0];" ::"l"(rp + w[u]));  // the next pass reads its row bounds
+      }
+  }
+  if constexpr (COUNT) {
+    bool ov = false;
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (dag[u]) ov |= S.add(w[u], sv[u]);
+    if (ov) c.ovf = 1;
+  }
+}
+
+// One level of the forward pass: the out-edges of queue entries [b, e) (at
+// level - 1). Short rows (up to 32 entries) of a run of 32 entries are walked
+// as one list of edges, 32 to a window: the threads whose rows start in a
+// window mark their first positions, and a visit's row is the last mark at or
+// before it. Long rows go to the whole warp, the longest to the CTA.
+template <int TIER, int T, bool COUNT>
+__device__ __forceinline__ void solo_push(const MGraph &G, const SoloMem<TIER> &S, SoloCtl &c, int level, int b, int e,
+                                          int &ph, uint64_t &maxc) {
+  constexpr int U = SOLO_U;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned lt = (1u << lane) - 1u, le = lt | (1u << lane);
+  uint8_t *own = c.own[warp];
+  solo_begin(c, ph);
+  for (int cb = solo_next(c, b, e, ph); cb < e; cb = solo_next(c, b, e, ph)) {
+    const int idx = cb + lane;
+    int beg = 0, d = 0;
+    uint64_t sv = 0ull;
+    if (idx < e) {
+      const int32_t v = S.queue[idx];
+      beg = G.rp[v];
+      d = G.rp[v + 1] - beg;
+      if constexpr (COUNT) sv = S.get(v);
+    }
+    if constexpr (COUNT) maxc = sv > maxc ? sv : maxc;
+    const int ds = d <= 32 ? d : 0;
+    int incl = ds;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const int y = __shfl_up_sync(FULL, incl, off);
+      if (lane >= off) incl += y;
+    }
+    const int E = __shfl_sync(FULL, incl, 31), start = incl - ds, first = beg - start;
+    const unsigned rows = __ballot_sync(FULL, ds > 0);
+    if (ds > 0) own[__popc(rows & lt)] = (uint8_t)lane;
+    __syncwarp();
+    uint32_t mask = 0u;
+    int before = -1;  // index of the last row that starts before the window
+    for (int i0 = 0; i0 < E; i0 += 32 * U) {
+      int32_t w[U];
+      uint64_t svu[U];
+      unsigned bal[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int s = start - (i0 + 32 * u);
+        const unsigned f = __reduce_or_sync(FULL, (ds > 0 && (unsigned)s < 32u) ? 1u << s : 0u);
+        const int i = i0 + 32 * u + lane;
+        const int o = i < E ? (int)own[before + __popc(f & le)] : 0;
+        before += __popc(f);
+        const int j = i + __shfl_sync(FULL, first, o);
+        if constexpr (COUNT) svu[u] = __shfl_sync(FULL, sv, o);
+        w[u] = i < E ? G.col[j] : -1;
+      }
+      solo_visit<TIER, U, COUNT>(S, c, level, w, svu, bal, G.rp);
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int s = start - (i0 + 32 * u);
+        if (s >= 0 && s < 32) mask |= bal[u] >> s;
+        else if (s < 0 && s > -32) mask |= bal[u] << -s;
+      }
+    }
+    if (idx < e) S.qmask[idx] = ds == 32 ? mask : mask & ((1u << ds) - 1u);
+    __syncwarp();
+    for (unsigned bm = __ballot_sync(FULL, d > 32); bm; bm &= bm - 1u) {
+      const int k = __ffs(bm) - 1;
+      const int hb = __shfl_sync(FULL, beg, k), he = hb + __shfl_sync(FULL, d, k);
+      if (he - hb > SOLO_HUGE_DEG) {
+        int slot = 0;
+        if (lane == 0) {
+          slot = atomicAdd(&c.nhuge[ph % 3], 1);
+          if (slot < SOLO_HUGE) c.huge[slot] = cb + k;
+        }
+        if (__shfl_sync(FULL, slot, 0) < SOLO_HUGE) continue;
+      }
+      uint32_t *words = S.lmask + (hb >> 4);
+      uint64_t svu[U];
+      svu[0] = __shfl_sync(FULL, sv, k);
+#pragma unroll
+      for (int u = 1; u < U; ++u) svu[u] = svu[0];
+      for (int j0 = hb; j0 < he; j0 += 32 * U) {
+        int32_t w[U];
+        unsigned bal[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int j = j0 + 32 * u + lane;
+          w[u] = j < he ? G.col[j] : -1;
+        }
+        solo_visit<TIER, U, COUNT>(S, c, level, w, svu, bal, G.rp);
+        if (lane == 0) {
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            if (j0 + 32 * u < he) words[((j0 - hb) >> 5) + u] = bal[u];
+        }
+      }
+    }
+  }
+  __syncthreads();
+  const int nh = min(c.nhuge[ph % 3], SOLO_HUGE);
+  ++ph;
+  if (nh) {
+    for (int k = 0; k < nh; ++k) {
+      const int32_t v = S.queue[c.huge[k]];
+      const int hb = G.rp[v], he = G.rp[v + 1];
+      uint64_t svu[1] = {0ull};
+      if constexpr (COUNT) svu[0] = S.get(v);
+      for (int j0 = hb + warp * 32; j0 < he; j0 += T) {
+        int32_t w[1];
+        unsigned bal[1];
+        w[0] = j0 + lane < he ? G.col[j0 + lane] : -1;
+        solo_visit<TIER, 1, COUNT>(S, c, level, w, svu, bal, G.rp);
+        if (lane == 0) S.lmask[(hb >> 4) + ((j0 - hb) >> 5)] = bal[0];
+      }
+    }
+    __syncthreads();
+  }
+}
+
+// 96-bit exact sums of coefficients in units of 2^-unit. With unit = 52 +
+// ceil(log2 of the largest count) every coefficient RN((1 + delta) / sigma) is
+// a whole number of units (it is at least 2^-ceil(log2 sigma)), and a
+// successor sum is delta_v / sigma_v <= n up to rounding, so the sum stays
+// below 2^96 while unit + ceil(log2 n) + 1 <= 96; a value outside the window
+// sets ERR_RANGE. Three limbs and 64-bit shifts take about half the
+// instructions of the 192-bit window.
+struct Acc3 {
+  uint32_t l0, l1, l2;
+};
+__device__ __forceinline__ void acc3_add3(Acc3 &a, uint32_t t0, uint32_t t1, uint32_t t2) {
+  asm("add.cc.u32 %0, %0, %3;\n\t"
+      "addc.cc.u32 %1, %1, %4;\n\t"
+      "addc.u32 %2, %2, %5;"
+      : "+r"(a.l0), "+r"(a.l1), "+r"(a.l2)
+      : "r"(t0), "r"(t1), "r"(t2));
+}
+// bias = 1075 - unit
+__device__ __forceinline__ void acc3_add(Acc3 &a, uint64_t bits, int bias, unsigned &err) {
+  const uint32_t hi = (uint32_t)(bits >> 32);
+  const int sh = (int)(hi >> 20) - bias;
+  if ((unsigned)sh > 43u) err |= ERR_RANGE;
+  const uint64_t m = (bits & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull;
+  const uint64_t lo = m << (sh & 63);
+  const uint32_t up = (uint32_t)((m >> 1) >> (63 - (sh & 63)));
+  acc3_add3(a, (uint32_t)lo, (uint32_t)(lo >> 32), up);
+}
+// The same value in the 192-bit window (unit 2^-128); 52 <= unit <= 95.
+__device__ __forceinline__ Acc acc3_widen(const Acc3 &a, int unit) {
+  const uint64_t w0 = (uint64_t)a.l0 | ((uint64_t)a.l1 << 32), w1 = a.l2;
+  const int s = 128 - unit;  // 33..76
+  if (s >= 64) {
+    const int r = s - 64;
+    return Acc{0ull, w0 << r, r ? ((w0 >> (64 - r)) | (w1 << r)) : w1};
+  }
+  return Acc{w0 << s, (w0 >> (64 - s)) | (w1 << s), w1 >> (64 - s)};
+}
+
+// Theorem 1 for the vertices of one level (queue entries [b, e)): exact sums of
+// the coefficients over the shortest-path edges the forward pass kept, then
+// delta and the vertex's own coefficient in place of its count. deliver(v,
+// delta) gets every vertex once.
+template <bool NARROW> struct SoloAcc {
+  using A = typename std::conditional<NARROW, Acc3, Acc>::type;
+  static __device__ __forceinline__ A zero() {
+    if constexpr (NARROW) return Acc3{0u, 0u, 0u};
+    else return acc_zero();
+  }
+  static __device__ __forceinline__ void add(A &a, uint64_t bits, int bias, unsigned &err) {
+    if constexpr (NARROW) acc3_add(a, bits, bias, err);
+    else acc_add(a, __longlong_as_double((long long)bits), err);
+  }
+  static __device__ __forceinline__ A warp_sum(A a) {
+    if constexpr (NARROW) {
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1)
+        acc3_add3(a, __shfl_xor_sync(FULL, a.l0, off), __shfl_xor_sync(FULL, a.l1, off),
+                  __shfl_xor_sync(FULL, a.l2, off));
+      return a;
+    } else {
+      return acc_warp_sum(a);
+    }
+  }
+  static __device__ __forceinline__ double round(const A &a, int unit) {
+    if constexpr (NARROW) return acc_round(acc3_widen(a, unit));
+    else return acc_round(a);
+  }
+  static __device__ __forceinline__ void put(unsigned long long *p, const A &a) {
+    if constexpr (NARROW) {
+      p[0] = a.l0;
+      p[1] = a.l1;
+      p[2] = a.l2;
+    } else {
+      p[0] = a.w0;
+      p[1] = a.w1;
+      p[2] = a.w2;
+    }
+  }
+  static __device__ __forceinline__ A take(const unsigned long long *p) {
+    if constexpr (NARROW) return Acc3{(uint32_t)p[0], (uint32_t)p[1], (uint32_t)p[2]};
+    else return Acc{p[0], p[1], p[2]};
+  }
+};
+
+// Adds the successors of words first, first + step, ... of a long row.
+template <int TIER, bool NARROW>
+__device__ __forceinline__ void solo_long_sum(const MGraph &G, const SoloMem<TIER> &S, int hb, int he, int first,
+                                              int step, int bias, typename SoloAcc<NARROW>::A &a, unsigned &err) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t *words = S.lmask + (hb >> 4);
+  const int nw = (he - hb + 31) >> 5;
+  for (int q = first; q < nw; q += 4 * step) {
+    uint64_t x[4];
+    int32_t w[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int i = q + u * step;
+      w[u] = (i < nw && ((words[i] >> lane) & 1u)) ? G.col[hb + 32 * i + lane] : -1;
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) x[u] = w[u] >= 0 ? S.get(w[u]) : 0ull;  // (a coefficient is never 0)
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (x[u]) SoloAcc<NARROW>::add(a, x[u], bias, err);
+  }
+}
+
+template <int TIER, bool NARROW, class F>
+__device__ __forceinline__ void solo_finish(const SoloMem<TIER> &S, int32_t v, const typename SoloAcc<NARROW>::A &a,
+                                            int unit, F &deliver) {
+  const uint64_t sg = S.get(v);
+  const double delta = delta_rn_fp(sg, SoloAcc<NARROW>::round(a, unit));
+  S.set(v, (uint64_t)__double_as_longlong(coef_of_fp(delta, sg)));
+  deliver(v, delta);
+}
+
+template <int TIER, int T, bool NARROW, class F>
+__device__ __forceinline__ void solo_back(const MGraph &G, const SoloMem<TIER> &S, SoloCtl &c, int b, int e, int unit,
+                                          int &ph, unsigned &err, F &deliver) {
+  using A = SoloAcc<NARROW>;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int bias = 1075 - unit;
+  solo_begin(c, ph);
+  for (int cb = solo_next(c, b, e, ph); cb < e; cb = solo_next(c, b, e, ph)) {
+    const int idx = cb + lane;
+    int32_t v = -1;
+    int beg = 0, d = 0;
+    uint32_t mask = 0u;
+    if (idx < e) {
+      v = S.queue[idx];
+      mask = S.qmask[idx];
+      beg = G.rp[v];
+      d = G.rp[v + 1] - beg;
+    }
+    typename A::A a = A::zero();
+    while (mask) {  // up to four successors in flight per thread
+      int32_t w[4];
+      uint64_t x[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        w[u] = mask ? G.col[beg + __ffs(mask) - 1] : -1;
+        mask &= mask - 1u;
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) x[u] = w[u] >= 0 ? S.get(w[u]) : 0ull;
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (x[u]) A::add(a, x[u], bias, err);
+    }
+    __syncwarp();
+    for (unsigned bm = __ballot_sync(FULL, d > 32); bm; bm &= bm - 1u) {
+      const int k = __ffs(bm) - 1;
+      const int hb = __shfl_sync(FULL, beg, k), he = hb + __shfl_sync(FULL, d, k);
+      if (he - hb > SOLO_HUGE_DEG) {
+        int slot = 0;
+        if (lane == 0) {
+          slot = atomicAdd(&c.nhuge[ph % 3], 1);
+          if (slot < SOLO_HUGE) c.huge[slot] = cb + k;
+        }
+        if (__shfl_sync(FULL, slot, 0) < SOLO_HUGE) {
+          if (lane == k) v = -1;  // finished after the others
+          continue;
+        }
+      }
+      typename A::A x = A::zero();
+      solo_long_sum<TIER, NARROW>(G, S, hb, he, 0, 1, bias, x, err);
+      x = A::warp_sum(x);
+      if (lane == k) a = x;
+    }
+    if (v >= 0) solo_finish<TIER, NARROW>(S, v, a, unit, deliver);
+    __syncwarp();
+  }
+  __syncthreads();
+  const int nh = min(c.nhuge[ph % 3], SOLO_HUGE);
+  ++ph;
+  if (nh) {
+    for (int k = 0; k < nh; ++k) {
+      const int32_t v = S.queue[c.huge[k]];
+      typename A::A x = A::zero();
+      solo_long_sum<TIER, NARROW>(G, S, G.rp[v], G.rp[v + 1], warp, T / 32, bias, x, err);
+      x = A::warp_sum(x);
+      if (lane == 0) A::put(c.red[warp], x);
+      __syncthreads();
+      if (warp == 0) {
+        typename A::A y = A::zero();
+        if (lane < T / 32) y = A::take(c.red[lane]);
+        y = A::warp_sum(y);
+        if (lane == 0) solo_finish<TIER, NARROW>(S, v, y, unit, deliver);
+      }
+      __syncthreads();
+    }
+  }
+}
+
+// ---- extended form (counts beyond 2^64-1; sums in CSR order of the vertex) --
+
+template <int TIER> __device__ __forceinline__ Xf solo_xf(const SoloMem<TIER> &S, int32_t v) {
+  return Xf{__longlong_as_double((long long)S.get(v)), S.exp[v]};
+}
+template <int TIER> __device__ __forceinline__ void solo_xf_set(const SoloMem<TIER> &S, int32_t v, Xf x) {
+  S.set(v, (uint64_t)__double_as_longlong(x.m));
+  S.exp[v] = x.e;
+}
+
+// Adds the warp's values x (threads with ok) to acc in thread order.
+__device__ __forceinline__ void solo_xf_warp(Xf &acc, bool ok, Xf x) {
+  for (unsigned b = __ballot_sync(FULL, ok); b; b &= b - 1u) {
+    const int k = __ffs(b) - 1;
+    acc = xf_add(acc, Xf{__shfl_sync(FULL, x.m, k), __shfl_sync(FULL, x.e, k)});
+  }
+}
+
+// Extended counts of the vertices of level l (queue entries [b, e)), pulled
+// over the in-neighbours in CSR order: a vertex per thread, rows above 32
+// entries by the whole warp.
+template <int TIER, int T>
+__device__ __forceinline__ void solo_xf_level(const MGraph &G, const SoloMem<TIER> &S, int l, int b, int e) {
+  const typename SoloMem<TIER>::D prev = solo_code<TIER>(l - 1);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int cb = b + warp * 32; cb < e; cb += T) {
+    const int idx = cb + lane;
+    int32_t v = -1;
+    int beg = 0, d = 0;
+    if (idx < e) {
+      v = S.queue[idx];
+      beg = G.rp_in[v];
+      d = G.rp_in[v + 1] - beg;
+    }
+    Xf acc{0.0, 0};
+    const int ds = d <= 32 ? d : 0;
+    for (int j = 0; j < ds; j += 4) {
+      int32_t u[4];
+      Xf x[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) u[q] = j + q < ds ? G.col_in[beg + j + q] : -1;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) x[q] = (u[q] >= 0 && S.dist[u[q]] == prev) ? solo_xf<TIER>(S, u[q]) : Xf{0.0, 0};
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc = xf_add(acc, x[q]);
+    }
+    __syncwarp();
+    for (unsigned bm = __ballot_sync(FULL, d > 32); bm; bm &= bm - 1u) {
+      const int k = __ffs(bm) - 1;
+      const int hb = __shfl_sync(FULL, beg, k), he = hb + __shfl_sync(FULL, d, k);
+      Xf tot{0.0, 0};
+      for (int j0 = hb; j0 < he; j0 += 32) {
+        bool ok = false;
+        Xf x{0.0, 0};
+        if (j0 + lane < he) {
+          const int32_t u = G.col_in[j0 + lane];
+          ok = S.dist[u] == prev;
+          if (ok) x = solo_xf<TIER>(S, u);
+        }
+        solo_xf_warp(tot, ok, x);
+      }
+      if (lane == k) acc = tot;
+    }
+    if (v >= 0) solo_xf_set<TIER>(S, v, acc);
+  }
+}
+
+// Theorem 1 for one level in the extended form (successors in CSR order).
+template <int TIER, int T, class F>
+__device__ __forceinline__ void solo_xf_back(const MGraph &G, const SoloMem<TIER> &S, int b, int e, F &deliver) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int cb = b + warp * 32; cb < e; cb += T) {
+    const int idx = cb + lane;
+    int32_t v = -1;
+    int beg = 0, d = 0;
+    uint32_t mask = 0u;
+    if (idx < e) {
+      v = S.queue[idx];
+      mask = S.qmask[idx];
+      beg = G.rp[v];
+      d = G.rp[v + 1] - beg;
+    }
+    Xf acc{0.0, 0};
+    while (mask) {
+      int32_t w[2];
+      Xf x[2];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        w[u] = mask ? G.col[beg + __ffs(mask) - 1] : -1;
+        mask &= mask - 1u;
+      }
+#pragma unroll
+      for (int u = 0; u < 2; ++u) x[u] = w[u] >= 0 ? solo_xf<TIER>(S, w[u]) : Xf{0.0, 0};
+      acc = xf_add(xf_add(acc, x[0]), x[1]);
+    }
+    __syncwarp();
+    for (unsigned bm = __ballot_sync(FULL, d > 32); bm; bm &= bm - 1u) {
+      const int k = __ffs(bm) - 1;
+      const int hb = __shfl_sync(FULL, beg, k), he = hb + __shfl_sync(FULL, d, k);
+      const uint32_t *words = S.lmask + (hb >> 4);
+      Xf tot{0.0, 0};
+      for (int q = 0; hb + 32 * q < he; ++q) {
+        const bool ok = (words[q] >> lane) & 1u;
+        solo_xf_warp(tot, ok, ok ? solo_xf<TIER>(S, G.col[hb + 32 * q + lane]) : Xf{0.0, 0});
+      }
+      if (lane == k) acc = tot;
+    }
+    if (v >= 0) {
+      const Xf sg = solo_xf<TIER>(S, v);
+      const double delta = xf_mul_to_double(sg, acc);
+      solo_xf_set<TIER>(S, v, xf_div(__dadd_rn(1.0, delta), sg));
+      deliver(v, delta);
+    }
+  }
+}
+
+// Forward pass of source s: distance codes, counts, level offsets and edge
+// bits; with dest >= 0 it stops once dest's level is settled. Returns the
+// deepest level; *ext: the counts are in the extended form (a count of the
+// settled levels exceeded 2^64-1); *maxc: the largest count of the levels
+// above the deepest and of the deepest too unless dest stopped the search
+// (when not extended).
+// Counts below 2^53 are exact in both forms, so a sample that overflows at
+// level L is converted, not recomputed, up to its first level with a count of
+// 2^53 or more, and goes on in the extended form from there.
+template <int TIER, int T>
+__device__ int solo_forward(const MGraph &G, int32_t s, int32_t dest, const SoloMem<TIER> &S, SoloCtl &c, int &ph,
+                            bool *ext, uint64_t *maxc) {
+  const int tid = threadIdx.x;
+  if constexpr (TIER == 2) {
+    for (int32_t v = tid; v < G.n; v += T) S.dist[v] = -1;
+  } else {
+    uint4 *d = reinterpret_cast<uint4 *>(S.dist);
+    const int words = (int)(((size_t)G.n * 2 + 15) / 16);
+    for (int i = tid; i < words; i += T) d[i] = make_uint4(~0u, ~0u, ~0u, ~0u);
+  }
+  if constexpr (TIER == 0) {
+    for (int32_t v = tid; v < G.n; v += T) S.lo[v] = S.hi[v] = 0u;
+  } else {
+    for (int32_t v = tid; v < G.n; v += T) S.val[v] = 0ull;
+  }
+  __syncthreads();
+  if (tid == 0) {
+    S.dist[s] = 0;
+    S.set(s, 1ull);
+    S.queue[0] = (typename SoloMem<TIER>::Q)s;
+    c.tail = 1;
+    c.near[0] = 0;
+    c.near[1] = 1;
+    c.ovf = 0;
+    c.l53 = 0x7FFFFFFF;
+    c.maxc = 1ull;
+  }
+  __syncthreads();
+  int L = 0, b = 0, e = 1;
+  bool xf = false;
+  uint64_t mymax = 1ull;
+  for (;;) {
+    if (xf) {
+      uint64_t none = 0ull;
+      solo_push<TIER, T, false>(G, S, c, L + 1, b, e, ph, none);
+    } else {
+      uint64_t lmax = 0ull;
+      solo_push<TIER, T, true>(G, S, c, L + 1, b, e, ph, lmax);
+      if (lmax >= (1ull << 53)) atomicMin(&c.l53, L);
+      mymax = lmax > mymax ? lmax : mymax;
+    }
+    const int nt = c.tail;
+    if (nt == e) break;  // no vertex at distance L + 1
+    if (xf) solo_xf_level<TIER, T>(G, S, L + 1, e, nt);
+    if (tid == 0) {
+      if (L + 2 < SOLO_NEAR) c.near[L + 2] = nt;
+      else S.far[L + 2] = nt;
+    }
+    __syncthreads();
+    ++L;
+    b = e;
+    e = nt;
+    if (!xf && c.ovf) {
+      // to the extended form: convert the exact levels, pull the rest
+      const int l53 = min(c.l53, L);
+      const int conv = solo_lo<TIER>(S, c, l53);
+      for (int i = tid; i < conv; i += T) {
+        const int32_t v = S.queue[i];
+        solo_xf_set<TIER>(S, v, xf_of_u64(S.get(v)));
+      }
+      __syncthreads();
+      for (int l = l53; l <= L; ++l) {
+        solo_xf_level<TIER, T>(G, S, l, solo_lo<TIER>(S, c, l), solo_lo<TIER>(S, c, l + 1));
+        __syncthreads();
+      }
+      xf = true;
+    }
+    if (dest >= 0 && S.dist[dest] != solo_unset<TIER>()) break;  // dest settled at level L
+  }
+  if (!xf) {
+    for (int off = 16; off > 0; off >>= 1) {
+      const uint64_t o = __shfl_xor_sync(FULL, mymax, off);
+      mymax = o > mymax ? o : mymax;
+    }
+    if ((tid & 31) == 0 && mymax > 1ull) atomicMax(&c.maxc, (unsigned long long)mymax);
+  }
+  __syncthreads();
+  *ext = xf;
+  *maxc = c.maxc;
+  return L;
+}
+
+// Theorem 1 for levels L..1 after solo_forward; deliver(v, delta) is called by
+// one thread for every vertex at distance >= 1.
+template <int TIER, int T, class F>
+__device__ __forceinline__ void solo_backward(const MGraph &G, int L, bool ext, uint64_t maxc, const SoloMem<TIER> &S,
+                                              SoloCtl &c, int &ph, unsigned &err, F deliver) {
+  if (ext) {
+    for (int l = L; l >= 1; --l) {
+      solo_xf_back<TIER, T>(G, S, solo_lo<TIER>(S, c, l), solo_lo<TIER>(S, c, l + 1), deliver);
+      __syncthreads();
+    }
+    return;
+  }
+  // ceil(log2) of the largest count and of n
+  const int unit = 52 + (maxc <= 1ull ? 0 : 64 - __clzll((long long)(maxc - 1ull)));
+  const int nlog = G.n <= 1 ? 0 : 32 - __clz(G.n - 1);
+  if (unit + nlog + 1 <= 96) {
+    for (int l = L; l >= 1; --l)
+      solo_back<TIER, T, true>(G, S, c, solo_lo<TIER>(S, c, l), solo_lo<TIER>(S, c, l + 1), unit, ph, err, deliver);
+  } else {
+    for (int l = L; l >= 1; --l)
+      solo_back<TIER, T, false>(G, S, c, solo_lo<TIER>(S, c, l), solo_lo<TIER>(S, c, l + 1), unit, ph, err, deliver);
+  }
+}
+
+}  // namespace bcg

@@ -1,0 +1,101 @@
+"""One source per CTA (csrc/bc_solo.cuh): the sizes where its tiles, tiers and
+tables end. Every sum is exact, so results equal the oracle's, and on graphs too
+large for it the 64-lane engine's, bit for bit."""
+import os
+
+import numpy as np
+import pytest
+
+import graphgen as gg
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+
+def _ctx(solo_n=None):
+    import paper_1608_04472_gb300 as pkg
+    old = os.environ.pop("BCG_SOLO_N", None)
+    try:
+        if solo_n is not None:
+            os.environ["BCG_SOLO_N"] = str(solo_n)
+        return pkg.Context(0, batch_width=64)
+    finally:
+        os.environ.pop("BCG_SOLO_N", None)
+        if old is not None:
+            os.environ["BCG_SOLO_N"] = old
+
+
+def _regular(n, d):
+    """Circulant graph: every row has exactly d entries (d even)."""
+    i = np.arange(n, dtype=np.int64)
+    eu = np.concatenate([i] * (d // 2))
+    ev = np.concatenate([(i + k) % n for k in range(1, d // 2 + 1)])
+    return gg.from_edges(n, eu, ev)
+
+
+def _bipartite(a, b):
+    u, v = np.divmod(np.arange(a * b, dtype=np.int64), b)
+    return gg.from_edges(a + b, u, a + v)
+
+
+SMALL = {
+    "one vertex": lambda: gg.from_edges(1, [], []),
+    "two vertices": lambda: gg.from_edges(2, [0], [1]),
+    "no edges": lambda: gg.from_edges(70, [], []),
+    "rows of 32": lambda: _regular(203, 32),
+    "rows of 34": lambda: _regular(203, 34),
+    "rows of 2 to 33": lambda: gg.erdos_renyi(333, 17, 5),
+    "star, row above 2048": lambda: _bipartite(1, 2500),
+    "70 rows of 2100": lambda: _bipartite(70, 2100),   # more longest rows than the CTA's list holds
+    "levels beyond the shared table": lambda: gg.from_edges(600, np.arange(599), np.arange(1, 600)),
+    "counts beyond 2^64": lambda: gg.grid(38),
+    "hubs and isolated vertices": lambda: gg.rmat(11, 8, 0.57, 0.19, 0.19, 7),
+}
+
+
+@pytest.mark.parametrize("name", list(SMALL))
+def test_small_graphs_equal_the_oracle(name):
+    g = SMALL[name]()
+    src = sorted({0, g.n // 2, g.n - 1})
+    with _ctx() as ctx:
+        h = ctx.load_graph(g.row_ptr, g.col)
+        delta, dist, sm, se, tier = ctx.source_dependencies_ext(h, src)
+        for i, s in enumerate(src):
+            d_o, dist_o = oracle.dependencies(g, s)[:2]
+            assert np.array_equal(dist[i], dist_o)
+            assert np.array_equal(delta[i], d_o)
+        assert np.array_equal(ctx.uniform_sources(h, 40, 3, 4), oracle.uniform_sources(g, 40, 3, 4))
+        if g.n > 1:
+            t = [0, g.n - 1]
+            got, ref = ctx.adaptive_sources(h, t, 2.0, 90, 5, 6), oracle.adaptive_sources(g, t, 2.0, 90, 5, 6)
+            assert np.array_equal(got["k"], ref["k"]) and np.array_equal(got["S"], ref["S"])
+
+
+# (n, degree, directed): the last size with everything in shared memory lies near 18,900;
+# 65,536 is the largest graph by rule; a directed graph's 16-bit codes end at 65,535
+@pytest.mark.parametrize("n,degree,directed", [(18_800, 6, False), (19_200, 6, False), (65_536, 5, False),
+                                               (65_535, 5, True), (65_536, 5, True)])
+def test_tier_edges_equal_the_64_lane_engine(n, degree, directed):
+    g = gg.directed_er(n, degree, 8) if directed else gg.erdos_renyi(n, degree, 8, pairwise=False)
+    out = []
+    for solo_n in (None, 0):
+        with _ctx(solo_n) as ctx:
+            h = ctx.load_graph(g.row_ptr, g.col, directed=directed)
+            delta, dist, sigma = ctx.source_dependencies(h, [0, n - 1], want_dist=True, want_sigma=True)
+            out.append((ctx.uniform_sources(h, 70, 9, 1), delta, dist, sigma))
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
+
+
+def test_more_levels_than_the_16_bit_codes():
+    """A path of 70,000 vertices: from s, delta_s(v) is the number of vertices beyond v."""
+    n = 70_000
+    g = gg.from_edges(n, np.arange(n - 1), np.arange(1, n))
+    targets = np.array([0, 1, 35_000, 69_998, 69_999], np.int32)
+    with _ctx() as ctx:
+        h = ctx.load_graph(g.row_ptr, g.col)
+        got = ctx.target_dependencies(h, targets, 4, 4, 0, 2)
+        src = ctx.draw_sources(4, 4, 0, 2, n)
+    for i, s in enumerate(src.tolist()):
+        want = [0.0 if v == s else float(n - 1 - v if v > s else v) for v in targets.tolist()]
+        assert got[:, i].tolist() == want
