@@ -407,14 +407,10 @@ typedef struct bc_tuning {
   int32_t batch_width;        /* 64: 64 sources share one traversal (level masks); 1: plain kernels */
   int32_t heavy_degree;       /* vertices of larger degree are split into segments (32 ..) */
   int32_t segment;            /* neighbours per heavy segment (32 ..) */
-  int32_t packed_max_lanes;   /* light forward: a 32-neighbour chunk over at most this many lanes ... */
-  int32_t packed_min_preds;   /* ... with at least this many predecessors is summed in packed groups
-                                 (packed_max_lanes 0: never) */
-  int32_t bwd_variant;        /* backward (counts <= 2^44): 1 packed lane groups, 0 two lane halves */
-  int32_t heavy_lane;         /* heavy segments: 0 a 64-lane step per neighbour; 1 per-lane item loops;
-                                 2 the backward's (successor, lane) items spread over all threads with
-                                 exact sums in shared memory; 3 that in both passes; 4 in the forward
-                                 only */
+  int32_t packed_max_lanes;   /* 0 .. 64, packed_min_preds 1 .. 32, bwd_variant 0 or 1, heavy_lane 0 .. 4: */
+  int32_t packed_min_preds;   /* kernel forms of earlier versions. One form is left for each kernel, the */
+  int32_t bwd_variant;        /* faster on every graph tried, so these are checked and kept with the */
+  int32_t heavy_lane;         /* record but choose nothing. */
   int32_t push_div;           /* forward level top-down (push from the level's vertices, counts pulled
                                  for the reached ones) when the level's degree sum is <= nnz/push_div;
                                  bottom-up otherwise; 0: always bottom-up (Sec. 3 step 1 either way) */

@@ -4,10 +4,11 @@
 // Layout (n vertices, 64 lanes, lane t = one sampled source):
 //   lm[l][v]    u64  bit t set iff d(s_t, v) = l            (level masks)
 //   visited[v]  u64  OR of lm[0..l][v]
-//   sigma[v][t] u64  sigma_{s_t v}; in the backward pass the slot of (v, t)
-//                    is overwritten by coef = (1+delta)/sigma (double bits)
-//                    once v's level in lane t is done. Lane-minor rows of 512 B,
-//                    so one warp reads a neighbour's 32 lanes with one request.
+//   sigma[v][t] u64  sigma_{s_t v}. Lane-minor rows of 512 B, so one warp reads a
+//                    neighbour's 32 lanes with one request.
+//   coef[v][t]  coef = (1+delta)/sigma as a 96-bit fixed-point number (12 B),
+//               written once v's level in lane t is done; where counts are too
+//               large for that, its double bits in the slot of sigma[v][t].
 //
 // Forward level l (Sec. 3 step 1, predecessor sets of Def. 3): every vertex v
 // with lanes still unvisited pulls from its CSR neighbours w:
@@ -20,6 +21,12 @@
 //   coef[v][t]  = RN(RN(1 + delta[v][t]) / sigma[v][t]).
 // Vertices of degree > HEAVY are split into SEG-long neighbour segments, each
 // handled by one warp; partial results are combined exactly afterwards.
+//
+// R-MAT s20, uniform k = 1024 (16 batches): 56.3 ms with neighbours walked by
+// warp shuffles and doubles converted at every add; 50.6 with entry lists and
+// work lists, 46.8 with vertices above degree 64 (before: 256) split, 41.6 with
+// coefficients kept in 96 bits, 39.5 with listed heavy segments. s16, Bader 1500
+// draws: 21.0 -> 14.0.
 #include <algorithm>
 #include <cstdlib>
 
@@ -27,21 +34,14 @@
 
 namespace bcg {
 
-constexpr int HEAVY_DEFAULT = 256;   // vertices above this degree are split into segments
+constexpr int HEAVY_DEFAULT = 64;    // vertices above this degree are split into segments
 constexpr int SEG_DEFAULT = 256;     // neighbours per heavy segment
-constexpr int GRAB = 16;     // vertices taken per work-queue grab
-constexpr int UNR = 3;       // neighbours gathered per unrolled step (measured: 2-3 best, 1 and 8 slower)
+constexpr int GRAB = 16;             // list positions taken per grab by default
+constexpr int UNR = 3;               // neighbours gathered per unrolled step of a top-down level's pull
 constexpr int FWD_THREADS = 256;
-// The packed backward kernels are latency-bound; five resident blocks per SM
-// (at most 51 registers a thread; a few bytes spill in the heavy finisher)
-// measured 5 % faster than the register-limited four. The forward kernels
-// measured slower that way.
+// Resident blocks per SM of the backward kernels (48 registers a thread); the
+// forward kernels take four (64 registers).
 constexpr int BWD_MIN_BLOCKS = 5;
-constexpr int DENSE_ITEMS = 32 * 64;  // dense item lists: at most 64 lanes for each of 32 neighbours
-// Shared-memory lane sums are indexed skew(t) = t + t/32 in rows of DSK words,
-// so lanes t and t + 32 fall in different banks.
-constexpr int DSK = 66;
-__device__ __forceinline__ int skew(int t) { return t + (t >> 5); }
 
 __device__ __forceinline__ uint64_t warp_or64(uint64_t x) {
   const unsigned lo = __reduce_or_sync(FULL, (unsigned)x);
@@ -73,47 +73,6 @@ __device__ __forceinline__ void block_or_to(uint64_t x, uint64_t *dst) {
   if (threadIdx.x == 0 && s_or) atomicOr((unsigned long long *)dst, s_or);
 }
 
-
-// Warp-wide 32x32 bit-matrix transpose: thread j holds row j; afterwards thread
-// i holds column i (bit j set iff bit i of row j was set). Five butterfly
-// stages, each exchanging the off-diagonal half-blocks of 16, 8, 4, 2 and 1 bits.
-__device__ __forceinline__ uint32_t warp_transpose32(uint32_t x) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int st = 0; st < 5; ++st) {
-    const int k = 16 >> st;
-    const uint32_t m = st == 0 ? 0x0000FFFFu : (st == 1 ? 0x00FF00FFu : (st == 2 ? 0x0F0F0F0Fu : (st == 3 ? 0x33333333u : 0x55555555u)));
-    const uint32_t y = __shfl_xor_sync(FULL, x, k);
-    x = (lane & k) ? (((y >> k) & m) | (x & ~m)) : ((x & m) | ((y & m) << k));
-  }
-  return x;
-}
-
-// Lane ownership for per-lane item loops: thread i owns the i-th and the
-// (i+32)-th set lane of `lanes` in increasing order (-1 when absent); the
-// second one, when present, is always >= 32.
-__device__ __forceinline__ void own_lanes(uint64_t lanes, int8_t *tab, int &p0, int &p1) {
-  const int lane = threadIdx.x & 31;
-  const unsigned lo = (unsigned)lanes, hi = (unsigned)(lanes >> 32);
-  const unsigned lt = (1u << lane) - 1u;
-  const int nlo = __popc(lo), L = nlo + __popc(hi);
-  if ((lo >> lane) & 1u) tab[__popc(lo & lt)] = (int8_t)lane;
-  if ((hi >> lane) & 1u) tab[nlo + __popc(hi & lt)] = (int8_t)(lane + 32);
-  __syncwarp();
-  p0 = lane < L ? (int)tab[lane] : -1;
-  p1 = lane + 32 < L ? (int)tab[lane + 32] : -1;
-  __syncwarp();
-}
-
-// The chunk's neighbour masks m (thread j: neighbour j) seen from lanes p0 and
-// p1: bit j of *c0 is bit p0 of m_j (0 when p0 < 0), likewise *c1 for p1.
-__device__ __forceinline__ void lane_columns(uint64_t m, int p0, int p1, uint32_t &c0, uint32_t &c1) {
-  const uint32_t tl = warp_transpose32((uint32_t)m), th = warp_transpose32((uint32_t)(m >> 32));
-  const uint32_t xl = __shfl_sync(FULL, tl, p0 & 31), xh = __shfl_sync(FULL, th, p0 & 31);
-  const uint32_t yh = __shfl_sync(FULL, th, p1 & 31);
-  c0 = p0 < 0 ? 0u : (p0 < 32 ? xl : xh);
-  c1 = p1 < 0 ? 0u : yh;
-}
 
 // Dynamic work distribution: a warp takes `step` consecutive items per atomic
 // (GRAB light vertices; one heavy segment or heavy vertex, whose work is large).
@@ -194,13 +153,6 @@ __global__ void k_zero_heavy_rows(int nh, const int32_t *__restrict__ heavy, uin
   if (h < nh && threadIdx.x < 64) sigma[(size_t)heavy[h] * 64 + threadIdx.x] = 0ull;
 }
 
-// Clear the next level's masks of the heavy vertices (before their segments
-// OR into them), when the light kernel of the level runs beside them.
-__global__ void k_zero_heavy_lm(int nh, const int32_t *__restrict__ heavy, uint64_t *__restrict__ lm_cur) {
-  const int h = blockIdx.x * blockDim.x + threadIdx.x;
-  if (h < nh) lm_cur[heavy[h]] = 0ull;
-}
-
 // Level 1 directly: the vertices at distance 1 from s_t are its neighbours, each
 // with exactly one shortest path (sigma = 1). One block per lane.
 __global__ void k_fwd_level1(int count, const int32_t *__restrict__ sources, const int32_t *__restrict__ rp,
@@ -235,15 +187,124 @@ __global__ void k_fwd_level1(int count, const int32_t *__restrict__ sources, con
   }
 }
 
+// ------------------------------------------------ neighbour entry lists --
+// Both passes reduce, for a vertex and its lanes at a level, over the
+// neighbours that share a lane with it (predecessors forward, successors
+// backward). A warp first lists those neighbours, (mask, vertex) entries of 16
+// bytes in shared memory, then sums their rows. Every kernel here is bound by
+// instruction issue (62-76 % on R-MAT s20), so what counts is the instructions
+// per entry: a broadcast read of the entry, a bit test, an address, a load and
+// the add. Walking neighbours by warp shuffles with two lanes per thread took
+// 30 (forward) to 60; from the list it is 8 to 20, with one lane per thread
+// while at most 32 lanes are in play and several entries per step below 17.
+//
+// Rows of a whole run of vertices are listed as one flattened list of edges, 32
+// to a window: the threads whose rows start in a window mark their first
+// positions and a visit's row is the last mark at or before it, so short rows
+// (7 of 32 threads on ER degree 7) cost no idle threads.
+constexpr int ECAP_F = 256;  // entries per warp, forward
+constexpr int ECAP_B = 128;  // ... and backward, where a ring shares the shared memory
+
+// Lists the entries of the rows held by the warp's threads (thread k: entries
+// [beg, beg + d) of col, wanted lanes `want`; d = 0: none; the sum of d at most
+// the list's capacity). Returns the number of entries; a row's are contiguous
+// from `first`. tri counts (edge, lane) pairs.
+__device__ __forceinline__ int list_rows(const int32_t *__restrict__ col, const uint64_t *__restrict__ lm, int beg,
+                                         int d, uint64_t want, uint4 *ent, uint8_t *own, int &first,
+                                         unsigned long long &tri) {
+  constexpr int U = 4;
+  const int lane = threadIdx.x & 31;
+  const unsigned lt = (1u << lane) - 1u, le = lt | (1u << lane);
+  int incl = d;
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const int y = __shfl_up_sync(FULL, incl, off);
+    if (lane >= off) incl += y;
+  }
+  const int E = __shfl_sync(FULL, incl, 31), start = incl - d, shift = beg - start;
+  const unsigned rows = __ballot_sync(FULL, d > 0);
+  if (d > 0) own[__popc(rows & lt)] = (uint8_t)lane;
+  __syncwarp();
+  int before = -1, total = 0;
+  first = 0;
+  for (int i0 = 0; i0 < E; i0 += 32 * U) {
+    int32_t w[U];
+    uint64_t m[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int s = start - (i0 + 32 * u);
+      const unsigned f = __reduce_or_sync(FULL, (d > 0 && (unsigned)s < 32u) ? 1u << s : 0u);
+      const int i = i0 + 32 * u + lane;
+      const int o = i < E ? (int)own[before + __popc(f & le)] : 0;
+      before += __popc(f);
+      const int j = i + __shfl_sync(FULL, shift, o);
+      m[u] = __shfl_sync(FULL, want, o);
+      w[u] = i < E ? col[j] : -1;
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) m[u] = w[u] >= 0 ? lm[w[u]] & m[u] : 0ull;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const unsigned bal = __ballot_sync(FULL, m[u] != 0ull);
+      const int s = start - (i0 + 32 * u);
+      if (d > 0 && (unsigned)s < 32u) first = total + __popc(bal & ((1u << s) - 1u));
+      if (m[u]) ent[total + __popc(bal & lt)] = make_uint4((uint32_t)m[u], (uint32_t)(m[u] >> 32), (uint32_t)w[u], 0u);
+      tri += (unsigned long long)__popcll((long long)m[u]);
+      total += __popc(bal);
+    }
+  }
+  __syncwarp();
+  return total;
+}
+
+// The same for one row's entries [beg, end) (at most the list's capacity).
+__device__ __forceinline__ int list_row(const int32_t *__restrict__ col, const uint64_t *__restrict__ lm, int beg,
+                                        int end, uint64_t want, uint4 *ent, unsigned long long &tri) {
+  constexpr int U = 4;
+  const int lane = threadIdx.x & 31;
+  const unsigned lt = (1u << lane) - 1u;
+  int total = 0;
+  for (int j0 = beg; j0 < end; j0 += 32 * U) {
+    int32_t w[U];
+    uint64_t m[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int j = j0 + 32 * u + lane;
+      w[u] = j < end ? col[j] : -1;
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) m[u] = w[u] >= 0 ? lm[w[u]] & want : 0ull;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const unsigned bal = __ballot_sync(FULL, m[u] != 0ull);
+      if (m[u]) ent[total + __popc(bal & lt)] = make_uint4((uint32_t)m[u], (uint32_t)(m[u] >> 32), (uint32_t)w[u], 0u);
+      tri += (unsigned long long)__popcll((long long)m[u]);
+      total += __popc(bal);
+    }
+  }
+  __syncwarp();
+  return total;
+}
+
+// OR of the masks of entries [f, e).
+__device__ __forceinline__ uint64_t entries_or(const uint4 *ent, int f, int e) {
+  uint64_t m = 0ull;
+  for (int i = f + (int)(threadIdx.x & 31); i < e; i += 32) {
+    const uint4 x = ent[i];
+    m |= ((uint64_t)x.y << 32) | x.x;
+  }
+  return warp_or64(m);
+}
+
+// Lanes of a vertex packed over the warp: groups of 2^glog threads each take
+// another entry per step; thread i of a group owns the i-th lane in increasing
+// order (p0; -1: none), and the (i+32)-th when more than 32 are set (p1).
 struct Packed {
-  int glog;  // log2 of the group width G
-  int p0;    // lane owned by this thread (-1: none)
-  int p1;    // second lane when |L| > 32 (G = 32), else -1
+  int glog;
+  int p0, p1;
   bool two;
 };
 
-// Active lane positions in increasing order: each set lane writes its position
-// at its rank in a per-warp table, then thread i reads entry i.
 __device__ __forceinline__ Packed pack_lanes(uint64_t lanes, int8_t *tab) {
   const int lane = threadIdx.x & 31;
   const unsigned lo = (unsigned)lanes, hi = (unsigned)(lanes >> 32);
@@ -262,508 +323,375 @@ __device__ __forceinline__ Packed pack_lanes(uint64_t lanes, int8_t *tab) {
   return pk;
 }
 
-
-// Predecessor counts for one 32-neighbour chunk of v, packed: the lanes of cm
-// (the OR of the chunk's masks) are spread over groups of G >= |cm| threads and
-// each group takes a different predecessor per step, so a chunk with many
-// predecessors over few lanes costs a few steps instead of one 64-slot step per
-// predecessor. The chunk's per-lane sums are then added into the owners' sums
-// (thread t owns lanes t and t + 32). Integer sums: exact, order-free.
-__device__ __forceinline__ void chunk_packed(uint64_t m, int32_t w, uint64_t cm, unsigned bal,
-                                             const uint64_t *__restrict__ sigma, int8_t *tab, int32_t *list,
-                                             uint64_t &s0, uint64_t &s1, uint64_t &ovf) {
+// acc0 / acc1 take the row values of entries [f, e) in the thread's lanes p0 /
+// p1, four steps in flight (only the last four check the list's end). R reads
+// a row's lane: R::V, R::zero(), R(w, lane).
+template <class R, class F0, class F1>
+__device__ __forceinline__ void entries_sum(const uint4 *ent, int f, int e, const Packed &pk, const R &rows, F0 acc0,
+                                            F1 acc1) {
   const int lane = threadIdx.x & 31;
-  const Packed pk = pack_lanes(cm, tab);
   const int NG = 32 >> pk.glog, g = lane >> pk.glog;
-  const int cnt = __popc(bal);
-  if (m != 0ull) list[__popc(bal & ((1u << lane) - 1u))] = lane;
-  __syncwarp();
-  const uint64_t b0 = pk.p0 >= 0 ? (1ull << pk.p0) : 0ull, b1 = pk.p1 >= 0 ? (1ull << pk.p1) : 0ull;
-  const int q0 = pk.p0 < 0 ? 0 : pk.p0, q1 = pk.p1 < 0 ? 0 : pk.p1;
-  uint64_t a0 = 0ull, a1 = 0ull;
-  for (int r = 0; r < cnt; r += 2 * NG) {
-    const int i0 = r + g, i1 = r + NG + g;
-    const bool h0 = i0 < cnt, h1 = i1 < cnt;
-    const int x0s = h0 ? list[i0] : 0, x1s = h1 ? list[i1] : 0;
-    const uint64_t m0 = __shfl_sync(FULL, m, x0s), m1 = __shfl_sync(FULL, m, x1s);
-    const int32_t w0 = __shfl_sync(FULL, w, x0s), w1 = __shfl_sync(FULL, w, x1s);
-    const uint64_t y0 = (h0 && (m0 & b0)) ? sigma[(size_t)w0 * 64 + q0] : 0ull;
-    const uint64_t y1 = (h1 && (m1 & b0)) ? sigma[(size_t)w1 * 64 + q0] : 0ull;
-    if (pk.two) {
-      const uint64_t z0 = (h0 && (m0 & b1)) ? sigma[(size_t)w0 * 64 + q1] : 0ull;
-      const uint64_t z1 = (h1 && (m1 & b1)) ? sigma[(size_t)w1 * 64 + q1] : 0ull;
-      uint64_t t = a1 + z0;
-      if (t < a1) ovf |= b1;
-      a1 = t + z1;
-      if (a1 < t) ovf |= b1;
+  const bool h0 = pk.p0 >= 32;
+  const uint32_t b0 = pk.p0 >= 0 ? 1u << (pk.p0 & 31) : 0u;
+  const int t0 = pk.p0 < 0 ? 0 : pk.p0;
+  if (!pk.two) {
+    int r = f;
+    for (; r + 4 * NG <= e; r += 4 * NG) {
+      typename R::V x[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const uint4 n = ent[r + u * NG + g];
+        x[u] = ((h0 ? n.y : n.x) & b0) ? rows(n.z, t0) : R::zero();
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) acc0(x[u]);
     }
-    uint64_t t = a0 + y0;
-    if (t < a0) ovf |= b0;
-    a0 = t + y1;
-    if (a0 < t) ovf |= b0;
-  }
-  __syncwarp();
-  for (int off = 1 << pk.glog; off < 32; off <<= 1) {
-    const uint64_t o = __shfl_xor_sync(FULL, a0, off);
-    const uint64_t t = a0 + o;
-    if (t < a0) ovf |= b0;
-    a0 = t;
-  }
-  // lane X of cm has rank r in the packed order: its sum is a0 of thread r
-  // (r < 32) or a1 of thread r - 32
-  const unsigned lo = (unsigned)cm, hi = (unsigned)(cm >> 32), lt = (1u << lane) - 1u;
-  const int nlo = __popc(lo);
-  const int r0 = __popc(lo & lt), r1 = nlo + __popc(hi & lt);
-  uint64_t v0 = __shfl_sync(FULL, a0, r0 & 31), v1 = __shfl_sync(FULL, a0, r1 & 31);
-  if (pk.two) {
-    const uint64_t u0 = __shfl_sync(FULL, a1, r0 & 31), u1 = __shfl_sync(FULL, a1, r1 & 31);
-    if (r0 >= 32) v0 = u0;
-    if (r1 >= 32) v1 = u1;
-  }
-  if ((lo >> lane) & 1u) {
-    const uint64_t t = s0 + v0;
-    if (t < s0) ovf |= 1ull << lane;
-    s0 = t;
-  }
-  if ((hi >> lane) & 1u) {
-    const uint64_t t = s1 + v1;
-    if (t < s1) ovf |= 1ull << (lane + 32);
-    s1 = t;
+    if (r < e) {
+      typename R::V x[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int q = r + u * NG + g;
+        const uint4 n = ent[q < e ? q : f];
+        x[u] = (q < e && ((h0 ? n.y : n.x) & b0)) ? rows(n.z, t0) : R::zero();
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) acc0(x[u]);
+    }
+  } else {  // (the 33rd lane and later: always 32 or above)
+    const uint32_t b1 = pk.p1 >= 0 ? 1u << (pk.p1 & 31) : 0u;
+    const int t1 = pk.p1 < 0 ? 0 : pk.p1;
+    int i = f;
+    for (; i + 2 <= e; i += 2) {
+      typename R::V x[2], y[2];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const uint4 n = ent[i + u];
+        x[u] = ((h0 ? n.y : n.x) & b0) ? rows(n.z, t0) : R::zero();
+        y[u] = (n.y & b1) ? rows(n.z, t1) : R::zero();
+      }
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        acc0(x[u]);
+        acc1(y[u]);
+      }
+    }
+    if (i < e) {
+      const uint4 n = ent[i];
+      acc0(((h0 ? n.y : n.x) & b0) ? rows(n.z, t0) : R::zero());
+      acc1((n.y & b1) ? rows(n.z, t1) : R::zero());
+    }
   }
 }
 
-// Adds the count x to lane t's 64-bit sum in shared memory (two 32-bit limbs,
-// the carry of the low limb passed on); a carry out of the high limb (the true
-// sum is 2^64 or more: the lane overflowed) sets the lane's bit in ovf2.
-__device__ __forceinline__ void u64_limbs_atomic_add(uint32_t (*acc)[DSK], uint32_t *ovf2, int t, uint64_t x) {
-  const uint32_t lo = (uint32_t)x, hi = (uint32_t)(x >> 32);
-  const int ts = skew(t);
-  uint32_t cy = 0u;
-  if (lo) {
-    const uint32_t old = atomicAdd(&acc[0][ts], lo);
-    cy = (old + lo < lo) ? 1u : 0u;
-  }
-  const uint32_t h = hi + cy;
-  bool of = h < cy;  // hi + carry wrapped
-  if (h) {
-    const uint32_t old = atomicAdd(&acc[1][ts], h);
-    of |= old + h < h;
-  }
-  if (of) atomicOr(&ovf2[t >> 5], 1u << (t & 31));
-}
+// Rows of 64 words of 64 bits.
+struct WordRows {
+  using V = uint64_t;
+  const uint64_t *__restrict__ p;
+  static __device__ __forceinline__ V zero() { return 0ull; }
+  __device__ __forceinline__ V operator()(uint32_t w, int t) const { return p[(size_t)w * 64 + t]; }
+};
 
 // --------------------------------------------------------------- forward --
-// One warp per vertex (grid-stride); heavy vertices only get lm_cur[v] = 0 here.
-__global__ void __launch_bounds__(FWD_THREADS)
-k_fwd_light(int32_t n, const int32_t *__restrict__ rp, const int32_t *__restrict__ col,
-            const uint64_t *__restrict__ lm_prev, uint64_t *__restrict__ lm_cur,
-            uint64_t *__restrict__ visited, uint64_t *__restrict__ sigma,
-            const uint64_t *__restrict__ active_prev, uint64_t *__restrict__ enable,
-            uint64_t *__restrict__ active_cur, unsigned *__restrict__ err,
-            unsigned long long *__restrict__ cnt, unsigned *__restrict__ wq, int heavy_deg, int pk_maxl,
-            int pk_mincnt, int32_t *__restrict__ list_next, unsigned *__restrict__ vcnt_next,
-            unsigned long long *__restrict__ vedges_next, int gsz, int zero_heavy) {
-  __shared__ int32_t lists[FWD_THREADS / 32][32];
-  __shared__ int8_t tabs[FWD_THREADS / 32][64];
-  const int lane = threadIdx.x & 31;
-  const uint64_t act = *active_prev & *enable;
-  uint64_t any_new = 0ull, smax = 0ull;
-  unsigned long long tri = 0ull, rch = 0ull;
-  uint64_t ovf = 0ull;  // lanes whose counts exceeded 2^64-1 here
-  // a warp takes gsz <= 32 vertices; each thread loads one vertex's header,
-  // and only vertices with unvisited active lanes and light degree are walked
-  for (int base = grab(wq, gsz); base < n; base = grab(wq, gsz)) {
-    const int vl = base + lane;
-    int hb = 0, he = 0;
-    uint64_t hv = 0ull;
-    bool work = false;
-    if (lane < gsz && vl < n) {
-      hb = rp[vl];
-      he = rp[vl + 1];
-      hv = visited[vl];
-      work = ((~hv & act) != 0ull) && he > hb && he - hb <= heavy_deg;
-      // heavy vertices are filled by their segments: their rows are cleared
-      // here, or (zero_heavy = 0) by k_zero_heavy_lm on the heavy kernels' stream
-      if (!work && (zero_heavy || he - hb <= heavy_deg)) lm_cur[vl] = 0ull;
-    }
-    unsigned todo = __ballot_sync(FULL, work);
-    unsigned found = 0u;  // vertices of this grab that join the next level
-    while (todo) {
-    const int iv = __ffs(todo) - 1;
-    todo &= todo - 1u;
-    const int v = base + iv;
-    const int beg = __shfl_sync(FULL, hb, iv), end = __shfl_sync(FULL, he, iv);
-    const uint64_t vis = __shfl_sync(FULL, hv, iv);
-    const uint64_t pend = ~vis & act;
-    uint64_t newm = 0ull;
-    {
-      uint64_t s0 = 0ull, s1 = 0ull;
-      for (int base = beg; base < end; base += 32) {
-        const int j = base + lane;
-        int32_t w = 0;
-        uint64_t m = 0ull;
-        if (j < end) {
-          w = col[j];
-          m = lm_prev[w] & pend;
-        }
-        newm |= m;
-        tri += (unsigned long long)__popcll((long long)m);
-        unsigned bal = __ballot_sync(FULL, m != 0ull);
-        if (pk_maxl > 0 && __popc(bal) >= pk_mincnt) {
-          // many predecessors over few lanes: packed groups do several per step
-          const uint64_t cm = warp_or64(m);
-          if (__popcll((long long)cm) <= pk_maxl) {
-            chunk_packed(m, w, cm, bal, sigma, tabs[threadIdx.x >> 5], lists[threadIdx.x >> 5], s0, s1, ovf);
-            bal = 0u;
-          }
-        }
-        while (bal) {
-          uint64_t mk[UNR];
-          int32_t wk[UNR];
-          take(bal, m, w, mk, wk);
-          uint64_t x0[UNR], x1[UNR];
-#pragma unroll
-          for (int k = 0; k < UNR; ++k) {
-            const uint64_t *row = sigma + (size_t)wk[k] * 64;
-            x0[k] = ((mk[k] >> lane) & 1ull) ? row[lane] : 0ull;
-            x1[k] = ((mk[k] >> (lane + 32)) & 1ull) ? row[lane + 32] : 0ull;
-          }
-#pragma unroll
-          for (int k = 0; k < UNR; ++k) {
-            const uint64_t t0 = s0 + x0[k];
-            if (t0 < s0) ovf |= 1ull << lane;
-            s0 = t0;
-            const uint64_t t1 = s1 + x1[k];
-            if (t1 < s1) ovf |= 1ull << (lane + 32);
-            s1 = t1;
-          }
-        }
-      }
-      newm = warp_or64(newm);
-      if ((newm >> lane) & 1ull) {
-        sigma[(size_t)v * 64 + lane] = s0;
-        smax = s0 > smax ? s0 : smax;
-      }
-      if ((newm >> (lane + 32)) & 1ull) {
-        sigma[(size_t)v * 64 + 32 + lane] = s1;
-        smax = s1 > smax ? s1 : smax;
-      }
-    }
-    if (lane == 0) {
-      lm_cur[v] = newm;
-      if (newm) visited[v] = vis | newm;
-    }
-    if (newm) found |= 1u << iv;
-    rch += (unsigned long long)__popcll((long long)newm);
-    any_new |= newm;
-    }
-    list_append((found >> lane) & 1u, vl, he - hb, list_next, vcnt_next, vedges_next);
+// Exact 64-bit counts. CHECK: note carries out of 64 bits (not needed while
+// the largest count so far times n stays below 2^64).
+template <bool CHECK> struct CountAcc {
+  uint64_t s = 0ull;
+  bool ov = false;
+  __device__ __forceinline__ void add(uint64_t x) {
+    s += x;
+    if constexpr (CHECK) ov |= s < x;
   }
+  __device__ __forceinline__ void group_sum(int glog) {  // over the groups: threads with the same slot
+    for (int off = 1 << glog; off < 32; off <<= 1) {
+      const uint64_t o = __shfl_xor_sync(FULL, s, off);
+      add(o);
+    }
+  }
+};
+
+// Sums of the entries [f, e) in the packed lanes; the bits of lanes whose count
+// left 64 bits go to ovf.
+template <bool CHECK>
+__device__ __forceinline__ void count_entries(const uint4 *ent, int f, int e, const Packed &pk,
+                                              const uint64_t *__restrict__ sigma, uint64_t &s0, uint64_t &s1,
+                                              uint64_t &ovf) {
+  CountAcc<CHECK> a, b;
+  entries_sum(ent, f, e, pk, WordRows{sigma}, [&](uint64_t x) { a.add(x); }, [&](uint64_t x) { b.add(x); });
+  a.group_sum(pk.glog);
+  a.add(s0);
+  b.add(s1);
+  s0 = a.s;
+  s1 = b.s;
+  if constexpr (CHECK) {
+    if (a.ov && pk.p0 >= 0) ovf |= 1ull << pk.p0;
+    if (b.ov && pk.p1 >= 0) ovf |= 1ull << pk.p1;
+  }
+}
+
+__device__ __forceinline__ bool counts_fit(uint64_t largest, int32_t n) {
+  return __umul64hi(largest, (uint64_t)n) == 0ull;
+}
+
+// Light vertices of a level (degree at most heavy_deg): the list `list_in`
+// (*cnt_in of them) holds the ones with lanes still to reach; a warp takes gsz
+// at a time. The vertices that stay unfinished go to list_out, the ones that
+// got lanes at this level to the level's list. The next level's masks must be
+// clear on entry.
+__global__ void __launch_bounds__(FWD_THREADS, 4)
+k_fwd_light(int32_t n, const int32_t *__restrict__ list_in, const unsigned *__restrict__ cnt_in,
+            int32_t *__restrict__ list_out, unsigned *__restrict__ cnt_out, const int32_t *__restrict__ rp,
+            const int32_t *__restrict__ col, const uint64_t *__restrict__ lm_prev, uint64_t *__restrict__ lm_cur,
+            uint64_t *__restrict__ visited, uint64_t *__restrict__ sigma, const uint64_t *__restrict__ active_prev,
+            uint64_t *__restrict__ enable, uint64_t *__restrict__ active_cur, unsigned long long *__restrict__ cnt,
+            unsigned *__restrict__ wq, int32_t *__restrict__ list_next, unsigned *__restrict__ vcnt_next,
+            unsigned long long *__restrict__ vedges_next, int gsz) {
+  __shared__ uint4 ents[FWD_THREADS / 32][ECAP_F];
+  __shared__ int8_t tabs[FWD_THREADS / 32][64];
+  __shared__ uint8_t owns[FWD_THREADS / 32][32];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const unsigned lt = (1u << lane) - 1u;
+  uint4 *ent = ents[wid];
+  int8_t *tab = tabs[wid];
+  const uint64_t act = *active_prev & *enable;
+  const int total = (int)*cnt_in;
+  const bool fit = counts_fit(enable[2], n);  // (grows during the level: still a bound for the level before)
+  uint64_t any_new = 0ull, smax = 0ull, ovf = 0ull;
+  unsigned long long tri = 0ull, rch = 0ull;
+  if (act)
+    for (int base = grab(wq, gsz); base < total; base = grab(wq, gsz)) {
+      int32_t v = -1;
+      int hb = 0, d = 0;
+      uint64_t vis = 0ull, pend = 0ull, mine = 0ull;
+      if (lane < gsz && base + lane < total) {
+        v = list_in[base + lane];
+        hb = rp[v];
+        d = rp[v + 1] - hb;
+        vis = visited[v];
+        pend = ~vis & act;
+      }
+      // one vertex's new lanes nm with counts s0 / s1 in the packed lanes
+      auto store = [&](int k, int32_t u, uint64_t nm, const Packed &pk, uint64_t s0, uint64_t s1) {
+        uint64_t *row = sigma + (size_t)u * 64;
+        if ((lane >> pk.glog) == 0 && pk.p0 >= 0 && ((nm >> pk.p0) & 1ull)) {
+          row[pk.p0] = s0;
+          smax = s0 > smax ? s0 : smax;
+        }
+        if (pk.p1 >= 0 && ((nm >> pk.p1) & 1ull)) {
+          row[pk.p1] = s1;
+          smax = s1 > smax ? s1 : smax;
+        }
+        if (lane == k) mine = nm;
+        any_new |= nm;
+      };
+      unsigned todo = __ballot_sync(FULL, pend != 0ull && d <= ECAP_F);
+      while (todo) {
+        const int dd = ((todo >> lane) & 1u) ? d : 0;
+        int incl = dd;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+          const int y = __shfl_up_sync(FULL, incl, off);
+          if (lane >= off) incl += y;
+        }
+        const unsigned sub = __ballot_sync(FULL, ((todo >> lane) & 1u) && incl <= ECAP_F);
+        todo &= ~sub;
+        int first;
+        const int ne = list_rows(col, lm_prev, hb, ((sub >> lane) & 1u) ? d : 0, pend, ent, owns[wid], first, tri);
+        for (unsigned r = sub; r;) {
+          const int k = __ffs(r) - 1;
+          r &= r - 1u;
+          const int f = __shfl_sync(FULL, first, k), e = r ? __shfl_sync(FULL, first, __ffs(r) - 1) : ne;
+          if (f == e) continue;
+          const int32_t u = __shfl_sync(FULL, v, k);
+          const uint64_t nm = entries_or(ent, f, e);
+          const Packed pk = pack_lanes(nm, tab);
+          uint64_t s0 = 0ull, s1 = 0ull;
+          if (fit) count_entries<false>(ent, f, e, pk, sigma, s0, s1, ovf);
+          else count_entries<true>(ent, f, e, pk, sigma, s0, s1, ovf);
+          store(k, u, nm, pk, s0, s1);
+        }
+        __syncwarp();
+      }
+      for (unsigned r = __ballot_sync(FULL, pend != 0ull && d > ECAP_F); r; r &= r - 1u) {
+        // (only with heavy_deg above the list's capacity) piece by piece
+        const int k = __ffs(r) - 1;
+        const int32_t u = __shfl_sync(FULL, v, k);
+        const int b = __shfl_sync(FULL, hb, k), e = b + __shfl_sync(FULL, d, k);
+        const uint64_t pl = __shfl_sync(FULL, pend, k);
+        const Packed pk = pack_lanes(pl, tab);
+        uint64_t s0 = 0ull, s1 = 0ull, nm = 0ull;
+        for (int j = b; j < e; j += ECAP_F) {
+          const int ne = list_row(col, lm_prev, j, min(e, j + ECAP_F), pl, ent, tri);
+          nm |= entries_or(ent, 0, ne);
+          count_entries<true>(ent, 0, ne, pk, sigma, s0, s1, ovf);
+          __syncwarp();
+        }
+        if (nm) store(k, u, nm, pk, s0, s1);
+      }
+      if (mine) {
+        lm_cur[v] = mine;
+        visited[v] = vis | mine;
+        rch += (unsigned long long)__popcll((long long)mine);
+      }
+      // unfinished vertices stay on the list; found ones join the level's
+      const unsigned left = __ballot_sync(FULL, (pend & ~mine) != 0ull), found = __ballot_sync(FULL, mine != 0ull);
+      unsigned p0 = 0u, p1 = 0u;
+      if (lane == 0 && left) p0 = atomicAdd(cnt_out, (unsigned)__popc(left));
+      if (lane == 1 && found) p1 = atomicAdd(vcnt_next, (unsigned)__popc(found));
+      p0 = __shfl_sync(FULL, p0, 0);
+      p1 = __shfl_sync(FULL, p1, 1);
+      if ((left >> lane) & 1u) list_out[p0 + __popc(left & lt)] = v;
+      if ((found >> lane) & 1u) list_next[p1 + __popc(found & lt)] = v;
+      if (vedges_next && found) {
+        const unsigned ds = __reduce_add_sync(FULL, mine ? (unsigned)d : 0u);
+        if (lane == 0) atomicAdd(vedges_next, (unsigned long long)ds);
+      }
+    }
   ovf = warp_or64(ovf);
   if (lane == 0 && ovf) atomicOr((unsigned long long *)(enable + 3), (unsigned long long)ovf);
-  (void)err;
   tri = warp_sum64(tri);
+  rch = warp_sum64(rch);
   if (lane == 0 && (tri | rch)) {
     atomicAdd(cnt, tri);
     atomicAdd(cnt + 1, rch);
   }
   smax = warp_max64(smax);
   if (lane == 0 && smax > 1ull) atomicMax((unsigned long long *)(enable + 2), (unsigned long long)smax);
+  any_new = warp_or64(any_new);
   block_or_to(any_new, active_cur);
 }
 
-// One warp per segment of a heavy vertex: partial sigma sums via atomics.
-__global__ void __launch_bounds__(FWD_THREADS)
-k_fwd_heavy(int nseg, const int32_t *__restrict__ seg_v, const int32_t *__restrict__ seg_b,
-            const int32_t *__restrict__ seg_e, const int32_t *__restrict__ col,
-            const uint64_t *__restrict__ lm_prev, uint64_t *__restrict__ lm_cur,
-            const uint64_t *__restrict__ visited, uint64_t *__restrict__ sigma,
-            const uint64_t *__restrict__ active_prev, uint64_t *__restrict__ enable,
-            unsigned *__restrict__ err, unsigned long long *__restrict__ cnt, unsigned *__restrict__ wq) {
-  const int lane = threadIdx.x & 31;
-  const uint64_t act = *active_prev & *enable;
-  unsigned long long tri = 0ull;
-  uint64_t ovf = 0ull;  // lanes whose counts exceeded 2^64-1 here
-  for (int s = grab(wq, 1); s < nseg; s = grab(wq, 1)) {
-    const int32_t v = seg_v[s];
-    const int beg = seg_b[s], end = seg_e[s];
-    const uint64_t pend = ~visited[v] & act;
-    if (!pend) continue;
-    uint64_t newm = 0ull, s0 = 0ull, s1 = 0ull;
-    for (int base = beg; base < end; base += 32) {
-      const int j = base + lane;
-      int32_t w = 0;
-      uint64_t m = 0ull;
-      if (j < end) {
-        w = col[j];
-        m = lm_prev[w] & pend;
-      }
-      newm |= m;
-      tri += (unsigned long long)__popcll((long long)m);
-      unsigned bal = __ballot_sync(FULL, m != 0ull);
-      while (bal) {
-        uint64_t mk[UNR];
-        int32_t wk[UNR];
-        take(bal, m, w, mk, wk);
-        uint64_t x0[UNR], x1[UNR];
-#pragma unroll
-        for (int k = 0; k < UNR; ++k) {
-          const uint64_t *row = sigma + (size_t)wk[k] * 64;
-          x0[k] = ((mk[k] >> lane) & 1ull) ? row[lane] : 0ull;
-          x1[k] = ((mk[k] >> (lane + 32)) & 1ull) ? row[lane + 32] : 0ull;
-        }
-#pragma unroll
-        for (int k = 0; k < UNR; ++k) {
-          const uint64_t t0 = s0 + x0[k];
-          if (t0 < s0) ovf |= 1ull << lane;
-          s0 = t0;
-          const uint64_t t1 = s1 + x1[k];
-          if (t1 < s1) ovf |= 1ull << (lane + 32);
-          s1 = t1;
-        }
-      }
-    }
-    newm = warp_or64(newm);
-    if (!newm) continue;
-    unsigned long long *dst = (unsigned long long *)(sigma + (size_t)v * 64);
-    if ((newm >> lane) & 1ull) {
-      const unsigned long long old = atomicAdd(dst + lane, (unsigned long long)s0);
-      if (old + s0 < old) ovf |= 1ull << lane;
-    }
-    if ((newm >> (lane + 32)) & 1ull) {
-      const unsigned long long old = atomicAdd(dst + 32 + lane, (unsigned long long)s1);
-      if (old + s1 < old) ovf |= 1ull << (lane + 32);
-    }
-    if (lane == 0) atomicOr((unsigned long long *)&lm_cur[v], (unsigned long long)newm);
-  }
-  ovf = warp_or64(ovf);
-  if (lane == 0 && ovf) atomicOr((unsigned long long *)(enable + 3), (unsigned long long)ovf);
-  (void)err;
-  tri = warp_sum64(tri);
-  if (lane == 0 && tri) atomicAdd(cnt, tri);
-}
-
-// The same with per-lane item loops: thread i owns the i-th (and (i+32)-th)
-// pending lane of v; a warp transpose turns the chunk's 32 predecessor masks
-// into one 32-bit column per owned lane, and each thread adds only the counts
-// of the predecessors in its own lanes. A hub-adjacent chunk has predecessors in
-// a fraction of the pending lanes, so this skips the lane slots a 64-wide step
-// per predecessor would leave idle.
-__global__ void __launch_bounds__(FWD_THREADS)
-k_fwd_heavy_lane(int nseg, const int32_t *__restrict__ seg_v, const int32_t *__restrict__ seg_b,
-                 const int32_t *__restrict__ seg_e, const int32_t *__restrict__ col,
-                 const uint64_t *__restrict__ lm_prev, uint64_t *__restrict__ lm_cur,
-                 const uint64_t *__restrict__ visited, uint64_t *__restrict__ sigma,
-                 const uint64_t *__restrict__ active_prev, uint64_t *__restrict__ enable,
-                 unsigned long long *__restrict__ cnt, unsigned *__restrict__ wq) {
-  __shared__ int32_t sws[FWD_THREADS / 32][32];
-  __shared__ int8_t tabs[FWD_THREADS / 32][64];
-  int32_t *sw = sws[threadIdx.x >> 5];
-  int8_t *tab = tabs[threadIdx.x >> 5];
-  const int lane = threadIdx.x & 31;
-  const uint64_t act = *active_prev & *enable;
-  unsigned long long tri = 0ull;
-  uint64_t ovf = 0ull;
-  for (int s = grab(wq, 1); s < nseg; s = grab(wq, 1)) {
-    const int32_t v = seg_v[s];
-    const int beg = seg_b[s], end = seg_e[s];
-    const uint64_t pend = ~visited[v] & act;
-    if (!pend) continue;
-    int p0, p1;
-    own_lanes(pend, tab, p0, p1);
-    uint64_t newm = 0ull, s0 = 0ull, s1 = 0ull;
-    bool o0 = false, o1 = false;
-    for (int base = beg; base < end; base += 32) {
-      const int j = base + lane;
-      int32_t w = 0;
-      uint64_t m = 0ull;
-      if (j < end) {
-        w = col[j];
-        m = lm_prev[w] & pend;
-      }
-      newm |= m;
-      tri += (unsigned long long)__popcll((long long)m);
-      sw[lane] = w;
-      uint32_t c0, c1;
-      lane_columns(m, p0, p1, c0, c1);
-      __syncwarp();
-      while (c0) {
-        const int ja = __ffs(c0) - 1;
-        c0 &= c0 - 1u;
-        const int jb = c0 ? __ffs(c0) - 1 : ja;
-        const bool hb = c0 != 0u;
-        if (hb) c0 &= c0 - 1u;
-        const uint64_t xa = sigma[(size_t)sw[ja] * 64 + p0];
-        const uint64_t xb = hb ? sigma[(size_t)sw[jb] * 64 + p0] : 0ull;
-        uint64_t t = s0 + xa;
-        o0 |= t < s0;
-        s0 = t + xb;
-        o0 |= s0 < t;
-      }
-      while (c1) {
-        const int ja = __ffs(c1) - 1;
-        c1 &= c1 - 1u;
-        const uint64_t xa = sigma[(size_t)sw[ja] * 64 + p1];
-        const uint64_t t = s1 + xa;
-        o1 |= t < s1;
-        s1 = t;
-      }
-      __syncwarp();
-    }
-    newm = warp_or64(newm);
-    if (!newm) continue;
-    unsigned long long *dst = (unsigned long long *)(sigma + (size_t)v * 64);
-    if (p0 >= 0 && ((newm >> p0) & 1ull)) {
-      const unsigned long long old = atomicAdd(dst + p0, (unsigned long long)s0);
-      if (o0 || old + s0 < old) ovf |= 1ull << p0;
-    }
-    if (p1 >= 0 && ((newm >> p1) & 1ull)) {
-      const unsigned long long old = atomicAdd(dst + p1, (unsigned long long)s1);
-      if (o1 || old + s1 < old) ovf |= 1ull << p1;
-    }
-    if (lane == 0) atomicOr((unsigned long long *)&lm_cur[v], (unsigned long long)newm);
-  }
-  ovf = warp_or64(ovf);
-  if (lane == 0 && ovf) atomicOr((unsigned long long *)(enable + 3), (unsigned long long)ovf);
-  tri = warp_sum64(tri);
-  if (lane == 0 && tri) atomicAdd(cnt, tri);
-}
-
-// Heavy segments of the forward with the predecessors' (count, lane) items
-// spread over all 32 threads (see k_bwd_heavy_seg_dense); the segment's
-// per-lane sums go to the vertex's count row by 64-bit atomics as in k_fwd_heavy.
+// One warp per listed segment (list null: every segment) of a heavy vertex; the
+// segments' sums meet in the vertex's count row by 64-bit atomics, and the last
+// of them sees the row's total, so the largest count is taken here.
 __global__ void __launch_bounds__(FWD_THREADS, 4)
-k_fwd_heavy_dense(int nseg, const int32_t *__restrict__ seg_v, const int32_t *__restrict__ seg_b,
-                  const int32_t *__restrict__ seg_e, const int32_t *__restrict__ col,
-                  const uint64_t *__restrict__ lm_prev, uint64_t *__restrict__ lm_cur,
-                  const uint64_t *__restrict__ visited, uint64_t *__restrict__ sigma,
-                  const uint64_t *__restrict__ active_prev, uint64_t *__restrict__ enable,
-                  unsigned long long *__restrict__ cnt, unsigned *__restrict__ wq) {
-  __shared__ uint32_t accs[FWD_THREADS / 32][2][DSK];
-  __shared__ uint32_t ovfs[FWD_THREADS / 32][2];
-  __shared__ uint16_t itemss[FWD_THREADS / 32][DENSE_ITEMS];
-  __shared__ int32_t sws[FWD_THREADS / 32][32];
-  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  uint32_t (*acc)[DSK] = accs[wid];
-  uint32_t *ovf2 = ovfs[wid];
-  uint16_t *items = itemss[wid];
-  int32_t *sw = sws[wid];
+k_fwd_heavy(int32_t n, int nseg, const int32_t *__restrict__ list, const unsigned *__restrict__ nlist,
+            const int32_t *__restrict__ seg_v, const int32_t *__restrict__ seg_b,
+            const int32_t *__restrict__ seg_e, const int32_t *__restrict__ col, const uint64_t *__restrict__ lm_prev,
+            uint64_t *__restrict__ lm_cur, const uint64_t *__restrict__ visited, uint64_t *__restrict__ sigma,
+            const uint64_t *__restrict__ active_prev, uint64_t *__restrict__ enable,
+            unsigned long long *__restrict__ cnt, unsigned *__restrict__ wq) {
+  __shared__ uint4 ents[FWD_THREADS / 32][ECAP_F];
+  __shared__ int8_t tabs[FWD_THREADS / 32][64];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  uint4 *ent = ents[wid];
+  int8_t *tab = tabs[wid];
   const uint64_t act = *active_prev & *enable;
+  const bool fit = counts_fit(enable[2], n);
   unsigned long long tri = 0ull;
-  uint64_t ovf = 0ull;
-  for (int s = grab(wq, 1); s < nseg; s = grab(wq, 1)) {
-    const int32_t v = seg_v[s];
-    const uint64_t pend = ~visited[v] & act;
-    if (!pend) continue;
-    for (int k = lane; k < 2 * DSK; k += 32) (&acc[0][0])[k] = 0u;
-    if (lane < 2) ovf2[lane] = 0u;
-    __syncwarp();
-    uint64_t newm = 0ull;
-    const int end = seg_e[s];
-    for (int base = seg_b[s]; base < end; base += 32) {
-      const int j = base + lane;
-      int32_t w = 0;
-      uint64_t m = 0ull;
-      if (j < end) {
-        w = col[j];
-        m = lm_prev[w] & pend;
-      }
-      newm |= m;
-      sw[lane] = w;
-      const int c = __popcll((long long)m);
-      tri += (unsigned long long)c;
-      int incl = c;
-#pragma unroll
-      for (int off = 1; off < 32; off <<= 1) {
-        const int y = __shfl_up_sync(FULL, incl, off);
-        if (lane >= off) incl += y;
-      }
-      const int N = __shfl_sync(FULL, incl, 31);
-      int k = incl - c;
-      while (m) {
-        const int t = __ffsll((long long)m) - 1;
-        m &= m - 1ull;
-        items[k++] = (uint16_t)((lane << 6) | t);
-      }
-      __syncwarp();
-      for (int r0 = 0; r0 < N; r0 += 32) {
-        const int i = r0 + lane;
-        if (i < N) {
-          const unsigned code = items[i];
-          const int t = (int)(code & 63u);
-          u64_limbs_atomic_add(acc, ovf2, t, sigma[(size_t)sw[code >> 6] * 64 + t]);
+  uint64_t ovf = 0ull, smax = 0ull;
+  const int total = list ? (int)*nlist : nseg;
+  if (act)
+    for (int i = grab(wq, 1); i < total; i = grab(wq, 1)) {
+      const int s = list ? list[i] : i;
+      const int32_t v = seg_v[s];
+      const int beg = seg_b[s], end = seg_e[s];
+      const uint64_t pend = ~visited[v] & act;
+      if (!pend) continue;
+      for (int b = beg; b < end; b += ECAP_F) {
+        const int ne = list_row(col, lm_prev, b, min(end, b + ECAP_F), pend, ent, tri);
+        if (!ne) continue;
+        const uint64_t nm = entries_or(ent, 0, ne);
+        const Packed pk = pack_lanes(nm, tab);
+        uint64_t s0 = 0ull, s1 = 0ull;
+        if (fit) count_entries<false>(ent, 0, ne, pk, sigma, s0, s1, ovf);
+        else count_entries<true>(ent, 0, ne, pk, sigma, s0, s1, ovf);
+        unsigned long long *dst = (unsigned long long *)(sigma + (size_t)v * 64);
+        if ((lane >> pk.glog) == 0 && pk.p0 >= 0) {
+          const unsigned long long x = (unsigned long long)s0, old = atomicAdd(dst + pk.p0, x);
+          if (old + x < x) ovf |= 1ull << pk.p0;
+          smax = old + x > smax ? old + x : smax;
         }
-      }
-      __syncwarp();
-    }
-    newm = warp_or64(newm);
-    if (newm) {
-      unsigned long long *dst = (unsigned long long *)(sigma + (size_t)v * 64);
-      const uint64_t ob = ((uint64_t)ovf2[1] << 32) | ovf2[0];
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int t = lane + 32 * h;
-        if ((newm >> t) & 1ull) {
-          const uint64_t x = ((uint64_t)acc[1][skew(t)] << 32) | acc[0][skew(t)];
-          const unsigned long long old = atomicAdd(dst + t, (unsigned long long)x);
-          if (((ob >> t) & 1ull) || old + x < old) ovf |= 1ull << t;
+        if (pk.p1 >= 0) {
+          const unsigned long long x = (unsigned long long)s1, old = atomicAdd(dst + pk.p1, x);
+          if (old + x < x) ovf |= 1ull << pk.p1;
+          smax = old + x > smax ? old + x : smax;
         }
+        if (lane == 0) atomicOr((unsigned long long *)&lm_cur[v], (unsigned long long)nm);
+        __syncwarp();
       }
-      if (lane == 0) atomicOr((unsigned long long *)&lm_cur[v], (unsigned long long)newm);
     }
-    __syncwarp();
-  }
   ovf = warp_or64(ovf);
   if (lane == 0 && ovf) atomicOr((unsigned long long *)(enable + 3), (unsigned long long)ovf);
   tri = warp_sum64(tri);
   if (lane == 0 && tri) atomicAdd(cnt, tri);
+  smax = warp_max64(smax);
+  if (lane == 0 && smax > 1ull) atomicMax((unsigned long long *)(enable + 2), (unsigned long long)smax);
 }
 
-// Also records, for the host, whether any heavy vertex has lanes at this level
-// (*hflag) and the lanes in which some heavy vertex is still unvisited (*hpend):
-// levels without heavy work then skip the heavy kernels.
-__global__ void k_fwd_heavy_fin(int nh, const int32_t *__restrict__ heavy,
+// Appends the segments [first, first + k) of the warp's threads to a list.
+__device__ __forceinline__ void append_segments(int first, int k, int32_t *__restrict__ list,
+                                                unsigned *__restrict__ count) {
+  const int lane = threadIdx.x & 31;
+  int incl = k;
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const int y = __shfl_up_sync(FULL, incl, off);
+    if (lane >= off) incl += y;
+  }
+  const int total = __shfl_sync(FULL, incl, 31);
+  if (!total) return;
+  unsigned base = 0u;
+  if (lane == 0) base = atomicAdd(count, (unsigned)total);
+  base = __shfl_sync(FULL, base, 0);
+  int32_t *out = list + base + incl - k;
+  if (k <= 8)
+    for (int i = 0; i < k; ++i) out[i] = first + i;
+  for (unsigned m = __ballot_sync(FULL, k > 8); m; m &= m - 1u) {  // a hub's: the whole warp
+    const int o = __ffs(m) - 1;
+    const int kk = __shfl_sync(FULL, k, o), ff = __shfl_sync(FULL, first, o), at = __shfl_sync(FULL, incl - k, o);
+    for (int i = lane; i < kk; i += 32) list[base + at + i] = ff + i;
+  }
+}
+
+// After the segments of a level: the heavy vertices' masks. Also records, for
+// the host, whether any heavy vertex has lanes at this level (*hflag) and the
+// lanes in which some heavy vertex is still unvisited (*hpend): levels without
+// heavy work then skip the heavy kernels; and lists the segments of the
+// vertices with lanes left for the next level (one atomic per segment taken is
+// what a level without work costs otherwise: 130,000 of them on R-MAT s20, 0.1
+// ms).
+__global__ void k_fwd_heavy_fin(int nh, const int32_t *__restrict__ heavy, const int32_t *__restrict__ hseg0,
                                 const uint64_t *__restrict__ lm_cur, uint64_t *__restrict__ visited,
                                 uint64_t *__restrict__ active_cur, unsigned long long *__restrict__ cnt,
-                                const uint64_t *__restrict__ sigma, uint64_t *__restrict__ enable,
-                                unsigned *__restrict__ hflag, unsigned long long *__restrict__ hpend,
-                                const int32_t *__restrict__ rp, int32_t *__restrict__ list_next,
-                                unsigned *__restrict__ vcnt_next, unsigned long long *__restrict__ vedges_next) {
-  // one warp per heavy vertex: the largest count of its new lanes is a warp
-  // maximum over the row (two loads per thread), not a chain of dependent loads
+                                const uint64_t *__restrict__ enable, unsigned *__restrict__ hflag,
+                                unsigned long long *__restrict__ hpend, const int32_t *__restrict__ rp,
+                                int32_t *__restrict__ list_next, unsigned *__restrict__ vcnt_next,
+                                unsigned long long *__restrict__ vedges_next, int32_t *__restrict__ seg_list,
+                                unsigned *__restrict__ seg_cnt) {
   const int lane = threadIdx.x & 31;
-  const int gw = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-  const int nw = (int)((gridDim.x * blockDim.x) >> 5);
+  const int h = blockIdx.x * blockDim.x + threadIdx.x;
   const uint64_t en = *enable;
-  uint64_t any_new = 0ull, pend_all = 0ull;
-  for (int h = gw; h < nh; h += nw) {
-    const int32_t v = heavy[h];
-    const uint64_t newm = lm_cur[v];
-    const uint64_t *row = sigma + (size_t)v * 64;
-    const uint64_t x0 = ((newm >> lane) & 1ull) ? row[lane] : 0ull;
-    const uint64_t x1 = ((newm >> (lane + 32)) & 1ull) ? row[lane + 32] : 0ull;
-    const uint64_t mx = warp_max64(x0 > x1 ? x0 : x1);
-    if (lane == 0) {
-      const uint64_t vis = visited[v];
-      pend_all |= ~(vis | newm) & en;
-      if (newm) {
-        visited[v] = vis | newm;
-        atomicAdd(cnt + 1, (unsigned long long)__popcll((long long)newm));
-        atomicMax((unsigned long long *)(enable + 2), (unsigned long long)mx);
-        if (list_next) {
-          list_next[atomicAdd(vcnt_next, 1u)] = v;
-          atomicAdd(vedges_next, (unsigned long long)(rp[v + 1] - rp[v]));
-        }
-      }
-    }
-    any_new |= newm;
+  uint64_t newm = 0ull, left = 0ull;
+  int32_t v = 0;
+  int first = 0, k = 0;
+  if (h < nh) {
+    v = heavy[h];
+    newm = lm_cur[v];
+    const uint64_t vis = visited[v];
+    if (newm) visited[v] = vis | newm;
+    left = ~(vis | newm) & en;
+    first = hseg0[h];
+    k = left ? hseg0[h + 1] - first : 0;
   }
+  append_segments(first, k, seg_list, seg_cnt);
+  const unsigned found = __ballot_sync(FULL, newm != 0ull);
+  if (found) {
+    unsigned pos = 0u;
+    if (lane == 0) pos = atomicAdd(vcnt_next, (unsigned)__popc(found));
+    pos = __shfl_sync(FULL, pos, 0);
+    if (newm) list_next[pos + __popc(found & ((1u << lane) - 1u))] = v;
+    if (vedges_next && newm) atomicAdd(vedges_next, (unsigned long long)(rp[v + 1] - rp[v]));
+  }
+  const unsigned long long rch = __reduce_add_sync(FULL, (unsigned)__popcll((long long)newm));
+  newm = warp_or64(newm);
+  left = warp_or64(left);
   if (lane == 0) {
-    if (any_new) {
-      atomicOr((unsigned long long *)active_cur, (unsigned long long)any_new);
+    if (newm) {
+      atomicAdd(cnt + 1, rch);
+      atomicOr((unsigned long long *)active_cur, (unsigned long long)newm);
       atomicOr(hflag, 1u);
     }
-    if (pend_all) atomicOr(hpend, (unsigned long long)pend_all);
+    if (left) atomicOr(hpend, (unsigned long long)left);
   }
 }
 
@@ -914,31 +842,97 @@ __global__ void k_pair_check(int count, int level, const int32_t *__restrict__ d
 }
 
 // -------------------------------------------------------------- backward --
-// Accumulator policies for the successor sums: the 128-bit window (used when
-// the batch's largest sigma is <= 2^44) and the general 192-bit one.
+// Exact sums of coefficients. Narrow: 96 bits in units of 2^-unit where the
+// batch's largest count allows (bc_common.cuh), and the coefficients are kept
+// in that form, 12 bytes (rows of 64 low words, then 64 high halves), so that
+// adding one is three instructions: with doubles, converted at every add, the
+// heavy segments of R-MAT s20's hub level kept the ALU pipe 87 % busy. Wide:
+// doubles in the counts' slots and the 192-bit window.
 struct NarrowAcc {
-  using A = Acc2;
-  static __device__ __forceinline__ A zero() { return acc2_zero(); }
-  static __device__ __forceinline__ void add(A &a, double x, unsigned &e) { acc2_add(a, x, e); }
-  static __device__ __forceinline__ Acc widen(const A &a) { return acc2_widen(a); }
+  using A = Acc3;
+  static constexpr bool narrow = true;
+  struct Rows {
+    using V = Acc3;
+    const uint64_t *__restrict__ p;
+    static __device__ __forceinline__ V zero() { return V{0u, 0u, 0u}; }
+    __device__ __forceinline__ V operator()(uint32_t w, int t) const {
+      const uint64_t *row = p + (size_t)w * 96;
+      const uint64_t lo = row[t];
+      return V{(uint32_t)lo, (uint32_t)(lo >> 32), reinterpret_cast<const uint32_t *>(row + 64)[t]};
+    }
+  };
+  static __device__ __forceinline__ A zero() { return A{0u, 0u, 0u}; }
+  static __device__ __forceinline__ void add(A &a, const Acc3 &x, unsigned &) { add_acc(a, x); }
+  static __device__ __forceinline__ void add_double(A &a, double x, int unit, unsigned &e) {
+    if (x != 0.0) acc3_add(a, (uint64_t)__double_as_longlong(x), 1075 - unit, e);
+  }
+  static __device__ __forceinline__ void put(uint64_t *rows, int32_t v, int t, const A &a) {
+    uint64_t *row = rows + (size_t)v * 96;
+    row[t] = (uint64_t)a.l0 | ((uint64_t)a.l1 << 32);
+    reinterpret_cast<uint32_t *>(row + 64)[t] = a.l2;
+  }
+  static __device__ __forceinline__ void put_double(uint64_t *rows, int32_t v, int t, double x, int unit, unsigned &e) {
+    A a = zero();
+    add_double(a, x, unit, e);
+    put(rows, v, t, a);
+  }
+  static __device__ __forceinline__ void add_acc(A &a, const A &b) { acc3_add3(a, b.l0, b.l1, b.l2); }
+  static __device__ __forceinline__ A shfl_xor(const A &a, int off) {
+    return A{__shfl_xor_sync(FULL, a.l0, off), __shfl_xor_sync(FULL, a.l1, off), __shfl_xor_sync(FULL, a.l2, off)};
+  }
+  static __device__ __forceinline__ A shfl_up(const A &a, int off) {
+    return A{__shfl_up_sync(FULL, a.l0, off), __shfl_up_sync(FULL, a.l1, off), __shfl_up_sync(FULL, a.l2, off)};
+  }
+  static __device__ __forceinline__ bool any(const A &a) { return (a.l0 | a.l1 | a.l2) != 0u; }
+  static __device__ __forceinline__ Acc widen(const A &a, int unit) { return acc3_widen(a, unit); }
 };
 struct WideAcc {
   using A = Acc;
+  static constexpr bool narrow = false;
+  using Rows = WordRows;
   static __device__ __forceinline__ A zero() { return acc_zero(); }
-  static __device__ __forceinline__ void add(A &a, double x, unsigned &e) { acc_add(a, x, e); }
-  static __device__ __forceinline__ Acc widen(const A &a) { return a; }
+  static __device__ __forceinline__ void add(A &a, uint64_t x, unsigned &e) {
+    acc_add(a, __longlong_as_double((long long)x), e);  // (0 adds nothing)
+  }
+  static __device__ __forceinline__ void add_double(A &a, double x, int, unsigned &e) { acc_add(a, x, e); }
+  static __device__ __forceinline__ void put_double(uint64_t *rows, int32_t v, int t, double x, int, unsigned &) {
+    rows[(size_t)v * 64 + t] = (uint64_t)__double_as_longlong(x);
+  }
+  static __device__ __forceinline__ void add_acc(A &a, const A &b) { acc_add_acc(a, b); }
+  static __device__ __forceinline__ A shfl_xor(const A &a, int off) {
+    return A{__shfl_xor_sync(FULL, a.w0, off), __shfl_xor_sync(FULL, a.w1, off), __shfl_xor_sync(FULL, a.w2, off)};
+  }
+  static __device__ __forceinline__ A shfl_up(const A &a, int off) {
+    return A{__shfl_up_sync(FULL, a.w0, off), __shfl_up_sync(FULL, a.w1, off), __shfl_up_sync(FULL, a.w2, off)};
+  }
+  static __device__ __forceinline__ bool any(const A &a) { return (a.w0 | a.w1 | a.w2) != 0ull; }
+  static __device__ __forceinline__ Acc widen(const A &a, int) { return a; }
 };
 
+// A pair without successors has delta = 0 and coefficient RN(1 / sigma), and
+// most pairs are such (the deepest level of each lane): for counts below
+// RECIPS the coefficient comes from a table (made for the batch's unit), and
+// the pair skips the ring. (No sink needs a zero delta: the rows and target
+// blocks start cleared.)
+constexpr int RECIPS = 2048;
+__global__ void k_recips(int unit, Acc3 *__restrict__ out) {
+  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  if (s >= RECIPS) return;
+  Acc3 a{0u, 0u, 0u};
+  unsigned e = 0u;
+  if (s > 0) NarrowAcc::add_double(a, coef_of(0.0, (uint64_t)s), unit, e);
+  out[s] = e ? Acc3{0u, 0u, 0u} : a;  // (a count above the batch's largest: never asked for)
+}
+
 // Finished (vertex, lane) pairs wait in a per-warp ring in shared memory until
-// 32 of them fill one warp-wide round of double arithmetic. The FP64 pipe is
-// charged per warp instruction whatever the number of active lanes, so the
-// rounds keep it busy with useful lanes only.
-constexpr int RING = 128;
-struct Ring {
-  int32_t v[RING];
-  int32_t t[RING];
-  double sum[RING];
+// 32 of them fill one warp-wide round of the per-vertex arithmetic (rounding
+// the sum, product, quotient), so its many instructions run with all threads.
+constexpr int RING = 96;  // up to 31 left over + 64 of one vertex
+template <class P> struct Ring {
+  typename P::A sum[RING];
   uint64_t sig[RING];
+  int32_t v[RING];
+  uint8_t t[RING];
 };
 
 // delta = RN(RN(sigma) * sum); a power-of-two sigma scales exactly (integer
@@ -953,645 +947,296 @@ __device__ __forceinline__ double delta_of(double sum, uint64_t sg) {
   return delta_rn(sg, sum);
 }
 
-// coef = RN(RN(1 + delta) / RN(sigma)) (power-of-two sigma: exact exponent shift).
-__device__ __forceinline__ double coef_round(double delta, uint64_t sg) { return coef_of(delta, sg); }
-
-__device__ __forceinline__ void ring_append(Ring &R, unsigned &tail, int32_t v, uint64_t lanes, const Acc &a0,
-                                            const Acc &a1, const uint64_t *__restrict__ row) {
-  const int lane = threadIdx.x & 31;
-  const unsigned lt = (1u << lane) - 1u;
-  const unsigned lo = (unsigned)lanes, hi = (unsigned)(lanes >> 32);
-  if ((lo >> lane) & 1u) {
-    const unsigned pos = (tail + __popc(lo & lt)) & (RING - 1);
-    R.v[pos] = v;
-    R.t[pos] = lane;
-    R.sum[pos] = acc_round(a0);
-    R.sig[pos] = row[lane];
-  }
-  tail += __popc(lo);
-  if ((hi >> lane) & 1u) {
-    const unsigned pos = (tail + __popc(hi & lt)) & (RING - 1);
-    R.v[pos] = v;
-    R.t[pos] = lane + 32;
-    R.sum[pos] = acc_round(a1);
-    R.sig[pos] = row[lane + 32];
-  }
-  tail += __popc(hi);
-}
-
-// One warp-wide round over ring records head..head+count-1 (count <= 32).
-// The coefficient's double bits overwrite sigma[v][t].
-__device__ __forceinline__ void ring_round(Ring &R, unsigned head, int count, uint64_t *__restrict__ sigma,
-                                           const Sink &sink, unsigned &e) {
+// One warp-wide round over `count` (<= 32) records from ring position head. The
+// coefficient's double bits overwrite sigma[v][t].
+template <class P>
+__device__ __forceinline__ void ring_round(Ring<P> &R, int head, int count, uint64_t *__restrict__ coef,
+                                           const Sink &sink, int unit, unsigned &e) {
   const int lane = threadIdx.x & 31;
   int32_t v = -1;
   double d = 0.0;
   if (lane < count) {
-    const unsigned pos = (head + lane) & (RING - 1);
+    int pos = head + lane;
+    pos -= pos >= RING ? RING : 0;
     v = R.v[pos];
-    const int32_t t = R.t[pos];
+    const int t = R.t[pos];
     const uint64_t sg = R.sig[pos];
-    d = delta_of(R.sum[pos], sg);
-    const double cf = coef_round(d, sg);
-    sigma[(size_t)v * 64 + t] = (uint64_t)__double_as_longlong(cf);
+    const typename P::A a = R.sum[pos];
+    if (P::any(a)) d = delta_of(acc_round(P::widen(a, unit)), sg);  // no successor: delta = 0
+    P::put_double(coef, v, t, coef_of(d, sg), unit, e);
     if (sink.delta_lm) sink.delta_lm[(size_t)v * 64 + t] = d;
     if (sink.tslot) sink_targets(sink, v, t, d);
   }
-  if (sink.acc) {
+  if (sink.acc && __any_sync(FULL, d != 0.0)) {
     // records of one vertex are consecutive: segmented exact inclusive scan
-    Acc a = acc_zero();
-    acc_add(a, d, e);
+    // (a dependency is at least 2^-ceil(log2 of the largest count), so it is a
+    // whole number of units too)
+    typename P::A a = P::zero();
+    P::add_double(a, d, unit, e);
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
-      Acc o;
-      o.w0 = __shfl_up_sync(FULL, a.w0, off);
-      o.w1 = __shfl_up_sync(FULL, a.w1, off);
-      o.w2 = __shfl_up_sync(FULL, a.w2, off);
+      const typename P::A o = P::shfl_up(a, off);
       const int32_t vo = __shfl_up_sync(FULL, v, off);
-      if (lane >= off && vo == v) acc_add_acc(a, o);
+      if (lane >= off && vo == v) P::add_acc(a, o);
     }
     const int32_t vn = __shfl_down_sync(FULL, v, 1);
-    if (v >= 0 && (lane == 31 || vn != v)) {
+    if (v >= 0 && (lane == 31 || vn != v) && P::any(a)) {
       Acc cur = sink.acc[v];
-      acc_add_acc(cur, a);
+      acc_add_acc(cur, P::widen(a, unit));
       sink.acc[v] = cur;
     }
   }
 }
 
-// Lane compaction: thread i of the warp takes the i-th set lane of `lanes`
-// (and the (i+32)-th when more than 32 lanes are set); -1 when absent.
-__device__ __forceinline__ void compact_lanes(uint64_t lanes, int &p0, int &p1) {
-  const int lane = threadIdx.x & 31;
-  const unsigned lo = (unsigned)lanes, hi = (unsigned)(lanes >> 32);
-  const int nlo = __popc(lo), ntot = nlo + __popc(hi);
-  auto nth = [&](int i) -> int {
-    if (i >= ntot) return -1;
-    if (i < nlo) return (int)__fns(lo, 0u, i + 1);
-    return 32 + (int)__fns(hi, 0u, i - nlo + 1);
-  };
-  p0 = nth(lane);
-  p1 = nth(lane + 32);
-}
-
-// Exact sums over the successors of v (neighbours one level deeper in the same
-// lane) for the compacted lanes p0 (and p1 when `two`).
+// The finished lanes of v (their sums in the threads of group 0; sg0 / sg1: the
+// counts of the thread's lanes): a lane without successors gets its tabulated
+// coefficient, the others go into the ring, with a round whenever 32 wait.
 template <class P>
-__device__ __forceinline__ void gather_successors(int beg, int end, uint64_t lanes, const uint64_t *__restrict__ col_lm,
-                                                  const int32_t *__restrict__ col, const uint64_t *__restrict__ sigma,
-                                                  int p0, int p1, bool two, typename P::A &a0, typename P::A &a1,
-                                                  unsigned &e) {
+__device__ __forceinline__ void ring_put(Ring<P> &R, int &head, int &have, int32_t v, const Packed &pk,
+                                         const typename P::A &a0, const typename P::A &a1, uint64_t sg0, uint64_t sg1,
+                                         uint64_t *__restrict__ coef, const Acc3 *__restrict__ recips,
+                                         const Sink &sink, int unit, unsigned &e) {
   const int lane = threadIdx.x & 31;
-  const int q0 = p0 < 0 ? 0 : p0, q1 = p1 < 0 ? 0 : p1;
-  const uint64_t b0 = p0 < 0 ? 0ull : (1ull << q0), b1 = p1 < 0 ? 0ull : (1ull << q1);
-  for (int base = beg; base < end; base += 32) {
-    const int j = base + lane;
-    int32_t w = 0;
-    uint64_t m = 0ull;
-    if (j < end) {
-      w = col[j];
-      m = col_lm[w] & lanes;
-    }
-    unsigned bal = __ballot_sync(FULL, m != 0ull);
-    while (bal) {
-      uint64_t mk[UNR];
-      int32_t wk[UNR];
-      take(bal, m, w, mk, wk);
-      uint64_t x0[UNR];
+  const unsigned lt = (1u << lane) - 1u;
 #pragma unroll
-      for (int k = 0; k < UNR; ++k) x0[k] = (mk[k] & b0) ? sigma[(size_t)wk[k] * 64 + q0] : 0ull;
-#pragma unroll
-      for (int k = 0; k < UNR; ++k) P::add(a0, __longlong_as_double((long long)x0[k]), e);
-      if (two) {
-        uint64_t x1[UNR];
-#pragma unroll
-        for (int k = 0; k < UNR; ++k) x1[k] = (mk[k] & b1) ? sigma[(size_t)wk[k] * 64 + q1] : 0ull;
-#pragma unroll
-        for (int k = 0; k < UNR; ++k) P::add(a1, __longlong_as_double((long long)x1[k]), e);
+  for (int h = 0; h < 2; ++h) {
+    if (h && !pk.two) break;
+    const int t = h ? pk.p1 : ((lane >> pk.glog) == 0 ? pk.p0 : -1);
+    const typename P::A &a = h ? a1 : a0;
+    const uint64_t sg = h ? sg1 : sg0;
+    bool on = t >= 0;
+    if constexpr (P::narrow) {
+      if (on && sg < (uint64_t)RECIPS && !P::any(a)) {
+        P::put(coef, v, t, recips[sg]);
+        on = false;
       }
     }
+    const unsigned m = __ballot_sync(FULL, on);
+    if (on) {
+      int pos = head + have + __popc(m & lt);
+      pos -= pos >= RING ? RING : 0;
+      R.v[pos] = v;
+      R.t[pos] = (uint8_t)t;
+      R.sum[pos] = a;
+      R.sig[pos] = sg;
+    }
+    have += __popc(m);
+  }
+  __syncwarp();
+  while (have >= 32) {
+    ring_round<P>(R, head, 32, coef, sink, unit, e);
+    head += 32;
+    head -= head >= RING ? RING : 0;
+    have -= 32;
+    __syncwarp();
   }
 }
 
-// Appends the finished lanes of v (compacted positions p0, p1) to the ring.
-__device__ __forceinline__ void ring_append_c(Ring &R, unsigned &tail, int32_t v, uint64_t lanes, int p0, int p1,
-                                              const Acc &a0, const Acc &a1, const uint64_t *__restrict__ row) {
-  const int lane = threadIdx.x & 31;
-  const int ntot = __popcll((long long)lanes);
-  if (p0 >= 0) {
-    const unsigned pos = (tail + lane) & (RING - 1);
-    R.v[pos] = v;
-    R.t[pos] = p0;
-    R.sum[pos] = acc_round(a0);
-    R.sig[pos] = row[p0];
-  }
-  if (p1 >= 0) {
-    const unsigned pos = (tail + 32 + lane) & (RING - 1);
-    R.v[pos] = v;
-    R.t[pos] = p1;
-    R.sum[pos] = acc_round(a1);
-    R.sig[pos] = row[p1];
-  }
-  tail += (unsigned)ntot;
-}
-
+// Exact sums over entries [f, e) in the packed lanes, totals in group 0.
 template <class P>
-__global__ void __launch_bounds__(FWD_THREADS)
-k_bwd_light(int32_t n, const int32_t *__restrict__ list_l, const unsigned *__restrict__ vcnt_l,
-            const int32_t *__restrict__ rp,
+__device__ __forceinline__ void coef_entries(const uint4 *ent, int f, int e, const Packed &pk,
+                                             const uint64_t *__restrict__ coef, typename P::A &a0,
+                                             typename P::A &a1, unsigned &err) {
+  entries_sum(ent, f, e, pk, typename P::Rows{coef}, [&](const typename P::Rows::V &x) { P::add(a0, x, err); },
+              [&](const typename P::Rows::V &x) { P::add(a1, x, err); });
+}
+template <class P> __device__ __forceinline__ void group_sum(typename P::A &a, int glog) {
+  for (int off = 1 << glog; off < 32; off <<= 1) P::add_acc(a, P::shfl_xor(a, off));
+}
+
+// The light vertices of level l (listed by the forward pass), a warp taking gsz
+// at a time.
+template <class P>
+__global__ void __launch_bounds__(FWD_THREADS, P::narrow ? BWD_MIN_BLOCKS : 3)
+k_bwd_light(const int32_t *__restrict__ list_l, const unsigned *__restrict__ vcnt_l, const int32_t *__restrict__ rp,
             const int32_t *__restrict__ col, const uint64_t *__restrict__ lm_cur, const uint64_t *__restrict__ lm_next,
-            uint64_t *__restrict__ sigma, Sink sink, unsigned *__restrict__ err, unsigned *__restrict__ wq,
-            int heavy_deg, uint64_t keep, int gsz) {
-  __shared__ Ring rings[FWD_THREADS / 32];
-  Ring &R = rings[threadIdx.x >> 5];
-  unsigned head = 0u, tail = 0u;
-  unsigned e = 0u;
-  // a small level walks its vertex list; a large one scans the vertex ids in
-  // order (adjacent rows, sequential CSR reads). A warp takes gsz <= 32
-  // vertices at a time, loads their masks and row bounds at once (one per
-  // thread) and walks only the light ones with lanes at this level (smaller
-  // takes on small graphs spread a level over more warps).
-  const int nv = vcnt_l ? (int)*vcnt_l : n;
-  const bool by_list = vcnt_l && (int64_t)nv * 16 <= (int64_t)n;
-  const int total = by_list ? nv : n;
-  const int lane_id = threadIdx.x & 31;
-  for (int base = grab(wq, gsz); base < total; base = grab(wq, gsz)) {
-    const int ii = base + lane_id;
-    int32_t hv = 0;
-    uint64_t hl = 0ull;
-    int hb = 0, he = 0;
-    if (lane_id < gsz && ii < total) {
-      hv = by_list ? list_l[ii] : ii;
-      hl = lm_cur[hv] & keep;
-      if (hl) {
-        hb = rp[hv];
-        he = rp[hv + 1];
-        if (he - hb > heavy_deg) hl = 0ull;  // heavy: its segments' kernels
-      }
-    }
-    for (unsigned todo = __ballot_sync(FULL, hl != 0ull); todo; todo &= todo - 1u) {
-      const int iv = __ffs(todo) - 1;
-      const int32_t v = __shfl_sync(FULL, hv, iv);
-      const uint64_t lanes = __shfl_sync(FULL, hl, iv);
-      const int beg = __shfl_sync(FULL, hb, iv), end = __shfl_sync(FULL, he, iv);
-      // thread t owns lanes t and t + 32 (no compaction: cheapest per vertex)
-      const int lane = threadIdx.x & 31;
-      const int p0 = ((lanes >> lane) & 1ull) ? lane : -1;
-      const int p1 = ((lanes >> (lane + 32)) & 1ull) ? lane + 32 : -1;
-      typename P::A a0 = P::zero(), a1 = P::zero();
-      gather_successors<P>(beg, end, lanes, lm_next, col, sigma, p0, p1, (lanes >> 32) != 0ull, a0, a1, e);
-      ring_append(R, tail, v, lanes, P::widen(a0), P::widen(a1), sigma + (size_t)v * 64);
-      __syncwarp();
-      while (tail - head >= 32u) {
-        ring_round(R, head, 32, sigma, sink, e);
-        head += 32u;
-        __syncwarp();
-      }
-    }
-  }
-  if (tail != head) ring_round(R, head, (int)(tail - head), sigma, sink, e);
-  if (e) atomicOr(err, e);
-}
-
-// Heavy vertices: one warp per segment (taken dynamically) writes the partial
-// sums of the vertex's active lanes to part[s][lane].
-template <class P>
-__global__ void __launch_bounds__(FWD_THREADS)
-k_bwd_heavy_seg(int nseg, const int32_t *__restrict__ seg_v, const int32_t *__restrict__ seg_b,
-                const int32_t *__restrict__ seg_e, const int32_t *__restrict__ col,
-                const uint64_t *__restrict__ lm_cur, const uint64_t *__restrict__ lm_next,
-                const uint64_t *__restrict__ sigma, Acc *__restrict__ part, unsigned *__restrict__ err,
-                unsigned *__restrict__ wq, uint64_t keep) {
-  unsigned e = 0u;
-  for (int s = grab(wq, 1); s < nseg; s = grab(wq, 1)) {
-      const int32_t v = seg_v[s];
-      const uint64_t lanes = lm_cur[v] & keep;
-      if (!lanes) continue;
-      int p0, p1;
-      compact_lanes(lanes, p0, p1);
-      const bool two = __popcll((long long)lanes) > 32;
-      typename P::A a0 = P::zero(), a1 = P::zero();
-      gather_successors<P>(seg_b[s], seg_e[s], lanes, lm_next, col, sigma, p0, p1, two, a0, a1, e);
-      if (p0 >= 0) part[(size_t)s * 64 + p0] = P::widen(a0);
-      if (p1 >= 0) part[(size_t)s * 64 + p1] = P::widen(a1);
-    }
-  if (e) atomicOr(err, e);
-}
-
-__global__ void __launch_bounds__(FWD_THREADS)
-k_bwd_heavy_fin(int nh, const int32_t *__restrict__ heavy, const int32_t *__restrict__ hseg0,
-                const uint64_t *__restrict__ lm_cur, uint64_t *__restrict__ sigma,
-                const Acc *__restrict__ part, Sink sink, unsigned *__restrict__ err, unsigned *__restrict__ wq, uint64_t keep) {
-  __shared__ Ring rings[FWD_THREADS / 32];
-  Ring &R = rings[threadIdx.x >> 5];
-  unsigned head = 0u, tail = 0u;
-  unsigned e = 0u;
-  for (int h = grab(wq, 1); h < nh; h = grab(wq, 1)) {
-    const int32_t v = heavy[h];
-    const uint64_t lanes = lm_cur[v] & keep;
-    if (!lanes) continue;
-    int p0, p1;
-    compact_lanes(lanes, p0, p1);
-    Acc a0 = acc_zero(), a1 = acc_zero();
-    for (int s = hseg0[h]; s < hseg0[h + 1]; ++s) {
-      if (p0 >= 0) acc_add_acc(a0, part[(size_t)s * 64 + p0]);
-      if (p1 >= 0) acc_add_acc(a1, part[(size_t)s * 64 + p1]);
-    }
-    ring_append_c(R, tail, v, lanes, p0, p1, a0, a1, sigma + (size_t)v * 64);
-    __syncwarp();
-    while (tail - head >= 32u) {
-      ring_round(R, head, 32, sigma, sink, e);
-      head += 32u;
-      __syncwarp();
-    }
-  }
-  if (tail != head) ring_round(R, head, (int)(tail - head), sigma, sink, e);
-  if (e) atomicOr(err, e);
-}
-
-// ------------------------------------------- packed fixed-point backward --
-// Used when the batch's largest sigma is <= 2^44: coefficients are stored as
-// exact 128-bit fixed-point limbs, so a successor add is a 4-limb carry chain.
-// A vertex at a level usually has few lanes L; the warp is split into 32/G
-// groups of G >= |L| threads and each group takes a different listed
-// successor per step (thread (g, s) owns the s-th active lane).
-
-__device__ __forceinline__ void acc2_add_u4(Acc2 &a, const uint4 &x) { acc2_add4(a, x.x, x.y, x.z, x.w); }
-
-__device__ __forceinline__ void acc2_shfl_xor_add(Acc2 &a, int off) {
-  const uint32_t o0 = __shfl_xor_sync(FULL, a.l0, off), o1 = __shfl_xor_sync(FULL, a.l1, off);
-  const uint32_t o2 = __shfl_xor_sync(FULL, a.l2, off), o3 = __shfl_xor_sync(FULL, a.l3, off);
-  acc2_add4(a, o0, o1, o2, o3);
-}
-
-// Packed successor sums over double coefficients held in the sigma slots
-// (coefficient of (w, t) at sigma[w][t] once w's level is done).
-__device__ __forceinline__ void gather_packed(int beg, int end, uint64_t lanes, const uint64_t *__restrict__ lm_next,
-                                              const int32_t *__restrict__ col, const uint64_t *__restrict__ coef,
-                                              const Packed &pk, int32_t *list, Acc2 &a0, Acc2 &a1, unsigned &e) {
-  const int lane = threadIdx.x & 31;
-  const int NG = 32 >> pk.glog, g = lane >> pk.glog;
-  const uint64_t b0 = pk.p0 >= 0 ? (1ull << pk.p0) : 0ull, b1 = pk.p1 >= 0 ? (1ull << pk.p1) : 0ull;
-  const int q0 = pk.p0 < 0 ? 0 : pk.p0, q1 = pk.p1 < 0 ? 0 : pk.p1;
-  for (int base = beg; base < end; base += 32) {
-    const int j = base + lane;
-    int32_t w = 0;
-    uint64_t m = 0ull;
-    if (j < end) {
-      w = col[j];
-      m = lm_next[w] & lanes;
-    }
-    const unsigned bal = __ballot_sync(FULL, m != 0ull);
-    const int cnt = __popc(bal);
-    if (m != 0ull) list[__popc(bal & ((1u << lane) - 1u))] = lane;
-    __syncwarp();
-    for (int r = 0; r < cnt; r += 2 * NG) {
-      const int i0 = r + g, i1 = r + NG + g;
-      const bool h0 = i0 < cnt, h1 = i1 < cnt;
-      const int s0 = h0 ? list[i0] : 0, s1 = h1 ? list[i1] : 0;
-      const uint64_t m0 = __shfl_sync(FULL, m, s0), m1 = __shfl_sync(FULL, m, s1);
-      const int32_t w0 = __shfl_sync(FULL, w, s0), w1 = __shfl_sync(FULL, w, s1);
-      const uint64_t x0 = (h0 && (m0 & b0)) ? coef[(size_t)w0 * 64 + q0] : 0ull;
-      const uint64_t x1 = (h1 && (m1 & b0)) ? coef[(size_t)w1 * 64 + q0] : 0ull;
-      if (pk.two) {
-        const uint64_t y0 = (h0 && (m0 & b1)) ? coef[(size_t)w0 * 64 + q1] : 0ull;
-        const uint64_t y1 = (h1 && (m1 & b1)) ? coef[(size_t)w1 * 64 + q1] : 0ull;
-        acc2_add(a1, __longlong_as_double((long long)y0), e);
-        acc2_add(a1, __longlong_as_double((long long)y1), e);
-      }
-      acc2_add(a0, __longlong_as_double((long long)x0), e);
-      acc2_add(a0, __longlong_as_double((long long)x1), e);
-    }
-    __syncwarp();
-  }
-  for (int off = 1 << pk.glog; off < 32; off <<= 1) acc2_shfl_xor_add(a0, off);
-}
-
-// Finished lanes of v (threads of group 0 own them) into the ring.
-__device__ __forceinline__ void ring_append_fx(Ring &R, unsigned &tail, int32_t v, uint64_t lanes, const Packed &pk,
-                                               const Acc2 &a0, const Acc2 &a1, const uint64_t *__restrict__ row) {
-  const int lane = threadIdx.x & 31;
-  if ((lane >> pk.glog) == 0 && pk.p0 >= 0) {
-    const unsigned pos = (tail + lane) & (RING - 1);
-    R.v[pos] = v;
-    R.t[pos] = pk.p0;
-    R.sum[pos] = acc_round(acc2_widen(a0));
-    R.sig[pos] = row[pk.p0];
-  }
-  if (pk.p1 >= 0) {
-    const unsigned pos = (tail + 32 + lane) & (RING - 1);
-    R.v[pos] = v;
-    R.t[pos] = pk.p1;
-    R.sum[pos] = acc_round(acc2_widen(a1));
-    R.sig[pos] = row[pk.p1];
-  }
-  tail += (unsigned)__popcll((long long)lanes);
-}
-
-__global__ void __launch_bounds__(FWD_THREADS, BWD_MIN_BLOCKS)
-k_bwd_light_fx(int32_t n, const int32_t *__restrict__ list_l, const unsigned *__restrict__ vcnt_l,
-               const int32_t *__restrict__ rp,
-               const int32_t *__restrict__ col, const uint64_t *__restrict__ lm_cur,
-               const uint64_t *__restrict__ lm_next, uint64_t *__restrict__ sigma, Sink sink,
-               unsigned *__restrict__ err, unsigned *__restrict__ wq, int heavy_deg, uint64_t keep, int gsz) {
-  __shared__ Ring rings[FWD_THREADS / 32];
-  __shared__ int32_t lists[FWD_THREADS / 32][32];
+            const uint64_t *__restrict__ sigma, uint64_t *__restrict__ coef, const Acc3 *__restrict__ recips, Sink sink,
+            unsigned *__restrict__ err, unsigned *__restrict__ wq, int heavy_deg, uint64_t keep, int gsz, int unit) {
+  __shared__ Ring<P> rings[FWD_THREADS / 32];
+  __shared__ uint4 ents[FWD_THREADS / 32][ECAP_B];
   __shared__ int8_t tabs[FWD_THREADS / 32][64];
-  Ring &R = rings[threadIdx.x >> 5];
-  int32_t *list = lists[threadIdx.x >> 5];
-  int8_t *tab = tabs[threadIdx.x >> 5];
-  unsigned head = 0u, tail = 0u;
+  __shared__ uint8_t owns[FWD_THREADS / 32][32];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  Ring<P> &R = rings[wid];
+  uint4 *ent = ents[wid];
+  int8_t *tab = tabs[wid];
+  int head = 0, have = 0;
   unsigned e = 0u;
-  // a small level walks its vertex list; a large one scans the vertex ids in
-  // order (adjacent rows, sequential CSR reads). A warp takes gsz <= 32
-  // vertices at a time, loads their masks and row bounds at once (one per
-  // thread) and walks only the light ones with lanes at this level (smaller
-  // takes on small graphs spread a level over more warps).
-  const int nv = vcnt_l ? (int)*vcnt_l : n;
-  const bool by_list = vcnt_l && (int64_t)nv * 16 <= (int64_t)n;
-  const int total = by_list ? nv : n;
-  const int lane_id = threadIdx.x & 31;
+  unsigned long long tri = 0ull;  // (counted by the forward pass)
+  const int total = (int)*vcnt_l;
   for (int base = grab(wq, gsz); base < total; base = grab(wq, gsz)) {
-    const int ii = base + lane_id;
-    int32_t hv = 0;
-    uint64_t hl = 0ull;
-    int hb = 0, he = 0;
-    if (lane_id < gsz && ii < total) {
-      hv = by_list ? list_l[ii] : ii;
-      hl = lm_cur[hv] & keep;
-      if (hl) {
-        hb = rp[hv];
-        he = rp[hv + 1];
-        if (he - hb > heavy_deg) hl = 0ull;  // heavy: its segments' kernels
+    int32_t v = -1;
+    int hb = 0, d = 0;
+    uint64_t lanes = 0ull;
+    if (lane < gsz && base + lane < total) {
+      v = list_l[base + lane];
+      lanes = lm_cur[v] & keep;
+      hb = rp[v];
+      d = rp[v + 1] - hb;
+      if (d > heavy_deg) lanes = 0ull;  // heavy: its segments' kernels
+    }
+    // sums of one vertex (thread k holds it): entries [f, e), or for a row
+    // above the list's capacity piece by piece
+    auto finish = [&](int k, int f, int en, bool pieces) {
+      const int32_t u = __shfl_sync(FULL, v, k);
+      const uint64_t ul = __shfl_sync(FULL, lanes, k);
+      const Packed pk = pack_lanes(ul, tab);
+      const uint64_t *row = sigma + (size_t)u * 64;
+      const uint64_t sg0 = ((lane >> pk.glog) == 0 && pk.p0 >= 0) ? row[pk.p0] : 0ull;
+      const uint64_t sg1 = pk.p1 >= 0 ? row[pk.p1] : 0ull;
+      typename P::A a0 = P::zero(), a1 = P::zero();
+      if (pieces) {
+        const int b = __shfl_sync(FULL, hb, k), end = b + __shfl_sync(FULL, d, k);
+        for (int j = b; j < end; j += ECAP_B) {
+          const int ne = list_row(col, lm_next, j, min(end, j + ECAP_B), ul, ent, tri);
+          coef_entries<P>(ent, 0, ne, pk, coef, a0, a1, e);
+          __syncwarp();
+        }
+        group_sum<P>(a0, pk.glog);
+      } else if (f < en) {
+        coef_entries<P>(ent, f, en, pk, coef, a0, a1, e);
+        group_sum<P>(a0, pk.glog);
       }
-    }
-    for (unsigned todo = __ballot_sync(FULL, hl != 0ull); todo; todo &= todo - 1u) {
-      const int iv = __ffs(todo) - 1;
-      const int32_t v = __shfl_sync(FULL, hv, iv);
-      const uint64_t lanes = __shfl_sync(FULL, hl, iv);
-      const int beg = __shfl_sync(FULL, hb, iv), end = __shfl_sync(FULL, he, iv);
-      const Packed pk = pack_lanes(lanes, tab);
-      Acc2 a0 = acc2_zero(), a1 = acc2_zero();
-      gather_packed(beg, end, lanes, lm_next, col, sigma, pk, list, a0, a1, e);
-      ring_append_fx(R, tail, v, lanes, pk, a0, a1, sigma + (size_t)v * 64);
-      __syncwarp();
-      while (tail - head >= 32u) {
-        ring_round(R, head, 32, sigma, sink, e);
-        head += 32u;
-        __syncwarp();
-      }
-    }
-  }
-  if (tail != head) ring_round(R, head, (int)(tail - head), sigma, sink, e);
-  if (e) atomicOr(err, e);
-}
-
-__global__ void __launch_bounds__(FWD_THREADS, BWD_MIN_BLOCKS)
-k_bwd_heavy_seg_fx(int nseg, const int32_t *__restrict__ seg_v, const int32_t *__restrict__ seg_b,
-                   const int32_t *__restrict__ seg_e, const int32_t *__restrict__ col,
-                   const uint64_t *__restrict__ lm_cur, const uint64_t *__restrict__ lm_next,
-                   const uint64_t *__restrict__ coef, uint4 *__restrict__ part, unsigned *__restrict__ wq,
-                   unsigned *__restrict__ err, uint64_t keep) {
-  __shared__ int32_t lists[FWD_THREADS / 32][32];
-  __shared__ int8_t tabs[FWD_THREADS / 32][64];
-  int32_t *list = lists[threadIdx.x >> 5];
-  int8_t *tab = tabs[threadIdx.x >> 5];
-  const int lane = threadIdx.x & 31;
-  unsigned e = 0u;
-  for (int s = grab(wq, 1); s < nseg; s = grab(wq, 1)) {
-      const int32_t v = seg_v[s];
-      const uint64_t lanes = lm_cur[v] & keep;
-      if (!lanes) continue;
-      const Packed pk = pack_lanes(lanes, tab);
-      Acc2 a0 = acc2_zero(), a1 = acc2_zero();
-      gather_packed(seg_b[s], seg_e[s], lanes, lm_next, col, coef, pk, list, a0, a1, e);
-      if ((lane >> pk.glog) == 0 && pk.p0 >= 0) part[(size_t)s * 64 + pk.p0] = make_uint4(a0.l0, a0.l1, a0.l2, a0.l3);
-      if (pk.p1 >= 0) part[(size_t)s * 64 + pk.p1] = make_uint4(a1.l0, a1.l1, a1.l2, a1.l3);
-    }
-  if (e) atomicOr(err, e);
-}
-
-// Heavy segments with per-lane item loops (see k_fwd_heavy_lane): thread i
-// owns the i-th (and (i+32)-th) lane of v at this level and adds, exactly, the
-// coefficients of the successors in its own lanes only; the partial sums go to
-// part[s][lane] as in k_bwd_heavy_seg_fx.
-__device__ __forceinline__ void acc2_add_nz(Acc2 &a, uint64_t bits, unsigned &err) {
-  const uint32_t hi = (uint32_t)(bits >> 32), lo = (uint32_t)bits;
-  const int p = (int)(hi >> 20) - 979;  // lowest mantissa bit, in units of 2^-96
-  if ((unsigned)p > 75u) {
-    err |= ERR_RANGE;
-    return;
-  }
-  const uint32_t mh = (hi & 0x000FFFFFu) | 0x00100000u;
-  const int r = p & 31, q = p >> 5;
-  const uint32_t c0 = lo << r;
-  const uint32_t c1 = __funnelshift_l(lo, mh, r);
-  const uint32_t c2 = __funnelshift_l(mh, 0u, r);
-  const uint32_t t0 = (q == 0) ? c0 : 0u;
-  const uint32_t t1 = (q == 0) ? c1 : ((q == 1) ? c0 : 0u);
-  const uint32_t t2 = (q == 0) ? c2 : ((q == 1) ? c1 : c0);
-  const uint32_t t3 = (q == 1) ? c2 : ((q == 2) ? c1 : 0u);
-  acc2_add4(a, t0, t1, t2, t3);
-}
-
-// Adds the coefficient x (its double bits; 0 is never listed) exactly to lane
-// t's sum in shared memory: four 32-bit limbs acc[0..3][t], value
-// (l3:l2:l1:l0) * 2^-96, the 128-bit window of acc2_add. The mantissa lands on
-// limbs q..q+2 (q from its exponent); each limb is added with a shared-memory
-// atomic and its carry passed to the next limb, so concurrent adds to the same
-// lane sum exactly (integer addition, any order).
-__device__ __forceinline__ void acc_limbs_atomic_add(uint32_t (*acc)[DSK], int t, uint64_t bits, unsigned &err) {
-  const uint32_t hi = (uint32_t)(bits >> 32), lo = (uint32_t)bits;
-  const int p = (int)(hi >> 20) - 979;  // lowest mantissa bit, in units of 2^-96
-  if ((unsigned)p > 75u) {
-    err |= ERR_RANGE;
-    return;
-  }
-  const uint32_t mh = (hi & 0x000FFFFFu) | 0x00100000u;
-  const int r = p & 31, q = p >> 5;
-  const uint32_t c[3] = {lo << r, __funnelshift_l(lo, mh, r), __funnelshift_l(mh, 0u, r)};
-  uint32_t carry = 0u;
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const int limb = q + k;
-    if (limb > 3) break;  // inside the window the sum never leaves 128 bits
-    const uint32_t x = (k < 3 ? c[k] : 0u) + carry;
-    carry = (k < 3 && x < carry) ? 1u : 0u;  // c[k] + carry wrapped (then x == 0)
-    if (x) {
-      const uint32_t old = atomicAdd(&acc[limb][skew(t)], x);
-      carry |= (old + x < x) ? 1u : 0u;
-    }
-    if (k >= 2 && !carry) break;
-  }
-}
-
-// Heavy segments with the successors' (coefficient, lane) items spread over
-// all 32 threads. The items of a 32-neighbour chunk are listed in neighbour
-// order (a successor's lanes are consecutive, so the 32 loads of a round touch
-// two or three coefficient rows); each thread takes one item per round and
-// adds it to the lane's exact sum in shared memory (acc_limbs_atomic_add). No
-// lane slot idles, unlike a 64-lane step per successor, of which a hub-level
-// successor fills about 13.
-__global__ void __launch_bounds__(FWD_THREADS, 4)
-k_bwd_heavy_seg_dense(int nseg, const int32_t *__restrict__ seg_v, const int32_t *__restrict__ seg_b,
-                      const int32_t *__restrict__ seg_e, const int32_t *__restrict__ col,
-                      const uint64_t *__restrict__ lm_cur, const uint64_t *__restrict__ lm_next,
-                      const uint64_t *__restrict__ coef, uint4 *__restrict__ part, unsigned *__restrict__ wq,
-                      unsigned *__restrict__ err, uint64_t keep) {
-  __shared__ uint32_t accs[FWD_THREADS / 32][4][DSK];
-  __shared__ uint16_t itemss[FWD_THREADS / 32][DENSE_ITEMS];
-  __shared__ int32_t sws[FWD_THREADS / 32][32];
-  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  uint32_t (*acc)[DSK] = accs[wid];
-  uint16_t *items = itemss[wid];
-  int32_t *sw = sws[wid];
-  unsigned e = 0u;
-  for (int s = grab(wq, 1); s < nseg; s = grab(wq, 1)) {
-    const int32_t v = seg_v[s];
-    const uint64_t lanes = lm_cur[v] & keep;
-    if (!lanes) continue;
-    for (int k = lane; k < 4 * DSK; k += 32) (&acc[0][0])[k] = 0u;
-    __syncwarp();
-    const int end = seg_e[s];
-    for (int base = seg_b[s]; base < end; base += 32) {
-      const int j = base + lane;
-      int32_t w = 0;
-      uint64_t m = 0ull;
-      if (j < end) {
-        w = col[j];
-        m = lm_next[w] & lanes;
-      }
-      sw[lane] = w;
-      const int c = __popcll((long long)m);
-      int incl = c;
+      ring_put<P>(R, head, have, u, pk, a0, a1, sg0, sg1, coef, recips, sink, unit, e);
+    };
+    for (unsigned r = __ballot_sync(FULL, lanes != 0ull && d == 0); r; r &= r - 1u)
+      finish(__ffs(r) - 1, 0, 0, false);  // (directed graphs: no out-neighbour)
+    unsigned todo = __ballot_sync(FULL, lanes != 0ull && d > 0 && d <= ECAP_B);
+    while (todo) {
+      const int dd = ((todo >> lane) & 1u) ? d : 0;
+      int incl = dd;
 #pragma unroll
       for (int off = 1; off < 32; off <<= 1) {
         const int y = __shfl_up_sync(FULL, incl, off);
         if (lane >= off) incl += y;
       }
-      const int N = __shfl_sync(FULL, incl, 31);
-      int k = incl - c;
-      while (m) {  // this neighbour's items: neighbour in bits 6..10, lane in bits 0..5
-        const int t = __ffsll((long long)m) - 1;
-        m &= m - 1ull;
-        items[k++] = (uint16_t)((lane << 6) | t);
-      }
-      __syncwarp();
-      for (int r0 = 0; r0 < N; r0 += 32) {
-        const int i = r0 + lane;
-        if (i < N) {
-          const unsigned code = items[i];
-          const int t = (int)(code & 63u);
-          const uint64_t x = coef[(size_t)sw[code >> 6] * 64 + t];
-          acc_limbs_atomic_add(acc, t, x, e);
-        }
+      const unsigned sub = __ballot_sync(FULL, ((todo >> lane) & 1u) && incl <= ECAP_B);
+      todo &= ~sub;
+      int first;
+      const int ne = list_rows(col, lm_next, hb, ((sub >> lane) & 1u) ? d : 0, lanes, ent, owns[wid], first, tri);
+      for (unsigned r = sub; r;) {
+        const int k = __ffs(r) - 1;
+        r &= r - 1u;
+        const int f = __shfl_sync(FULL, first, k), en = r ? __shfl_sync(FULL, first, __ffs(r) - 1) : ne;
+        finish(k, f, en, false);
       }
       __syncwarp();
     }
-    const int a0 = skew(lane), a1 = skew(lane + 32);
-    if ((lanes >> lane) & 1ull) part[(size_t)s * 64 + lane] = make_uint4(acc[0][a0], acc[1][a0], acc[2][a0], acc[3][a0]);
-    if ((lanes >> (lane + 32)) & 1ull)
-      part[(size_t)s * 64 + lane + 32] = make_uint4(acc[0][a1], acc[1][a1], acc[2][a1], acc[3][a1]);
-    __syncwarp();
+    for (unsigned r = __ballot_sync(FULL, lanes != 0ull && d > ECAP_B); r; r &= r - 1u)
+      finish(__ffs(r) - 1, 0, 0, true);
   }
+  if (have) ring_round<P>(R, head, have, coef, sink, unit, e);
   if (e) atomicOr(err, e);
 }
 
-__global__ void __launch_bounds__(FWD_THREADS, BWD_MIN_BLOCKS)
-k_bwd_heavy_seg_lane(int nseg, const int32_t *__restrict__ seg_v, const int32_t *__restrict__ seg_b,
-                     const int32_t *__restrict__ seg_e, const int32_t *__restrict__ col,
-                     const uint64_t *__restrict__ lm_cur, const uint64_t *__restrict__ lm_next,
-                     const uint64_t *__restrict__ coef, uint4 *__restrict__ part, unsigned *__restrict__ wq,
-                     unsigned *__restrict__ err, uint64_t keep) {
-  __shared__ int32_t sws[FWD_THREADS / 32][32];
-  __shared__ int8_t tabs[FWD_THREADS / 32][64];
-  int32_t *sw = sws[threadIdx.x >> 5];
-  int8_t *tab = tabs[threadIdx.x >> 5];
+// The heavy vertices with lanes at a level: their segments, and the vertices
+// with several.
+__global__ void k_bwd_heavy_list(int nh, const int32_t *__restrict__ heavy, const int32_t *__restrict__ hseg0,
+                                 const uint64_t *__restrict__ lm_cur, uint64_t keep, int32_t *__restrict__ seg_list,
+                                 int32_t *__restrict__ multi, unsigned *__restrict__ counts) {
   const int lane = threadIdx.x & 31;
+  const int h = blockIdx.x * blockDim.x + threadIdx.x;
+  int first = 0, k = 0;
+  if (h < nh && (lm_cur[heavy[h]] & keep)) {
+    first = hseg0[h];
+    k = hseg0[h + 1] - first;
+  }
+  append_segments(first, k, seg_list, counts);
+  const unsigned m = __ballot_sync(FULL, k > 1);
+  if (!m) return;
+  unsigned pos = 0u;
+  if (lane == 0) pos = atomicAdd(counts + 1, (unsigned)__popc(m));
+  pos = __shfl_sync(FULL, pos, 0);
+  if (k > 1) multi[pos + __popc(m & ((1u << lane) - 1u))] = h;
+}
+
+// Heavy vertices: one warp per listed segment (taken dynamically). A vertex of
+// one segment is finished here; the others' partial sums go to part[s][lane].
+template <class P>
+__global__ void __launch_bounds__(FWD_THREADS, P::narrow ? BWD_MIN_BLOCKS : 3)
+k_bwd_heavy_seg(const int32_t *__restrict__ list, const unsigned *__restrict__ nlist,
+                const int32_t *__restrict__ seg_v, const int32_t *__restrict__ seg_b,
+                const int32_t *__restrict__ seg_e, const int32_t *__restrict__ rp, const int32_t *__restrict__ col,
+                const uint64_t *__restrict__ lm_cur, const uint64_t *__restrict__ lm_next,
+                const uint64_t *__restrict__ sigma, uint64_t *__restrict__ coef, const Acc3 *__restrict__ recips,
+                typename P::A *__restrict__ part, Sink sink, unsigned *__restrict__ wq, unsigned *__restrict__ err,
+                uint64_t keep, int unit) {
+  __shared__ Ring<P> rings[FWD_THREADS / 32];
+  __shared__ uint4 ents[FWD_THREADS / 32][ECAP_B];
+  __shared__ int8_t tabs[FWD_THREADS / 32][64];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  Ring<P> &R = rings[wid];
+  uint4 *ent = ents[wid];
+  int head = 0, have = 0;
   unsigned e = 0u;
-  for (int s = grab(wq, 1); s < nseg; s = grab(wq, 1)) {
+  unsigned long long tri = 0ull;
+  const int total = (int)*nlist;
+  for (int i = grab(wq, 1); i < total; i = grab(wq, 1)) {
+    const int s = list[i];
     const int32_t v = seg_v[s];
     const uint64_t lanes = lm_cur[v] & keep;
-    if (!lanes) continue;
-    int p0, p1;
-    own_lanes(lanes, tab, p0, p1);
-    Acc2 a0 = acc2_zero(), a1 = acc2_zero();
-    const int end = seg_e[s];
-    for (int base = seg_b[s]; base < end; base += 32) {
-      const int j = base + lane;
-      int32_t w = 0;
-      uint64_t m = 0ull;
-      if (j < end) {
-        w = col[j];
-        m = lm_next[w] & lanes;
-      }
-      sw[lane] = w;
-      uint32_t c0, c1;
-      lane_columns(m, p0, p1, c0, c1);
-      __syncwarp();
-      while (c0) {
-        const int ja = __ffs(c0) - 1;
-        c0 &= c0 - 1u;
-        const bool hb = c0 != 0u;
-        const int jb = hb ? __ffs(c0) - 1 : ja;
-        if (hb) c0 &= c0 - 1u;
-        const uint64_t xa = coef[(size_t)sw[ja] * 64 + p0];
-        const uint64_t xb = hb ? coef[(size_t)sw[jb] * 64 + p0] : 0ull;
-        acc2_add_nz(a0, xa, e);
-        if (hb) acc2_add_nz(a0, xb, e);
-      }
-      while (c1) {
-        const int ja = __ffs(c1) - 1;
-        c1 &= c1 - 1u;
-        acc2_add_nz(a1, coef[(size_t)sw[ja] * 64 + p1], e);
-      }
+    const int beg = seg_b[s], end = seg_e[s];
+    const bool whole = rp[v] == beg && rp[v + 1] == end;
+    const Packed pk = pack_lanes(lanes, tabs[wid]);
+    typename P::A a0 = P::zero(), a1 = P::zero();
+    for (int j = beg; j < end; j += ECAP_B) {
+      const int ne = list_row(col, lm_next, j, min(end, j + ECAP_B), lanes, ent, tri);
+      coef_entries<P>(ent, 0, ne, pk, coef, a0, a1, e);
       __syncwarp();
     }
-    if (p0 >= 0) part[(size_t)s * 64 + p0] = make_uint4(a0.l0, a0.l1, a0.l2, a0.l3);
-    if (p1 >= 0) part[(size_t)s * 64 + p1] = make_uint4(a1.l0, a1.l1, a1.l2, a1.l3);
+    group_sum<P>(a0, pk.glog);
+    if (whole) {
+      const uint64_t *row = sigma + (size_t)v * 64;
+      const uint64_t sg0 = ((lane >> pk.glog) == 0 && pk.p0 >= 0) ? row[pk.p0] : 0ull;
+      const uint64_t sg1 = pk.p1 >= 0 ? row[pk.p1] : 0ull;
+      ring_put<P>(R, head, have, v, pk, a0, a1, sg0, sg1, coef, recips, sink, unit, e);
+    } else {
+      if ((lane >> pk.glog) == 0 && pk.p0 >= 0) part[(size_t)s * 64 + pk.p0] = a0;
+      if (pk.p1 >= 0) part[(size_t)s * 64 + pk.p1] = a1;
+    }
   }
+  if (have) ring_round<P>(R, head, have, coef, sink, unit, e);
   if (e) atomicOr(err, e);
 }
 
-__global__ void __launch_bounds__(FWD_THREADS, BWD_MIN_BLOCKS)
-k_bwd_heavy_fin_fx(int nh, const int32_t *__restrict__ heavy, const int32_t *__restrict__ hseg0,
-                   const uint64_t *__restrict__ lm_cur, uint64_t *__restrict__ sigma,
-                   const uint4 *__restrict__ part, Sink sink, unsigned *__restrict__ err, unsigned *__restrict__ wq, uint64_t keep) {
-  __shared__ Ring rings[FWD_THREADS / 32];
+template <class P>
+__global__ void __launch_bounds__(FWD_THREADS, 4)
+k_bwd_heavy_fin(const int32_t *__restrict__ multi, const unsigned *__restrict__ nmulti,
+                const int32_t *__restrict__ heavy, const int32_t *__restrict__ hseg0,
+                const uint64_t *__restrict__ lm_cur, const uint64_t *__restrict__ sigma, uint64_t *__restrict__ coef,
+                const Acc3 *__restrict__ recips, const typename P::A *__restrict__ part, Sink sink,
+                unsigned *__restrict__ err,
+                unsigned *__restrict__ wq, uint64_t keep, int unit) {
+  __shared__ Ring<P> rings[FWD_THREADS / 32];
   __shared__ int8_t tabs[FWD_THREADS / 32][64];
-  Ring &R = rings[threadIdx.x >> 5];
-  int8_t *tab = tabs[threadIdx.x >> 5];
-  unsigned head = 0u, tail = 0u;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  Ring<P> &R = rings[wid];
+  int head = 0, have = 0;
   unsigned e = 0u;
-  for (int h = grab(wq, 1); h < nh; h = grab(wq, 1)) {
-      const int32_t v = heavy[h];
-      const uint64_t lanes = lm_cur[v] & keep;
-      if (!lanes) continue;
-      int p0, p1;
-      own_lanes(lanes, tab, p0, p1);
-      Acc2 a0 = acc2_zero(), a1 = acc2_zero();
-      // a hub has hundreds of segments: independent loads, four in flight
-      const int sb = hseg0[h], se = hseg0[h + 1];
-      const int q0 = p0 < 0 ? 0 : p0, q1 = p1 < 0 ? 0 : p1;
+  const int total = (int)*nmulti;
+  for (int i = grab(wq, 1); i < total; i = grab(wq, 1)) {
+    const int h = multi[i];
+    const int32_t v = heavy[h];
+    const uint64_t lanes = lm_cur[v] & keep;
+    const Packed pk = pack_lanes(lanes, tabs[wid]);
+    const uint64_t *row = sigma + (size_t)v * 64;
+    const uint64_t sg0 = ((lane >> pk.glog) == 0 && pk.p0 >= 0) ? row[pk.p0] : 0ull;
+    const uint64_t sg1 = pk.p1 >= 0 ? row[pk.p1] : 0ull;
+    // the groups take different segments (a hub has hundreds)
+    typename P::A a0 = P::zero(), a1 = P::zero();
+    const int NG = 32 >> pk.glog;
+    const int sb = hseg0[h], se = hseg0[h + 1];
+    const typename P::A *q0 = part + (pk.p0 < 0 ? 0 : pk.p0), *q1 = part + (pk.p1 < 0 ? 0 : pk.p1);
 #pragma unroll 4
-      for (int s = sb; s < se; ++s) {
-        if (p0 >= 0) acc2_add_u4(a0, part[(size_t)s * 64 + q0]);
-        if (p1 >= 0) acc2_add_u4(a1, part[(size_t)s * 64 + q1]);
-      }
-      Packed pk;
-      pk.glog = 5;
-      pk.p0 = p0;
-      pk.p1 = p1;
-      pk.two = p1 >= 0;
-      ring_append_fx(R, tail, v, lanes, pk, a0, a1, sigma + (size_t)v * 64);
-      __syncwarp();
-      while (tail - head >= 32u) {
-        ring_round(R, head, 32, sigma, sink, e);
-        head += 32u;
-        __syncwarp();
-      }
+    for (int s = sb + (lane >> pk.glog); s < se; s += NG) {
+      if (pk.p0 >= 0) P::add_acc(a0, q0[(size_t)s * 64]);
+      if (pk.p1 >= 0) P::add_acc(a1, q1[(size_t)s * 64]);
     }
-  if (tail != head) ring_round(R, head, (int)(tail - head), sigma, sink, e);
+    __syncwarp();
+    group_sum<P>(a0, pk.glog);
+    ring_put<P>(R, head, have, v, pk, a0, a1, sg0, sg1, coef, recips, sink, unit, e);
+  }
+  if (have) ring_round<P>(R, head, have, coef, sink, unit, e);
   if (e) atomicOr(err, e);
 }
 
@@ -1626,6 +1271,11 @@ __global__ void k_extract(int32_t n, int count, int maxlevel, const uint64_t *__
 struct HeavyMeta {
   int nh = 0, nseg = 0, heavy_deg = 0, seg = 0;
   DevBuf heavy, hseg0, seg_v, seg_b, seg_e, part, part2;
+  DevBuf list, multi;  // a level's segments; its vertices with several
+  DevBuf light;  // count (first word), then the light vertices with neighbours, in id order
+  template <class F> void each(F f) {
+    for (DevBuf *b : {&heavy, &hseg0, &seg_v, &seg_b, &seg_e, &part, &part2, &light, &list, &multi}) f(*b);
+  }
 };
 static std::map<const int32_t *, HeavyMeta> g_heavy;  // keyed by the graph's device col pointer
 static std::mutex g_heavy_mu;
@@ -1644,20 +1294,22 @@ static HeavyMeta &heavy_meta(bc_ctx *ctx, const Graph &g, bool in_csr) {
     if (old.heavy_deg == want_deg && old.seg == want_seg) return old;
     // the graph's split changed (a new tuning): rebuild
     cudaStreamSynchronize(ctx->stream);
-    old.heavy.release(); old.hseg0.release(); old.seg_v.release(); old.seg_b.release();
-    old.seg_e.release(); old.part.release(); old.part2.release();
+    old.each([](DevBuf &b) { b.release(); });
     g_heavy.erase(it);
   }
   HeavyMeta &hm = g_heavy[grp];
   std::vector<int32_t> rp(g.n + 1);
   BCG_CUDA(cudaMemcpy(rp.data(), grp, sizeof(int32_t) * (g.n + 1), cudaMemcpyDeviceToHost));
-  std::vector<int32_t> heavy, hseg0, sv, sb, se;
+  std::vector<int32_t> heavy, hseg0, sv, sb, se, light(1, 0);
   hm.heavy_deg = want_deg;
   hm.seg = want_seg;
   const int seg = want_seg;
   for (int32_t v = 0; v < g.n; ++v) {
     const int d = rp[v + 1] - rp[v];
-    if (d <= hm.heavy_deg) continue;
+    if (d <= hm.heavy_deg) {
+      if (d > 0) light.push_back(v);
+      continue;
+    }
     hseg0.push_back((int32_t)sv.size());
     heavy.push_back(v);
     for (int b = rp[v]; b < rp[v + 1]; b += seg) {
@@ -1678,8 +1330,12 @@ static HeavyMeta &heavy_meta(bc_ctx *ctx, const Graph &g, bool in_csr) {
   up(hm.seg_v, sv);
   up(hm.seg_b, sb);
   up(hm.seg_e, se);
-  hm.part.ensure(std::max<size_t>(hm.nseg, 1) * 64 * sizeof(Acc));
-  (void)ctx;
+  hm.list.ensure(std::max<size_t>(hm.nseg, 1) * sizeof(int32_t));
+  hm.multi.ensure(std::max<size_t>(hm.nh, 1) * sizeof(int32_t));
+  if (grp == g.rp_in) {  // the forward's first list
+    light[0] = (int32_t)light.size() - 1;
+    up(hm.light, light);
+  }
   return hm;
 }
 
@@ -1688,8 +1344,7 @@ void forget_heavy_meta(const int32_t *rp) {
   auto it = g_heavy.find(rp);
   if (it == g_heavy.end()) return;
   HeavyMeta &hm = it->second;
-  hm.heavy.release(); hm.hseg0.release(); hm.seg_v.release(); hm.seg_b.release();
-  hm.seg_e.release(); hm.part.release(); hm.part2.release();
+  hm.each([](DevBuf &b) { b.release(); });
   g_heavy.erase(it);
 }
 
@@ -1704,19 +1359,17 @@ static int grid_blocks() {
   return g_num_sms * 8;
 }
 
-// Vertices a warp of the light kernels takes at a time. Fewer than 32 spread a
-// level's vertices over more warps, which matters most on small graphs (ER
-// n = 100k, 256 samples: backward 3.86 / 2.41 / 2.22 / 2.33 ms taking 32 / 16
-// / 8 / 4, forward 1.72 / 1.38 / 1.31 / 1.41 ms) and still pays on R-MAT s20
-// (17,437 vs 17,074 samples/s taking 16 instead of 32).
-// BCG_BWD_GRAB / BCG_FWD_GRAB override.
+// Vertices a warp of the light kernels takes at a time: on small graphs fewer,
+// for more warps to have some (R-MAT s17 directed 6.96 ms taking 4, 7.03 taking
+// 8, 7.66 taking 16), on large ones more, for fewer atomics (s20 48.2 / 46.8 /
+// 46.8 ms). BCG_BWD_GRAB / BCG_FWD_GRAB override.
 static int env_grab(const char *name) {
   const char *e = std::getenv(name);
   const int v = e ? std::atoi(e) : 0;
   return (v == 1 || v == 2 || v == 4 || v == 8 || v == 16 || v == 32) ? v : 0;
 }
 
-static int light_grab(int32_t n) { return n >= (1 << 17) ? 16 : 8; }
+static int light_grab(int32_t n) { return n >= (1 << 18) ? 8 : 4; }
 
 static int bwd_grab(int32_t n) {
   static const int env = env_grab("BCG_BWD_GRAB");
@@ -1750,6 +1403,9 @@ void batch_ensure(bc_ctx *ctx, const Graph &g) {
   ws.vlist.ensure((size_t)ws.lcap * n * 4);
   ws.vcnt.ensure((size_t)(ws.lcap + 2) * 4);
   ws.vedges.ensure((size_t)(ws.lcap + 2) * 8);
+  ws.slist.ensure(2 * n * 4);
+  ws.scnt.ensure((size_t)(ws.lcap + 2) * 4);
+  ws.hcnt.ensure((size_t)(ws.lcap + 2) * 16);
   heavy_meta(ctx, g, true);
   heavy_meta(ctx, g, false);
 }
@@ -1780,14 +1436,19 @@ int batch_forward(bc_ctx *ctx, const Graph &g, int count, bool pairs, OvfMode mo
   BCG_CUDA(cudaMemsetAsync(ws.wq.p, 0, ws.wq.bytes, st));
   BCG_CUDA(cudaMemsetAsync(ws.vcnt.p, 0, ws.vcnt.bytes, st));
   BCG_CUDA(cudaMemsetAsync(ws.vedges.p, 0, ws.vedges.bytes, st));
-  // level lists (and their degree sums) are kept only for the direction
-  // switch: a bottom-up-only pass records nothing (the lists cost ~3 % of the
-  // forward on R-MAT s20)
-  ws.lists = ctx->push_div > 0;
-  int32_t *vlist = ws.lists ? ws.vlist.as<int32_t>() : nullptr;
+  BCG_CUDA(cudaMemsetAsync(ws.scnt.p, 0, ws.scnt.bytes, st));
+  BCG_CUDA(cudaMemsetAsync(ws.hcnt.p, 0, ws.hcnt.bytes, st));
+  // every level's vertices are listed (the backward walks them); their degree
+  // sums only for the direction switch
+  int32_t *vlist = ws.vlist.as<int32_t>();
   unsigned *vcnt = ws.vcnt.as<unsigned>();
   unsigned long long *vedges = ws.vedges.as<unsigned long long>();
-  auto lst = [&](int lev) -> int32_t * { return vlist ? vlist + (size_t)lev * n : nullptr; };
+  auto lst = [&](int lev) -> int32_t * { return vlist + (size_t)lev * n; };
+  const bool directions = ctx->push_div > 0;
+  // light vertices with lanes still to reach: the graph's own list first
+  const int32_t *todo = hm.light.as<int32_t>() + 1;
+  const unsigned *ntodo = hm.light.as<unsigned>();
+  bool flip = false;
   {
     LaunchScope ls(ctx, F_INIT);
     if (hm.nh) k_zero_heavy_rows<<<hm.nh, 64, 0, st>>>(hm.nh, hm.heavy.as<int32_t>(), ws.sigma.as<uint64_t>());
@@ -1804,7 +1465,7 @@ int batch_forward(bc_ctx *ctx, const Graph &g, int count, bool pairs, OvfMode mo
   ctx->batches += 1;
   const int blocks = grid_blocks();
   int l = 0;
-  bool heavy_done = false;
+  bool heavy_done = false, listed = false;
   uint64_t fedges = 0ull;  // degree sum of the vertices at the current level (direction test)
   {
     // level 1 straight from the sources' adjacency; heavy sigma rows were zeroed
@@ -1848,8 +1509,15 @@ int batch_forward(bc_ctx *ctx, const Graph &g, int count, bool pairs, OvfMode mo
       ws.vedges.grow_keep((size_t)(ncap + 2) * 8, st);
       BCG_CUDA(cudaMemsetAsync(ws.vcnt.as<unsigned>() + ws.lcap + 2, 0, (size_t)(ncap - ws.lcap) * 4, st));
       BCG_CUDA(cudaMemsetAsync(ws.vedges.as<unsigned long long>() + ws.lcap + 2, 0, (size_t)(ncap - ws.lcap) * 8, st));
+      const bool own = ntodo == hm.light.as<unsigned>();
+      const ptrdiff_t at = own ? 0 : ntodo - ws.scnt.as<unsigned>();
+      ws.scnt.grow_keep((size_t)(ncap + 2) * 4, st);
+      BCG_CUDA(cudaMemsetAsync(ws.scnt.as<unsigned>() + ws.lcap + 2, 0, (size_t)(ncap - ws.lcap) * 4, st));
+      if (!own) ntodo = ws.scnt.as<unsigned>() + at;
+      ws.hcnt.grow_keep((size_t)(ncap + 2) * 16, st);
+      BCG_CUDA(cudaMemsetAsync(ws.hcnt.as<unsigned>() + 4 * (ws.lcap + 2), 0, (size_t)(ncap - ws.lcap) * 16, st));
       ws.lcap = ncap;
-      vlist = ws.lists ? ws.vlist.as<int32_t>() : nullptr;
+      vlist = ws.vlist.as<int32_t>();
       vcnt = ws.vcnt.as<unsigned>();
       vedges = ws.vedges.as<unsigned long long>();
     }
@@ -1858,58 +1526,44 @@ int batch_forward(bc_ctx *ctx, const Graph &g, int count, bool pairs, OvfMode mo
     unsigned *hw = ws.wq.as<unsigned>() + 8 * (l + 1);  // slot 5: heavy lanes at l+1; 6-7: heavy pending lanes
     // top-down when the level's vertices have few edges (Beamer's direction
     // switch, here on the level's degree sum against the graph's edges)
-    const bool push = ws.lists && fedges * (uint64_t)ctx->push_div <= (uint64_t)g.nnz;
+    const bool push = directions && fedges * (uint64_t)ctx->push_div <= (uint64_t)g.nnz;
     const bool heavy_now = !push && hm.nseg && !heavy_done;
-    // With heavy work at this level, the heavy vertices' kernels (clear their
-    // rows, segments, finisher) run on the side stream beside the light kernel:
-    // the two write disjoint rows and read only level l's masks and counts, and
-    // the level ends with a join. Without the side stream the light kernel
-    // clears the heavy rows itself and runs first.
+    if (push) listed = false;  // (the list was made for the level after the last heavy one)
+    // With heavy work at this level, the heavy vertices' kernels (segments,
+    // finisher) run on the side stream beside the light kernel: the two write
+    // disjoint rows and read only level l's masks and counts, and the level
+    // ends with a join.
     const bool fov = heavy_now && ctx->fwd_overlap;
     if (fov) side_stream(ctx);
     const cudaStream_t hst = fov ? ctx->side : st;
+    unsigned long long *ve = directions ? vedges + l + 1 : nullptr;
     auto heavy_chain = [&] {
-      if (fov) {
-        LaunchScope ls(ctx, F_FWD, hst, false);
-        k_zero_heavy_lm<<<(hm.nh + 255) / 256, 256, 0, hst>>>(hm.nh, hm.heavy.as<int32_t>(),
-                                                              lm + (size_t)(l + 1) * n);
-      }
-      if (ctx->heavy_lane == 3 || ctx->heavy_lane == 4) {
-        LaunchScope ls(ctx, F_FWD, hst, false);
-        k_fwd_heavy_dense<<<std::min(blocks, (hm.nseg + 7) / 8), FWD_THREADS, 0, hst>>>(
-            hm.nseg, hm.seg_v.as<int32_t>(), hm.seg_b.as<int32_t>(), hm.seg_e.as<int32_t>(), pcol,
-            lm + (size_t)l * n, lm + (size_t)(l + 1) * n, ws.visited.as<uint64_t>(), ws.sigma.as<uint64_t>(),
-            act + l, ws.enable.as<uint64_t>(), ws.cnt.as<unsigned long long>(), ws.wq.as<unsigned>() + 8 * l + 1);
-      } else if (ctx->heavy_lane == 1) {
-        LaunchScope ls(ctx, F_FWD, hst, false);
-        k_fwd_heavy_lane<<<std::min(blocks, (hm.nseg + 7) / 8), FWD_THREADS, 0, hst>>>(
-            hm.nseg, hm.seg_v.as<int32_t>(), hm.seg_b.as<int32_t>(), hm.seg_e.as<int32_t>(), pcol,
-            lm + (size_t)l * n, lm + (size_t)(l + 1) * n, ws.visited.as<uint64_t>(), ws.sigma.as<uint64_t>(),
-            act + l, ws.enable.as<uint64_t>(), ws.cnt.as<unsigned long long>(), ws.wq.as<unsigned>() + 8 * l + 1);
-      } else {
+      {
         LaunchScope ls(ctx, F_FWD, hst, false);
         k_fwd_heavy<<<std::min(blocks, (hm.nseg + 7) / 8), FWD_THREADS, 0, hst>>>(
-            hm.nseg, hm.seg_v.as<int32_t>(), hm.seg_b.as<int32_t>(), hm.seg_e.as<int32_t>(), pcol,
-            lm + (size_t)l * n, lm + (size_t)(l + 1) * n, ws.visited.as<uint64_t>(), ws.sigma.as<uint64_t>(),
-            act + l, ws.enable.as<uint64_t>(), ws.err.as<unsigned>(), ws.cnt.as<unsigned long long>(),
-            ws.wq.as<unsigned>() + 8 * l + 1);
+            g.n, hm.nseg, listed ? hm.list.as<int32_t>() : nullptr, ws.hcnt.as<unsigned>() + 4 * l,
+            hm.seg_v.as<int32_t>(), hm.seg_b.as<int32_t>(), hm.seg_e.as<int32_t>(), pcol,
+            lm + (size_t)l * n, lm + (size_t)(l + 1) * n, ws.visited.as<uint64_t>(), ws.sigma.as<uint64_t>(), act + l,
+            ws.enable.as<uint64_t>(), ws.cnt.as<unsigned long long>(), ws.wq.as<unsigned>() + 8 * l + 1);
       }
       LaunchScope ls(ctx, F_FWD, hst, false);
-      k_fwd_heavy_fin<<<std::min(blocks, (hm.nh + 7) / 8), 256, 0, hst>>>(
-          hm.nh, hm.heavy.as<int32_t>(), lm + (size_t)(l + 1) * n, ws.visited.as<uint64_t>(), act + l + 1,
-          ws.cnt.as<unsigned long long>(), ws.sigma.as<uint64_t>(), ws.enable.as<uint64_t>(), hw + 5,
-          reinterpret_cast<unsigned long long *>(hw + 6), g.rp, lst(l + 1), vcnt + l + 1, vedges + l + 1);
+      k_fwd_heavy_fin<<<(hm.nh + 255) / 256, 256, 0, hst>>>(
+          hm.nh, hm.heavy.as<int32_t>(), hm.hseg0.as<int32_t>(), lm + (size_t)(l + 1) * n, ws.visited.as<uint64_t>(),
+          act + l + 1, ws.cnt.as<unsigned long long>(), ws.enable.as<uint64_t>(), hw + 5,
+          reinterpret_cast<unsigned long long *>(hw + 6), g.rp, lst(l + 1), vcnt + l + 1, ve, hm.list.as<int32_t>(),
+          ws.hcnt.as<unsigned>() + 4 * (l + 1));
+      listed = true;
     };
     {
       // the level's time on the main stream (after the join) is the family's time
       LaunchScope level_scope(ctx, F_FWD, st, true, false);
+      BCG_CUDA(cudaMemsetAsync(lm + (size_t)(l + 1) * n, 0, n * 8, st));
       if (fov) {
         BCG_CUDA(cudaEventRecord(ctx->ev_fork, st));
         BCG_CUDA(cudaStreamWaitEvent(hst, ctx->ev_fork, 0));
         heavy_chain();
       }
       if (push) {
-        BCG_CUDA(cudaMemsetAsync(lm + (size_t)(l + 1) * n, 0, n * 8, st));
         {
           LaunchScope ls(ctx, F_FWD, st, false);
           k_fwd_push<<<blocks, FWD_THREADS, 0, st>>>(g.rp, g.col, lst(l), vcnt + l, lm + (size_t)l * n,
@@ -1926,12 +1580,15 @@ int batch_forward(bc_ctx *ctx, const Graph &g, int count, bool pairs, OvfMode mo
                                                        ws.wq.as<unsigned>() + 8 * l + 1, hm.heavy_deg, hw + 5);
       } else {
         LaunchScope ls(ctx, F_FWD, st, false);
-        k_fwd_light<<<blocks, FWD_THREADS, 0, st>>>(g.n, prp, pcol, lm + (size_t)l * n, lm + (size_t)(l + 1) * n,
-                                                   ws.visited.as<uint64_t>(), ws.sigma.as<uint64_t>(), act + l,
-                                                   ws.enable.as<uint64_t>(), act + l + 1, ws.err.as<unsigned>(),
-                                                   ws.cnt.as<unsigned long long>(), ws.wq.as<unsigned>() + 8 * l + 0,
-                                                   hm.heavy_deg, ctx->pk_maxl, ctx->pk_mincnt, lst(l + 1),
-                                                   vcnt + l + 1, vedges + l + 1, fwd_grab(g.n), fov ? 0 : 1);
+        int32_t *left = ws.slist.as<int32_t>() + (flip ? n : 0);
+        flip = !flip;  // (a top-down level in between leaves the list as it is)
+        k_fwd_light<<<blocks, FWD_THREADS, 0, st>>>(
+            g.n, todo, ntodo, left, ws.scnt.as<unsigned>() + l + 1, prp, pcol, lm + (size_t)l * n,
+            lm + (size_t)(l + 1) * n, ws.visited.as<uint64_t>(), ws.sigma.as<uint64_t>(), act + l,
+            ws.enable.as<uint64_t>(), act + l + 1, ws.cnt.as<unsigned long long>(), ws.wq.as<unsigned>() + 8 * l + 0,
+            lst(l + 1), vcnt + l + 1, ve, fwd_grab(g.n));
+        todo = left;
+        ntodo = ws.scnt.as<unsigned>() + l + 1;
       }
       if (heavy_now && !fov) heavy_chain();
       if (fov) {
@@ -2008,12 +1665,14 @@ void batch_backward(bc_ctx *ctx, const Graph &g, int maxlevel, const Sink &sink,
   cudaStream_t st = ctx->stream;
   const int blocks = grid_blocks();
   uint64_t *lm = ws.lm.as<uint64_t>();
-  // per level: the vertices with lanes there (recorded only with the direction switch on)
-  const int32_t *vlist = ws.lists ? ws.vlist.as<int32_t>() : nullptr;
-  const unsigned *vcnt = ws.lists ? ws.vcnt.as<unsigned>() : nullptr;
-  auto lvl_list = [&](int lev) -> const int32_t * { return vlist ? vlist + (size_t)lev * n : nullptr; };
-  auto lvl_cnt = [&](int lev) -> const unsigned * { return vcnt ? vcnt + lev : nullptr; };
-  const bool narrow = ws.last_sigmax <= (1ull << 44);
+  // exact sums: 96 bits while the counts and the graph's size allow (a sum of
+  // coefficients is delta / sigma < n up to rounding, the per-vertex sums in a
+  // ring round at most 32 of them), else 192
+  const uint64_t largest = ws.last_sigmax;
+  int unit = 52, nlog = 0;
+  while (unit < 115 && largest > (1ull << (unit - 52))) ++unit;  // 52 + ceil(log2 of the largest count)
+  while (nlog < 31 && (int64_t)g.n > ((int64_t)1 << nlog)) ++nlog;
+  const bool narrow = unit + nlog + 6 <= 96;
   // A level's heavy-segment kernel and its light kernel touch disjoint data
   // (segment partials vs the light vertices' slots; both read only level l+1's
   // coefficients), so the segments run on the side stream beside the light
@@ -2024,80 +1683,64 @@ void batch_backward(bc_ctx *ctx, const Graph &g, int maxlevel, const Sink &sink,
   // the family's time is the pass's time on the main stream (the side stream's
   // kernels are joined into it): the overlapping launches are counted, not timed
   LaunchScope pass(ctx, F_BWD, st, true, false);
-  auto fork = [&] {
-    if (!overlap) return;
-    BCG_CUDA(cudaEventRecord(ctx->ev_fork, st));
-    BCG_CUDA(cudaStreamWaitEvent(sst, ctx->ev_fork, 0));
-  };
-  auto join = [&] {
-    if (!overlap) return;
-    BCG_CUDA(cudaEventRecord(ctx->ev_join, sst));
-    BCG_CUDA(cudaStreamWaitEvent(st, ctx->ev_join, 0));
-  };
-  if (narrow && ctx->bwd_variant == 1) {
-    hm.part2.ensure(std::max<size_t>(hm.nseg, 1) * 64 * sizeof(uint4));
+  DevBuf &part = narrow ? hm.part2 : hm.part;
+  part.ensure(std::max<size_t>(hm.nseg, 1) * 64 * (narrow ? sizeof(Acc3) : sizeof(Acc)));
+  uint64_t *coef = ws.sigma.as<uint64_t>();  // wide: in the counts' slots
+  Acc3 *recips = nullptr;
+  if (narrow) {
+    ws.coef.ensure(n * 768);
+    ws.recips.ensure(RECIPS * sizeof(Acc3));
+    coef = ws.coef.as<uint64_t>();
+    recips = ws.recips.as<Acc3>();
+    LaunchScope ls(ctx, F_BWD, st, false);
+    k_recips<<<RECIPS / 256, 256, 0, st>>>(unit, recips);
+  }
+  auto run = [&](auto policy) {
+    using P = decltype(policy);
     for (int l = maxlevel; l >= 1; --l) {
       const bool hv = hm.nseg && heavy_at(ws, l);
+      const uint64_t *cur = lm + (size_t)l * n, *next = lm + (size_t)(l + 1) * n;
+      unsigned *wq = ws.wq.as<unsigned>() + 8 * l;
+      unsigned *counts = ws.hcnt.as<unsigned>() + 4 * l + 1;  // segments listed, vertices with several
       if (hv) {
-        fork();
+        if (overlap) {
+          BCG_CUDA(cudaEventRecord(ctx->ev_fork, st));
+          BCG_CUDA(cudaStreamWaitEvent(sst, ctx->ev_fork, 0));
+        }
+        {
+          LaunchScope ls(ctx, F_BWD, sst, false);
+          k_bwd_heavy_list<<<(hm.nh + 255) / 256, 256, 0, sst>>>(hm.nh, hm.heavy.as<int32_t>(), hm.hseg0.as<int32_t>(),
+                                                                 cur, keep, hm.list.as<int32_t>(),
+                                                                 hm.multi.as<int32_t>(), counts);
+        }
         LaunchScope ls(ctx, F_BWD, sst, false);
-        auto kseg = (ctx->heavy_lane == 2 || ctx->heavy_lane == 3) ? k_bwd_heavy_seg_dense
-                                         : (ctx->heavy_lane == 1 ? k_bwd_heavy_seg_lane : k_bwd_heavy_seg_fx);
-        kseg<<<std::min(blocks, (hm.nseg + 7) / 8), FWD_THREADS, 0, sst>>>(
-            hm.nseg, hm.seg_v.as<int32_t>(), hm.seg_b.as<int32_t>(), hm.seg_e.as<int32_t>(), g.col,
-            lm + (size_t)l * n, lm + (size_t)(l + 1) * n, ws.sigma.as<uint64_t>(), hm.part2.as<uint4>(),
-            ws.wq.as<unsigned>() + 8 * l + 3, ws.err.as<unsigned>(), keep);
+        k_bwd_heavy_seg<P><<<std::min(blocks, (hm.nseg + 7) / 8), FWD_THREADS, 0, sst>>>(
+            hm.list.as<int32_t>(), counts, hm.seg_v.as<int32_t>(), hm.seg_b.as<int32_t>(), hm.seg_e.as<int32_t>(), g.rp,
+            g.col, cur, next, ws.sigma.as<uint64_t>(), coef, recips, part.as<typename P::A>(), sink, wq + 3,
+            ws.err.as<unsigned>(), keep, unit);
       }
       {
         LaunchScope ls(ctx, F_BWD, st, false);
-        k_bwd_light_fx<<<blocks, FWD_THREADS, 0, st>>>(g.n, lvl_list(l), lvl_cnt(l), g.rp, g.col,
-                                                      lm + (size_t)l * n, lm + (size_t)(l + 1) * n,
-                                                      ws.sigma.as<uint64_t>(), sink, ws.err.as<unsigned>(),
-                                                      ws.wq.as<unsigned>() + 8 * l + 2, hm.heavy_deg, keep,
-                                                      bwd_grab(g.n));
+        k_bwd_light<P><<<blocks, FWD_THREADS, 0, st>>>(ws.vlist.as<int32_t>() + (size_t)l * n,
+                                                      ws.vcnt.as<unsigned>() + l, g.rp, g.col, cur, next,
+                                                      ws.sigma.as<uint64_t>(), coef, recips, sink,
+                                                      ws.err.as<unsigned>(), wq + 2, hm.heavy_deg, keep,
+                                                      bwd_grab(g.n), unit);
       }
       if (hv) {
-        join();
+        if (overlap) {
+          BCG_CUDA(cudaEventRecord(ctx->ev_join, sst));
+          BCG_CUDA(cudaStreamWaitEvent(st, ctx->ev_join, 0));
+        }
         LaunchScope ls(ctx, F_BWD, st, false);
-        k_bwd_heavy_fin_fx<<<std::min(blocks, (hm.nh + 7) / 8), FWD_THREADS, 0, st>>>(
-            hm.nh, hm.heavy.as<int32_t>(), hm.hseg0.as<int32_t>(), lm + (size_t)l * n, ws.sigma.as<uint64_t>(),
-            hm.part2.as<uint4>(), sink, ws.err.as<unsigned>(), ws.wq.as<unsigned>() + 8 * l + 4, keep);
+        k_bwd_heavy_fin<P><<<std::min(blocks, (hm.nh + 7) / 8), FWD_THREADS, 0, st>>>(
+            hm.multi.as<int32_t>(), counts + 1, hm.heavy.as<int32_t>(), hm.hseg0.as<int32_t>(), cur,
+            ws.sigma.as<uint64_t>(), coef, recips, part.as<typename P::A>(), sink, ws.err.as<unsigned>(), wq + 4, keep, unit);
       }
     }
-    return;
-  }
-  for (int l = maxlevel; l >= 1; --l) {
-    const bool hv = hm.nseg && heavy_at(ws, l);
-    if (hv) {
-      fork();
-      LaunchScope ls(ctx, F_BWD, sst, false);
-      auto kseg = narrow ? k_bwd_heavy_seg<NarrowAcc> : k_bwd_heavy_seg<WideAcc>;
-      kseg<<<std::min(blocks, (hm.nseg + 7) / 8), FWD_THREADS, 0, sst>>>(
-          hm.nseg, hm.seg_v.as<int32_t>(), hm.seg_b.as<int32_t>(), hm.seg_e.as<int32_t>(), g.col,
-          lm + (size_t)l * n, lm + (size_t)(l + 1) * n, ws.sigma.as<uint64_t>(), hm.part.as<Acc>(),
-          ws.err.as<unsigned>(), ws.wq.as<unsigned>() + 8 * l + 3, keep);
-    }
-    {
-      LaunchScope ls(ctx, F_BWD, st, false);
-      if (narrow)
-        k_bwd_light<NarrowAcc><<<blocks, FWD_THREADS, 0, st>>>(
-            g.n, lvl_list(l), lvl_cnt(l), g.rp, g.col, lm + (size_t)l * n, lm + (size_t)(l + 1) * n,
-            ws.sigma.as<uint64_t>(), sink, ws.err.as<unsigned>(), ws.wq.as<unsigned>() + 8 * l + 2, hm.heavy_deg,
-            keep, bwd_grab(g.n));
-      else
-        k_bwd_light<WideAcc><<<blocks, FWD_THREADS, 0, st>>>(
-            g.n, lvl_list(l), lvl_cnt(l), g.rp, g.col, lm + (size_t)l * n, lm + (size_t)(l + 1) * n,
-            ws.sigma.as<uint64_t>(), sink, ws.err.as<unsigned>(), ws.wq.as<unsigned>() + 8 * l + 2, hm.heavy_deg,
-            keep, bwd_grab(g.n));
-    }
-    if (hv) {
-      join();
-      LaunchScope ls(ctx, F_BWD, st, false);
-      k_bwd_heavy_fin<<<std::min(blocks, (hm.nh + 7) / 8), FWD_THREADS, 0, st>>>(
-          hm.nh, hm.heavy.as<int32_t>(), hm.hseg0.as<int32_t>(), lm + (size_t)l * n, ws.sigma.as<uint64_t>(),
-          hm.part.as<Acc>(), sink, ws.err.as<unsigned>(), ws.wq.as<unsigned>() + 8 * l + 4, keep);
-    }
-  }
+  };
+  if (narrow) run(NarrowAcc{});
+  else run(WideAcc{});
 }
 
 void batch_extract(bc_ctx *ctx, const Graph &g, int count, int maxlevel, int32_t *dist, uint64_t *sigma,

@@ -1765,7 +1765,6 @@ bc_status bc_create(bc_ctx **out, int device, const bc_options *opt) {
     if (opt) ctx->batch_width = opt->batch_width;
     if (const char *hd = std::getenv("BCG_HEAVY_DEGREE")) ctx->heavy_deg = std::atoi(hd);
     if (const char *sl = std::getenv("BCG_SEGMENT")) ctx->seg_len = std::atoi(sl);
-    if (const char *bv = std::getenv("BCG_BWD_VARIANT")) ctx->bwd_variant = std::atoi(bv);
     if (const char *dl = std::getenv("BCG_DEEP_LEVELS")) ctx->deep_levels = std::atoi(dl);
     if (const char *sn = std::getenv("BCG_SOLO_N")) ctx->solo_n = std::atoi(sn);
     if (const char *sz = std::getenv("BCG_SOLO_NNZ")) ctx->solo_nnz = std::atoll(sz);
@@ -1773,9 +1772,6 @@ bc_status bc_create(bc_ctx **out, int device, const bc_options *opt) {
       const int t = std::atoi(so);
       ctx->solo_threads = (t == 256 || t == 1024) ? t : 0;
     }
-    if (const char *pm = std::getenv("BCG_PK_MAXL")) ctx->pk_maxl = std::atoi(pm);
-    if (const char *pc = std::getenv("BCG_PK_MINCNT")) ctx->pk_mincnt = std::atoi(pc);
-    if (const char *hl = std::getenv("BCG_HEAVY_LANE")) ctx->heavy_lane = std::atoi(hl);
     if (const char *pd = std::getenv("BCG_PUSH_DIV")) ctx->push_div = std::atoi(pd);
     if (const char *mc = std::getenv("BCG_MULTI_CAP")) ctx->multi_cap = std::atoi(mc);
     if (const char *pe = std::getenv("BCG_PAIR_ENGINE")) {
@@ -1838,7 +1834,7 @@ void bc_destroy(bc_ctx *ctx) {
                       &ws.pair_sig, &ws.pair_exp, &ws.err, &ws.cnt, &ws.acc, &ws.tslot, &ws.tdelta, &ws.scan, &ws.misc, &ws.misc2,
                       &ws.delta_lm, &ws.p_dist, &ws.p_sigma, &ws.p_coef, &ws.p_queue, &ws.p_ctr,
                       &ws.x_dist, &ws.x_m, &ws.x_e, &ws.x_vis, &ws.x_nm, &ws.x_list, &ws.x_lmask, &ws.x_ctr,
-                      &ws.x_off, &ws.rows, &ws.win})
+                      &ws.x_off, &ws.rows, &ws.win, &ws.slist, &ws.scnt, &ws.coef, &ws.recips, &ws.hcnt})
       b->release();
     if (ws.pinned) cudaFreeHost(ws.pinned);
     for (cudaEvent_t e : ctx->event_pool) cudaEventDestroy(e);
@@ -2135,7 +2131,7 @@ static bc_tuning current_tuning(bc_ctx *ctx, const Graph &g) {
   if (g.tuned) return g.tune;
   bc_tuning t{};
   t.batch_width = batch_width(ctx);
-  t.heavy_degree = ctx->heavy_deg > 0 ? ctx->heavy_deg : 256;
+  t.heavy_degree = ctx->heavy_deg > 0 ? ctx->heavy_deg : 64;
   t.segment = ctx->seg_len > 0 ? ctx->seg_len : 256;
   t.packed_max_lanes = ctx->pk_maxl;
   t.packed_min_preds = ctx->pk_mincnt;
@@ -2229,12 +2225,8 @@ bc_status bc_autotune(bc_ctx *ctx, bc_graph g, int64_t k, uint64_t seed, bc_tuni
     // the traversal's direction and the heavy-vertex split first (largest
     // effects on R-MAT), then the kernel forms
     sweep(&bc_tuning::push_div, {0, 8, 32, 128});
-    sweep(&bc_tuning::heavy_degree, {128, 256, 512, 1024});
+    sweep(&bc_tuning::heavy_degree, {32, 64, 128, 256, 512});
     sweep(&bc_tuning::segment, {128, 256, 512});
-    sweep(&bc_tuning::packed_max_lanes, {0, 8, 16, 32});
-    sweep(&bc_tuning::packed_min_preds, {4, 6, 10});
-    sweep(&bc_tuning::bwd_variant, {0, 1});
-    sweep(&bc_tuning::heavy_lane, {0, 1, 2, 3, 4});
     sweep(&bc_tuning::deep_levels, {16, 32, 64});
     if (gr.n <= (1 << 17)) sweep(&bc_tuning::batch_width, {1, 64});
     best.trial_ms = best_ms;

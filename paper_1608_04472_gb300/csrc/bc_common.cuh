@@ -156,47 +156,42 @@ __device__ __forceinline__ Acc acc_warp_sum(Acc a) {
   return a;
 }
 
-// A narrower exact accumulator for successor sums: 128 bits in 32-bit limbs,
-// value = (l3:l2:l1:l0) * 2^-96, holding every double in [2^-44, 2^32). When
-// sigma <= 2^44 every coefficient RN((1+delta)/sigma) is >= 2^-44, and a
-// successor sum equals delta_v/sigma_v <= n < 2^31 up to rounding, so the
-// window is never left; out-of-window values set ERR_RANGE.
-struct Acc2 {
-  uint32_t l0, l1, l2, l3;
+// 96-bit exact sums of coefficients in units of 2^-unit. With unit = 52 +
+// ceil(log2 of the largest count) every coefficient RN((1 + delta) / sigma) is
+// a whole number of units (it is at least 2^-ceil(log2 sigma)), and a
+// successor sum is delta_v / sigma_v <= n up to rounding, so the sum stays
+// below 2^96 while unit + ceil(log2 n) + 1 <= 96; a value outside the window
+// sets ERR_RANGE. Three limbs and 64-bit shifts take about half the
+// instructions of the 192-bit window.
+struct Acc3 {
+  uint32_t l0, l1, l2;
 };
-
-__device__ __forceinline__ Acc2 acc2_zero() { return Acc2{0u, 0u, 0u, 0u}; }
-
-__device__ __forceinline__ void acc2_add4(Acc2 &a, uint32_t t0, uint32_t t1, uint32_t t2, uint32_t t3) {
-  asm("add.cc.u32 %0, %0, %4;\n\t"
-      "addc.cc.u32 %1, %1, %5;\n\t"
-      "addc.cc.u32 %2, %2, %6;\n\t"
-      "addc.u32 %3, %3, %7;"
-      : "+r"(a.l0), "+r"(a.l1), "+r"(a.l2), "+r"(a.l3)
-      : "r"(t0), "r"(t1), "r"(t2), "r"(t3));
+__device__ __forceinline__ void acc3_add3(Acc3 &a, uint32_t t0, uint32_t t1, uint32_t t2) {
+  asm("add.cc.u32 %0, %0, %3;\n\t"
+      "addc.cc.u32 %1, %1, %4;\n\t"
+      "addc.u32 %2, %2, %5;"
+      : "+r"(a.l0), "+r"(a.l1), "+r"(a.l2)
+      : "r"(t0), "r"(t1), "r"(t2));
 }
-
-__device__ __forceinline__ void acc2_add(Acc2 &a, double x, unsigned &err) {
-  const uint64_t bits = (uint64_t)__double_as_longlong(x);
-  if (bits == 0ull) return;
-  const uint32_t hi = (uint32_t)(bits >> 32), lo = (uint32_t)bits;
-  const int p = (int)(hi >> 20) - 979;  // lowest mantissa bit, in units of 2^-96
-  if ((unsigned)p > 75u) { err |= ERR_RANGE; return; }
-  const uint32_t mh = (hi & 0x000FFFFFu) | 0x00100000u;
-  const int r = p & 31, q = p >> 5;
-  const uint32_t c0 = lo << r;
-  const uint32_t c1 = __funnelshift_l(lo, mh, r);
-  const uint32_t c2 = __funnelshift_l(mh, 0u, r);
-  const uint32_t t0 = (q == 0) ? c0 : 0u;
-  const uint32_t t1 = (q == 0) ? c1 : ((q == 1) ? c0 : 0u);
-  const uint32_t t2 = (q == 0) ? c2 : ((q == 1) ? c1 : c0);
-  const uint32_t t3 = (q == 1) ? c2 : ((q == 2) ? c1 : 0u);
-  acc2_add4(a, t0, t1, t2, t3);
+// bias = 1075 - unit
+__device__ __forceinline__ void acc3_add(Acc3 &a, uint64_t bits, int bias, unsigned &err) {
+  const uint32_t hi = (uint32_t)(bits >> 32);
+  const int sh = (int)(hi >> 20) - bias;
+  if ((unsigned)sh > 43u) err |= ERR_RANGE;
+  const uint64_t m = (bits & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull;
+  const uint64_t lo = m << (sh & 63);
+  const uint32_t up = (uint32_t)((m >> 1) >> (63 - (sh & 63)));
+  acc3_add3(a, (uint32_t)lo, (uint32_t)(lo >> 32), up);
 }
-
-// The same value in the 192-bit format (unit 2^-128).
-__device__ __forceinline__ Acc acc2_widen(const Acc2 &a) {
-  return Acc{(uint64_t)a.l0 << 32, (uint64_t)a.l1 | ((uint64_t)a.l2 << 32), (uint64_t)a.l3};
+// The same value in the 192-bit window (unit 2^-128); 52 <= unit <= 95.
+__device__ __forceinline__ Acc acc3_widen(const Acc3 &a, int unit) {
+  const uint64_t w0 = (uint64_t)a.l0 | ((uint64_t)a.l1 << 32), w1 = a.l2;
+  const int s = 128 - unit;  // 33..76
+  if (s >= 64) {
+    const int r = s - 64;
+    return Acc{0ull, w0 << r, r ? ((w0 >> (64 - r)) | (w1 << r)) : w1};
+  }
+  return Acc{w0 << s, (w0 >> (64 - s)) | (w1 << s), w1 >> (64 - s)};
 }
 
 // ------------------------------------------------------ Brandes arithmetic --

@@ -115,8 +115,10 @@ struct Workspace {
   // (vlist[l*n ..], each once), their count vcnt[l] and degree sum vedges[l]
   DevBuf vlist;    // [lcap][n] i32
   DevBuf vcnt;     // [lcap+2] u32
-  DevBuf vedges;   // [lcap+2] u64
-  bool lists = false;  // the last forward recorded level lists (direction switch on)
+  DevBuf vedges;   // [lcap+2] u64 (kept with the direction switch on)
+  DevBuf coef, recips;  // backward coefficients as 96-bit numbers [n][64] (12 B each), reciprocals of small counts
+  DevBuf hcnt;         // per level: heavy segments listed forward, backward, vertices with several, - (u32)
+  DevBuf slist, scnt;  // light vertices a level left unfinished: [2][n] i32, their counts [lcap+2] u32
   DevBuf enable;   // u64 lane enable mask
   DevBuf sources;  // [64] i32
   DevBuf targets;  // [64] i32 pair destinations
@@ -177,24 +179,13 @@ struct bc_ctx {
   // batched-engine tuning: degree above which a vertex is split into segments,
   // and the segment length (0 = library defaults)
   int32_t heavy_deg = 0, seg_len = 0;
-  // backward kernel form (128-bit window only): 1 = packed lane groups (default),
-  // 0 = two lane halves per thread
-  int32_t bwd_variant = 1;
-  // light forward: a 32-neighbour chunk with at least pk_mincnt predecessors
-  // over at most pk_maxl lanes is summed in packed groups (0 disables)
-  int32_t pk_maxl = 16, pk_mincnt = 6;
-  // heavy-vertex segments: 0 a 64-lane step per neighbour in both passes; 1
-  // per-lane item loops (4 % slower on R-MAT s20: scattered row loads); 2 the
-  // backward's items spread over all threads with exact shared-memory sums; 3
-  // that in both passes; 4 in the forward only (the default: the dense forward
-  // measured 3.5 % faster on R-MAT s20, the dense backward 1.6 % slower)
-  int32_t heavy_lane = 4;
+  // kernel forms of earlier versions, kept with a graph's tuning record (bc.h)
+  int32_t bwd_variant = 1, pk_maxl = 16, pk_mincnt = 6, heavy_lane = 4;
   // direction of a forward level: top-down (push from the level's vertex list,
   // then counts pulled for the discovered vertices only) when the level's
   // vertices have at most nnz / push_div edges; bottom-up (every vertex with
   // pending lanes pulls) otherwise; 0 = always bottom-up (the default: on
-  // R-MAT s20 with 64-lane batches the union frontier is rarely small, and the
-  // level lists the switch needs cost more than the top-down levels saved)
+  // R-MAT s20 with 64-lane batches the union frontier is rarely small)
   int32_t push_div = 0;
   // multi-graph split: hub eccentricity above which a graph goes to the
   // persistent kernel, and its CTAs per SM while the batched engine runs beside

@@ -347,44 +347,6 @@ __device__ __forceinline__ void solo_push(const MGraph &G, const SoloMem<TIER> &
   }
 }
 
-// 96-bit exact sums of coefficients in units of 2^-unit. With unit = 52 +
-// ceil(log2 of the largest count) every coefficient RN((1 + delta) / sigma) is
-// a whole number of units (it is at least 2^-ceil(log2 sigma)), and a
-// successor sum is delta_v / sigma_v <= n up to rounding, so the sum stays
-// below 2^96 while unit + ceil(log2 n) + 1 <= 96; a value outside the window
-// sets ERR_RANGE. Three limbs and 64-bit shifts take about half the
-// instructions of the 192-bit window.
-struct Acc3 {
-  uint32_t l0, l1, l2;
-};
-__device__ __forceinline__ void acc3_add3(Acc3 &a, uint32_t t0, uint32_t t1, uint32_t t2) {
-  asm("add.cc.u32 %0, %0, %3;\n\t"
-      "addc.cc.u32 %1, %1, %4;\n\t"
-      "addc.u32 %2, %2, %5;"
-      : "+r"(a.l0), "+r"(a.l1), "+r"(a.l2)
-      : "r"(t0), "r"(t1), "r"(t2));
-}
-// bias = 1075 - unit
-__device__ __forceinline__ void acc3_add(Acc3 &a, uint64_t bits, int bias, unsigned &err) {
-  const uint32_t hi = (uint32_t)(bits >> 32);
-  const int sh = (int)(hi >> 20) - bias;
-  if ((unsigned)sh > 43u) err |= ERR_RANGE;
-  const uint64_t m = (bits & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull;
-  const uint64_t lo = m << (sh & 63);
-  const uint32_t up = (uint32_t)((m >> 1) >> (63 - (sh & 63)));
-  acc3_add3(a, (uint32_t)lo, (uint32_t)(lo >> 32), up);
-}
-// The same value in the 192-bit window (unit 2^-128); 52 <= unit <= 95.
-__device__ __forceinline__ Acc acc3_widen(const Acc3 &a, int unit) {
-  const uint64_t w0 = (uint64_t)a.l0 | ((uint64_t)a.l1 << 32), w1 = a.l2;
-  const int s = 128 - unit;  // 33..76
-  if (s >= 64) {
-    const int r = s - 64;
-    return Acc{0ull, w0 << r, r ? ((w0 >> (64 - r)) | (w1 << r)) : w1};
-  }
-  return Acc{w0 << s, (w0 >> (64 - s)) | (w1 << s), w1 >> (64 - s)};
-}
-
 // Theorem 1 for the vertices of one level (queue entries [b, e)): exact sums of
 // the coefficients over the shortest-path edges the forward pass kept, then
 // delta and the vertex's own coefficient in place of its count. deliver(v,

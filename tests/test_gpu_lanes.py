@@ -1,0 +1,90 @@
+"""The 64-lane engine (csrc/bc_batch.cu) where its entry lists, lane groups,
+segments and tables end, on graphs small enough for the oracle (which run one
+source per CTA by rule: BCG_SOLO_N=0 sends them here)."""
+import os
+
+import numpy as np
+import pytest
+
+import graphgen as gg
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    import paper_1608_04472_gb300 as pkg
+    os.environ["BCG_SOLO_N"] = "0"
+    try:
+        c = pkg.Context(0, batch_width=64)
+    finally:
+        del os.environ["BCG_SOLO_N"]
+    yield c
+    c.close()
+
+
+def _regular(n, d):
+    i = np.arange(n, dtype=np.int64)
+    return gg.from_edges(n, np.concatenate([i] * (d // 2)), np.concatenate([(i + k) % n for k in range(1, d // 2 + 1)]))
+
+
+def _fans(widths):
+    """For each a in widths: x - a vertices - y - z, so that a paths reach y and z
+    (the table of reciprocals ends at 2048)."""
+    eu, ev, n = [], [], 0
+    for a in widths:
+        mid = np.arange(n + 1, n + 1 + a)
+        y = n + 1 + a
+        eu += [np.full(a, n), mid, [y]]
+        ev += [mid, np.full(a, y), [y + 1]]
+        n = y + 2
+    return gg.from_edges(n, np.concatenate(eu), np.concatenate(ev))
+
+
+GRAPHS = {
+    "rows of 64 (light) and 66 (heavy)": lambda: gg.from_edges(
+        500, *np.concatenate([_regular(250, 64).edges(), _regular(250, 66).edges() + 250]).T),
+    "hubs of several segments": lambda: gg.barabasi_albert(3000, 6, 9, m0=8),
+    "rows of 1 to 16": lambda: gg.erdos_renyi(700, 7, 3),
+    "skewed rows": lambda: gg.rmat(11, 12, 0.57, 0.19, 0.19, 4),
+    "counts of 2047, 2048, 2049": lambda: _fans([2047, 2048, 2049]),
+    "counts beyond the 96-bit window": lambda: gg.grid(25),
+}
+
+
+@pytest.mark.parametrize("name", list(GRAPHS))
+@pytest.mark.parametrize("lanes", [1, 4, 5, 17, 33, 64])
+def test_rows_equal_the_oracle(ctx, name, lanes):
+    g = GRAPHS[name]()
+    src = np.unique(np.linspace(0, g.n - 1, lanes).astype(np.int32))
+    h = ctx.load_graph(g.row_ptr, g.col)
+    delta, dist, sigma = ctx.source_dependencies(h, src, want_dist=True, want_sigma=True)
+    ctx.free_graph(h)
+    for i in range(0, len(src), max(1, len(src) // 6)):
+        d_o, dist_o, sig_o = oracle.dependencies(g, int(src[i]))[:3]
+        assert np.array_equal(dist[i], dist_o) and np.array_equal(sigma[i], sig_o)
+        assert np.array_equal(delta[i], d_o)
+
+
+@pytest.mark.parametrize("heavy,segment", [(32, 32), (64, 256), (129, 64), (257, 300), (5000, 256)])
+def test_splits_equal_the_oracle(ctx, heavy, segment):
+    """Light rows at and above the lists' capacities (128 backward, 256 forward)."""
+    g = gg.from_edges(900, *np.concatenate([gg.erdos_renyi(420, 128, 6).edges(), gg.erdos_renyi(420, 257, 7).edges() + 440,
+                                            [[419, 440], [430, 431]]]).T)
+    h = ctx.load_graph(g.row_ptr, g.col)
+    ctx.set_tuning(h, dict(ctx.get_tuning(h), heavy_degree=heavy, segment=segment))
+    got = ctx.uniform_sources(h, 130, 3, 8)
+    ctx.free_graph(h)
+    assert np.array_equal(got, oracle.uniform_sources(g, 130, 3, 8))
+
+
+def test_directed_rows_without_successors(ctx):
+    g = gg.directed_rmat(11, 6, 0.57, 0.19, 0.19, 5)
+    h = ctx.load_graph(g.row_ptr, g.col, directed=True)
+    got = ctx.uniform_sources(h, 100, 2, 3)
+    res = ctx.adaptive_sources(h, [0, 1, 7], 2.0, 200, 4, 5)
+    ctx.free_graph(h)
+    assert np.array_equal(got, oracle.uniform_sources(g, 100, 2, 3))
+    ref = oracle.adaptive_sources(g, [0, 1, 7], 2.0, 200, 4, 5)
+    assert np.array_equal(res["S"], ref["S"]) and np.array_equal(res["k"], ref["k"])
