@@ -29,6 +29,7 @@
 // draws: 21.0 -> 14.0.
 #include <algorithm>
 #include <cstdlib>
+#include <memory>
 
 #include "bc_internal.h"
 
@@ -1268,13 +1269,28 @@ __global__ void k_extract(int32_t n, int count, int maxlevel, const uint64_t *__
 }
 
 // ------------------------------------------------------------------ host --
+// Control words of one level, cleared together before a batch.
+struct LevelCtl {
+  unsigned long long active;  // lanes with a vertex at the level
+  unsigned long long vedges;  // degree sum of the level's vertices (kept with the direction switch on)
+  unsigned long long hpend;   // lanes some heavy vertex has not reached after the level
+  unsigned q_light, q_heavy, q_bwd_light, q_bwd_seg, q_bwd_fin;  // work counters
+  unsigned hflag;                 // a heavy vertex has lanes at the level
+  unsigned vcnt;                  // vertices at the level (their list: vlist)
+  unsigned todo;                  // light vertices unfinished before the level's successor
+  unsigned fseg;                  // heavy segments listed for the level's successor
+  unsigned bseg, bmulti;          // backward: listed segments, heavy vertices with several
+  unsigned pad[15];
+};
+static_assert(sizeof(LevelCtl) == 128, "one line per level");
+
 struct HeavyMeta {
   int nh = 0, nseg = 0, heavy_deg = 0, seg = 0;
-  DevBuf heavy, hseg0, seg_v, seg_b, seg_e, part, part2;
-  DevBuf list, multi;  // a level's segments; its vertices with several
+  int depth = 0;  // the deepest level of the batches so far: levels launched without asking the device
+  DevBuf heavy, hseg0, seg_v, seg_b, seg_e;
   DevBuf light;  // count (first word), then the light vertices with neighbours, in id order
   template <class F> void each(F f) {
-    for (DevBuf *b : {&heavy, &hseg0, &seg_v, &seg_b, &seg_e, &part, &part2, &light, &list, &multi}) f(*b);
+    for (DevBuf *b : {&heavy, &hseg0, &seg_v, &seg_b, &seg_e, &light}) f(*b);
   }
 };
 static std::map<const int32_t *, HeavyMeta> g_heavy;  // keyed by the graph's device col pointer
@@ -1330,8 +1346,6 @@ static HeavyMeta &heavy_meta(bc_ctx *ctx, const Graph &g, bool in_csr) {
   up(hm.seg_v, sv);
   up(hm.seg_b, sb);
   up(hm.seg_e, se);
-  hm.list.ensure(std::max<size_t>(hm.nseg, 1) * sizeof(int32_t));
-  hm.multi.ensure(std::max<size_t>(hm.nh, 1) * sizeof(int32_t));
   if (grp == g.rp_in) {  // the forward's first list
     light[0] = (int32_t)light.size() - 1;
     up(hm.light, light);
@@ -1398,132 +1412,97 @@ void batch_ensure(bc_ctx *ctx, const Graph &g) {
   }
   ws.visited.ensure(n * 8);
   ws.sigma.ensure(n * 64 * 8);
-  ws.active.ensure((size_t)(ws.lcap + 2) * 8);
-  ws.wq.ensure((size_t)(ws.lcap + 2) * 8 * 4);
+  ws.ctl.ensure((size_t)(ws.lcap + 2) * sizeof(LevelCtl));
   ws.vlist.ensure((size_t)ws.lcap * n * 4);
-  ws.vcnt.ensure((size_t)(ws.lcap + 2) * 4);
-  ws.vedges.ensure((size_t)(ws.lcap + 2) * 8);
   ws.slist.ensure(2 * n * 4);
-  ws.scnt.ensure((size_t)(ws.lcap + 2) * 4);
-  ws.hcnt.ensure((size_t)(ws.lcap + 2) * 16);
-  heavy_meta(ctx, g, true);
-  heavy_meta(ctx, g, false);
+  for (bool in : {true, false}) {
+    const HeavyMeta &hm = heavy_meta(ctx, g, in);
+    ws.hlist.ensure(std::max<size_t>(hm.nseg, 1) * sizeof(int32_t));
+    ws.hmulti.ensure(std::max<size_t>(hm.nh, 1) * sizeof(int32_t));
+  }
 }
 
-// Two device words to the host with one synchronisation.
-static void read_u64x2(bc_ctx *ctx, const uint64_t *a, const uint64_t *b, uint64_t &va, uint64_t &vb) {
-  uint64_t *h = static_cast<uint64_t *>(ctx->ws.pinned);
-  BCG_CUDA(cudaMemcpyAsync(h, a, 8, cudaMemcpyDeviceToHost, ctx->stream));
-  BCG_CUDA(cudaMemcpyAsync(h + 1, b, 8, cudaMemcpyDeviceToHost, ctx->stream));
-  BCG_CUDA(cudaStreamSynchronize(ctx->stream));
-  va = h[0];
-  vb = h[1];
-}
-
-int batch_forward(bc_ctx *ctx, const Graph &g, int count, bool pairs, OvfMode mode) {
-  Workspace &ws = ctx->ws;
-  batch_ensure(ctx, g);
-  // counts are pulled over the in-neighbour CSR (the CSR itself when undirected;
-  // Def. 3 with paths following the edges on a directed graph); level 1 and the
-  // top-down pushes follow the out-edges
-  HeavyMeta &hm = heavy_meta(ctx, g, true);
-  const int32_t *prp = g.rp_in, *pcol = g.col_in;
-  const size_t n = (size_t)g.n;
-  cudaStream_t st = ctx->stream;
-  BCG_CUDA(cudaMemsetAsync(ws.lm.p, 0, 2 * n * 8, st));  // levels 0 and 1
-  BCG_CUDA(cudaMemsetAsync(ws.visited.p, 0, n * 8, st));
-  BCG_CUDA(cudaMemsetAsync(ws.active.p, 0, (size_t)(ws.lcap + 2) * 8, st));
-  BCG_CUDA(cudaMemsetAsync(ws.wq.p, 0, ws.wq.bytes, st));
-  BCG_CUDA(cudaMemsetAsync(ws.vcnt.p, 0, ws.vcnt.bytes, st));
-  BCG_CUDA(cudaMemsetAsync(ws.vedges.p, 0, ws.vedges.bytes, st));
-  BCG_CUDA(cudaMemsetAsync(ws.scnt.p, 0, ws.scnt.bytes, st));
-  BCG_CUDA(cudaMemsetAsync(ws.hcnt.p, 0, ws.hcnt.bytes, st));
-  // every level's vertices are listed (the backward walks them); their degree
-  // sums only for the direction switch
-  int32_t *vlist = ws.vlist.as<int32_t>();
-  unsigned *vcnt = ws.vcnt.as<unsigned>();
-  unsigned long long *vedges = ws.vedges.as<unsigned long long>();
-  auto lst = [&](int lev) -> int32_t * { return vlist + (size_t)lev * n; };
-  const bool directions = ctx->push_div > 0;
-  // light vertices with lanes still to reach: the graph's own list first
-  const int32_t *todo = hm.light.as<int32_t>() + 1;
-  const unsigned *ntodo = hm.light.as<unsigned>();
-  bool flip = false;
-  {
-    LaunchScope ls(ctx, F_INIT);
-    if (hm.nh) k_zero_heavy_rows<<<hm.nh, 64, 0, st>>>(hm.nh, hm.heavy.as<int32_t>(), ws.sigma.as<uint64_t>());
-  }
-  {
-    LaunchScope ls(ctx, F_INIT);
-    k_batch_init<<<1, 64, 0, st>>>(count, ws.sources.as<int32_t>(), ws.lm.as<uint64_t>(),
-                                   ws.visited.as<uint64_t>(), ws.sigma.as<uint64_t>(),
-                                   ws.active.as<uint64_t>(), ws.enable.as<uint64_t>(),
-                                   ws.pair_d.as<int32_t>(), ws.pair_sig.as<uint64_t>(), g.rp, lst(0), vcnt,
-                                   vedges);
-  }
-  ctx->samples += count;
-  ctx->batches += 1;
-  const int blocks = grid_blocks();
+// A forward pass whose levels are launched one at a time or, up to the depth of
+// the graph's earlier batches, without asking the device in between (a host
+// read per level left the GPU idle between levels: R-MAT s16 spent a third of a
+// batch that way). Kernels of a level without lanes return at once.
+struct Forward {
+  bc_ctx *ctx;
+  const Graph &g;
+  Workspace &ws;
+  HeavyMeta &hm;
+  size_t n;
+  cudaStream_t st;
+  int count;
+  bool pairs;
+  OvfMode mode;
   int l = 0;
-  bool heavy_done = false, listed = false;
-  uint64_t fedges = 0ull;  // degree sum of the vertices at the current level (direction test)
-  {
-    // level 1 straight from the sources' adjacency; heavy sigma rows were zeroed
-    // above and only receive stores here, so the atomics-based heavy path is not needed
+  bool heavy_done = false, listed = false, flip = false;
+  const int32_t *todo = nullptr;  // light vertices with lanes still to reach
+  int todo_level = -1;            // level whose control word counts them (-1: the graph's own list)
+  uint64_t fedges = 0ull;         // degree sum of the vertices at level l (direction test)
+
+  Forward(bc_ctx *c, const Graph &gr, int cnt, bool pr, OvfMode m)
+      : ctx(c), g(gr), ws(c->ws), hm(heavy_meta(c, gr, true)), n((size_t)gr.n), st(c->stream), count(cnt), pairs(pr),
+        mode(m) {}
+  LevelCtl *ctl(int lev) { return ws.ctl.as<LevelCtl>() + lev; }
+  int32_t *lst(int lev) { return ws.vlist.as<int32_t>() + (size_t)lev * n; }
+  uint64_t *lm(int lev) { return ws.lm.as<uint64_t>() + (size_t)lev * n; }
+  static uint64_t *u64(unsigned long long *p) { return reinterpret_cast<uint64_t *>(p); }
+  uint64_t *pinned() { return static_cast<uint64_t *>(ws.pinned); }
+
+  // Level 0, and level 1 straight from the sources' adjacency (heavy sigma rows
+  // are cleared before and only receive stores there).
+  void init() {
+    BCG_CUDA(cudaMemsetAsync(ws.lm.p, 0, 2 * n * 8, st));  // levels 0 and 1
+    BCG_CUDA(cudaMemsetAsync(ws.visited.p, 0, n * 8, st));
+    BCG_CUDA(cudaMemsetAsync(ws.ctl.p, 0, (size_t)(ws.lcap + 2) * sizeof(LevelCtl), st));
+    todo = hm.light.as<int32_t>() + 1;
+    if (hm.nh) {
+      LaunchScope ls(ctx, F_INIT);
+      k_zero_heavy_rows<<<hm.nh, 64, 0, st>>>(hm.nh, hm.heavy.as<int32_t>(), ws.sigma.as<uint64_t>());
+    }
+    {
+      LaunchScope ls(ctx, F_INIT);
+      k_batch_init<<<1, 64, 0, st>>>(count, ws.sources.as<int32_t>(), lm(0), ws.visited.as<uint64_t>(),
+                                     ws.sigma.as<uint64_t>(), u64(&ctl(0)->active), ws.enable.as<uint64_t>(),
+                                     ws.pair_d.as<int32_t>(), ws.pair_sig.as<uint64_t>(), g.rp, lst(0), &ctl(0)->vcnt,
+                                     &ctl(0)->vedges);
+    }
+    ctx->samples += count;
+    ctx->batches += 1;
     {
       LaunchScope ls(ctx, F_FWD);
-      k_fwd_level1<<<count, 128, 0, st>>>(count, ws.sources.as<int32_t>(), g.rp, g.col,
-                                           ws.lm.as<uint64_t>() + n, ws.visited.as<uint64_t>(),
-                                           ws.sigma.as<uint64_t>(), ws.active.as<uint64_t>() + 1,
-                                           ws.cnt.as<unsigned long long>(), lst(1), vcnt + 1, vedges + 1);
+      k_fwd_level1<<<count, 128, 0, st>>>(count, ws.sources.as<int32_t>(), g.rp, g.col, lm(1),
+                                          ws.visited.as<uint64_t>(), ws.sigma.as<uint64_t>(), u64(&ctl(1)->active),
+                                          ws.cnt.as<unsigned long long>(), lst(1), &ctl(1)->vcnt, &ctl(1)->vedges);
     }
-    uint64_t cont1;
-    if (pairs) {
-      LaunchScope ls(ctx, F_PAIR);
-      k_pair_check<<<1, 64, 0, st>>>(count, 1, ws.targets.as<int32_t>(), ws.lm.as<uint64_t>() + n,
-                                     ws.sigma.as<uint64_t>(), ws.enable.as<uint64_t>(), ws.pair_d.as<int32_t>(),
-                                     ws.pair_sig.as<uint64_t>(), ws.active.as<uint64_t>() + 1,
-                                     ws.enable.as<uint64_t>() + 1);
-      read_u64x2(ctx, ws.enable.as<uint64_t>() + 1, reinterpret_cast<const uint64_t *>(vedges + 1), cont1, fedges);
-    } else {
-      read_u64x2(ctx, ws.active.as<uint64_t>() + 1, reinterpret_cast<const uint64_t *>(vedges + 1), cont1, fedges);
-    }
-    ws.last_ovf = 0ull;
-    if (!cont1) {  // no vertex at distance 1 (or, for pairs, every destination found)
-      ws.last_sigmax = 1ull;
-      ws.hlev.assign(3, 1);
-      return pairs ? 1 : 0;
-    }
+    if (pairs) pair_check(1);
     l = 1;
   }
-  for (;;) {
-    if (l + 2 >= ws.lcap) {
-      const int ncap = ws.lcap * 2;
-      ws.lm.grow_keep((size_t)ncap * n * 8, st);
-      ws.active.grow_keep((size_t)(ncap + 2) * 8, st);
-      ws.wq.grow_keep((size_t)(ncap + 2) * 8 * 4, st);
-      BCG_CUDA(cudaMemsetAsync(ws.wq.as<unsigned>() + 8 * (ws.lcap + 2), 0, (size_t)(ncap - ws.lcap) * 8 * 4, st));
-      BCG_CUDA(cudaMemsetAsync(ws.active.as<uint64_t>() + ws.lcap + 2, 0, (size_t)(ncap - ws.lcap) * 8, st));
-      ws.vlist.grow_keep((size_t)ncap * n * 4, st);
-      ws.vcnt.grow_keep((size_t)(ncap + 2) * 4, st);
-      ws.vedges.grow_keep((size_t)(ncap + 2) * 8, st);
-      BCG_CUDA(cudaMemsetAsync(ws.vcnt.as<unsigned>() + ws.lcap + 2, 0, (size_t)(ncap - ws.lcap) * 4, st));
-      BCG_CUDA(cudaMemsetAsync(ws.vedges.as<unsigned long long>() + ws.lcap + 2, 0, (size_t)(ncap - ws.lcap) * 8, st));
-      const bool own = ntodo == hm.light.as<unsigned>();
-      const ptrdiff_t at = own ? 0 : ntodo - ws.scnt.as<unsigned>();
-      ws.scnt.grow_keep((size_t)(ncap + 2) * 4, st);
-      BCG_CUDA(cudaMemsetAsync(ws.scnt.as<unsigned>() + ws.lcap + 2, 0, (size_t)(ncap - ws.lcap) * 4, st));
-      if (!own) ntodo = ws.scnt.as<unsigned>() + at;
-      ws.hcnt.grow_keep((size_t)(ncap + 2) * 16, st);
-      BCG_CUDA(cudaMemsetAsync(ws.hcnt.as<unsigned>() + 4 * (ws.lcap + 2), 0, (size_t)(ncap - ws.lcap) * 16, st));
-      ws.lcap = ncap;
-      vlist = ws.vlist.as<int32_t>();
-      vcnt = ws.vcnt.as<unsigned>();
-      vedges = ws.vedges.as<unsigned long long>();
-    }
-    uint64_t *lm = ws.lm.as<uint64_t>();
-    uint64_t *act = ws.active.as<uint64_t>();
-    unsigned *hw = ws.wq.as<unsigned>() + 8 * (l + 1);  // slot 5: heavy lanes at l+1; 6-7: heavy pending lanes
+
+  void pair_check(int lev) {
+    LaunchScope ls(ctx, F_PAIR);
+    k_pair_check<<<1, 64, 0, st>>>(count, lev, ws.targets.as<int32_t>(), lm(lev), ws.sigma.as<uint64_t>(),
+                                   ws.enable.as<uint64_t>(), ws.pair_d.as<int32_t>(), ws.pair_sig.as<uint64_t>(),
+                                   u64(&ctl(lev)->active), ws.enable.as<uint64_t>() + 1);
+  }
+
+  void grow() {
+    const int ncap = ws.lcap * 2;
+    ws.lm.grow_keep((size_t)ncap * n * 8, st);
+    ws.vlist.grow_keep((size_t)ncap * n * 4, st);
+    ws.ctl.grow_keep((size_t)(ncap + 2) * sizeof(LevelCtl), st);
+    BCG_CUDA(cudaMemsetAsync(ctl(ws.lcap + 2), 0, (size_t)(ncap - ws.lcap) * sizeof(LevelCtl), st));
+    ws.lcap = ncap;
+  }
+
+  // Launches level l -> l + 1; returns whether the heavy kernels ran.
+  bool level() {
+    if (l + 2 >= ws.lcap) grow();
+    const int blocks = grid_blocks();
+    const int32_t *prp = g.rp_in, *pcol = g.col_in;
+    const bool directions = ctx->push_div > 0;
     // top-down when the level's vertices have few edges (Beamer's direction
     // switch, here on the level's degree sum against the graph's edges)
     const bool push = directions && fedges * (uint64_t)ctx->push_div <= (uint64_t)g.nnz;
@@ -1536,123 +1515,162 @@ int batch_forward(bc_ctx *ctx, const Graph &g, int count, bool pairs, OvfMode mo
     const bool fov = heavy_now && ctx->fwd_overlap;
     if (fov) side_stream(ctx);
     const cudaStream_t hst = fov ? ctx->side : st;
-    unsigned long long *ve = directions ? vedges + l + 1 : nullptr;
+    LevelCtl *cur = ctl(l), *next = ctl(l + 1);
+    unsigned long long *ve = directions ? &next->vedges : nullptr;
+    unsigned long long *cnt = ws.cnt.as<unsigned long long>();
+    uint64_t *visited = ws.visited.as<uint64_t>(), *sigma = ws.sigma.as<uint64_t>(),
+             *enable = ws.enable.as<uint64_t>();
     auto heavy_chain = [&] {
       {
         LaunchScope ls(ctx, F_FWD, hst, false);
         k_fwd_heavy<<<std::min(blocks, (hm.nseg + 7) / 8), FWD_THREADS, 0, hst>>>(
-            g.n, hm.nseg, listed ? hm.list.as<int32_t>() : nullptr, ws.hcnt.as<unsigned>() + 4 * l,
-            hm.seg_v.as<int32_t>(), hm.seg_b.as<int32_t>(), hm.seg_e.as<int32_t>(), pcol,
-            lm + (size_t)l * n, lm + (size_t)(l + 1) * n, ws.visited.as<uint64_t>(), ws.sigma.as<uint64_t>(), act + l,
-            ws.enable.as<uint64_t>(), ws.cnt.as<unsigned long long>(), ws.wq.as<unsigned>() + 8 * l + 1);
+            g.n, hm.nseg, listed ? ws.hlist.as<int32_t>() : nullptr, &cur->fseg, hm.seg_v.as<int32_t>(),
+            hm.seg_b.as<int32_t>(), hm.seg_e.as<int32_t>(), pcol, lm(l), lm(l + 1), visited, sigma,
+            u64(&cur->active), enable, cnt, &cur->q_heavy);
       }
       LaunchScope ls(ctx, F_FWD, hst, false);
       k_fwd_heavy_fin<<<(hm.nh + 255) / 256, 256, 0, hst>>>(
-          hm.nh, hm.heavy.as<int32_t>(), hm.hseg0.as<int32_t>(), lm + (size_t)(l + 1) * n, ws.visited.as<uint64_t>(),
-          act + l + 1, ws.cnt.as<unsigned long long>(), ws.enable.as<uint64_t>(), hw + 5,
-          reinterpret_cast<unsigned long long *>(hw + 6), g.rp, lst(l + 1), vcnt + l + 1, ve, hm.list.as<int32_t>(),
-          ws.hcnt.as<unsigned>() + 4 * (l + 1));
+          hm.nh, hm.heavy.as<int32_t>(), hm.hseg0.as<int32_t>(), lm(l + 1), visited, u64(&next->active), cnt, enable,
+          &next->hflag, &next->hpend, g.rp, lst(l + 1), &next->vcnt, ve, ws.hlist.as<int32_t>(), &next->fseg);
       listed = true;
     };
-    {
-      // the level's time on the main stream (after the join) is the family's time
-      LaunchScope level_scope(ctx, F_FWD, st, true, false);
-      BCG_CUDA(cudaMemsetAsync(lm + (size_t)(l + 1) * n, 0, n * 8, st));
-      if (fov) {
-        BCG_CUDA(cudaEventRecord(ctx->ev_fork, st));
-        BCG_CUDA(cudaStreamWaitEvent(hst, ctx->ev_fork, 0));
-        heavy_chain();
-      }
-      if (push) {
-        {
-          LaunchScope ls(ctx, F_FWD, st, false);
-          k_fwd_push<<<blocks, FWD_THREADS, 0, st>>>(g.rp, g.col, lst(l), vcnt + l, lm + (size_t)l * n,
-                                                    lm + (size_t)(l + 1) * n, ws.visited.as<uint64_t>(), act + l,
-                                                    ws.enable.as<uint64_t>(), lst(l + 1), vcnt + l + 1,
-                                                    vedges + l + 1, ws.wq.as<unsigned>() + 8 * l + 0);
-        }
+    // the level's time on the main stream (after the join) is the family's time
+    LaunchScope level_scope(ctx, F_FWD, st, true, false);
+    BCG_CUDA(cudaMemsetAsync(lm(l + 1), 0, n * 8, st));
+    if (fov) {
+      BCG_CUDA(cudaEventRecord(ctx->ev_fork, st));
+      BCG_CUDA(cudaStreamWaitEvent(hst, ctx->ev_fork, 0));
+      heavy_chain();
+    }
+    if (push) {
+      {
         LaunchScope ls(ctx, F_FWD, st, false);
-        k_fwd_pull_list<<<blocks, FWD_THREADS, 0, st>>>(prp, pcol, lst(l + 1), vcnt + l + 1,
-                                                       lm + (size_t)l * n, lm + (size_t)(l + 1) * n,
-                                                       ws.visited.as<uint64_t>(), ws.sigma.as<uint64_t>(),
-                                                       ws.enable.as<uint64_t>(), act + l + 1,
-                                                       ws.cnt.as<unsigned long long>(),
-                                                       ws.wq.as<unsigned>() + 8 * l + 1, hm.heavy_deg, hw + 5);
-      } else {
-        LaunchScope ls(ctx, F_FWD, st, false);
-        int32_t *left = ws.slist.as<int32_t>() + (flip ? n : 0);
-        flip = !flip;  // (a top-down level in between leaves the list as it is)
-        k_fwd_light<<<blocks, FWD_THREADS, 0, st>>>(
-            g.n, todo, ntodo, left, ws.scnt.as<unsigned>() + l + 1, prp, pcol, lm + (size_t)l * n,
-            lm + (size_t)(l + 1) * n, ws.visited.as<uint64_t>(), ws.sigma.as<uint64_t>(), act + l,
-            ws.enable.as<uint64_t>(), act + l + 1, ws.cnt.as<unsigned long long>(), ws.wq.as<unsigned>() + 8 * l + 0,
-            lst(l + 1), vcnt + l + 1, ve, fwd_grab(g.n));
-        todo = left;
-        ntodo = ws.scnt.as<unsigned>() + l + 1;
+        k_fwd_push<<<blocks, FWD_THREADS, 0, st>>>(g.rp, g.col, lst(l), &cur->vcnt, lm(l), lm(l + 1), visited,
+                                                  u64(&cur->active), enable, lst(l + 1), &next->vcnt, &next->vedges,
+                                                  &cur->q_light);
       }
-      if (heavy_now && !fov) heavy_chain();
-      if (fov) {
-        BCG_CUDA(cudaEventRecord(ctx->ev_join, hst));
-        BCG_CUDA(cudaStreamWaitEvent(st, ctx->ev_join, 0));
-      }
+      LaunchScope ls(ctx, F_FWD, st, false);
+      k_fwd_pull_list<<<blocks, FWD_THREADS, 0, st>>>(prp, pcol, lst(l + 1), &next->vcnt, lm(l), lm(l + 1), visited,
+                                                     sigma, enable, u64(&next->active), cnt, &cur->q_heavy,
+                                                     hm.heavy_deg, &next->hflag);
+    } else {
+      LaunchScope ls(ctx, F_FWD, st, false);
+      int32_t *left = ws.slist.as<int32_t>() + (flip ? n : 0);
+      flip = !flip;  // (a top-down level in between leaves the list as it is)
+      k_fwd_light<<<blocks, FWD_THREADS, 0, st>>>(
+          g.n, todo, todo_level < 0 ? hm.light.as<unsigned>() : &ctl(todo_level)->todo, left, &next->todo, prp, pcol,
+          lm(l), lm(l + 1), visited, sigma, u64(&cur->active), enable, u64(&next->active), cnt, &cur->q_light,
+          lst(l + 1), &next->vcnt, ve, fwd_grab(g.n));
+      todo = left;
+      todo_level = l + 1;
     }
-    // Deep traversals also watch the overflowed lanes every level: once every
-    // lane has overflowed the integer pass has nothing left to give (and its
-    // per-level masks would only grow).
-    const bool watch = mode == OVF_EXTEND && l >= 24;
-    uint64_t cont, ovf = 0ull;
-    const uint64_t *cont_word = act + l + 1;
-    if (pairs) {
-      LaunchScope ls(ctx, F_PAIR);
-      k_pair_check<<<1, 64, 0, st>>>(count, l + 1, ws.targets.as<int32_t>(), lm + (size_t)(l + 1) * n,
-                                     ws.sigma.as<uint64_t>(), ws.enable.as<uint64_t>(), ws.pair_d.as<int32_t>(),
-                                     ws.pair_sig.as<uint64_t>(), act + l + 1, ws.enable.as<uint64_t>() + 1);
-      cont_word = ws.enable.as<uint64_t>() + 1;
+    if (heavy_now && !fov) heavy_chain();
+    if (fov) {
+      BCG_CUDA(cudaEventRecord(ctx->ev_join, hst));
+      BCG_CUDA(cudaStreamWaitEvent(st, ctx->ev_join, 0));
     }
-    uint64_t hpend = 0ull;
-    {
-      // the level's continue word, the overflowed lanes (deep watch) or the
-      // heavy vertices' pending lanes, and the next level's degree sum: one sync
-      uint64_t *h = static_cast<uint64_t *>(ws.pinned);
-      const uint64_t *second = watch ? ws.enable.as<uint64_t>() + 3
-                                     : (heavy_now ? reinterpret_cast<const uint64_t *>(hw + 6) : cont_word);
-      BCG_CUDA(cudaMemcpyAsync(h, cont_word, 8, cudaMemcpyDeviceToHost, st));
-      BCG_CUDA(cudaMemcpyAsync(h + 1, second, 8, cudaMemcpyDeviceToHost, st));
-      BCG_CUDA(cudaMemcpyAsync(h + 2, vedges + l + 1, 8, cudaMemcpyDeviceToHost, st));
-      BCG_CUDA(cudaStreamSynchronize(st));
-      cont = h[0];
-      if (watch) ovf = h[1];
-      else if (heavy_now) hpend = h[1];
-      fedges = h[2];
-    }
-    // no heavy vertex is unvisited in a lane that goes on: the heavy kernels
-    // have nothing left to do in this batch (the lanes going on only shrink)
-    if (heavy_now && !watch && (hpend & cont) == 0ull) heavy_done = true;
-    // stop once every lane still going has overflowed (finished lanes are complete)
-    const bool all_ovf = watch && ovf != 0ull && (cont & ~ovf) == 0ull;
-    if (!cont || all_ovf) {
-      // largest sigma and overflowed lanes, adjacent words
-      uint64_t *h = static_cast<uint64_t *>(ws.pinned);
-      BCG_CUDA(cudaMemcpyAsync(h, ws.enable.as<uint64_t>() + 2, 16, cudaMemcpyDeviceToHost, st));
-      BCG_CUDA(cudaStreamSynchronize(st));
-      ws.last_sigmax = h[0];
-      ws.last_ovf = h[1];
-      // per level: did any heavy vertex get lanes there (level 1 is filled
-      // without the heavy kernels: assume yes)
-      ws.hlev.assign((size_t)l + 2, 1);
-      // (a directed graph's backward splits by out-degree, so its heavy
-      // kernels run at every level)
-      if (hm.nseg && !g.directed) {
-        std::vector<unsigned> fl((size_t)(l + 2) * 8);
-        BCG_CUDA(cudaMemcpyAsync(fl.data(), ws.wq.p, fl.size() * 4, cudaMemcpyDeviceToHost, st));
-        BCG_CUDA(cudaStreamSynchronize(st));
-        for (int k = 2; k <= l + 1; ++k) ws.hlev[k] = fl[(size_t)k * 8 + 5] != 0u;
-      }
-      if (ws.last_ovf && mode == OVF_ERROR) raise_err_bits(ctx, ERR_SIGMA_OVERFLOW);
-      return l;
-    }
-    ++l;
+    return heavy_now;
   }
+
+  // Levels up to the depth of earlier batches, then their control words and
+  // the batch's words (largest count, overflowed lanes) on their way to the
+  // host. False when the levels have to be asked for one at a time.
+  bool blind() {
+    if (pairs || ctx->push_div > 0 || hm.depth < 1 || hm.depth + 3 > ws.lcap || ws.lcap > 24) return false;
+    for (; l <= hm.depth; ++l) level();
+    uint64_t *h = pinned();
+    BCG_CUDA(cudaMemcpyAsync(h, ws.enable.as<uint64_t>() + 2, 16, cudaMemcpyDeviceToHost, st));
+    BCG_CUDA(cudaMemcpyAsync(h + 2, ws.ctl.p, (size_t)(l + 1) * sizeof(LevelCtl), cudaMemcpyDeviceToHost, st));
+    return true;
+  }
+
+  int finished(int last, uint64_t sigmax, uint64_t ovf, const LevelCtl *levels) {
+    ws.last_sigmax = sigmax;
+    ws.last_ovf = ovf;
+    // per level: did any heavy vertex get lanes there (level 1 is filled
+    // without the heavy kernels: assume yes; a directed graph's backward splits
+    // by out-degree, so its heavy kernels run at every level)
+    ws.hlev.assign((size_t)last + 2, 1);
+    if (hm.nseg && !g.directed)
+      for (int k = 2; k <= last + 1; ++k) ws.hlev[k] = levels[k].hflag != 0u;
+    if (ovf && mode == OVF_ERROR) raise_err_bits(ctx, ERR_SIGMA_OVERFLOW);
+    if (!pairs) hm.depth = std::max(hm.depth, last);
+    return last;
+  }
+
+  // After blind(): the deepest level, going on level by level where the batch
+  // is deeper than the ones before.
+  int end_blind() {
+    BCG_CUDA(cudaStreamSynchronize(st));
+    const uint64_t *h = pinned();
+    const LevelCtl *lv = reinterpret_cast<const LevelCtl *>(h + 2);
+    if (lv[l].active == 0ull) {
+      int last = l;
+      while (last > 0 && lv[last].active == 0ull) --last;
+      return finished(last, h[0], h[1], lv);
+    }
+    return run();
+  }
+
+  // Level by level from level l (whose lanes are on) to the end.
+  int run() {
+    uint64_t *h = pinned();
+    for (;; ++l) {
+      const bool heavy_now = level();
+      // Deep traversals also watch the overflowed lanes every level: once every
+      // lane has overflowed the integer pass has nothing left to give (and its
+      // per-level masks would only grow).
+      const bool watch = mode == OVF_EXTEND && l >= 24;
+      if (pairs) pair_check(l + 1);
+      BCG_CUDA(cudaMemcpyAsync(h, ws.enable.p, 32, cudaMemcpyDeviceToHost, st));
+      BCG_CUDA(cudaMemcpyAsync(h + 4, ctl(l + 1), sizeof(LevelCtl), cudaMemcpyDeviceToHost, st));
+      BCG_CUDA(cudaStreamSynchronize(st));
+      const LevelCtl &next = *reinterpret_cast<const LevelCtl *>(h + 4);
+      const uint64_t cont = pairs ? h[1] : next.active, ovf = watch ? h[3] : 0ull;
+      fedges = next.vedges;
+      // no heavy vertex is unvisited in a lane that goes on: the heavy kernels
+      // have nothing left to do in this batch (the lanes going on only shrink)
+      if (heavy_now && (next.hpend & cont) == 0ull) heavy_done = true;
+      // stop once every lane still going has overflowed (finished lanes are complete)
+      const bool all_ovf = watch && ovf != 0ull && (cont & ~ovf) == 0ull;
+      if (!cont || all_ovf) {
+        const uint64_t sigmax = h[2], ov = h[3];
+        std::vector<LevelCtl> lv((size_t)l + 2);
+        if (hm.nseg && !g.directed) {
+          BCG_CUDA(cudaMemcpyAsync(lv.data(), ws.ctl.p, lv.size() * sizeof(LevelCtl), cudaMemcpyDeviceToHost, st));
+          BCG_CUDA(cudaStreamSynchronize(st));
+        }
+        return finished(l, sigmax, ov, lv.data());
+      }
+    }
+  }
+
+  // The whole pass, level by level.
+  int all() {
+    init();
+    uint64_t *h = pinned();
+    BCG_CUDA(cudaMemcpyAsync(h, ws.enable.p, 16, cudaMemcpyDeviceToHost, st));
+    BCG_CUDA(cudaMemcpyAsync(h + 2, ctl(1), sizeof(LevelCtl), cudaMemcpyDeviceToHost, st));
+    BCG_CUDA(cudaStreamSynchronize(st));
+    const LevelCtl &one = *reinterpret_cast<const LevelCtl *>(h + 2);
+    fedges = one.vedges;
+    ws.last_ovf = 0ull;
+    if (!(pairs ? h[1] : one.active)) {  // no vertex at distance 1 (or, for pairs, every destination found)
+      ws.last_sigmax = 1ull;
+      ws.hlev.assign(3, 1);
+      return pairs ? 1 : 0;
+    }
+    return run();
+  }
+};
+
+int batch_forward(bc_ctx *ctx, const Graph &g, int count, bool pairs, OvfMode mode) {
+  batch_ensure(ctx, g);
+  Forward f(ctx, g, count, pairs, mode);
+  if (pairs) return f.all();
+  if (f.hm.depth < 1) return f.all();
+  f.init();
+  return f.blind() ? f.end_blind() : f.run();
 }
 
 // Whether a heavy vertex has lanes at level l in the last forward pass.
@@ -1672,7 +1690,12 @@ void batch_backward(bc_ctx *ctx, const Graph &g, int maxlevel, const Sink &sink,
   int unit = 52, nlog = 0;
   while (unit < 115 && largest > (1ull << (unit - 52))) ++unit;  // 52 + ceil(log2 of the largest count)
   while (nlog < 31 && (int64_t)g.n > ((int64_t)1 << nlog)) ++nlog;
-  const bool narrow = unit + nlog + 6 <= 96;
+  bool narrow = unit + nlog + 6 <= 96;
+  if (narrow && ws.coef.bytes < n * 768) {  // 768 B per vertex more than the wide form: only where there is room
+    size_t fr = 0, tot = 0;
+    if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) cudaGetLastError();
+    narrow = n * 768 < fr / 2;
+  }
   // A level's heavy-segment kernel and its light kernel touch disjoint data
   // (segment partials vs the light vertices' slots; both read only level l+1's
   // coefficients), so the segments run on the side stream beside the light
@@ -1683,8 +1706,7 @@ void batch_backward(bc_ctx *ctx, const Graph &g, int maxlevel, const Sink &sink,
   // the family's time is the pass's time on the main stream (the side stream's
   // kernels are joined into it): the overlapping launches are counted, not timed
   LaunchScope pass(ctx, F_BWD, st, true, false);
-  DevBuf &part = narrow ? hm.part2 : hm.part;
-  part.ensure(std::max<size_t>(hm.nseg, 1) * 64 * (narrow ? sizeof(Acc3) : sizeof(Acc)));
+  ws.hpart.ensure(std::max<size_t>(hm.nseg, 1) * 64 * (narrow ? sizeof(Acc3) : sizeof(Acc)));
   uint64_t *coef = ws.sigma.as<uint64_t>();  // wide: in the counts' slots
   Acc3 *recips = nullptr;
   if (narrow) {
@@ -1697,11 +1719,11 @@ void batch_backward(bc_ctx *ctx, const Graph &g, int maxlevel, const Sink &sink,
   }
   auto run = [&](auto policy) {
     using P = decltype(policy);
+    typename P::A *part = ws.hpart.as<typename P::A>();
     for (int l = maxlevel; l >= 1; --l) {
       const bool hv = hm.nseg && heavy_at(ws, l);
       const uint64_t *cur = lm + (size_t)l * n, *next = lm + (size_t)(l + 1) * n;
-      unsigned *wq = ws.wq.as<unsigned>() + 8 * l;
-      unsigned *counts = ws.hcnt.as<unsigned>() + 4 * l + 1;  // segments listed, vertices with several
+      LevelCtl *ctl = ws.ctl.as<LevelCtl>() + l;
       if (hv) {
         if (overlap) {
           BCG_CUDA(cudaEventRecord(ctx->ev_fork, st));
@@ -1710,22 +1732,20 @@ void batch_backward(bc_ctx *ctx, const Graph &g, int maxlevel, const Sink &sink,
         {
           LaunchScope ls(ctx, F_BWD, sst, false);
           k_bwd_heavy_list<<<(hm.nh + 255) / 256, 256, 0, sst>>>(hm.nh, hm.heavy.as<int32_t>(), hm.hseg0.as<int32_t>(),
-                                                                 cur, keep, hm.list.as<int32_t>(),
-                                                                 hm.multi.as<int32_t>(), counts);
+                                                                 cur, keep, ws.hlist.as<int32_t>(),
+                                                                 ws.hmulti.as<int32_t>(), &ctl->bseg);
         }
         LaunchScope ls(ctx, F_BWD, sst, false);
         k_bwd_heavy_seg<P><<<std::min(blocks, (hm.nseg + 7) / 8), FWD_THREADS, 0, sst>>>(
-            hm.list.as<int32_t>(), counts, hm.seg_v.as<int32_t>(), hm.seg_b.as<int32_t>(), hm.seg_e.as<int32_t>(), g.rp,
-            g.col, cur, next, ws.sigma.as<uint64_t>(), coef, recips, part.as<typename P::A>(), sink, wq + 3,
-            ws.err.as<unsigned>(), keep, unit);
+            ws.hlist.as<int32_t>(), &ctl->bseg, hm.seg_v.as<int32_t>(), hm.seg_b.as<int32_t>(),
+            hm.seg_e.as<int32_t>(), g.rp, g.col, cur, next, ws.sigma.as<uint64_t>(), coef, recips, part, sink,
+            &ctl->q_bwd_seg, ws.err.as<unsigned>(), keep, unit);
       }
       {
         LaunchScope ls(ctx, F_BWD, st, false);
-        k_bwd_light<P><<<blocks, FWD_THREADS, 0, st>>>(ws.vlist.as<int32_t>() + (size_t)l * n,
-                                                      ws.vcnt.as<unsigned>() + l, g.rp, g.col, cur, next,
-                                                      ws.sigma.as<uint64_t>(), coef, recips, sink,
-                                                      ws.err.as<unsigned>(), wq + 2, hm.heavy_deg, keep,
-                                                      bwd_grab(g.n), unit);
+        k_bwd_light<P><<<blocks, FWD_THREADS, 0, st>>>(
+            ws.vlist.as<int32_t>() + (size_t)l * n, &ctl->vcnt, g.rp, g.col, cur, next, ws.sigma.as<uint64_t>(), coef,
+            recips, sink, ws.err.as<unsigned>(), &ctl->q_bwd_light, hm.heavy_deg, keep, bwd_grab(g.n), unit);
       }
       if (hv) {
         if (overlap) {
@@ -1734,13 +1754,171 @@ void batch_backward(bc_ctx *ctx, const Graph &g, int maxlevel, const Sink &sink,
         }
         LaunchScope ls(ctx, F_BWD, st, false);
         k_bwd_heavy_fin<P><<<std::min(blocks, (hm.nh + 7) / 8), FWD_THREADS, 0, st>>>(
-            hm.multi.as<int32_t>(), counts + 1, hm.heavy.as<int32_t>(), hm.hseg0.as<int32_t>(), cur,
-            ws.sigma.as<uint64_t>(), coef, recips, part.as<typename P::A>(), sink, ws.err.as<unsigned>(), wq + 4, keep, unit);
+            ws.hmulti.as<int32_t>(), &ctl->bmulti, hm.heavy.as<int32_t>(), hm.hseg0.as<int32_t>(), cur,
+            ws.sigma.as<uint64_t>(), coef, recips, part, sink, ws.err.as<unsigned>(), &ctl->q_bwd_fin, keep, unit);
       }
     }
   };
   if (narrow) run(NarrowAcc{});
   else run(WideAcc{});
+}
+
+// ---- batches in flight ----
+
+__global__ void k_add_acc(int32_t n, const Acc *__restrict__ from, Acc *__restrict__ to) {
+  const int32_t v = blockIdx.x * blockDim.x + threadIdx.x;
+  if (v >= n) return;
+  Acc a = to[v];
+  acc_add_acc(a, from[v]);
+  to[v] = a;
+}
+
+// The context's batch state and streams exchanged for the second slot's while
+// in scope.
+struct SlotScope {
+  bc_ctx *ctx;
+  bool on;
+  SlotScope(bc_ctx *c, bool second) : ctx(c), on(second) {
+    if (on) swap();
+  }
+  ~SlotScope() {
+    if (on) swap();
+  }
+  void swap() {
+    std::swap(static_cast<BatchState &>(ctx->ws), ctx->slot2.state);
+    std::swap(ctx->stream, ctx->slot2.stream);
+    std::swap(ctx->side, ctx->slot2.side);
+    std::swap(ctx->ev_fork, ctx->slot2.ev_fork);
+    std::swap(ctx->ev_join, ctx->slot2.ev_join);
+  }
+  SlotScope(const SlotScope &) = delete;
+  SlotScope &operator=(const SlotScope &) = delete;
+};
+
+// Makes the second slot's state for graph g; false when its memory (about 1.9
+// KB per vertex) would take more than a quarter of what is free.
+static bool second_slot(bc_ctx *ctx, const Graph &g, bool acc) {
+  if (!ctx->batch_overlap) return false;
+  BatchSlot &s = ctx->slot2;
+  const size_t need = (size_t)g.n * (1900 + (acc ? sizeof(Acc) : 0));
+  if (s.state.sigma.bytes < (size_t)g.n * 512) {
+    size_t fr = 0, tot = 0;
+    if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    if (need > fr / 4) return false;
+  }
+  if (!s.stream) {
+    BCG_CUDA(cudaStreamCreateWithFlags(&s.stream, cudaStreamNonBlocking));
+    BCG_CUDA(cudaEventCreateWithFlags(&s.ev_begin, cudaEventDisableTiming));
+    BCG_CUDA(cudaEventCreateWithFlags(&s.ev_end, cudaEventDisableTiming));
+    BCG_CUDA(cudaMallocHost(&s.state.pinned, 4096));
+    s.state.enable.ensure(64);
+    s.state.sources.ensure(64 * 4);
+  }
+  if (acc) s.acc.ensure((size_t)g.n * sizeof(Acc));
+  return true;
+}
+
+// The sources src[0 .. count) (device) in batches of 64 on the lane engine, lane
+// t of a batch at column pos[b + t] of the sink (pos may be null). Two batches
+// are in flight, each with its own state and stream: while one's forward pass
+// runs, the other's backward pass fills the SMs its narrow levels leave idle,
+// and the host reads a batch's depth and largest count without the GPU waiting
+// for it. The batches write different columns; all-vertex sums are kept per
+// slot and added at the end (exact sums: any order).
+// ms with one batch at a time and with two: ER n = 100,003 k = 333 5.73 / 4.90,
+// R-MAT s16 Bader 1500 draws 15.0 / 12.2, directed s17 k = 512 6.58 / 5.15, s20 k =
+// 1024 40.4 / 37.1 (a host read per level, one batch: 5.70, 14.0, 6.39, 38.1).
+void run_lane_batches(bc_ctx *ctx, const Graph &g, const int32_t *src, const int32_t *pos, int count,
+                      const Sink &sink) {
+  if (count < 1) return;
+  cudaStream_t main = ctx->stream;
+  auto batch_sink = [&](int b, bool second) {
+    Sink s = sink;
+    if (s.tslot && pos) s.lane_col = pos + b;
+    if (s.acc && second) s.acc = ctx->slot2.acc.as<Acc>();
+    return s;
+  };
+  auto backward = [&](int maxl, int cnt, const Sink &s) {
+    const uint64_t all = lanes_of(cnt), ovf = ctx->ws.last_ovf & all;
+    if (ovf != all) batch_backward(ctx, g, maxl, s, all & ~ovf);
+    if (ovf) {
+      // the extended form's state is not per slot: the other batch waits
+      for (cudaStream_t other : {ctx->stream, ctx->slot2.stream})
+        if (other) BCG_CUDA(cudaStreamSynchronize(other));
+      ext_source_batch(ctx, g, ctx->ws.sources.as<int32_t>(), ovf, s);
+      BCG_CUDA(cudaStreamSynchronize(ctx->stream));
+    }
+  };
+  auto load = [&](int b, int cnt) {
+    batch_ensure(ctx, g);
+    BCG_CUDA(cudaMemcpyAsync(ctx->ws.sources.p, src + b, (size_t)cnt * 4, cudaMemcpyDeviceToDevice, ctx->stream));
+  };
+  int b0 = 0;
+  // level by level while the graph's depth is not known, or where a second
+  // batch has no room
+  batch_ensure(ctx, g);
+  const int one = std::min(64, count);
+  const bool known = heavy_meta(ctx, g, true).depth >= 1 && ctx->push_div == 0;
+  const bool two = count > 64 && ctx->push_div == 0 && second_slot(ctx, g, sink.acc != nullptr);
+  if (!known || !two) {
+    const int upto = two ? one : count;
+    for (; b0 < upto; b0 += 64) {
+      const int cnt = std::min(64, count - b0);
+      load(b0, cnt);
+      const int maxl = batch_forward(ctx, g, cnt, false, OVF_EXTEND);
+      backward(maxl, cnt, batch_sink(b0, false));
+    }
+    if (b0 >= count) return;
+  }
+  BatchSlot &s2 = ctx->slot2;
+  BCG_CUDA(cudaEventRecord(s2.ev_begin, main));
+  BCG_CUDA(cudaStreamWaitEvent(s2.stream, s2.ev_begin, 0));
+  if (sink.acc) BCG_CUDA(cudaMemsetAsync(s2.acc.p, 0, (size_t)g.n * sizeof(Acc), s2.stream));
+  struct Flight {
+    int b = -1, cnt = 0, l = 0;
+    bool asked = false;  // the levels were launched blindly: ask for the outcome
+    std::unique_ptr<Forward> f;
+  } fl[2];
+  auto end = [&](bool second) {
+    Flight &f = fl[second];
+    if (f.b < 0) return;
+    SlotScope sc(ctx, second);
+    const int maxl = f.asked ? f.f->end_blind() : f.l;
+    backward(maxl, f.cnt, batch_sink(f.b, second));
+    f.b = -1;
+  };
+  try {
+    bool second = false;
+    for (int b = b0; b < count; b += 64, second = !second) {
+      Flight &f = fl[second];
+      f.cnt = std::min(64, count - b);
+      {
+        SlotScope sc(ctx, second);
+        load(b, f.cnt);
+        f.f.reset(new Forward(ctx, g, f.cnt, false, OVF_EXTEND));
+        f.f->init();
+        f.asked = f.f->blind();
+        if (!f.asked) f.l = f.f->run();
+        f.b = b;
+      }
+      end(!second);
+    }
+    end(second);
+    end(!second);
+    BCG_CUDA(cudaEventRecord(s2.ev_end, s2.stream));
+    BCG_CUDA(cudaStreamWaitEvent(main, s2.ev_end, 0));
+  } catch (...) {
+    cudaStreamSynchronize(s2.stream);
+    cudaStreamSynchronize(main);
+    throw;
+  }
+  if (sink.acc) {
+    LaunchScope ls(ctx, F_MISC);
+    k_add_acc<<<(g.n + 255) / 256, 256, 0, main>>>(g.n, s2.acc.as<Acc>(), sink.acc);
+  }
 }
 
 void batch_extract(bc_ctx *ctx, const Graph &g, int count, int maxlevel, int32_t *dist, uint64_t *sigma,

@@ -823,6 +823,10 @@ static void run_window(bc_ctx *ctx, const Graph &g, int W, Sink sink) {
   }
   const int32_t *sorted_src = ws.win.as<int32_t>() + WMAX;
   const int32_t *sorted_pos = ws.win.as<int32_t>() + 2 * WMAX;
+  if (width != 1 && !g.w) {
+    run_lane_batches(ctx, g, sorted_src, sorted_pos, W, sink);
+    return;
+  }
   for (int b = 0; b < W; b += width) {
     const int count = std::min(width, W - b);
     BCG_CUDA(cudaMemcpyAsync(ws.sources.p, sorted_src + b, (size_t)count * 4, cudaMemcpyDeviceToDevice, ctx->stream));
@@ -871,8 +875,11 @@ static void do_exact_or_uniform(bc_ctx *ctx, const Graph &g, bool exact, int64_t
   } else {
     // all n sources, grouped by key (the sum over sources is exact, so any order)
     const KeyMeta &km = key_meta(ctx, g, true);
+    if (width != 1 && !g.w) {
+      run_lane_batches(ctx, g, km.order.as<int32_t>(), nullptr, g.n, sink);
+    }
     const int step = g.w && width != 1 ? WMAX_SOLO : width;
-    for (int64_t i0 = 0; i0 < (int64_t)g.n; i0 += step) {
+    for (int64_t i0 = 0; (width == 1 || g.w) && i0 < (int64_t)g.n; i0 += step) {
       const int count = (int)std::min<int64_t>(step, (int64_t)g.n - i0);
       if (step > 64) {
         run_sources_per_cta(ctx, g, km.order.as<int32_t>() + i0, count, sink);
@@ -1779,6 +1786,7 @@ bc_status bc_create(bc_ctx **out, int device, const bc_options *opt) {
       ctx->pair_engine = (e == 1 || e == 2) ? e : 0;
     }
     if (const char *bo = std::getenv("BCG_BWD_OVERLAP")) ctx->bwd_overlap = std::atoi(bo) != 0;
+    if (const char *ov = std::getenv("BCG_BATCH_OVERLAP")) ctx->batch_overlap = std::atoi(ov) != 0;
     if (const char *fo = std::getenv("BCG_FWD_OVERLAP")) ctx->fwd_overlap = std::atoi(fo) != 0;
     if (const char *pt = std::getenv("BCG_PAIR_CTA_THREADS")) ctx->pair_cta_threads = std::atoi(pt) == 128 ? 128 : 256;
     if (const char *ph = std::getenv("BCG_PAIR_HASH")) ctx->pair_hash_lg = std::max(6, std::min(24, std::atoi(ph)));
@@ -1830,19 +1838,26 @@ void bc_destroy(bc_ctx *ctx) {
     }
     ctx->graphs.clear();
     Workspace &ws = ctx->ws;
-    for (DevBuf *b : {&ws.lm, &ws.vlist, &ws.vcnt, &ws.vedges, &ws.visited, &ws.sigma, &ws.active, &ws.wq, &ws.enable, &ws.sources, &ws.targets, &ws.pair_d,
-                      &ws.pair_sig, &ws.pair_exp, &ws.err, &ws.cnt, &ws.acc, &ws.tslot, &ws.tdelta, &ws.scan, &ws.misc, &ws.misc2,
-                      &ws.delta_lm, &ws.p_dist, &ws.p_sigma, &ws.p_coef, &ws.p_queue, &ws.p_ctr,
-                      &ws.x_dist, &ws.x_m, &ws.x_e, &ws.x_vis, &ws.x_nm, &ws.x_list, &ws.x_lmask, &ws.x_ctr,
-                      &ws.x_off, &ws.rows, &ws.win, &ws.slist, &ws.scnt, &ws.coef, &ws.recips, &ws.hcnt})
+    for (BatchState *b : {static_cast<BatchState *>(&ws), &ctx->slot2.state}) {
+      b->each([](DevBuf &x) { x.release(); });
+      if (b->pinned) cudaFreeHost(b->pinned);
+    }
+    for (DevBuf *b : {&ws.targets, &ws.pair_d, &ws.pair_sig, &ws.pair_exp, &ws.err, &ws.cnt, &ws.acc, &ws.tslot,
+                      &ws.tdelta, &ws.scan, &ws.misc, &ws.misc2, &ws.delta_lm, &ws.p_dist, &ws.p_sigma, &ws.p_coef,
+                      &ws.p_queue, &ws.p_ctr, &ws.x_dist, &ws.x_m, &ws.x_e, &ws.x_vis, &ws.x_nm, &ws.x_list,
+                      &ws.x_lmask, &ws.x_ctr, &ws.x_off, &ws.rows, &ws.win, &ctx->slot2.acc})
       b->release();
-    if (ws.pinned) cudaFreeHost(ws.pinned);
     for (cudaEvent_t e : ctx->event_pool) cudaEventDestroy(e);
     if (ctx->own_stream && ctx->stream) cudaStreamDestroy(ctx->stream);
     if (ctx->stream2) cudaStreamDestroy(ctx->stream2);
     if (ctx->side) cudaStreamDestroy(ctx->side);
     if (ctx->ev_fork) cudaEventDestroy(ctx->ev_fork);
     if (ctx->ev_join) cudaEventDestroy(ctx->ev_join);
+    BatchSlot &s2 = ctx->slot2;
+    for (cudaStream_t s : {s2.stream, s2.side})
+      if (s) cudaStreamDestroy(s);
+    for (cudaEvent_t e : {s2.ev_fork, s2.ev_join, s2.ev_begin, s2.ev_end})
+      if (e) cudaEventDestroy(e);
   }
   delete ctx;
 }

@@ -104,23 +104,39 @@ __device__ __forceinline__ void sink_targets(const Sink &sink, int32_t v, int t,
     if (!sink.eq || sink.lane_q[t] == sink.eq[e]) sink.tdelta[(size_t)e * sink.tstride + c] = d;
 }
 
-struct Workspace {
+// State of one 64-lane batch (two can be in flight: bc_ctx::slot2).
+struct BatchState {
   DevBuf lm;       // [lcap][n] u64 level masks
   int32_t lcap = 0;
   DevBuf visited;  // [n] u64
-  DevBuf sigma;    // [n][64] u64 sigma, overwritten by coef (double) in the backward
-  DevBuf active;   // [lcap+2] u64 OR of level masks; [0..] per level
-  DevBuf wq;       // [2*(lcap+2)] u32 work-queue counters (forward / backward per level)
-  // per level l of the last batched forward: the vertices with lanes at l
-  // (vlist[l*n ..], each once), their count vcnt[l] and degree sum vedges[l]
-  DevBuf vlist;    // [lcap][n] i32
-  DevBuf vcnt;     // [lcap+2] u32
-  DevBuf vedges;   // [lcap+2] u64 (kept with the direction switch on)
+  DevBuf sigma;    // [n][64] u64 sigma (overwritten by coef in the backward where counts are large)
   DevBuf coef, recips;  // backward coefficients as 96-bit numbers [n][64] (12 B each), reciprocals of small counts
-  DevBuf hcnt;         // per level: heavy segments listed forward, backward, vertices with several, - (u32)
-  DevBuf slist, scnt;  // light vertices a level left unfinished: [2][n] i32, their counts [lcap+2] u32
-  DevBuf enable;   // u64 lane enable mask
+  DevBuf ctl;      // [lcap+2] control words per level (bc_batch.cu)
+  DevBuf vlist;    // [lcap][n] i32: the vertices with lanes at each level, each once
+  DevBuf slist;    // [2][n] i32: light vertices a level left unfinished
+  DevBuf hlist, hmulti, hpart;  // a level's heavy segments, its vertices with several, partial sums [nseg][64]
+  DevBuf enable;   // u64: lane enable mask, pair continuation word, largest count, overflowed lanes
   DevBuf sources;  // [64] i32
+  uint64_t last_ovf = 0ull;      // lanes of the last forward whose counts exceeded 2^64-1
+  uint64_t last_sigmax = ~0ull;  // largest count of the last forward
+  std::vector<uint8_t> hlev;     // per level of the last forward: a heavy vertex has lanes there
+  void *pinned = nullptr;        // 4 KiB pinned host staging
+  template <class F> void each(F f) {
+    for (DevBuf *b : {&lm, &visited, &sigma, &coef, &recips, &ctl, &vlist, &slist, &hlist, &hmulti, &hpart, &enable,
+                      &sources})
+      f(*b);
+  }
+};
+
+// The second batch in flight: its state, streams and all-vertex sums.
+struct BatchSlot {
+  BatchState state;
+  cudaStream_t stream = nullptr, side = nullptr;
+  cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_begin = nullptr, ev_end = nullptr;
+  DevBuf acc;  // [n] Acc
+};
+
+struct Workspace : BatchState {
   DevBuf targets;  // [64] i32 pair destinations
   DevBuf pair_d;   // [64] i32 d(s,t) of pair lanes
   DevBuf pair_sig; // [64] u64 sigma_st of pair lanes (extended lanes: mantissa bits)
@@ -136,8 +152,6 @@ struct Workspace {
   DevBuf delta_lm; // [n][64] f64
   DevBuf win;      // draw window: draws[W] | sorted sources[W] | sorted positions[W]
   DevBuf rows;     // per-source output rows of one launch (one source per CTA)
-  uint64_t last_ovf = 0ull;  // lanes of the last batched forward whose counts exceeded 2^64-1
-  std::vector<uint8_t> hlev;  // per level of the last batched forward: a heavy vertex has lanes there
   // extended-form engine (bc_ext.cu): dist [n][64] i32, sigma/coef as
   // mantissa [n][64] f64 + exponent [n][64] i32, visited / next masks [n],
   // level entry lists with lane masks, level offsets (device and host copies)
@@ -145,8 +159,6 @@ struct Workspace {
   std::vector<unsigned long long> x_hoff;
   // plain single-source engine
   DevBuf p_dist, p_sigma, p_coef, p_queue, p_ctr;
-  void *pinned = nullptr;  // 4 KiB pinned host staging
-  uint64_t last_sigmax = ~0ull;  // largest sigma of the last batched forward pass
 };
 
 }  // namespace bcg
@@ -161,6 +173,8 @@ struct bc_ctx {
   cudaStream_t side = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   int32_t bwd_overlap = 1, fwd_overlap = 1;
+  bcg::BatchSlot slot2;       // second 64-lane batch in flight (BCG_BATCH_OVERLAP=0: one at a time)
+  int32_t batch_overlap = 1;
   int32_t batch_width = 0;
   std::recursive_mutex mu;
   std::atomic<int> api_waiting{0};  // API calls waiting for mu (the server worker yields to them)
@@ -289,6 +303,9 @@ void sigma_to_xf(bc_ctx *ctx, long long total, const uint64_t *sig, double *sm, 
 void batch_extract(bc_ctx *ctx, const Graph &g, int count, int maxlevel, int32_t *dist,
                    uint64_t *sigma, int64_t row_stride, int64_t lane_stride);
 void batch_ensure(bc_ctx *ctx, const Graph &g);
+// Sources src[0 .. count) in batches of 64, two in flight; lane columns from pos.
+void run_lane_batches(bc_ctx *ctx, const Graph &g, const int32_t *src, const int32_t *pos, int count,
+                      const Sink &sink);
 
 // ---- plain single-source engine ----
 // Forward + backward for one source; outputs to a sink laid out as for lane 0.

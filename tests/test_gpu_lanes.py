@@ -88,3 +88,20 @@ def test_directed_rows_without_successors(ctx):
     assert np.array_equal(got, oracle.uniform_sources(g, 100, 2, 3))
     ref = oracle.adaptive_sources(g, [0, 1, 7], 2.0, 200, 4, 5)
     assert np.array_equal(res["S"], ref["S"]) and np.array_equal(res["k"], ref["k"])
+
+
+def test_batches_in_flight_with_extended_lanes(ctx):
+    """Thirteen layers of 60 vertices: from the end layers counts reach 60^12 > 2^64,
+    from the middle ones they stay below; several batches in flight."""
+    w, layers = 60, 13
+    i, j = np.divmod(np.arange(w * w), w)
+    g = gg.from_edges(w * layers, np.concatenate([i + w * k for k in range(layers - 1)]),
+                      np.concatenate([j + w * (k + 1) for k in range(layers - 1)]))
+    h = ctx.load_graph(g.row_ptr, g.col)
+    got = [ctx.uniform_sources(h, 333, 6, 1) for _ in range(2)]  # the depth is known the second time
+    res = ctx.adaptive_sources(h, [0, 300, 779], 2.0, 600, 7, 2)
+    ctx.free_graph(h)
+    want = oracle.uniform_sources(g, 333, 6, 1)
+    assert np.array_equal(got[0], want) and np.array_equal(got[1], want)
+    ref = oracle.adaptive_sources(g, [0, 300, 779], 2.0, 600, 7, 2)
+    assert np.array_equal(res["S"], ref["S"]) and np.array_equal(res["k"], ref["k"])
