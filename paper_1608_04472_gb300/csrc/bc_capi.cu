@@ -180,26 +180,53 @@ struct ScanState {
 
 // Sequential stop test per target, in draw order (Sec. 4 step 3; Algorithm 1's
 // while-condition): S <- S + x_i, k <- k + 1, stop at the first S*scale > cn.
+// One warp per target: 32 values are read at once and only the non-zero ones
+// enter the serial chain (adding 0 changes neither S nor the test's outcome:
+// it failed for the S before, and for the first S = 0 as c*n > 0). Most pair values are 0. With a
+// thread per target reading its row on its own, a window of 4096 draws was
+// 4096 dependent steps of uncoalesced loads: 1.6 ms of the 12.1 ms of 6,000
+// pair draws with 64 targets, 0.8 of 2.5 ms of Bader's loop on ER n = 2000;
+// this way 0.08 and 0.2 ms (the whole: 6.4 ms with larger first windows, 1.15 ms).
 __global__ void k_stop_scan(int T, int count, const double *__restrict__ vals, ScanState st, int64_t k0,
                             double cn, double scale, int stride) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  const int lane = threadIdx.x & 31;
+  const int j = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
   if (j >= T || st.done[j]) return;
+  const double *row = vals + (size_t)j * stride;
   double S = st.S[j];
-  int64_t k = k0;
-  bool stop = false;
-  for (int t = 0; t < count; ++t) {
-    S = __dadd_rn(S, vals[(size_t)j * stride + t]);
-    k = k0 + t + 1;
-    if (__dmul_rn(S, scale) > cn) {
-      stop = true;
-      break;
+  int stop = -1;  // position of the draw that stops the target
+  double x = lane < count ? row[lane] : 0.0;
+  for (int t0 = 0; t0 < count && stop < 0; t0 += 32) {
+    const double next = t0 + 32 + lane < count ? row[t0 + 32 + lane] : 0.0;
+    unsigned m = __ballot_sync(FULL, x != 0.0);
+    if (__popc(m) >= 8) {
+      // values are not negative, so S never falls: if the test fails after the
+      // 32 draws it failed after each of them
+      double all = S;
+#pragma unroll
+      for (int i = 0; i < 32; ++i) all = __dadd_rn(all, __shfl_sync(FULL, x, i));
+      if (!(__dmul_rn(all, scale) > cn)) {
+        S = all;
+        m = 0u;
+      }
     }
+    for (; m; m &= m - 1u) {
+      const int i = __ffs(m) - 1;
+      S = __dadd_rn(S, __shfl_sync(FULL, x, i));
+      if (__dmul_rn(S, scale) > cn) {
+        stop = t0 + i;
+        break;
+      }
+    }
+    x = next;
   }
-  st.S[j] = S;
-  st.k[j] = k;
-  if (stop) {
-    st.done[j] = 1;
-    atomicSub(st.remaining, 1);
+  if (lane == 0) {
+    st.S[j] = S;
+    st.k[j] = k0 + (stop < 0 ? count : stop + 1);
+    if (stop >= 0) {
+      st.done[j] = 1;
+      atomicSub(st.remaining, 1);
+    }
   }
 }
 
@@ -960,7 +987,7 @@ static void do_adaptive_sources(bc_ctx *ctx, const Graph &g, const int32_t *targ
     run_window(ctx, g, W, sink);
     {
       LaunchScope ls(ctx, F_SCAN);
-      k_stop_scan<<<(T + 127) / 128, 128, 0, st>>>(T, W, ws.tdelta.as<double>(), ss, i0, cn, 1.0, W);
+      k_stop_scan<<<(T + 3) / 4, 128, 0, st>>>(T, W, ws.tdelta.as<double>(), ss, i0, cn, 1.0, W);
     }
     remaining = read_remaining(ctx, ss);
     i0 += W;
@@ -1129,6 +1156,7 @@ static void pair_window(bc_ctx *ctx, const Graph &g, int W, int32_t *wsrc, int32
 // warp search keeps that many pairs in flight at once) while the window's
 // T x W values stay small, else 1024.
 static int pair_window_max(int32_t T) { return T <= 4096 ? 4096 : WMAX; }
+constexpr int PAIR_FIRST = 1024;  // pairs in the first windows (about one per resident CTA)
 
 // The tables of the targets of the last pair-value block (d(v_j, .) and
 // sigma_{v_j .}, [n][Tp]), kept for the next block of the same query (graph
@@ -1247,11 +1275,14 @@ static void do_adaptive_pairs(bc_ctx *ctx, const Graph &g, const int32_t *target
     for (DevBuf *b : {&wsrc, &wdst, &wpd, &wpexp, &wpxf}) b->ensure(pwmax * 4);
     wpsig.ensure(pwmax * 8);
     int32_t remaining = T;
-    // windows of draws as in Bader's loop (64 .. 1024, growing with the draws
-    // made; one draw at a time with the plain width); the stop scan walks each
-    // window in draw order
+    // windows of draws as in Bader's loop, growing with the draws made (one draw
+    // at a time with the plain width); the stop scan walks each window in draw
+    // order. A window takes as long as its slowest pair while there are CTAs
+    // left, so the first ones hold a pair for every CTA (with 64 pairs first,
+    // 6,000 draws on BA n = 300,007 took 13 windows instead of 6).
+    const int64_t first = ctx->pair_engine == 1 ? 64 : PAIR_FIRST;
     for (int64_t i0 = 0; i0 < cap && remaining > 0;) {
-      const int64_t want = width == 1 ? 1 : std::max<int64_t>(64, i0 / 2);
+      const int64_t want = width == 1 ? 1 : std::max<int64_t>(first, i0 / 2);
       const int W = (int)std::min<int64_t>(std::min<int64_t>(pwmax, want), cap - i0);
       {
         LaunchScope ls(ctx, F_DRAW);
@@ -1269,7 +1300,7 @@ static void do_adaptive_pairs(bc_ctx *ctx, const Graph &g, const int32_t *target
       }
       {
         LaunchScope ls(ctx, F_SCAN);
-        k_stop_scan<<<(T + 127) / 128, 128, 0, st>>>(T, W, ws.tdelta.as<double>(), ss, i0, cn, scale, W);
+        k_stop_scan<<<(T + 3) / 4, 128, 0, st>>>(T, W, ws.tdelta.as<double>(), ss, i0, cn, scale, W);
       }
       remaining = read_remaining(ctx, ss);
       i0 += W;
