@@ -59,6 +59,7 @@ struct Graph {
   uint32_t *w = nullptr;
   uint32_t *w_in = nullptr;
   uint64_t w_step = 0;
+  uint64_t w_max = 1;  // longest edge
   // launch settings of this graph (bc_set_tuning / bc_autotune); unset: the
   // context's defaults
   bc_tuning tune{};
@@ -221,7 +222,7 @@ struct bc_ctx {
   int32_t pair_cta_threads = 256;
   int64_t pair_fallbacks = 0;  // pairs that search handed to the CTA form
   // weighted graphs: near-far threshold increment for graphs loaded later
-  // (0 = a sixth of the graph's mean edge length)
+  // (0 = by the graph's mean edge and row length)
   long long w_step = 0;
 };
 
