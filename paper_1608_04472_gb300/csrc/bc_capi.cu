@@ -370,43 +370,59 @@ __global__ void k_validate(int32_t n, const int32_t *__restrict__ rp, const int3
   }
 }
 
-// Key of a vertex for grouping sampled sources: its distance from the graph's
-// highest-degree vertex (capped at 254), 255 when unreachable from it.
 // Source keys (Sec. 3's per-sample step is the same for every source; only
 // which sources share a 64-lane batch changes the work): the distances of each
 // vertex to K landmarks, projected on their first principal component and
-// quantised to 8 bits, so that sources with similar BFS level structure sort
-// next to each other. Landmark 0 is the hub; landmark i+1 is the vertex reached
-// from the hub that is farthest from landmarks 0..i (smallest index on ties).
+// quantised to 8 bits (255: not reached from the hub), so that sources with
+// similar BFS level structure sort next to each other. Landmark 0 is the hub,
+// the others are vertices drawn at random from those with edges that reach it,
+// so that one 64-lane forward pass gives all their distances. (Before, one
+// plain search per landmark, each the farthest from those before: first call /
+// later calls in ms on R-MAT s20 k = 1024 112 / 35.8 -> 49 / 34.6, s16 Bader 1500
+// draws 29 / 11.6 -> 14.3 / 11.4, directed s17 k = 512 17 / 5.2 -> 8.8 / 5.2. With 1, 8,
+// 16, 32 landmarks s20 takes 44.7, 38.5, 37.6, 37.0.)
 
-// Row l of the landmark distances as bytes (254 caps a distance, 255: not
-// reached) and the running minimum over landmarks (-1: not reached from the
-// hub). The first row also gives the hub's eccentricity.
-__global__ void k_land_row(int32_t n, const int32_t *__restrict__ dist, uint8_t *__restrict__ row,
-                           int32_t *__restrict__ mind, int first, int *__restrict__ maxd) {
+// Row 0: the hub's distances as bytes (254 caps a distance, 255: not reached)
+// and its eccentricity.
+__global__ void k_land_hub(int32_t n, const int32_t *__restrict__ dist, uint8_t *__restrict__ row,
+                           int *__restrict__ maxd) {
   const int32_t v = blockIdx.x * blockDim.x + threadIdx.x;
-  if (v >= n) return;
-  const int32_t d = dist[v];
-  row[v] = d < 0 ? 255 : (uint8_t)(d > 254 ? 254 : d);
-  if (first) {
-    mind[v] = d;
-    if (d > 0) atomicMax(maxd, d);
-  } else if (mind[v] >= 0 && d >= 0 && d < mind[v]) {
-    mind[v] = d;
+  int d = -1;
+  if (v < n) {
+    d = dist[v];
+    row[v] = d < 0 ? 255 : (uint8_t)(d > 254 ? 254 : d);
   }
+  d = __reduce_max_sync(FULL, d);
+  if ((threadIdx.x & 31) == 0 && d > 0) atomicMax(maxd, d);
 }
 
-// (mind << 32) | ~v, maximised over the vertices: the farthest vertex, the
-// smallest index among equals.
-__global__ void k_land_far(int32_t n, const int32_t *__restrict__ mind, unsigned long long *__restrict__ best) {
+// Candidate landmarks: vertices with edges, by the draws of a fixed stream (a
+// vertex without edges gives way to the next one with some, in id order).
+__global__ void k_land_draw(int32_t n, const int32_t *__restrict__ rp, int32_t *__restrict__ out) {
+  int32_t v = draw_source(0x6C616E646D61726Bull, 0ull, (uint64_t)threadIdx.x, n);
+  for (int i = 0; i < 4096 && rp[v + 1] == rp[v]; ++i) v = v + 1 < n ? v + 1 : 0;
+  out[threadIdx.x] = v;
+}
+
+// Rows 1..K-1 from the level masks of a forward pass: row r has the distances
+// from the lane with row_of_lane = r (rows start at 255).
+__global__ void k_land_rows(int32_t n, int K, int maxlevel, const uint64_t *__restrict__ lm,
+                            const int8_t *__restrict__ row_of_lane, uint8_t *__restrict__ rows) {
   const int32_t v = blockIdx.x * blockDim.x + threadIdx.x;
-  unsigned long long x = 0;
-  if (v < n && mind[v] >= 0) x = ((unsigned long long)mind[v] << 32) | (uint32_t)~(uint32_t)v;
-  for (int o = 16; o > 0; o >>= 1) {
-    const unsigned long long y = __shfl_xor_sync(0xffffffffu, x, o);
-    x = y > x ? y : x;
-  }
-  if ((threadIdx.x & 31) == 0 && x) atomicMax(best, x);
+  if (v >= n) return;
+  for (int l = 0; l <= maxlevel; ++l)
+    for (uint64_t m = lm[(size_t)l * n + v]; m; m &= m - 1ull) {
+      const int r = row_of_lane[__ffsll((long long)m) - 1];
+      if (r > 0) rows[(size_t)r * n + v] = (uint8_t)(l > 254 ? 254 : l);
+    }
+}
+
+// The lanes whose source reaches the hub.
+__global__ void k_land_reach(int32_t n, int32_t hub, int maxlevel, const uint64_t *__restrict__ lm,
+                             unsigned long long *__restrict__ out) {
+  unsigned long long m = 0;
+  for (int l = 0; l <= maxlevel; ++l) m |= lm[(size_t)l * n + hub];
+  *out = m;
 }
 
 constexpr int KEY_LM_MAX = 32;
@@ -625,7 +641,7 @@ static void copy_scan_out(bc_ctx *ctx, int32_t T, const ScanState &st, double sc
 // ---------------------------------------------------------------- drivers ---
 
 // Per-graph source keys (landmark projection, above) and, for exact BC, all
-// vertices ordered by key; computed on first use from K BFSs (K = 32, or
+// vertices ordered by key; computed on first use from K landmarks (K = 32, or
 // BCG_KEY_LANDMARKS; 1 gives the hub distance alone, rescaled).
 struct KeyMeta {
   DevBuf key, order;
@@ -680,56 +696,74 @@ static void build_key(bc_ctx *ctx, const Graph &g, KeyMeta &km) {
   Workspace &ws = ctx->ws;
   cudaStream_t st = ctx->stream;
   const size_t n = (size_t)g.n;
-  const int K = key_landmarks();
+  // edge lengths: a source has a CTA of its own, so the hub's row is enough
+  const int K = g.w ? 1 : key_landmarks();
   const unsigned nb = (unsigned)((n + 255) / 256);
   const int64_t s0 = ctx->samples, b0 = ctx->batches;
-  DevBuf dist, mind, rows, proj, small;
+  DevBuf dist, rows, proj, small;
   auto release_all = [&] {
-    for (DevBuf *b : {&dist, &mind, &rows, &proj, &small}) b->release();
+    for (DevBuf *b : {&dist, &rows, &proj, &small}) b->release();
   };
   try {
     dist.ensure(n * 4 + 8);
-    mind.ensure(n * 4);
-    rows.ensure(n * K);
-    // small: [0] landmark, [8] max distance, [16] farthest (u64), [32] range, [64] w|mu, [512] moments
-    small.ensure(512 + 8 * KEY_MOM_THREADS);
+    rows.ensure(n);
+    // small: [0] the hub, [8] max distance, [16] lanes that reach the hub (u64), [32] range, [64] w|mu,
+    // [320] row of each lane, [384] the caller's sources (64), [1024] moments
+    small.ensure(1024 + 8 * KEY_MOM_THREADS);
     char *sm = small.as<char>();
     int32_t *d_src = reinterpret_cast<int32_t *>(sm);
     int *d_maxd = reinterpret_cast<int *>(sm + 8);
-    unsigned long long *d_far = reinterpret_cast<unsigned long long *>(sm + 16);
+    unsigned long long *d_reach = reinterpret_cast<unsigned long long *>(sm + 16);
     int *d_range = reinterpret_cast<int *>(sm + 32);
     float *d_wmu = reinterpret_cast<float *>(sm + 64);  // w[KEY_LM_MAX] | mu[KEY_LM_MAX]
-    unsigned long long *d_mom = reinterpret_cast<unsigned long long *>(sm + 512);
+    unsigned long long *d_mom = reinterpret_cast<unsigned long long *>(sm + 1024);
     BCG_CUDA(cudaMemsetAsync(sm, 0, small.bytes, st));
-    int32_t L = g.hub;
-    int Kused = 0;
-    for (int i = 0; i < K; ++i) {
-      BCG_CUDA(cudaMemcpyAsync(d_src, &L, 4, cudaMemcpyHostToDevice, st));
-      plain_distances(ctx, g, d_src, dist.as<int32_t>());  // any depth
+    BCG_CUDA(cudaMemcpyAsync(d_src, &g.hub, 4, cudaMemcpyHostToDevice, st));
+    plain_distances(ctx, g, d_src, dist.as<int32_t>());  // any depth
+    {
+      LaunchScope ls(ctx, F_MISC);
+      k_land_hub<<<nb, 256, 0, st>>>(g.n, dist.as<int32_t>(), rows.as<uint8_t>(), d_maxd);
+    }
+    BCG_CUDA(cudaMemcpyAsync(ws.pinned, d_maxd, 4, cudaMemcpyDeviceToHost, st));
+    sync(ctx);
+    km.ecc = *static_cast<int32_t *>(ws.pinned);
+    int Kused = 1;
+    // deep graphs run one source per persistent CTA, where batches do not
+    // share traversals: the hub distance alone (also where a forward pass's
+    // state, about 700 B per vertex, would not leave room)
+    bool more = K > 1 && km.ecc > 0 && km.ecc <= 64;
+    if (more) {
+      size_t fr = 0, tot = 0;
+      if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) cudaGetLastError();
+      more = n * (size_t)(K + (ws.sigma.bytes < n * 512 ? 700 : 0)) < fr / 2;
+    }
+    if (more) {
+      // (the caller may have its batch's sources in place already)
+      BCG_CUDA(cudaMemcpyAsync(sm + 384, ws.sources.p, 64 * 4, cudaMemcpyDeviceToDevice, st));
       {
         LaunchScope ls(ctx, F_MISC);
-        k_land_row<<<nb, 256, 0, st>>>(g.n, dist.as<int32_t>(), rows.as<uint8_t>() + (size_t)i * n,
-                                       mind.as<int32_t>(), i == 0, d_maxd);
+        k_land_draw<<<1, 64, 0, st>>>(g.n, g.rp, ws.sources.as<int32_t>());
       }
-      ++Kused;
-      if (i == 0) {
-        BCG_CUDA(cudaMemcpyAsync(ws.pinned, d_maxd, 4, cudaMemcpyDeviceToHost, st));
-        sync(ctx);
-        km.ecc = *static_cast<int32_t *>(ws.pinned);
-      }
-      // deep graphs run one source per persistent CTA, where batches do not
-      // share traversals: the hub distance alone
-      if (i + 1 == K || km.ecc > 64) break;
+      const int maxl = batch_forward(ctx, g, 64, false, OVF_IGNORE);
       {
         LaunchScope ls(ctx, F_MISC);
-        BCG_CUDA(cudaMemsetAsync(d_far, 0, 8, st));
-        k_land_far<<<nb, 256, 0, st>>>(g.n, mind.as<int32_t>(), d_far);
-        BCG_CUDA(cudaMemcpyAsync(ws.pinned, d_far, 8, cudaMemcpyDeviceToHost, st));
+        k_land_reach<<<1, 1, 0, st>>>(g.n, g.hub, maxl, ws.lm.as<uint64_t>(), d_reach);
       }
+      BCG_CUDA(cudaMemcpyAsync(ws.pinned, d_reach, 8, cudaMemcpyDeviceToHost, st));
       sync(ctx);
-      const unsigned long long far = *static_cast<unsigned long long *>(ws.pinned);
-      if ((far >> 32) == 0) break;  // every vertex reached from the hub is a landmark
-      L = (int32_t)~(uint32_t)(far & 0xFFFFFFFFull);
+      const uint64_t reach = *static_cast<uint64_t *>(ws.pinned);
+      int8_t row[64] = {};
+      for (int t = 0; t < 64 && Kused < K; ++t)
+        if ((reach >> t) & 1ull) row[t] = (int8_t)Kused++;
+      BCG_CUDA(cudaMemcpyAsync(sm + 320, row, 64, cudaMemcpyHostToDevice, st));
+      if (Kused > 1) {
+        rows.grow_keep(n * (size_t)Kused, st);
+        BCG_CUDA(cudaMemsetAsync(rows.as<uint8_t>() + n, 255, n * (size_t)(Kused - 1), st));
+        LaunchScope ls(ctx, F_MISC);
+        k_land_rows<<<nb, 256, 0, st>>>(g.n, Kused, maxl, ws.lm.as<uint64_t>(),
+                                        reinterpret_cast<const int8_t *>(sm + 320), rows.as<uint8_t>());
+      }
+      BCG_CUDA(cudaMemcpyAsync(ws.sources.p, sm + 384, 64 * 4, cudaMemcpyDeviceToDevice, st));
     }
     const int nmom = 1 + Kused + Kused * (Kused + 1) / 2;
     {

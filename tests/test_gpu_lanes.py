@@ -105,3 +105,22 @@ def test_batches_in_flight_with_extended_lanes(ctx):
     assert np.array_equal(got[0], want) and np.array_equal(got[1], want)
     ref = oracle.adaptive_sources(g, [0, 300, 779], 2.0, 600, 7, 2)
     assert np.array_equal(res["S"], ref["S"]) and np.array_equal(res["k"], ref["k"])
+
+
+@pytest.mark.parametrize("shape", ["edgeless", "matching", "star", "two_stars", "complete", "chain_into_hub"])
+def test_source_key_where_landmarks_run_out(ctx, shape):
+    """No landmark but the hub, none that reaches it, none of another distance;
+    a directed chain of 150 arcs into the hub (deeper than the hub's own reach)."""
+    i = np.arange(60)
+    edges = {"edgeless": (i[:0], i[:0]), "matching": (i[0:40:2], i[1:40:2]), "star": (0 * i[1:], i[1:]),
+             "two_stars": (np.repeat([0, 30], 29), np.delete(i, [0, 30])), "complete": np.triu_indices(60, 1)}
+    if shape == "chain_into_hub":
+        c = np.arange(150)
+        g = gg.from_edges_directed(200, np.r_[c, np.full(49, 150)], np.r_[c + 1, np.arange(151, 200)])
+    else:
+        g = gg.from_edges(60, *edges[shape])
+    h = ctx.load_graph(g.row_ptr, g.col, directed=shape == "chain_into_hub")
+    got, exact = ctx.uniform_sources(h, 300, 4, 6), ctx.exact(h)
+    ctx.free_graph(h)
+    assert np.array_equal(got, oracle.uniform_sources(g, 300, 4, 6))
+    assert np.array_equal(exact, oracle.exact_bc(g))
