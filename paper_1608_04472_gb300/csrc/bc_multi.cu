@@ -16,6 +16,8 @@
 // in the extended form (bc_xf.cuh; sums in CSR order of the vertex).
 #include <algorithm>
 #include <cstring>
+#include <map>
+#include <tuple>
 #include <vector>
 
 #include "bc_internal.h"
@@ -32,6 +34,11 @@ struct MItem {
 
 extern __shared__ uint4 solo_shared[];
 
+__device__ __forceinline__ void prefetch_acc(const Acc *a) {
+  asm volatile("prefetch.global.L1 [%0];" ::"l"(a));
+  asm volatile("prefetch.global.L1 [%0];" ::"l"(&a->w2));
+}
+
 // Sources [0, count) delivered to the sink (lane t = source t; all-vertex sums
 // to per-CTA partials) and, where asked, to per-source rows.
 template <int TIER, int T>
@@ -44,7 +51,7 @@ k_solo(MGraph G, SoloSources src, int count, unsigned *__restrict__ next, unsign
   Acc *part = partials ? partials + (size_t)blockIdx.x * G.n : nullptr;
   if (part)
     for (int32_t v = threadIdx.x; v < G.n; v += T) part[v] = acc_zero();
-  if (threadIdx.x == 0) c.nhuge[0] = c.nhuge[1] = c.nhuge[2] = c.grab[0] = c.grab[1] = 0;
+  solo_init(c);
   int ph = 0;
   unsigned e = 0u;
   for (;;) {
@@ -90,6 +97,9 @@ k_solo(MGraph G, SoloSources src, int count, unsigned *__restrict__ next, unsign
         acc_add(cur, delta, e);
         part[v] = cur;
       }
+    }, [&](int32_t v) {
+      if (part) prefetch_acc(part + v);
+      if (sink.tslot) asm volatile("prefetch.global.L1 [%0];" ::"l"(sink.tslot + v));
     });
     __syncthreads();
   }
@@ -103,7 +113,7 @@ k_multi(const MGraph *__restrict__ graphs, const MItem *__restrict__ items, int 
         unsigned char *__restrict__ scratch, size_t stride, Acc *__restrict__ partials, unsigned *__restrict__ err) {
   __shared__ SoloCtl c;
   unsigned e = 0u;
-  if (threadIdx.x == 0) c.nhuge[0] = c.nhuge[1] = c.nhuge[2] = c.grab[0] = c.grab[1] = 0;
+  solo_init(c);
   int ph = 0;
   for (;;) {
     if (threadIdx.x == 0) c.item = (int)atomicAdd(next, 1u);
@@ -124,7 +134,7 @@ k_multi(const MGraph *__restrict__ graphs, const MItem *__restrict__ items, int 
         Acc cur = part[v];
         acc_add(cur, delta, e);
         part[v] = cur;
-      });
+      }, [&](int32_t v) { prefetch_acc(part + v); });
     }
     __syncthreads();  // c.item is rewritten only after every thread has used it
   }
@@ -145,7 +155,7 @@ k_solo_targets(MGraph G, const int32_t *__restrict__ targets, int count, int Tp,
   __shared__ SoloCtl c;
   const SoloMem<TIER> S =
       solo_mem<TIER>(reinterpret_cast<unsigned char *>(solo_shared), scratch + (size_t)blockIdx.x * stride, G.n, G.nnz);
-  if (threadIdx.x == 0) c.nhuge[0] = c.nhuge[1] = c.nhuge[2] = c.grab[0] = c.grab[1] = 0;
+  solo_init(c);
   int ph = 0;
   for (;;) {
     if (threadIdx.x == 0) c.item = (int)atomicAdd(next, 1u);
@@ -186,7 +196,7 @@ k_solo_pairs(MGraph G, const int32_t *__restrict__ sources, const int32_t *__res
   __shared__ SoloCtl c;
   const SoloMem<TIER> S =
       solo_mem<TIER>(reinterpret_cast<unsigned char *>(solo_shared), scratch + (size_t)blockIdx.x * stride, G.n, G.nnz);
-  if (threadIdx.x == 0) c.nhuge[0] = c.nhuge[1] = c.nhuge[2] = c.grab[0] = c.grab[1] = 0;
+  solo_init(c);
   int ph = 0;
   for (;;) {
     if (threadIdx.x == 0) c.item = (int)atomicAdd(next, 1u);
@@ -249,6 +259,10 @@ __global__ void k_multi_reduce(const MGraph *__restrict__ graphs, const int32_t 
 // Shared memory a CTA can have for its state beside SoloCtl.
 constexpr size_t SOLO_SMEM_MAX = (size_t)227 * 1024 - sizeof(SoloCtl) - 64;
 
+// An SM's shared memory and what a CTA takes of it.
+constexpr size_t SOLO_SM_SMEM = (size_t)228 * 1024;
+static size_t solo_cta_smem(int tier, int32_t n) { return solo_smem(tier, n) + sizeof(SoloCtl) + 1024; }
+
 struct SoloCfg {
   int tier = 2, threads = 256, ncta = 1;
   size_t smem = 0, stride = 0;
@@ -293,7 +307,9 @@ template <class F> static auto solo_form(const SoloCfg &c, F fn) {
 
 template <class K> static int solo_resident(K kern, const SoloCfg &c) {
   int per = 0;
-  if (c.smem) BCG_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c.smem));
+  // (the most any graph asks for, so that another graph's launch, in this plan or
+  // on another thread, does not lower it)
+  if (c.smem) BCG_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SOLO_SMEM_MAX));
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, c.threads, c.smem) != cudaSuccess || per < 1) {
     cudaGetLastError();
     per = 1;
@@ -314,15 +330,23 @@ static SoloCfg solo_cfg(bc_ctx *ctx, int tier, int32_t n, int64_t nnz, int64_t c
   c.smem = solo_smem(tier, n);
   c.stride = solo_stride(tier, n, nnz);
   if (tier < 2 && !deep) {
-    const size_t cta = c.smem + sizeof(SoloCtl) + 1024;
     const bool few = count <= solo_sms() && n >= 4096;
-    c.threads = (tier == 0 && 3 * cta <= (size_t)228 * 1024 && !few) ? 256 : 1024;
+    c.threads = (tier == 0 && 3 * solo_cta_smem(tier, n) <= SOLO_SM_SMEM && !few) ? 256 : 1024;
   }
   if (tier < 2 && ctx->solo_threads) c.threads = ctx->solo_threads;
   return c;
 }
+//
+// A deep graph's levels keep few of an SM's threads busy, so what counts is how
+// many sources an SM has at once: where four CTAs' counts don't fit its shared
+// memory (n > 4,700) they go to L2 (tier 1), unless there is no more than one
+// source per SM. 4096 sources on square grids, ms, tier 0 / tier 1: n = 2500 3.2 /
+// 3.9, 5000 5.9 / 5.7, 10,000 21.3 / 8.6, 18,000 31.8 / 13.2.
 static SoloCfg solo_cfg(bc_ctx *ctx, const Graph &g, int64_t count) {
-  return solo_cfg(ctx, solo_tier(g), g.n, g.nnz, count, graph_depth_hint(ctx, g) > ctx->deep_levels);
+  const bool deep = graph_depth_hint(ctx, g) > ctx->deep_levels;
+  int tier = solo_tier(g);
+  if (tier == 0 && deep && count > solo_sms() && 4 * solo_cta_smem(0, g.n) > SOLO_SM_SMEM) tier = 1;
+  return solo_cfg(ctx, tier, g.n, g.nnz, count, deep);
 }
 
 // Resident CTAs over all SMs (at most `cap` per SM when cap > 0, at most
@@ -429,17 +453,20 @@ static void enqueue_multi(bc_ctx *ctx, MultiPlan &P) {
 
 // Items: each graph's draws are cut into runs of about equal cost (cost of a
 // source ~ n + nnz), at least 4 runs per CTA overall. Graphs whose state has
-// the same tier and CTA size form a group with its own launch; a group's runs
-// are queued largest first so its CTAs finish close together.
+// the same tier and CTA size and fits an SM as often (up to four times) form a
+// group with its own launch, so that the largest graph's shared memory does not
+// set the CTAs per SM for all; a group's runs are queued largest first so its
+// CTAs finish close together.
 static void build_plan(bc_ctx *ctx, MultiPlan &P, const std::vector<const Graph *> &gs) {
   const int G = (int)gs.size();
   P.G = G;
   P.nmax = 1;
   P.total_n = 0;
-  std::map<std::pair<int, int>, std::vector<int>> by;  // (tier, threads) -> graphs
+  std::map<std::tuple<int, int, int>, std::vector<int>> by;  // (tier, threads, 4 - CTAs per SM) -> graphs
   for (int g = 0; g < G; ++g) {
-    const int tier = solo_tier(*gs[g]);
-    by[{tier, solo_cfg(ctx, *gs[g], (int64_t)1 << 30).threads}].push_back(g);
+    const SoloCfg c = solo_cfg(ctx, *gs[g], (int64_t)1 << 30);
+    const int per_sm = (int)std::min<size_t>(c.threads == 1024 ? 1 : 4, SOLO_SM_SMEM / solo_cta_smem(c.tier, gs[g]->n));
+    by[{c.tier, c.threads, 4 - per_sm}].push_back(g);
     P.nmax = std::max(P.nmax, gs[g]->n);
     P.total_n += gs[g]->n;
   }
@@ -456,8 +483,8 @@ static void build_plan(bc_ctx *ctx, MultiPlan &P, const std::vector<const Graph 
       zmax = std::max(zmax, gs[g]->nnz);
       total += (double)P.k[g] * (double)(gs[g]->n + gs[g]->nnz);
     }
-    m.cfg = solo_cfg(ctx, it->first.first, nmax, zmax, (int64_t)1 << 30, false);
-    m.cfg.threads = it->first.second;
+    m.cfg = solo_cfg(ctx, std::get<0>(it->first), nmax, zmax, (int64_t)1 << 30, false);
+    m.cfg.threads = std::get<1>(it->first);
     solo_form(m.cfg, [&](auto f) {
       solo_ctas(m.cfg, k_multi<decltype(f)::tier, decltype(f)::threads>, (int64_t)1 << 30, m.cfg.stride, P.cap_per_sm);
       return 0;

@@ -12,11 +12,16 @@
 // and, on deep graphs, the latency of a level's chain of dependent loads. Two
 // passes over all edges forward and one backward, a row per group of threads,
 // took 190 instructions per edge visit on ER n = 2000 (issue 56 %, 0.50 us a
-// source); hence the single flattened pass and the edge bits. The state tiers:
+// source); hence the single flattened pass and the edge bits. On deep graphs a
+// level is one round of a few warps, so its chain was shortened: a level's
+// entries also in shared memory, one barrier a level forward, the next level's
+// entries and row bounds loaded a level ahead in the backward pass, in the
+// extended form one pass instead of a push and a pull, no FP64 multiplication by
+// powers of two (256 sources on a 200x200 grid 3.21 -> 2.55 ms). The state tiers:
 //   tier 0  distances, queue and counts in shared memory, 12 B per vertex
 //           (n up to ~18,500);
 //   tier 1  distances (2 B) in shared memory, queue and counts in global
-//           memory, where 152 CTAs' arrays mostly fit L2 (n up to ~113,000);
+//           memory, where 152 CTAs' arrays mostly fit L2 (n up to ~111,000);
 //   tier 2  everything in global memory (any n).
 // Where each is taken, with the times: solo_fits (bc_multi.cu).
 #pragma once
@@ -44,11 +49,13 @@ constexpr int SOLO_NEAR = 512;  // level offsets kept in shared memory (the rest
 constexpr int SOLO_HUGE = 64;   // rows taken by the whole CTA per pass (more fall back to a warp)
 constexpr int SOLO_HUGE_DEG = 2048;
 constexpr int SOLO_U = 4;       // 32-edge windows a warp has in flight at once
+constexpr int SOLO_RING = 512;  // tiers 1, 2: entries of a level kept in shared memory too
 
 struct SoloCtl {
   int item, tail;
+  int ovf;                      // a count left 64 bits (tail, ovf: the weighted engine's)
   int nhuge[3];                 // longest rows found by pass ph in slot ph % 3
-  int ovf;                      // a count of the last level left 64 bits
+  int found[3], over[3];        // vertices reached by pass ph; a count left 64 bits in it
   int l53;                      // first level with a count of 2^53 or more
   int grab[2];                  // next list position of the running and of the next pass
   unsigned long long maxc;      // largest count
@@ -71,6 +78,7 @@ template <int TIER> struct SoloMem {
   using Q = typename std::conditional<TIER == 0, uint16_t, int32_t>::type;
   D *dist;
   Q *queue;
+  int32_t *ring;       // tiers 1, 2: the first SOLO_RING entries of level l at (l & 1) * SOLO_RING
   uint64_t *val;       // tiers 1, 2: counts, then coefficients (double bits; mantissas in the extended form)
   uint32_t *lo, *hi;   // tier 0: the same in halves (shared memory adds 32 bits at once)
   int32_t *exp;        // exponents of the extended form
@@ -107,7 +115,7 @@ __host__ __device__ inline size_t solo_al(size_t x) { return (x + 255) / 256 * 2
 // Shared and global bytes of one CTA's state.
 __host__ __device__ inline size_t solo_smem(int tier, int32_t n) {
   const size_t d = ((size_t)n * 2 + 15) / 16 * 16, w = ((size_t)n * 4 + 15) / 16 * 16;
-  return tier == 0 ? 2 * d + 2 * w : (tier == 1 ? d : 0);
+  return tier == 0 ? 2 * d + 2 * w : (tier == 1 ? d : 0) + 8 * SOLO_RING;
 }
 __host__ __device__ inline size_t solo_stride(int tier, int32_t n, int64_t nnz) {
   const size_t a4 = solo_al((size_t)n * 4 + 8);
@@ -133,7 +141,8 @@ __device__ __forceinline__ SoloMem<TIER> solo_mem(unsigned char *sm, unsigned ch
   } else {
     S.queue = reinterpret_cast<int32_t *>(gm);
     S.val = reinterpret_cast<uint64_t *>(gm + a4);
-    if constexpr (TIER == 1) S.dist = reinterpret_cast<uint16_t *>(sm);
+    S.ring = reinterpret_cast<int32_t *>(sm);
+    if constexpr (TIER == 1) S.dist = reinterpret_cast<uint16_t *>(sm + 8 * SOLO_RING);
     else S.dist = reinterpret_cast<int32_t *>(gm + a4 + solo_al((size_t)n * 8));
   }
   return S;
@@ -166,19 +175,33 @@ template <int TIER> __device__ __forceinline__ int solo_lo(const SoloMem<TIER> &
   return l < SOLO_NEAR ? c.near[l] : S.far[l];
 }
 
+// Queue entry idx of level l, which starts at position b. A level's entries go
+// to shared memory as they are found, so a narrow level's next pass starts
+// without a round trip to L2.
+template <int TIER> __device__ __forceinline__ int32_t solo_entry(const SoloMem<TIER> &S, int l, int b, int idx) {
+  if constexpr (TIER != 0)
+    if (idx - b < SOLO_RING) return S.ring[(l & 1) * SOLO_RING + idx - b];
+  return S.queue[idx];
+}
+
+__device__ __forceinline__ void solo_init(SoloCtl &c) {
+  if (threadIdx.x < 3) c.nhuge[threadIdx.x] = c.found[threadIdx.x] = c.over[threadIdx.x] = 0;
+  if (threadIdx.x < 2) c.grab[threadIdx.x] = 0;
+}
+
 // A pass over list positions [b, e) in runs of 32 from a shared counter (uneven
 // rows spread over the warps). Returns the warp's next run or e. ph counts the
 // passes, the same in every thread. A pass clears the next one's counters: that
-// pass's list position was last used one pass ago, its count of longest rows
-// was last read two passes ago, each before the barrier that ended the pass
-// before this one.
+// pass's list position was last used one pass ago, what it finds was last read
+// two passes ago, each before the barrier that ended the pass before this one.
 __device__ __forceinline__ void solo_begin(SoloCtl &c, int ph) {
   if (threadIdx.x == 0) {
     c.grab[(ph + 1) & 1] = 0;
-    c.nhuge[(ph + 1) % 3] = 0;
+    c.nhuge[(ph + 1) % 3] = c.found[(ph + 1) % 3] = c.over[(ph + 1) % 3] = 0;
   }
 }
 __device__ __forceinline__ int solo_next(SoloCtl &c, int b, int e, int ph) {
+  if (b >= e) return e;  // (the first run is the warp's by its number: a narrow level has no other)
   int k = 0;
   if ((threadIdx.x & 31) == 0) k = atomicAdd(&c.grab[ph & 1], 32);
   return min(e, b + __shfl_sync(FULL, k, 0));
@@ -186,10 +209,12 @@ __device__ __forceinline__ int solo_next(SoloCtl &c, int b, int e, int ph) {
 
 // U edge visits per thread (w[u] < 0: none): finds the vertices not reached so
 // far (they join `level` and the queue), adds sv[u] to the count of every
-// endpoint at `level`, and returns the warp's shortest-path bits in bal[u].
+// endpoint at `level`, and returns the warp's shortest-path bits in bal[u]. The
+// level starts at queue position e; slot: the pass's counters.
 template <int TIER, int U, bool COUNT>
-__device__ __forceinline__ void solo_visit(const SoloMem<TIER> &S, SoloCtl &c, int level, const int32_t (&w)[U],
-                                           const uint64_t (&sv)[U], unsigned (&bal)[U], const int32_t *rp) {
+__device__ __forceinline__ void solo_visit(const SoloMem<TIER> &S, SoloCtl &c, int level, int e, int slot,
+                                           const int32_t (&w)[U], const uint64_t (&sv)[U], unsigned (&bal)[U],
+                                           const int32_t *rp) {
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
   const typename SoloMem<TIER>::D code = solo_code<TIER>(level);
@@ -213,12 +238,15 @@ __device__ __forceinline__ void solo_visit(const SoloMem<TIER> &S, SoloCtl &c, i
   }
   if (total) {  // one queue reservation for the warp's finds
     int base = 0;
-    if (lane == 0) base = atomicAdd(&c.tail, total);
+    if (lane == 0) base = atomicAdd(&c.found[slot], total);
     base = __shfl_sync(FULL, base, 0);
 #pragma unroll
     for (int u = 0; u < U; ++u)
       if (won[u]) {
-        S.queue[base + at[u]] = (typename SoloMem<TIER>::Q)w[u];
+        const int q = base + at[u];
+        S.queue[e + q] = (typename SoloMem<TIER>::Q)w[u];
+        if constexpr (TIER != 0)
+          if (q < SOLO_RING) S.ring[(level & 1) * SOLO_RING + q] = w[u];
         asm volatile("prefetch.global.L1 [%0];" ::"l"(rp + w[u]));  // the next pass reads its row bounds
       }
   }
@@ -227,7 +255,7 @@ __device__ __forceinline__ void solo_visit(const SoloMem<TIER> &S, SoloCtl &c, i
 #pragma unroll
     for (int u = 0; u < U; ++u)
       if (dag[u]) ov |= S.add(w[u], sv[u]);
-    if (ov) c.ovf = 1;
+    if (ov) c.over[slot] = 1;
   }
 }
 
@@ -243,13 +271,14 @@ __device__ __forceinline__ void solo_push(const MGraph &G, const SoloMem<TIER> &
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned lt = (1u << lane) - 1u, le = lt | (1u << lane);
   uint8_t *own = c.own[warp];
+  const int slot = ph % 3;
   solo_begin(c, ph);
-  for (int cb = solo_next(c, b, e, ph); cb < e; cb = solo_next(c, b, e, ph)) {
+  for (int cb = b + warp * 32; cb < e; cb = solo_next(c, b + T, e, ph)) {
     const int idx = cb + lane;
     int beg = 0, d = 0;
     uint64_t sv = 0ull;
     if (idx < e) {
-      const int32_t v = S.queue[idx];
+      const int32_t v = solo_entry<TIER>(S, level - 1, b, idx);
       beg = G.rp[v];
       d = G.rp[v + 1] - beg;
       if constexpr (COUNT) sv = S.get(v);
@@ -270,6 +299,7 @@ __device__ __forceinline__ void solo_push(const MGraph &G, const SoloMem<TIER> &
     int before = -1;  // index of the last row that starts before the window
     for (int i0 = 0; i0 < E; i0 += 32 * U) {
       int32_t w[U];
+      int o[U];
       uint64_t svu[U];
       unsigned bal[U];
 #pragma unroll
@@ -277,13 +307,16 @@ __device__ __forceinline__ void solo_push(const MGraph &G, const SoloMem<TIER> &
         const int s = start - (i0 + 32 * u);
         const unsigned f = __reduce_or_sync(FULL, (ds > 0 && (unsigned)s < 32u) ? 1u << s : 0u);
         const int i = i0 + 32 * u + lane;
-        const int o = i < E ? (int)own[before + __popc(f & le)] : 0;
+        o[u] = i < E ? (int)own[before + __popc(f & le)] : 0;
         before += __popc(f);
-        const int j = i + __shfl_sync(FULL, first, o);
-        if constexpr (COUNT) svu[u] = __shfl_sync(FULL, sv, o);
+        const int j = i + __shfl_sync(FULL, first, o[u]);
         w[u] = i < E ? G.col[j] : -1;
       }
-      solo_visit<TIER, U, COUNT>(S, c, level, w, svu, bal, G.rp);
+      if constexpr (COUNT) {  // (the counts may still be on their way when the columns are asked for)
+#pragma unroll
+        for (int u = 0; u < U; ++u) svu[u] = __shfl_sync(FULL, sv, o[u]);
+      }
+      solo_visit<TIER, U, COUNT>(S, c, level, e, slot, w, svu, bal, G.rp);
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const int s = start - (i0 + 32 * u);
@@ -297,12 +330,12 @@ __device__ __forceinline__ void solo_push(const MGraph &G, const SoloMem<TIER> &
       const int k = __ffs(bm) - 1;
       const int hb = __shfl_sync(FULL, beg, k), he = hb + __shfl_sync(FULL, d, k);
       if (he - hb > SOLO_HUGE_DEG) {
-        int slot = 0;
+        int at = 0;
         if (lane == 0) {
-          slot = atomicAdd(&c.nhuge[ph % 3], 1);
-          if (slot < SOLO_HUGE) c.huge[slot] = cb + k;
+          at = atomicAdd(&c.nhuge[slot], 1);
+          if (at < SOLO_HUGE) c.huge[at] = cb + k;
         }
-        if (__shfl_sync(FULL, slot, 0) < SOLO_HUGE) continue;
+        if (__shfl_sync(FULL, at, 0) < SOLO_HUGE) continue;
       }
       uint32_t *words = S.lmask + (hb >> 4);
       uint64_t svu[U];
@@ -317,7 +350,7 @@ __device__ __forceinline__ void solo_push(const MGraph &G, const SoloMem<TIER> &
           const int j = j0 + 32 * u + lane;
           w[u] = j < he ? G.col[j] : -1;
         }
-        solo_visit<TIER, U, COUNT>(S, c, level, w, svu, bal, G.rp);
+        solo_visit<TIER, U, COUNT>(S, c, level, e, slot, w, svu, bal, G.rp);
         if (lane == 0) {
 #pragma unroll
           for (int u = 0; u < U; ++u)
@@ -327,7 +360,7 @@ __device__ __forceinline__ void solo_push(const MGraph &G, const SoloMem<TIER> &
     }
   }
   __syncthreads();
-  const int nh = min(c.nhuge[ph % 3], SOLO_HUGE);
+  const int nh = min(c.nhuge[slot], SOLO_HUGE);
   ++ph;
   if (nh) {
     for (int k = 0; k < nh; ++k) {
@@ -339,7 +372,7 @@ __device__ __forceinline__ void solo_push(const MGraph &G, const SoloMem<TIER> &
         int32_t w[1];
         unsigned bal[1];
         w[0] = j0 + lane < he ? G.col[j0 + lane] : -1;
-        solo_visit<TIER, 1, COUNT>(S, c, level, w, svu, bal, G.rp);
+        solo_visit<TIER, 1, COUNT>(S, c, level, e, slot, w, svu, bal, G.rp);
         if (lane == 0) S.lmask[(hb >> 4) + ((j0 - hb) >> 5)] = bal[0];
       }
     }
@@ -425,24 +458,61 @@ __device__ __forceinline__ void solo_finish(const SoloMem<TIER> &S, int32_t v, c
   deliver(v, delta);
 }
 
-template <int TIER, int T, bool NARROW, class F>
-__device__ __forceinline__ void solo_back(const MGraph &G, const SoloMem<TIER> &S, SoloCtl &c, int b, int e, int unit,
-                                          int &ph, unsigned &err, F &deliver) {
+// A thread's entry in the first run of a level of the backward pass: its loads
+// are issued a level ahead (they depend on nothing that the level between
+// changes), so a narrow level's chain is the successors' coefficients and the
+// arithmetic alone.
+struct SoloAhead {
+  int32_t v = -1;
+  uint32_t mask = 0u;
+  int beg = 0, d = 0;
+};
+template <int TIER> __device__ __forceinline__ SoloAhead solo_ahead(const SoloMem<TIER> &S, int b, int e) {
+  SoloAhead p;
+  const int idx = b + (int)threadIdx.x;
+  if (idx < e) {
+    p.v = S.queue[idx];
+    p.mask = S.qmask[idx];
+  }
+  return p;
+}
+template <class H>
+__device__ __forceinline__ void solo_ahead_row(const MGraph &G, SoloAhead &p, bool narrow_level, H &hint) {
+  if (p.v < 0) return;
+  p.beg = G.rp[p.v];
+  p.d = G.rp[p.v + 1] - p.beg;
+  if (!narrow_level) return;  // (a wide level has other runs to hide the loads behind)
+  if (p.mask) asm volatile("prefetch.global.L1 [%0];" ::"l"(G.col + p.beg));
+  hint(p.v);
+}
+
+// (p: this level's first run; [nb, b): the next level to come, loaded into p)
+template <int TIER, int T, bool NARROW, class F, class H>
+__device__ __forceinline__ void solo_back(const MGraph &G, const SoloMem<TIER> &S, SoloCtl &c, int nb, int b, int e,
+                                          int unit, int &ph, unsigned &err, F &deliver, H &hint, SoloAhead &p) {
   using A = SoloAcc<NARROW>;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int bias = 1075 - unit;
   solo_begin(c, ph);
-  for (int cb = solo_next(c, b, e, ph); cb < e; cb = solo_next(c, b, e, ph)) {
-    const int idx = cb + lane;
-    int32_t v = -1;
-    int beg = 0, d = 0;
-    uint32_t mask = 0u;
-    if (idx < e) {
-      v = S.queue[idx];
-      mask = S.qmask[idx];
-      beg = G.rp[v];
-      d = G.rp[v + 1] - beg;
+  int32_t v = p.v;
+  int beg = p.beg, d = p.d;
+  uint32_t mask = p.mask;
+  p = solo_ahead<TIER>(S, nb, b);
+  bool first = true;
+  for (int cb = b + warp * 32; cb < e; cb = solo_next(c, b + T, e, ph)) {
+    if (!first) {
+      const int idx = cb + lane;
+      v = -1;
+      beg = d = 0;
+      mask = 0u;
+      if (idx < e) {
+        v = S.queue[idx];
+        mask = S.qmask[idx];
+        beg = G.rp[v];
+        d = G.rp[v + 1] - beg;
+      }
     }
+    first = false;
     typename A::A a = A::zero();
     while (mask) {  // up to four successors in flight per thread
       int32_t w[4];
@@ -481,6 +551,7 @@ __device__ __forceinline__ void solo_back(const MGraph &G, const SoloMem<TIER> &
     if (v >= 0) solo_finish<TIER, NARROW>(S, v, a, unit, deliver);
     __syncwarp();
   }
+  solo_ahead_row(G, p, b - nb <= T, hint);
   __syncthreads();
   const int nh = min(c.nhuge[ph % 3], SOLO_HUGE);
   ++ph;
@@ -570,20 +641,96 @@ __device__ __forceinline__ void solo_xf_level(const MGraph &G, const SoloMem<TIE
   }
 }
 
-// Theorem 1 for one level in the extended form (successors in CSR order).
-template <int TIER, int T, class F>
-__device__ __forceinline__ void solo_xf_back(const MGraph &G, const SoloMem<TIER> &S, int b, int e, F &deliver) {
+// The same pull fused with the push from the same vertices (an undirected
+// graph's rows are both): counts of level l = level - 1 from the neighbours a
+// level below, the next level from those not reached yet, one pass and one
+// barrier a level. Rows up to 32 entries by a thread in CSR order, four at a
+// time; longer ones by the warp.
+template <int TIER, int T>
+__device__ __forceinline__ void solo_xf_push(const MGraph &G, const SoloMem<TIER> &S, SoloCtl &c, int level, int b,
+                                             int e, int &ph) {
+  const typename SoloMem<TIER>::D prev = solo_code<TIER>(level - 2 + (level < 2));
+  const bool pull = level >= 2;  // the source's count stands
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int slot = ph % 3;
+  const uint64_t none[4] = {0ull, 0ull, 0ull, 0ull};
+  solo_begin(c, ph);
   for (int cb = b + warp * 32; cb < e; cb += T) {
     const int idx = cb + lane;
     int32_t v = -1;
     int beg = 0, d = 0;
-    uint32_t mask = 0u;
     if (idx < e) {
-      v = S.queue[idx];
-      mask = S.qmask[idx];
+      v = solo_entry<TIER>(S, level - 1, b, idx);
       beg = G.rp[v];
       d = G.rp[v + 1] - beg;
+    }
+    Xf acc{0.0, 0};
+    uint32_t mask = 0u;
+    const int ds = d <= 32 ? d : 0, most = __reduce_max_sync(FULL, ds);
+    for (int j = 0; j < most; j += 4) {
+      int32_t w[4];
+      Xf x[4];
+      unsigned bal[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) w[u] = j + u < ds ? G.col[beg + j + u] : -1;
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        x[u] = (pull && w[u] >= 0 && S.dist[w[u]] == prev) ? solo_xf<TIER>(S, w[u]) : Xf{0.0, 0};
+      solo_visit<TIER, 4, false>(S, c, level, e, slot, w, none, bal, G.rp);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) mask |= ((bal[u] >> lane) & 1u) << ((j + u) & 31);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc = xf_add(acc, x[q]);
+    }
+    __syncwarp();
+    for (unsigned bm = __ballot_sync(FULL, d > 32); bm; bm &= bm - 1u) {
+      const int k = __ffs(bm) - 1;
+      const int hb = __shfl_sync(FULL, beg, k), he = hb + __shfl_sync(FULL, d, k);
+      uint32_t *words = S.lmask + (hb >> 4);
+      Xf tot{0.0, 0};
+      for (int j0 = hb; j0 < he; j0 += 32) {
+        int32_t w[1];
+        const uint64_t zero[1] = {0ull};
+        unsigned bal[1];
+        w[0] = j0 + lane < he ? G.col[j0 + lane] : -1;
+        const bool ok = pull && w[0] >= 0 && S.dist[w[0]] == prev;
+        const Xf x = ok ? solo_xf<TIER>(S, w[0]) : Xf{0.0, 0};
+        solo_visit<TIER, 1, false>(S, c, level, e, slot, w, zero, bal, G.rp);
+        if (lane == 0) words[(j0 - hb) >> 5] = bal[0];
+        solo_xf_warp(tot, ok, x);
+      }
+      if (lane == k) acc = tot;
+    }
+    if (v >= 0) {
+      if (pull) solo_xf_set<TIER>(S, v, acc);
+      S.qmask[idx] = mask;
+    }
+  }
+  __syncthreads();
+  ++ph;
+}
+
+// Theorem 1 for one level in the extended form (successors in CSR order).
+template <int TIER, int T, class F, class H>
+__device__ __forceinline__ void solo_xf_back(const MGraph &G, const SoloMem<TIER> &S, int nb, int b, int e, F &deliver,
+                                             H &hint, SoloAhead &p) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int32_t v = p.v;
+  int beg = p.beg, d = p.d;
+  uint32_t mask = p.mask;
+  p = solo_ahead<TIER>(S, nb, b);
+  for (int cb = b + warp * 32; cb < e; cb += T) {
+    if (cb >= b + T) {
+      const int idx = cb + lane;
+      v = -1;
+      beg = d = 0;
+      mask = 0u;
+      if (idx < e) {
+        v = S.queue[idx];
+        mask = S.qmask[idx];
+        beg = G.rp[v];
+        d = G.rp[v + 1] - beg;
+      }
     }
     Xf acc{0.0, 0};
     while (mask) {
@@ -617,6 +764,7 @@ __device__ __forceinline__ void solo_xf_back(const MGraph &G, const SoloMem<TIER
       deliver(v, delta);
     }
   }
+  solo_ahead_row(G, p, b - nb <= T, hint);
 }
 
 // Forward pass of source s: distance codes, counts, level offsets and edge
@@ -649,19 +797,22 @@ __device__ int solo_forward(const MGraph &G, int32_t s, int32_t dest, const Solo
     S.dist[s] = 0;
     S.set(s, 1ull);
     S.queue[0] = (typename SoloMem<TIER>::Q)s;
-    c.tail = 1;
+    if constexpr (TIER != 0) S.ring[0] = s;
     c.near[0] = 0;
     c.near[1] = 1;
-    c.ovf = 0;
     c.l53 = 0x7FFFFFFF;
     c.maxc = 1ull;
   }
   __syncthreads();
   int L = 0, b = 0, e = 1;
   bool xf = false;
+  const bool fused = G.rp_in == G.rp;  // (extended form) level L's counts come with the push from it
   uint64_t mymax = 1ull;
   for (;;) {
-    if (xf) {
+    const int slot = ph % 3;
+    if (xf && fused) {
+      solo_xf_push<TIER, T>(G, S, c, L + 1, b, e, ph);
+    } else if (xf) {
       uint64_t none = 0ull;
       solo_push<TIER, T, false>(G, S, c, L + 1, b, e, ph, none);
     } else {
@@ -670,19 +821,23 @@ __device__ int solo_forward(const MGraph &G, int32_t s, int32_t dest, const Solo
       if (lmax >= (1ull << 53)) atomicMin(&c.l53, L);
       mymax = lmax > mymax ? lmax : mymax;
     }
-    const int nt = c.tail;
+    // (a pass's counters stand until the pass after the next one begins)
+    const int nt = e + c.found[slot];
     if (nt == e) break;  // no vertex at distance L + 1
-    if (xf) solo_xf_level<TIER, T>(G, S, L + 1, e, nt);
+    if (xf && !fused) {
+      solo_xf_level<TIER, T>(G, S, L + 1, e, nt);
+      __syncthreads();
+    }
     if (tid == 0) {
       if (L + 2 < SOLO_NEAR) c.near[L + 2] = nt;
       else S.far[L + 2] = nt;
     }
-    __syncthreads();
     ++L;
     b = e;
     e = nt;
-    if (!xf && c.ovf) {
+    if (!xf && c.over[slot]) {
       // to the extended form: convert the exact levels, pull the rest
+      __syncthreads();
       const int l53 = min(c.l53, L);
       const int conv = solo_lo<TIER>(S, c, l53);
       for (int i = tid; i < conv; i += T) {
@@ -696,7 +851,10 @@ __device__ int solo_forward(const MGraph &G, int32_t s, int32_t dest, const Solo
       }
       xf = true;
     }
-    if (dest >= 0 && S.dist[dest] != solo_unset<TIER>()) break;  // dest settled at level L
+    if (dest >= 0 && __syncthreads_or(S.dist[dest] != solo_unset<TIER>())) {  // dest settled at level L
+      if (xf && fused) solo_xf_level<TIER, T>(G, S, L, b, e);
+      break;
+    }
   }
   if (!xf) {
     for (int off = 16; off > 0; off >>= 1) {
@@ -711,27 +869,36 @@ __device__ int solo_forward(const MGraph &G, int32_t s, int32_t dest, const Solo
   return L;
 }
 
+struct SoloNoHint {
+  __device__ void operator()(int32_t) const {}
+};
+
 // Theorem 1 for levels L..1 after solo_forward; deliver(v, delta) is called by
-// one thread for every vertex at distance >= 1.
-template <int TIER, int T, class F>
+// one thread for every vertex at distance >= 1, hint(v) at least a level's
+// barrier earlier for some of them (to prefetch what deliver reads).
+template <int TIER, int T, class F, class H = SoloNoHint>
 __device__ __forceinline__ void solo_backward(const MGraph &G, int L, bool ext, uint64_t maxc, const SoloMem<TIER> &S,
-                                              SoloCtl &c, int &ph, unsigned &err, F deliver) {
-  if (ext) {
-    for (int l = L; l >= 1; --l) {
-      solo_xf_back<TIER, T>(G, S, solo_lo<TIER>(S, c, l), solo_lo<TIER>(S, c, l + 1), deliver);
-      __syncthreads();
-    }
-    return;
-  }
+                                              SoloCtl &c, int &ph, unsigned &err, F deliver, H hint = H{}) {
+  if (L < 1) return;
+  int b = solo_lo<TIER>(S, c, L), e = solo_lo<TIER>(S, c, L + 1);
+  SoloAhead p = solo_ahead<TIER>(S, b, e);
+  solo_ahead_row(G, p, e - b <= T, hint);
   // ceil(log2) of the largest count and of n
   const int unit = 52 + (maxc <= 1ull ? 0 : 64 - __clzll((long long)(maxc - 1ull)));
   const int nlog = G.n <= 1 ? 0 : 32 - __clz(G.n - 1);
-  if (unit + nlog + 1 <= 96) {
-    for (int l = L; l >= 1; --l)
-      solo_back<TIER, T, true>(G, S, c, solo_lo<TIER>(S, c, l), solo_lo<TIER>(S, c, l + 1), unit, ph, err, deliver);
-  } else {
-    for (int l = L; l >= 1; --l)
-      solo_back<TIER, T, false>(G, S, c, solo_lo<TIER>(S, c, l), solo_lo<TIER>(S, c, l + 1), unit, ph, err, deliver);
+  const bool narrow = unit + nlog + 1 <= 96;
+  for (int l = L; l >= 1; --l) {
+    const int nb = l > 1 ? solo_lo<TIER>(S, c, l - 1) : b;  // (level 0, the source, has no part in it)
+    if (ext) {
+      solo_xf_back<TIER, T>(G, S, nb, b, e, deliver, hint, p);
+      __syncthreads();
+    } else if (narrow) {
+      solo_back<TIER, T, true>(G, S, c, nb, b, e, unit, ph, err, deliver, hint, p);
+    } else {
+      solo_back<TIER, T, false>(G, S, c, nb, b, e, unit, ph, err, deliver, hint, p);
+    }
+    e = b;
+    b = nb;
   }
 }
 

@@ -538,7 +538,7 @@ extern __shared__ uint4 w_shared[];
 
 template <int TIER>
 __device__ __forceinline__ WMem<TIER> w_begin(const WGraph &W, unsigned char *scratch, size_t stride, WCtl &sh) {
-  if (threadIdx.x == 0) sh.c.nhuge[0] = sh.c.nhuge[1] = sh.c.nhuge[2] = sh.c.grab[0] = sh.c.grab[1] = 0;
+  solo_init(sh.c);
   return w_mem<TIER>(reinterpret_cast<unsigned char *>(w_shared), scratch + (size_t)blockIdx.x * stride, W.g.n,
                      W.g.nnz);
 }
@@ -675,6 +675,8 @@ static WGraph w_graph(const Graph &g) {
   return G;
 }
 
+constexpr size_t W_SMEM_MAX = (size_t)226 * 1024;  // state, control words and a margin
+
 struct WCfg {
   int tier, threads, ncta;
   size_t smem, stride;
@@ -694,7 +696,7 @@ static WCfg w_cfg(const Graph &g) {
   WCfg c{};
   const uint64_t longest = g.w ? g.w_max : 1ull;
   const bool narrow = longest * (uint64_t)std::max(1, g.n - 1) < 0xFFFFFFFFull;
-  c.tier = narrow && w_smem(0, g.n) + sizeof(WCtl) + 1024 <= (size_t)226 * 1024 ? 0 : 1;
+  c.tier = narrow && w_smem(0, g.n) + sizeof(WCtl) + 1024 <= W_SMEM_MAX ? 0 : 1;
   c.smem = w_smem(c.tier, g.n);
   c.stride = w_stride(c.tier, g.n, g.nnz);
   c.threads = (g.n < 4096 || g.nnz < 5 * (int64_t)g.n) ? 256 : 1024;
@@ -705,7 +707,10 @@ template <class K> static void w_ctas(WCfg &c, K kern, int count, size_t per) {
   int dev = 0, sms = 0, occ = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (c.smem) BCG_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c.smem));
+  // (the most any graph asks for: another thread's graph does not lower it)
+  if (c.smem)
+    BCG_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)(W_SMEM_MAX - sizeof(WCtl) - 1024)));
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, c.threads, c.smem) != cudaSuccess || occ < 1) {
     cudaGetLastError();
     occ = 1;

@@ -16,6 +16,12 @@ struct Xf {
 // 2^k as a double, k in [-1022, 1023]
 __device__ __forceinline__ double pow2(int k) { return __longlong_as_double((long long)(k + 1023) << 52); }
 
+// x * 2^k, x and the product normal: exact, and an integer addition where an
+// FP64 multiplication would wait for its slow pipe
+__device__ __forceinline__ double scale2(double x, int k) {
+  return __longlong_as_double(__double_as_longlong(x) + ((long long)k << 52));
+}
+
 // x * 2^e normalised; x a positive normal double, or 0
 __device__ __forceinline__ Xf xf_make(double x, int e) {
   if (x == 0.0) return Xf{0.0, 0};
@@ -37,7 +43,7 @@ __device__ __forceinline__ Xf xf_add(Xf a, Xf b) {
   }
   const long long d = (long long)a.e - (long long)b.e;
   if (d > 60) return a;
-  return xf_make(__dadd_rn(a.m, __dmul_rn(b.m, pow2(-(int)d))), a.e);
+  return xf_make(__dadd_rn(a.m, scale2(b.m, -(int)d)), a.e);
 }
 
 // RN(a * b) as a double: the mantissa product rounds once; steps of 2^1000 are
@@ -46,6 +52,7 @@ __device__ __forceinline__ double xf_mul_to_double(Xf a, Xf b) {
   if (a.m == 0.0 || b.m == 0.0) return 0.0;
   double p = __dmul_rn(a.m, b.m);
   long long k = (long long)a.e + (long long)b.e;
+  if (k >= -1000 && k <= 1000) return scale2(p, (int)k);  // p in [1, 4)
   while (k > 1000) {
     p = __dmul_rn(p, pow2(1000));
     k -= 1000;

@@ -99,3 +99,37 @@ def test_more_levels_than_the_16_bit_codes():
     for i, s in enumerate(src.tolist()):
         want = [0.0 if v == s else float(n - 1 - v if v > s else v) for v in targets.tolist()]
         assert got[:, i].tolist() == want
+
+
+def _layers(w, layers):
+    i, j = np.divmod(np.arange(w * w), w)
+    k = w * np.arange(layers - 1)[:, None]
+    return gg.from_edges(w * layers, (i + k).ravel(), (j + w + k).ravel())
+
+
+@pytest.mark.parametrize("name,make", [("counts in L2 above one source per SM", lambda: gg.grid(80)),
+                                       ("long rows beyond 2^64", lambda: _layers(40, 36))])
+@pytest.mark.parametrize("k", [100, 200])
+def test_deep_graphs_equal_the_oracle(name, make, k):
+    """Narrow levels, in tier 0 or 1 by the number of sources; in the extended form
+    a level's counts are pulled by the pass that pushes from it."""
+    g = make()
+    with _ctx() as ctx:
+        h = ctx.load_graph(g.row_ptr, g.col)
+        got = ctx.uniform_sources(h, k, 3, 9)
+        pairs = ctx.adaptive_pairs(h, [5, g.n // 2, g.n - 7], 1.0, 64, 2, 3)  # searches that stop at a level
+    assert np.array_equal(got, oracle.uniform_sources(g, k, 3, 9))
+    ref = oracle.adaptive_pairs(g, [5, g.n // 2, g.n - 7], 1.0, 64, 2, 3)
+    assert np.array_equal(pairs["S"], ref["S"]) and np.array_equal(pairs["k"], ref["k"])
+
+
+def test_many_deep_graphs_of_every_residency():
+    """Square grids that fit an SM four times to once, in one call."""
+    gs = [gg.grid(s) for s in (40, 75, 150, 180, 210, 245)]
+    with _ctx() as ctx:
+        hs = [ctx.load_graph(g.row_ptr, g.col) for g in gs]
+        got = ctx.uniform_sources_multi(hs, [3] * 6, [7] * 6, list(range(6)))
+        for q, (g, h, e) in enumerate(zip(gs, hs, got)):
+            assert np.array_equal(e, ctx.uniform_sources(h, 3, 7, q))
+            if g.n < 6000:
+                assert np.array_equal(e, oracle.uniform_sources(g, 3, 7, q))
