@@ -375,7 +375,7 @@ __global__ void k_validate(int32_t n, const int32_t *__restrict__ rp, const int3
 // vertex to K landmarks, projected on their first principal component and
 // quantised to 8 bits (255: not reached from the hub), so that sources with
 // similar BFS level structure sort next to each other. Landmark 0 is the hub,
-// the others are vertices drawn at random from those with edges that reach it,
+// the others are vertices drawn at random from those it reaches and that reach it,
 // so that one 64-lane forward pass gives all their distances. (Before, one
 // plain search per landmark, each the farthest from those before: first call /
 // later calls in ms on R-MAT s20 k = 1024 112 / 35.8 -> 49 / 34.6, s16 Bader 1500
@@ -396,12 +396,19 @@ __global__ void k_land_hub(int32_t n, const int32_t *__restrict__ dist, uint8_t 
   if ((threadIdx.x & 31) == 0 && d > 0) atomicMax(maxd, d);
 }
 
-// Candidate landmarks: vertices with edges, by the draws of a fixed stream (a
-// vertex without edges gives way to the next one with some, in id order).
-__global__ void k_land_draw(int32_t n, const int32_t *__restrict__ rp, int32_t *__restrict__ out) {
+// Candidate landmarks: vertices with edges that the hub reaches, by the draws of
+// a fixed stream (another vertex gives way to the next such one in id order, or
+// to the hub). In the hub's component a landmark's distances are at most twice
+// the hub's; a long path elsewhere would take a level mask per level.
+__global__ void k_land_draw(int32_t n, const int32_t *__restrict__ rp, const uint8_t *__restrict__ hub_row,
+                            int32_t hub, int32_t *__restrict__ out) {
   int32_t v = draw_source(0x6C616E646D61726Bull, 0ull, (uint64_t)threadIdx.x, n);
-  for (int i = 0; i < 4096 && rp[v + 1] == rp[v]; ++i) v = v + 1 < n ? v + 1 : 0;
-  out[threadIdx.x] = v;
+  bool ok = false;
+  for (int i = 0; i < 4096 && !ok; ++i) {
+    ok = hub_row[v] != 255 && rp[v + 1] != rp[v];
+    if (!ok) v = v + 1 < n ? v + 1 : 0;
+  }
+  out[threadIdx.x] = ok ? v : hub;
 }
 
 // Rows 1..K-1 from the level masks of a forward pass: row r has the distances
@@ -730,19 +737,19 @@ static void build_key(bc_ctx *ctx, const Graph &g, KeyMeta &km) {
     int Kused = 1;
     // deep graphs run one source per persistent CTA, where batches do not
     // share traversals: the hub distance alone (also where a forward pass's
-    // state, about 700 B per vertex, would not leave room)
+    // state, about 700 B per vertex and 8 B per level, would not leave room)
     bool more = K > 1 && km.ecc > 0 && km.ecc <= 64;
     if (more) {
       size_t fr = 0, tot = 0;
       if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) cudaGetLastError();
-      more = n * (size_t)(K + (ws.sigma.bytes < n * 512 ? 700 : 0)) < fr / 2;
+      more = n * (size_t)(K + 16 * km.ecc + (ws.sigma.bytes < n * 512 ? 700 : 0)) < fr / 2;
     }
     if (more) {
       // (the caller may have its batch's sources in place already)
       BCG_CUDA(cudaMemcpyAsync(sm + 384, ws.sources.p, 64 * 4, cudaMemcpyDeviceToDevice, st));
       {
         LaunchScope ls(ctx, F_MISC);
-        k_land_draw<<<1, 64, 0, st>>>(g.n, g.rp, ws.sources.as<int32_t>());
+        k_land_draw<<<1, 64, 0, st>>>(g.n, g.rp, rows.as<uint8_t>(), g.hub, ws.sources.as<int32_t>());
       }
       const int maxl = batch_forward(ctx, g, 64, false, OVF_IGNORE);
       {

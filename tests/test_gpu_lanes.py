@@ -124,3 +124,22 @@ def test_source_key_where_landmarks_run_out(ctx, shape):
     ctx.free_graph(h)
     assert np.array_equal(got, oracle.uniform_sources(g, 300, 4, 6))
     assert np.array_equal(exact, oracle.exact_bc(g))
+
+
+def test_source_key_beside_a_long_path(ctx):
+    """A star and, in another component, a path of 30,000 levels: the landmarks'
+    pass stays in the hub's component (64 level masks per level of the path would
+    take 24 GB)."""
+    import torch
+    star, path = 70000, 30000
+    i = np.arange(1, star)
+    p = np.arange(star, star + path - 1)
+    g = gg.from_edges(star + path, np.r_[0 * i, p], np.r_[i, p + 1])
+    h = ctx.load_graph(g.row_ptr, g.col)
+    free = torch.cuda.mem_get_info()[0]
+    res = ctx.adaptive_pairs(h, [0, 5], 1.0, 6, 3, 1)
+    used = free - torch.cuda.mem_get_info()[0]
+    ctx.free_graph(h)
+    ref = oracle.adaptive_pairs(g, [0, 5], 1.0, 6, 3, 1)
+    assert np.array_equal(res["S"], ref["S"]) and np.array_equal(res["k"], ref["k"])
+    assert used < 12 << 30  # the pair search's own arrays: 34 B a vertex and resident CTA
