@@ -749,6 +749,7 @@ void do_uniform_multi(bc_ctx *ctx, const std::vector<bc_graph> &handles, const s
         build_plan(ctx, P, dg);
       } catch (...) {
         ctx->stream = main;
+        P.release();  // (a plan cut short, e.g. out of memory, must not pass for the same one next time)
         throw;
       }
       ctx->stream = main;
