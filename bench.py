@@ -675,7 +675,8 @@ def main():
     alg_bytes = bytes_bwd if dom == "bwd" else bytes_fwd
     dom_ms = kern[dom]["ms"]
     achieved = alg_bytes / (dom_ms / 1e3) / 1e9 if dom_ms > 0 else 0.0
-    kern_names = {"bwd": "backward pass: k_bwd_light_fx + k_bwd_heavy_seg_fx + k_bwd_heavy_fin_fx per level",
+    kern_names = {"bwd": "backward pass: k_bwd_heavy_list + k_bwd_heavy_seg + k_bwd_light + k_bwd_heavy_fin per level, "
+                         "timed beside the other batch in flight",
                   "fwd": "forward pass: k_fwd_light + the heavy-vertex kernels + k_fwd_heavy_fin per level"}
     ratio = recorded_traffic() if dom == "bwd" else None
     alg_per_launch = alg_bytes / max(kern[dom]["launches"], 1)
