@@ -128,7 +128,7 @@ def test_source_key_where_landmarks_run_out(ctx, shape):
 
 def test_source_key_beside_a_long_path(ctx):
     """A star and, in another component, a path of 30,000 levels: the landmarks'
-    pass stays in the hub's component (64 level masks per level of the path would
+    pass stays in the hub's component (a level mask for each level of the path would
     take 24 GB)."""
     import torch
     star, path = 70000, 30000
