@@ -350,6 +350,9 @@ __device__ __forceinline__ void w_source(const WGraph &W, int32_t s, const WMem<
               better[u] = better[u] && nd[u] < (unsigned long long)old;
               fresh[u] = better[u] && old == INF;
             }
+            // the improved distances come before the list bits: whoever clears a
+            // near bit after it was seen set here (load, above) reads them
+            __threadfence_block();
 #pragma unroll
             for (int u = 0; u < U; ++u) {
               const bool near = better[u] && nd[u] < Tn;
