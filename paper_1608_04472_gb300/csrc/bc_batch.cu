@@ -1667,8 +1667,8 @@ struct Forward {
 int batch_forward(bc_ctx *ctx, const Graph &g, int count, bool pairs, OvfMode mode) {
   batch_ensure(ctx, g);
   Forward f(ctx, g, count, pairs, mode);
-  if (pairs) return f.all();
-  if (f.hm.depth < 1) return f.all();
+  // (the direction switch needs level 1's degree sum before the first level)
+  if (pairs || f.hm.depth < 1 || ctx->push_div > 0) return f.all();
   f.init();
   return f.blind() ? f.end_blind() : f.run();
 }

@@ -143,3 +143,24 @@ def test_source_key_beside_a_long_path(ctx):
     ref = oracle.adaptive_pairs(g, [0, 5], 1.0, 6, 3, 1)
     assert np.array_equal(res["S"], ref["S"]) and np.array_equal(res["k"], ref["k"])
     assert used < 12 << 30  # the pair search's own arrays: 34 B a vertex and resident CTA
+
+
+def test_direction_switch_tests_the_first_level_in_every_batch(monkeypatch):
+    """A top-down level is two launches, a bottom-up one a single launch. With push_div
+    = 20 the level after the sources' neighbours (64 rows of about 9 entries are
+    more than 16,000 / 20) runs bottom-up, the last ones top-down; the same batch
+    takes the same levels whether or not the graph's depth is known."""
+    import paper_1608_04472_gb300 as pkg
+    monkeypatch.setenv("BCG_SOLO_N", "0")
+    g = gg.erdos_renyi(2000, 8, 3)
+    src = np.arange(0, 1920, 30, dtype=np.int32)
+    launches = []
+    with pkg.Context(0, batch_width=64) as c:
+        h = c.load_graph(g.row_ptr, g.col)
+        c.set_tuning(h, dict(c.get_tuning(h), push_div=20))
+        for _ in range(2):
+            c.reset_stats()
+            delta = c.source_dependencies(h, src)[0]
+            launches.append(c.stats()["kernels"]["fwd"]["launches"])
+            assert np.array_equal(delta[7], oracle.dependencies(g, int(src[7]))[0])
+    assert launches[0] == launches[1]
