@@ -1283,6 +1283,9 @@ struct LevelCtl {
   unsigned pad[15];
 };
 static_assert(sizeof(LevelCtl) == 128, "one line per level");
+// Levels launched without asking the device: as many as the pinned staging
+// holds control words of (two levels more than the depth, and 16 bytes before).
+constexpr int BLIND_DEPTH = (int)((4096 - 16) / sizeof(LevelCtl)) - 2;
 
 struct HeavyMeta {
   int nh = 0, nseg = 0, heavy_deg = 0, seg = 0;
@@ -1406,10 +1409,10 @@ static void side_stream(bc_ctx *ctx) {
 void batch_ensure(bc_ctx *ctx, const Graph &g) {
   Workspace &ws = ctx->ws;
   const size_t n = (size_t)g.n;
-  if (ws.lcap < 16 || ws.lm.bytes < (size_t)ws.lcap * n * 8) {
-    ws.lcap = std::max(ws.lcap, 16);
-    ws.lm.ensure((size_t)ws.lcap * n * 8);
-  }
+  // as many levels as this graph's batches have had (and 16 for the first),
+  // whatever graphs the buffers served before
+  ws.lcap = std::max(16, heavy_meta(ctx, g, true).depth + 3);
+  ws.lm.ensure((size_t)ws.lcap * n * 8);
   ws.visited.ensure(n * 8);
   ws.sigma.ensure(n * 64 * 8);
   ws.ctl.ensure((size_t)(ws.lcap + 2) * sizeof(LevelCtl));
@@ -1576,7 +1579,7 @@ struct Forward {
   // the batch's words (largest count, overflowed lanes) on their way to the
   // host. False when the levels have to be asked for one at a time.
   bool blind() {
-    if (pairs || ctx->push_div > 0 || hm.depth < 1 || hm.depth + 3 > ws.lcap || ws.lcap > 24) return false;
+    if (pairs || ctx->push_div > 0 || hm.depth < 1 || hm.depth > BLIND_DEPTH || hm.depth + 3 > ws.lcap) return false;
     for (; l <= hm.depth; ++l) level();
     uint64_t *h = pinned();
     BCG_CUDA(cudaMemcpyAsync(h, ws.enable.as<uint64_t>() + 2, 16, cudaMemcpyDeviceToHost, st));
@@ -1856,22 +1859,27 @@ void run_lane_batches(bc_ctx *ctx, const Graph &g, const int32_t *src, const int
     batch_ensure(ctx, g);
     BCG_CUDA(cudaMemcpyAsync(ctx->ws.sources.p, src + b, (size_t)cnt * 4, cudaMemcpyDeviceToDevice, ctx->stream));
   };
-  int b0 = 0;
-  // level by level while the graph's depth is not known, or where a second
-  // batch has no room
+  // one batch at a time while the graph's depth is not known, where levels are
+  // asked for one by one (a second batch would have nothing to run beside), or
+  // where a second batch has no room
   batch_ensure(ctx, g);
-  const int one = std::min(64, count);
-  const bool known = heavy_meta(ctx, g, true).depth >= 1 && ctx->push_div == 0;
-  const bool two = count > 64 && ctx->push_div == 0 && second_slot(ctx, g, sink.acc != nullptr);
-  if (!known || !two) {
-    const int upto = two ? one : count;
-    for (; b0 < upto; b0 += 64) {
-      const int cnt = std::min(64, count - b0);
-      load(b0, cnt);
-      const int maxl = batch_forward(ctx, g, cnt, false, OVF_EXTEND);
-      backward(maxl, cnt, batch_sink(b0, false));
-    }
-    if (b0 >= count) return;
+  const HeavyMeta &hm = heavy_meta(ctx, g, true);
+  auto single = [&](int b) {
+    const int cnt = std::min(64, count - b);
+    load(b, cnt);
+    const int maxl = batch_forward(ctx, g, cnt, false, OVF_EXTEND);
+    backward(maxl, cnt, batch_sink(b, false));
+  };
+  int b0 = 0;
+  if (hm.depth < 1) {
+    single(0);
+    b0 = 64;
+  }
+  const bool two = count - b0 > 64 && ctx->push_div == 0 && hm.depth >= 1 && hm.depth <= BLIND_DEPTH &&
+                   second_slot(ctx, g, sink.acc != nullptr);
+  if (!two) {
+    for (; b0 < count; b0 += 64) single(b0);
+    return;
   }
   BatchSlot &s2 = ctx->slot2;
   BCG_CUDA(cudaEventRecord(s2.ev_begin, main));

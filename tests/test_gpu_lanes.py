@@ -164,3 +164,33 @@ def test_direction_switch_tests_the_first_level_in_every_batch(monkeypatch):
             launches.append(c.stats()["kernels"]["fwd"]["launches"])
             assert np.array_equal(delta[7], oracle.dependencies(g, int(src[7]))[0])
     assert launches[0] == launches[1]
+
+
+def _path_and_star(path, leaves=50):
+    """A path 0 - 1 - .. and, in another component, a star around vertex `path`."""
+    p, i = np.arange(path - 1), np.arange(leaves)
+    return gg.from_edges(path + 1 + leaves, np.r_[p, 0 * i + path], np.r_[p + 1, path + 1 + i])
+
+
+@pytest.mark.parametrize("before", [None, 26])
+@pytest.mark.parametrize("path", [12, 21, 30, 33])
+def test_levels_launched_unasked_follow_the_graph_s_own_depth(monkeypatch, before, path):
+    """Once a batch from the path's end has shown the depth, a batch from the star is
+    launched that deep without asking (up to 29 levels), whatever graph the context
+    ran before."""
+    import paper_1608_04472_gb300 as pkg
+    monkeypatch.setenv("BCG_SOLO_N", "0")
+    g = _path_and_star(path)
+    with pkg.Context(0, batch_width=64) as c:
+        if before:
+            d = _path_and_star(before)
+            c.source_dependencies(c.load_graph(d.row_ptr, d.col), [0])
+        h = c.load_graph(g.row_ptr, g.col)
+        far = c.source_dependencies(h, [0])[0]
+        c.reset_stats()
+        near = c.source_dependencies(h, [path])[0]
+        levels = c.stats()["kernels"]["fwd"]["launches"] - 1  # (level 1 is a kernel of its own)
+        est = c.uniform_sources(h, 200, 3, 1)
+    assert np.array_equal(far[0], oracle.dependencies(g, 0)[0]) and np.array_equal(near[0], oracle.dependencies(g, path)[0])
+    assert np.array_equal(est, oracle.uniform_sources(g, 200, 3, 1))
+    assert levels == (path - 1 if path - 1 <= 29 else 1)
