@@ -1444,6 +1444,7 @@ struct Forward {
   const int32_t *todo = nullptr;  // light vertices with lanes still to reach
   int todo_level = -1;            // level whose control word counts them (-1: the graph's own list)
   uint64_t fedges = 0ull;         // degree sum of the vertices at level l (direction test)
+  int limit = 0x7FFFFFFF;         // levels wanted: vertices farther away may stay unreached
 
   Forward(bc_ctx *c, const Graph &gr, int cnt, bool pr, OvfMode m)
       : ctx(c), g(gr), ws(c->ws), hm(heavy_meta(c, gr, true)), n((size_t)gr.n), st(c->stream), count(cnt), pairs(pr),
@@ -1636,7 +1637,7 @@ struct Forward {
       if (heavy_now && (next.hpend & cont) == 0ull) heavy_done = true;
       // stop once every lane still going has overflowed (finished lanes are complete)
       const bool all_ovf = watch && ovf != 0ull && (cont & ~ovf) == 0ull;
-      if (!cont || all_ovf) {
+      if (!cont || all_ovf || l >= limit) {
         const uint64_t sigmax = h[2], ov = h[3];
         std::vector<LevelCtl> lv((size_t)l + 2);
         if (hm.nseg && !g.directed) {
@@ -1667,9 +1668,10 @@ struct Forward {
   }
 };
 
-int batch_forward(bc_ctx *ctx, const Graph &g, int count, bool pairs, OvfMode mode) {
+int batch_forward(bc_ctx *ctx, const Graph &g, int count, bool pairs, OvfMode mode, int limit) {
   batch_ensure(ctx, g);
   Forward f(ctx, g, count, pairs, mode);
+  f.limit = limit;
   // (the direction switch needs level 1's degree sum before the first level)
   if (pairs || f.hm.depth < 1 || ctx->push_div > 0) return f.all();
   f.init();

@@ -398,8 +398,10 @@ __global__ void k_land_hub(int32_t n, const int32_t *__restrict__ dist, uint8_t 
 
 // Candidate landmarks: vertices with edges that the hub reaches, by the draws of
 // a fixed stream (another vertex gives way to the next such one in id order, or
-// to the hub). In the hub's component a landmark's distances are at most twice
-// the hub's; a long path elsewhere would take a level mask per level.
+// to the hub). On an undirected graph a landmark's distances are then at most
+// twice the hub's; a directed one can have a landmark at the end of a long chain,
+// so the pass goes no deeper than that (a level takes 12 B a vertex, and a chain
+// of 10,000 arcs among 200,000 vertices took 24 GB for draws that never met it).
 __global__ void k_land_draw(int32_t n, const int32_t *__restrict__ rp, const uint8_t *__restrict__ hub_row,
                             int32_t hub, int32_t *__restrict__ out) {
   int32_t v = draw_source(0x6C616E646D61726Bull, 0ull, (uint64_t)threadIdx.x, n);
@@ -759,13 +761,16 @@ static void build_key(bc_ctx *ctx, const Graph &g, KeyMeta &km) {
     int Kused = 1;
     // deep graphs run one source per persistent CTA, where batches do not
     // share traversals: the hub distance alone (also where a forward pass's
-    // state, about 700 B per vertex and 8 B per level, would not leave room)
+    // state, about 700 B per vertex and 12 B per level, the levels' arrays
+    // doubled as they grow, would not leave room)
+    const int levels = 2 * km.ecc + 2;
     bool more = K > 1 && km.ecc > 0 && km.ecc <= 64;
     if (more) {
       size_t fr = 0, tot = 0;
       if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) cudaGetLastError();
-      more = n * (size_t)(K + 16 * km.ecc + (ws.sigma.bytes < n * 512 ? 700 : 0)) < fr / 2;
+      more = n * (size_t)(K + 36 * std::max(16, levels + 3) + (ws.sigma.bytes < n * 512 ? 700 : 0)) < fr / 2;
     }
+    int maxl = 0;
     if (more) {
       // (the caller may have its batch's sources in place already)
       BCG_CUDA(cudaMemcpyAsync(sm + 384, ws.sources.p, 64 * 4, cudaMemcpyDeviceToDevice, st));
@@ -773,7 +778,16 @@ static void build_key(bc_ctx *ctx, const Graph &g, KeyMeta &km) {
         LaunchScope ls(ctx, F_MISC);
         k_land_draw<<<1, 64, 0, st>>>(g.n, g.rp, rows.as<uint8_t>(), g.hub, ws.sources.as<int32_t>());
       }
-      const int maxl = batch_forward(ctx, g, 64, false, OVF_IGNORE);
+      try {
+        maxl = batch_forward(ctx, g, 64, false, OVF_IGNORE, levels);
+      } catch (const Error &e) {  // another user of the device took the room meanwhile
+        if (e.code != BC_E_NOMEM) throw;
+        BCG_CUDA(cudaStreamSynchronize(st));
+        BCG_CUDA(cudaMemcpyAsync(ws.sources.p, sm + 384, 64 * 4, cudaMemcpyDeviceToDevice, st));
+        more = false;
+      }
+    }
+    if (more) {
       {
         LaunchScope ls(ctx, F_MISC);
         k_land_reach<<<1, 1, 0, st>>>(g.n, g.hub, maxl, ws.lm.as<uint64_t>(), d_reach);

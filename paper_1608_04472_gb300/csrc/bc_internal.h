@@ -277,8 +277,10 @@ enum OvfMode { OVF_IGNORE = 0, OVF_ERROR = 1, OVF_EXTEND = 2 };
 inline uint64_t lanes_of(int count) { return count >= 64 ? ~0ull : ((1ull << count) - 1ull); }
 // Runs the forward BFS for `count` (<= 64) sources already on the device in
 // ws.sources. Returns the deepest level reached. With `pairs`, lane i stops
-// once ws.targets[i] is discovered and its d/sigma are recorded.
-int batch_forward(bc_ctx *ctx, const Graph &g, int count, bool pairs, OvfMode mode = OVF_ERROR);
+// once ws.targets[i] is discovered and its d/sigma are recorded. Levels beyond
+// `limit` are not looked for (unless earlier batches on the graph had them).
+int batch_forward(bc_ctx *ctx, const Graph &g, int count, bool pairs, OvfMode mode = OVF_ERROR,
+                  int limit = 0x7FFFFFFF);
 // Runs the backward accumulation for levels maxlevel..1 into the sink, for the
 // lanes in `keep`.
 void batch_backward(bc_ctx *ctx, const Graph &g, int maxlevel, const Sink &sink, uint64_t keep = ~0ull);

@@ -194,3 +194,34 @@ def test_levels_launched_unasked_follow_the_graph_s_own_depth(monkeypatch, befor
     assert np.array_equal(far[0], oracle.dependencies(g, 0)[0]) and np.array_equal(near[0], oracle.dependencies(g, path)[0])
     assert np.array_equal(est, oracle.uniform_sources(g, 200, 3, 1))
     assert levels == (path - 1 if path - 1 <= 29 else 1)
+
+
+@pytest.mark.parametrize("shape", ["star_and_path", "hub_to_all_and_chain"])
+def test_landmarks_take_no_level_per_vertex_of_a_long_path(ctx, shape):
+    """Draws that all miss a path of 3,000 vertices: another component's on the
+    undirected graph, a chain of arcs among the vertices the hub points to on the
+    directed one. The source key's pass takes a few levels of 12 B a vertex, not one
+    per path vertex (3.6 GB and as much again while they grow)."""
+    import torch
+    n, path, k = 100_000, 3000, 100
+    p = np.arange(n - path, n - 1)
+    if shape == "star_and_path":
+        i = np.arange(1, n - path)
+        g = gg.from_edges(n, np.r_[0 * i, p], np.r_[i, p + 1])
+    else:
+        i = np.arange(1, n)
+        g = gg.from_edges_directed(n, np.r_[0 * i, p], np.r_[i, p + 1])
+    seed = next(s for s in range(1000) if ctx.draw_sources(s, 1, 0, k, n).max() < n - path)
+    h = ctx.load_graph(g.row_ptr, g.col, directed=shape != "star_and_path")
+    free = torch.cuda.mem_get_info()[0]
+    got = ctx.uniform_sources(h, k, seed, 1)
+    used = free - torch.cuda.mem_get_info()[0]
+    ctx.free_graph(h)
+    # leaves of the star have one shortest path to every other one, through 0
+    s = ctx.draw_sources(seed, 1, 0, k, n)
+    leaves = n - path - 1
+    want = np.zeros(n)
+    if shape == "star_and_path":
+        want[0] = n * (float(np.sum(s != 0)) * (leaves - 1)) / k
+    assert np.array_equal(got, want)
+    assert used < 1 << 30  # the 64-lane state of 100,000 vertices: 2 KB each, twice
