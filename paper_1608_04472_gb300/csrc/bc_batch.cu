@@ -1316,7 +1316,7 @@ static HeavyMeta &heavy_meta(bc_ctx *ctx, const Graph &g, bool in_csr) {
     old.each([](DevBuf &b) { b.release(); });
     g_heavy.erase(it);
   }
-  HeavyMeta &hm = g_heavy[grp];
+  HeavyMeta hm;
   std::vector<int32_t> rp(g.n + 1);
   BCG_CUDA(cudaMemcpy(rp.data(), grp, sizeof(int32_t) * (g.n + 1), cudaMemcpyDeviceToHost));
   std::vector<int32_t> heavy, hseg0, sv, sb, se, light(1, 0);
@@ -1344,16 +1344,21 @@ static HeavyMeta &heavy_meta(bc_ctx *ctx, const Graph &g, bool in_csr) {
     b.ensure(std::max<size_t>(x.size(), 1) * sizeof(int32_t));
     if (!x.empty()) BCG_CUDA(cudaMemcpy(b.p, x.data(), x.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
   };
-  up(hm.heavy, heavy);
-  up(hm.hseg0, hseg0);
-  up(hm.seg_v, sv);
-  up(hm.seg_b, sb);
-  up(hm.seg_e, se);
-  if (grp == g.rp_in) {  // the forward's first list
-    light[0] = (int32_t)light.size() - 1;
-    up(hm.light, light);
+  try {
+    up(hm.heavy, heavy);
+    up(hm.hseg0, hseg0);
+    up(hm.seg_v, sv);
+    up(hm.seg_b, sb);
+    up(hm.seg_e, se);
+    if (grp == g.rp_in) {  // the forward's first list
+      light[0] = (int32_t)light.size() - 1;
+      up(hm.light, light);
+    }
+  } catch (...) {  // (a split cut short must not pass for the graph's next time)
+    hm.each([](DevBuf &b) { b.release(); });
+    throw;
   }
-  return hm;
+  return g_heavy[grp] = std::move(hm);
 }
 
 void forget_heavy_meta(const int32_t *rp) {
@@ -1814,14 +1819,13 @@ static bool second_slot(bc_ctx *ctx, const Graph &g, bool acc) {
     }
     if (need > fr / 4) return false;
   }
-  if (!s.stream) {
-    BCG_CUDA(cudaStreamCreateWithFlags(&s.stream, cudaStreamNonBlocking));
-    BCG_CUDA(cudaEventCreateWithFlags(&s.ev_begin, cudaEventDisableTiming));
-    BCG_CUDA(cudaEventCreateWithFlags(&s.ev_end, cudaEventDisableTiming));
-    BCG_CUDA(cudaMallocHost(&s.state.pinned, 4096));
-    s.state.enable.ensure(64);
-    s.state.sources.ensure(64 * 4);
-  }
+  // (each by itself: a failure here must not pass for a finished slot next time)
+  if (!s.stream) BCG_CUDA(cudaStreamCreateWithFlags(&s.stream, cudaStreamNonBlocking));
+  for (cudaEvent_t *e : {&s.ev_begin, &s.ev_end})
+    if (!*e) BCG_CUDA(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
+  if (!s.state.pinned) BCG_CUDA(cudaMallocHost(&s.state.pinned, 4096));
+  s.state.enable.ensure(64);
+  s.state.sources.ensure(64 * 4);
   if (acc) s.acc.ensure((size_t)g.n * sizeof(Acc));
   return true;
 }

@@ -225,3 +225,33 @@ def test_landmarks_take_no_level_per_vertex_of_a_long_path(ctx, shape):
         want[0] = n * (float(np.sum(s != 0)) * (leaves - 1)) / k
     assert np.array_equal(got, want)
     assert used < 1 << 30  # the 64-lane state of 100,000 vertices: 2 KB each, twice
+
+
+def test_a_call_that_ran_out_of_memory_leaves_nothing_half_built(monkeypatch):
+    """Calls of a fresh context with more and more of the memory they need: each gives
+    the result or BC_E_NOMEM, and the ones after it are right."""
+    import torch
+    import paper_1608_04472_gb300 as pkg
+    monkeypatch.setenv("BCG_SOLO_N", "0")
+    i, j = np.divmod(np.arange(60 * 60), 60)
+    g = gg.erdos_renyi(200_000, 6, 5, pairwise=False)
+    wide = gg.from_edges(60 * 13, np.concatenate([i + 60 * k for k in range(12)]),
+                         np.concatenate([j + 60 * (k + 1) for k in range(12)]))
+    with pkg.Context(0, batch_width=64) as c:  # every kernel is loaded before memory runs short
+        want = c.uniform_sources(c.load_graph(g.row_ptr, g.col), 150, 2, 2)
+        c.uniform_sources(c.load_graph(wide.row_ptr, wide.col), 150, 2, 2)
+    failed = 0
+    with pkg.Context(0, batch_width=64) as c:
+        h = c.load_graph(g.row_ptr, g.col)
+        for left in (2, 8, 24, 64, 128, 256, 512):
+            torch.cuda.empty_cache()
+            rest = torch.empty(torch.cuda.mem_get_info()[0] - (left << 20), dtype=torch.uint8, device="cuda")
+            try:
+                assert np.array_equal(c.uniform_sources(h, 150, 2, 2), want)
+            except pkg.BCError as e:
+                assert e.code == -2  # BC_E_NOMEM
+                failed += 1
+            del rest
+        torch.cuda.empty_cache()
+        assert np.array_equal(c.uniform_sources(h, 150, 2, 2), want)
+    assert failed
