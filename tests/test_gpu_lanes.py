@@ -227,6 +227,19 @@ def test_landmarks_take_no_level_per_vertex_of_a_long_path(ctx, shape):
     assert used < 1 << 30  # the 64-lane state of 100,000 vertices: 2 KB each, twice
 
 
+def _fill(torch, left):
+    """Holds the device's memory but for about `left` bytes."""
+    torch.cuda.empty_cache()
+    held, size = [], torch.cuda.mem_get_info()[0]
+    while size >= 2 << 20:
+        size = max(0, min(size, torch.cuda.mem_get_info()[0] - left)) >> 21 << 21
+        try:
+            held.append(torch.empty(size, dtype=torch.uint8, device="cuda"))
+        except torch.OutOfMemoryError:
+            size //= 2
+    return held
+
+
 def test_a_call_that_ran_out_of_memory_leaves_nothing_half_built(monkeypatch):
     """Calls of a fresh context with more and more of the memory they need: each gives
     the result or BC_E_NOMEM, and the ones after it are right."""
@@ -244,14 +257,13 @@ def test_a_call_that_ran_out_of_memory_leaves_nothing_half_built(monkeypatch):
     with pkg.Context(0, batch_width=64) as c:
         h = c.load_graph(g.row_ptr, g.col)
         for left in (2, 8, 24, 64, 128, 256, 512):
-            torch.cuda.empty_cache()
-            rest = torch.empty(torch.cuda.mem_get_info()[0] - (left << 20), dtype=torch.uint8, device="cuda")
+            rest = _fill(torch, left << 20)
             try:
                 assert np.array_equal(c.uniform_sources(h, 150, 2, 2), want)
             except pkg.BCError as e:
                 assert e.code == -2  # BC_E_NOMEM
                 failed += 1
-            del rest
-        torch.cuda.empty_cache()
+            rest.clear()
+            torch.cuda.empty_cache()
         assert np.array_equal(c.uniform_sources(h, 150, 2, 2), want)
     assert failed
