@@ -1381,26 +1381,29 @@ static int grid_blocks() {
   return g_num_sms * 8;
 }
 
-// Vertices a warp of the light kernels takes at a time: on small graphs fewer,
-// for more warps to have some (R-MAT s17 directed 6.96 ms taking 4, 7.03 taking
-// 8, 7.66 taking 16), on large ones more, for fewer atomics (s20 48.2 / 46.8 /
-// 46.8 ms). BCG_BWD_GRAB / BCG_FWD_GRAB override.
+// Vertices a warp of the light kernels takes at a time, by one atomic on a shared
+// counter. Forward 16: with 4 below 2^18 vertices (8 above) the wide levels of
+// sparse graphs waited for the counter and for windows filled by 4 short rows; ms
+// for 1024 draws with 4 / 8 / 16 / 32: directed ER n = 200,000 degree 2 66.8 / 54.4 /
+// 49.8 / 50.7, ER n = 100,003 degree 7 13.5 / 11.8 / 11.1 / 11.0, R-MAT s16 5.53 /
+// 5.38 / 5.35 / 5.64, directed s17 10.27 / 9.70 / 9.51 / 9.80, s20 37.9 / 35.1 / 34.4 /
+// 34.3. Backward 4 below 2^18 vertices and 8 above (a vertex's sums are more work, and
+// more warps then have some): ER degree 7 13.5 / 13.4 / 14.1 / 15.2, s16 5.51 / 5.55 /
+// 5.90 / 6.24, s20 35.7 / 35.2 / 35.2 / 35.3. BCG_FWD_GRAB / BCG_BWD_GRAB override.
 static int env_grab(const char *name) {
   const char *e = std::getenv(name);
   const int v = e ? std::atoi(e) : 0;
   return (v == 1 || v == 2 || v == 4 || v == 8 || v == 16 || v == 32) ? v : 0;
 }
 
-static int light_grab(int32_t n) { return n >= (1 << 18) ? 8 : 4; }
-
 static int bwd_grab(int32_t n) {
   static const int env = env_grab("BCG_BWD_GRAB");
-  return env ? env : light_grab(n);
+  return env ? env : (n >= (1 << 18) ? 8 : 4);
 }
 
-static int fwd_grab(int32_t n) {
+static int fwd_grab() {
   static const int env = env_grab("BCG_FWD_GRAB");
-  return env ? env : light_grab(n);
+  return env ? env : 16;
 }
 
 // The context's side stream and its fork / join events, made on first use.
@@ -1569,7 +1572,7 @@ struct Forward {
       k_fwd_light<<<blocks, FWD_THREADS, 0, st>>>(
           g.n, todo, todo_level < 0 ? hm.light.as<unsigned>() : &ctl(todo_level)->todo, left, &next->todo, prp, pcol,
           lm(l), lm(l + 1), visited, sigma, u64(&cur->active), enable, u64(&next->active), cnt, &cur->q_light,
-          lst(l + 1), &next->vcnt, ve, fwd_grab(g.n));
+          lst(l + 1), &next->vcnt, ve, fwd_grab());
       todo = left;
       todo_level = l + 1;
     }
