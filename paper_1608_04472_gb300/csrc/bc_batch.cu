@@ -1382,12 +1382,13 @@ static int grid_blocks() {
 }
 
 // Vertices a warp of the light kernels takes at a time, by one atomic on a shared
-// counter. Forward 16: with 4 below 2^18 vertices (8 above) the wide levels of
-// sparse graphs waited for the counter and for windows filled by 4 short rows; ms
-// for 1024 draws with 4 / 8 / 16 / 32: directed ER n = 200,000 degree 2 66.8 / 54.4 /
+// counter. Forward 16 (8 below 2^16 vertices, 4 below 2^14, for more warps to have
+// some): with 4 below 2^18 the wide levels of sparse graphs waited for the counter
+// and for windows filled by 4 short rows; ms for 1024 draws with 4 / 8 / 16 / 32: directed ER n = 200,000 degree 2 66.8 / 54.4 /
 // 49.8 / 50.7, ER n = 100,003 degree 7 13.5 / 11.8 / 11.1 / 11.0, R-MAT s16 5.53 /
 // 5.38 / 5.35 / 5.64, directed s17 10.27 / 9.70 / 9.51 / 9.80, s20 37.9 / 35.1 / 34.4 /
-// 34.3. Backward 4 below 2^18 vertices and 8 above (a vertex's sums are more work, and
+// 34.3; with 4 / 8 / 16: ER degree 8 n = 10,000 3.80 / 3.69 / 4.06, n = 30,000 5.74 /
+// 5.33 / 5.43, n = 50,000 7.79 / 7.07 / 6.70. Backward 4 below 2^18 vertices and 8 above (a vertex's sums are more work, and
 // more warps then have some): ER degree 7 13.5 / 13.4 / 14.1 / 15.2, s16 5.51 / 5.55 /
 // 5.90 / 6.24, s20 35.7 / 35.2 / 35.2 / 35.3. BCG_FWD_GRAB / BCG_BWD_GRAB override.
 static int env_grab(const char *name) {
@@ -1401,9 +1402,9 @@ static int bwd_grab(int32_t n) {
   return env ? env : (n >= (1 << 18) ? 8 : 4);
 }
 
-static int fwd_grab() {
+static int fwd_grab(int32_t n) {
   static const int env = env_grab("BCG_FWD_GRAB");
-  return env ? env : 16;
+  return env ? env : (n >= (1 << 16) ? 16 : n >= (1 << 14) ? 8 : 4);
 }
 
 // The context's side stream and its fork / join events, made on first use.
@@ -1572,7 +1573,7 @@ struct Forward {
       k_fwd_light<<<blocks, FWD_THREADS, 0, st>>>(
           g.n, todo, todo_level < 0 ? hm.light.as<unsigned>() : &ctl(todo_level)->todo, left, &next->todo, prp, pcol,
           lm(l), lm(l + 1), visited, sigma, u64(&cur->active), enable, u64(&next->active), cnt, &cur->q_light,
-          lst(l + 1), &next->vcnt, ve, fwd_grab());
+          lst(l + 1), &next->vcnt, ve, fwd_grab(g.n));
       todo = left;
       todo_level = l + 1;
     }
