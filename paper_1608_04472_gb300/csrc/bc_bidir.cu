@@ -770,7 +770,7 @@ std::vector<int32_t> pair_lanes(bc_ctx *ctx, const Graph &g, const int32_t *d_sr
   for (int i = 0; i < count; ++i)
     if (flags[(size_t)i]) bigs.push_back(i);
   Workspace &ws = ctx->ws;
-  const bool deep = lane_major(ctx, g);
+  const bool per_cta = lane_major(ctx, g, (int64_t)bigs.size());
   B.idx.ensure(64 * 4);
   for (size_t k0 = 0; k0 < bigs.size(); k0 += 64) {
     const int c = (int)std::min<size_t>(64, bigs.size() - k0);
@@ -780,7 +780,7 @@ std::vector<int32_t> pair_lanes(bc_ctx *ctx, const Graph &g, const int32_t *d_sr
       k_gather_pairs<<<1, 64, 0, st>>>(c, B.idx.as<int32_t>(), d_src, d_dst, ws.sources.as<int32_t>(),
                                        ws.targets.as<int32_t>());
     }
-    if (deep)
+    if (per_cta)
       lane_pairs(ctx, g, c);  // every lane overflows there, so each is extended
     else
       ext_pair_lanes(ctx, g, ws.sources.as<int32_t>(), ws.targets.as<int32_t>(), lanes_of(c));

@@ -571,16 +571,16 @@ static void launch_draw_sources(bc_ctx *ctx, uint64_t seed, uint64_t qid, uint64
 
 // Lanes whose path counts exceed 2^64-1 skip the integer backward pass and are
 // recomputed in the extended form (bc_ext.cu); the others are unaffected.
-// Graphs whose per-source state fits shared memory (solo_fits) and deep graphs
-// (the hub's eccentricity above ctx->deep_levels, e.g. grids) run one source
-// per CTA: on deep graphs level masks and 64-lane rows cost O(levels * n),
-// while each source's own BFS costs O(n + nnz).
+// Deep graphs (the hub's eccentricity above ctx->deep_levels, e.g. grids) and
+// graphs whose per-source state fits shared memory, where that is faster for so
+// many sources (solo_pays), run one source per CTA: on deep graphs level masks and
+// 64-lane rows cost O(levels * n), while each source's own BFS costs O(n + nnz).
 void run_source_batch(bc_ctx *ctx, const Graph &g, int count, const Sink &sink) {
   if (g.w) {  // edge lengths: the weighted engine at any width
     wlane_sink(ctx, g, ctx->ws.sources.as<int32_t>(), count, sink);
   } else if (batch_width(ctx) == 1) {
     plain_source(ctx, g, ctx->ws.sources.as<int32_t>(), sink, nullptr, nullptr);
-  } else if (lane_major(ctx, g)) {
+  } else if (lane_major(ctx, g, count)) {
     lane_sink(ctx, g, ctx->ws.sources.as<int32_t>(), count, sink);
   } else {
     const int maxl = batch_forward(ctx, g, count, false, OVF_EXTEND);
@@ -656,6 +656,7 @@ struct KeyMeta {
   DevBuf key, order;
   DevBuf hub;        // the hub's distances as bytes, from the depth until the key is built
   int32_t ecc = -1;  // largest finite distance from the hub (-1: not known yet)
+  int K = 0;         // landmarks the key was asked for with
 };
 static std::map<const int32_t *, KeyMeta> g_keys;
 static std::mutex g_keys_mu;
@@ -734,12 +735,10 @@ static void build_depth(bc_ctx *ctx, const Graph &g, KeyMeta &km) {
   dist.release();
 }
 
-static void build_key(bc_ctx *ctx, const Graph &g, KeyMeta &km) {
+static void build_key(bc_ctx *ctx, const Graph &g, KeyMeta &km, int K) {
   Workspace &ws = ctx->ws;
   cudaStream_t st = ctx->stream;
   const size_t n = (size_t)g.n;
-  // edge lengths: a source has a CTA of its own, so the hub's row is enough
-  const int K = g.w ? 1 : key_landmarks();
   const unsigned nb = (unsigned)((n + 255) / 256);
   const int64_t s0 = ctx->samples, b0 = ctx->batches;
   DevBuf rows, proj, small;
@@ -842,14 +841,25 @@ static void build_key(bc_ctx *ctx, const Graph &g, KeyMeta &km) {
   }
   ctx->samples = s0;
   ctx->batches = b0;
+  if (K == 1) std::swap(rows, km.hub);  // (a later call may want the landmarks)
+  km.K = K;
   release_all();
 }
 
-static KeyMeta &key_meta(bc_ctx *ctx, const Graph &g, bool need_order) {
+// The key for a call with `count` sources. Edge lengths: a source has a CTA of its
+// own, so the hub's row is enough. On graphs of at most 65,536 vertices it is as
+// well below 512 sources: the landmarks take 0.6 to 0.9 ms once and save 7 to 9 % of
+// a call of 300 and more (R-MAT s15, 200 / 1024 draws, hub alone and with landmarks:
+// 1.13 / 4.2 and 1.06 / 3.9 ms).
+static KeyMeta &key_meta(bc_ctx *ctx, const Graph &g, bool need_order, int64_t count) {
   std::lock_guard<std::mutex> lk(g_keys_mu);
   KeyMeta &km = g_keys[g.rp];
   const size_t n = (size_t)g.n;
-  if (!km.key.p) build_key(ctx, g, km);
+  const int K = g.w || (g.n <= 65536 && count < 512) ? 1 : key_landmarks();
+  if (!km.key.p || km.K < K) {
+    km.order.release();
+    build_key(ctx, g, km, K);
+  }
   if (need_order && !km.order.p) {
     std::vector<uint8_t> key(n);
     BCG_CUDA(cudaMemcpy(key.data(), km.key.p, n, cudaMemcpyDeviceToHost));
@@ -867,43 +877,46 @@ static KeyMeta &key_meta(bc_ctx *ctx, const Graph &g, bool need_order) {
 constexpr int WMAX = 1024;       // draws per window of the 64-lane engine
 constexpr int WMAX_SOLO = 4096;  // ... of the engines that run one source per CTA
 
-bool lane_major(bc_ctx *ctx, const Graph &g) {
-  return solo_fits(ctx, g) || graph_depth_hint(ctx, g) > ctx->deep_levels;  // (a fitting graph needs no depth here)
+bool lane_major(bc_ctx *ctx, const Graph &g, int64_t count, bool adaptive, int64_t beside) {
+  if (graph_depth_hint(ctx, g) > ctx->deep_levels) return true;
+  return solo_fits(ctx, g) && solo_pays(ctx, g, count, adaptive, beside);
 }
 
 // Engines that run one source per persistent CTA (edge lengths; deep graphs;
 // graphs whose state fits shared memory) take a whole window in one launch, so
 // every resident CTA has a source; the 64-lane engine and the plain width take
 // 64 or 1 at a time.
-bool one_source_per_cta(bc_ctx *ctx, const Graph &g) {
-  return batch_width(ctx) != 1 && (g.w || lane_major(ctx, g));
+bool one_source_per_cta(bc_ctx *ctx, const Graph &g, int64_t count, bool adaptive, int64_t beside) {
+  return batch_width(ctx) != 1 && (g.w || lane_major(ctx, g, count, adaptive, beside));
 }
 
-// The draws a window can hold and the size of the first one. Where a source
-// has a CTA of its own, fewer sources than CTAs leave SMs idle, so windows
-// start at one source per resident CTA (per SM on the weighted engine and on
-// deep graphs in global memory, where more sources at once compete for
-// bandwidth) instead of 64.
-static int window_max(bc_ctx *ctx, const Graph &g, int32_t T) {
-  return one_source_per_cta(ctx, g) && T <= 4096 ? WMAX_SOLO : WMAX;
-}
-static int window_first(bc_ctx *ctx, const Graph &g) {
-  if (!one_source_per_cta(ctx, g)) return 64;
-  return std::max(64, g.w ? 152 : solo_slots(ctx, g));
+// A window that the 64-lane engine takes as one batch, in draw order.
+static bool one_batch(bc_ctx *ctx, const Graph &g, int W) { return W <= 64 && batch_width(ctx) != 1 && !g.w; }
+
+// The draws a window can hold and the size of the first one, where sources have
+// a CTA each (per_cta) or not; a call keeps to one of the two. Where a source has a CTA
+// of its own, fewer sources than CTAs leave SMs idle, so windows start at one
+// source per resident CTA (per SM on the weighted engine and on deep graphs in
+// global memory, where more sources at once compete for bandwidth) instead of 64.
+static int window_max(bool per_cta, int32_t T) { return per_cta && T <= 4096 ? WMAX_SOLO : WMAX; }
+static int window_first(bc_ctx *ctx, const Graph &g, bool per_cta) {
+  return !per_cta ? 64 : std::max(64, g.w ? 152 : solo_slots(ctx, g));
 }
 
 // Draws [i0, i0+W) of (seed, qid): ws.win = draws[W] and, for the 64-lane
 // engine, grouped by source key, sorted sources[W] at WMAX and sorted draw
 // positions[W] at 2 WMAX (where a source has a CTA of its own, which sources
-// run together does not matter, and no key is built).
-static void draw_window(bc_ctx *ctx, const Graph &g, uint64_t seed, uint64_t qid, int64_t i0, int W) {
+// run together does not matter, nor in a window of one batch: no key is built).
+// total: the call's draws.
+static void draw_window(bc_ctx *ctx, const Graph &g, bool per_cta, int64_t total, uint64_t seed, uint64_t qid,
+                        int64_t i0, int W) {
   Workspace &ws = ctx->ws;
   ws.win.ensure(WMAX_SOLO * 4);
   static_assert(WMAX_SOLO >= 3 * WMAX, "the window buffer holds the draws and their sorted form");
   int32_t *draws = ws.win.as<int32_t>();
   launch_draw_sources(ctx, seed, qid, (uint64_t)i0, W, g.n, draws);
-  if (one_source_per_cta(ctx, g)) return;
-  const KeyMeta &km = key_meta(ctx, g, false);
+  if (per_cta || one_batch(ctx, g, W)) return;
+  const KeyMeta &km = key_meta(ctx, g, false, total);
   LaunchScope ls(ctx, F_DRAW);
   k_sort_window<<<1, 1024, 0, ctx->stream>>>(W, draws, km.key.as<uint8_t>(), draws + WMAX, draws + 2 * WMAX);
 }
@@ -918,11 +931,15 @@ static void run_sources_per_cta(bc_ctx *ctx, const Graph &g, const int32_t *d_so
 // Runs the window's sources: one launch where a source has a CTA, else batches
 // of the context's width (lane t of the batch starting at position b is the
 // window's sorted entry b + t).
-static void run_window(bc_ctx *ctx, const Graph &g, int W, Sink sink) {
+static void run_window(bc_ctx *ctx, const Graph &g, bool per_cta, int W, Sink sink) {
   Workspace &ws = ctx->ws;
   const int width = batch_width(ctx);
-  if (one_source_per_cta(ctx, g)) {  // column = draw position
+  if (per_cta) {  // column = draw position
     run_sources_per_cta(ctx, g, ws.win.as<int32_t>(), W, sink);
+    return;
+  }
+  if (one_batch(ctx, g, W)) {
+    run_lane_batches(ctx, g, ws.win.as<int32_t>(), nullptr, W, sink);
     return;
   }
   const int32_t *sorted_src = ws.win.as<int32_t>() + WMAX;
@@ -945,8 +962,8 @@ static void run_window(bc_ctx *ctx, const Graph &g, int W, Sink sink) {
 // in the kernel), else window by window.
 static void run_draws(bc_ctx *ctx, const Graph &g, uint64_t seed, uint64_t qid, int64_t i0, int64_t count,
                       const Sink &sink) {
-  const bool solo = batch_width(ctx) != 1 && !g.w && lane_major(ctx, g);
-  const int64_t most = solo ? (int64_t)1 << 30 : window_max(ctx, g, 0);
+  const bool per_cta = one_source_per_cta(ctx, g, count), solo = per_cta && !g.w;
+  const int64_t most = solo ? (int64_t)1 << 30 : window_max(per_cta, 0);
   for (int64_t a = 0; a < count; a += most) {
     const int W = (int)std::min<int64_t>(most, count - a);
     if (solo) {
@@ -957,8 +974,8 @@ static void run_draws(bc_ctx *ctx, const Graph &g, uint64_t seed, uint64_t qid, 
       src.draw = 1;
       solo_sources(ctx, g, src, W, sink, SoloRows{});
     } else {
-      draw_window(ctx, g, seed, qid, i0 + a, W);
-      run_window(ctx, g, W, sink);
+      draw_window(ctx, g, per_cta, count, seed, qid, i0 + a, W);
+      run_window(ctx, g, per_cta, W, sink);
     }
   }
 }
@@ -974,11 +991,11 @@ static void do_exact_or_uniform(bc_ctx *ctx, const Graph &g, bool exact, int64_t
   const int width = batch_width(ctx);
   if (!exact) {
     run_draws(ctx, g, seed, qid, 0, k, sink);
-  } else if (one_source_per_cta(ctx, g) && !g.w) {
+  } else if (!g.w && one_source_per_cta(ctx, g, g.n)) {
     solo_sources(ctx, g, SoloSources{}, g.n, sink, SoloRows{});  // every vertex once
   } else {
     // all n sources, grouped by key (the sum over sources is exact, so any order)
-    const KeyMeta &km = key_meta(ctx, g, true);
+    const KeyMeta &km = key_meta(ctx, g, true, g.n);
     if (width != 1 && !g.w) {
       run_lane_batches(ctx, g, km.order.as<int32_t>(), nullptr, g.n, sink);
     }
@@ -1007,13 +1024,14 @@ static void do_exact_or_uniform(bc_ctx *ctx, const Graph &g, bool exact, int64_t
 // The depth that decides between the level-mask engine and one source per
 // persistent CTA: the largest finite distance from the hub (along out-edges on
 // a directed graph; the level-mask engine pulls counts over the in-neighbour CSR).
-// Small graphs get it from one CTA's BFS.
+// Small graphs get it from one CTA's BFS (about 5 ns a vertex and 0.5 an entry;
+// the plain engine's takes 20 us a level, in all of 6 to 15 here).
 int graph_depth_hint(bc_ctx *ctx, const Graph &g) {
   {
     std::lock_guard<std::mutex> lk(g_keys_mu);
     KeyMeta &km = g_keys[g.rp];
     if (km.ecc >= 0) return km.ecc;
-    if (!solo_fits(ctx, g)) {
+    if (!solo_fits(ctx, g) || g.n + g.nnz / 10 > 40000) {
       const int64_t s0 = ctx->samples, b0 = ctx->batches;
       build_depth(ctx, g, km);
       ctx->samples = s0;
@@ -1042,7 +1060,8 @@ static void do_adaptive_sources(bc_ctx *ctx, const Graph &g, const int32_t *targ
   const size_t n = (size_t)g.n;
   cudaStream_t st = ctx->stream;
   ws.tslot.ensure(n * 4);
-  const int wmax = window_max(ctx, g, T);
+  const bool per_cta = one_source_per_cta(ctx, g, cap, true);
+  const int wmax = window_max(per_cta, T);
   ws.tdelta.ensure((size_t)std::max(T, 1) * wmax * 8);
   {
     LaunchScope ls(ctx, F_MISC);
@@ -1056,18 +1075,18 @@ static void do_adaptive_sources(bc_ctx *ctx, const Graph &g, const int32_t *targ
   }
   ScanState ss = make_scan(ctx, T);
   const double cn = c * (double)g.n;
-  const int64_t first = window_first(ctx, g);
+  const int64_t first = window_first(ctx, g, per_cta);
   int32_t remaining = T;
   for (int64_t i0 = 0; i0 < cap && remaining > 0;) {
     const int64_t want = std::max<int64_t>(first, i0 / 2);
     const int W = (int)std::min<int64_t>(std::min<int64_t>(wmax, want), cap - i0);
-    draw_window(ctx, g, seed, qid, i0, W);
+    draw_window(ctx, g, per_cta, cap, seed, qid, i0, W);
     BCG_CUDA(cudaMemsetAsync(ws.tdelta.p, 0, (size_t)T * W * 8, st));
     Sink sink;
     sink.tslot = ws.tslot.as<int32_t>();
     sink.tdelta = ws.tdelta.as<double>();
     sink.tstride = W;
-    run_window(ctx, g, W, sink);
+    run_window(ctx, g, per_cta, W, sink);
     {
       LaunchScope ls(ctx, F_SCAN);
       k_stop_scan<<<(T + 3) / 4, 128, 0, st>>>(T, W, ws.tdelta.as<double>(), ss, i0, cn, 1.0, W);
@@ -1090,7 +1109,8 @@ static void do_target_block(bc_ctx *ctx, const Graph &g, const int32_t *targets,
   const size_t n = (size_t)g.n;
   cudaStream_t st = ctx->stream;
   ws.tslot.ensure(n * 4);
-  const int wmax = window_max(ctx, g, T);
+  const bool per_cta = one_source_per_cta(ctx, g, count);
+  const int wmax = window_max(per_cta, T);
   ws.tdelta.ensure((size_t)std::max(T, 1) * wmax * 8);
   {
     LaunchScope ls(ctx, F_MISC);
@@ -1105,13 +1125,13 @@ static void do_target_block(bc_ctx *ctx, const Graph &g, const int32_t *targets,
   std::vector<double> h((size_t)T * wmax);
   for (int64_t a = 0; a < count; a += wmax) {
     const int W = (int)std::min<int64_t>(wmax, count - a);
-    draw_window(ctx, g, seed, qid, i0 + a, W);
+    draw_window(ctx, g, per_cta, count, seed, qid, i0 + a, W);
     BCG_CUDA(cudaMemsetAsync(ws.tdelta.p, 0, (size_t)T * W * 8, st));
     Sink sink;
     sink.tslot = ws.tslot.as<int32_t>();
     sink.tdelta = ws.tdelta.as<double>();
     sink.tstride = W;
-    run_window(ctx, g, W, sink);
+    run_window(ctx, g, per_cta, W, sink);
     BCG_CUDA(cudaMemcpyAsync(h.data(), ws.tdelta.p, (size_t)T * W * 8, cudaMemcpyDeviceToHost, st));
     sync(ctx);
     for (int32_t j = 0; j < T; ++j)
@@ -1153,7 +1173,7 @@ void target_bfs(bc_ctx *ctx, const Graph &g, const int32_t *d_targets, int T, in
   Workspace &ws = ctx->ws;
   const size_t n = (size_t)g.n;
   tx.assign((size_t)Tp, 0);
-  if (T > 0 && lane_major(ctx, g)) {
+  if (T > 0 && lane_major(ctx, g, T)) {
     // one BFS per CTA and target
     if (!texp.p) texp.ensure(n * (size_t)Tp * 4);
     DevBuf dtx;
@@ -1203,7 +1223,7 @@ uint64_t pair_batch(bc_ctx *ctx, const Graph &g, int count) {
   uint64_t ovf;
   if (batch_width(ctx) == 1) {
     ovf = plain_pair(ctx, g, ws.sources.as<int32_t>(), ws.targets.as<int32_t>()) ? 1ull : 0ull;
-  } else if (lane_major(ctx, g)) {
+  } else if (lane_major(ctx, g, count)) {
     ovf = lane_pairs(ctx, g, count);
   } else {
     batch_forward(ctx, g, count, true, OVF_EXTEND);
@@ -1518,7 +1538,7 @@ static void do_source_dependencies(bc_ctx *ctx, const Graph &g, const int32_t *s
     do_source_rows_weighted(ctx, g, sources, count, delta_out, nullptr, sigma_out, sm_out, se_out, tier_out);
     return;
   }
-  if (batch_width(ctx) != 1 && solo_fits(ctx, g)) {
+  if (batch_width(ctx) != 1 && solo_fits(ctx, g) && lane_major(ctx, g, count)) {
     do_source_rows_solo(ctx, g, sources, count, delta_out, dist_out, sigma_out, sm_out, se_out, tier_out);
     return;
   }
@@ -1854,7 +1874,10 @@ bc_status bc_create(bc_ctx **out, int device, const bc_options *opt) {
     if (const char *hd = std::getenv("BCG_HEAVY_DEGREE")) ctx->heavy_deg = std::atoi(hd);
     if (const char *sl = std::getenv("BCG_SEGMENT")) ctx->seg_len = std::atoi(sl);
     if (const char *dl = std::getenv("BCG_DEEP_LEVELS")) ctx->deep_levels = std::atoi(dl);
-    if (const char *sn = std::getenv("BCG_SOLO_N")) ctx->solo_n = std::atoi(sn);
+    if (const char *sn = std::getenv("BCG_SOLO_N")) {
+      ctx->solo_n = std::atoi(sn);
+      ctx->solo_always = ctx->solo_n > 0;
+    }
     if (const char *sz = std::getenv("BCG_SOLO_NNZ")) ctx->solo_nnz = std::atoll(sz);
     if (const char *so = std::getenv("BCG_SOLO_THREADS")) {
       const int t = std::atoi(so);

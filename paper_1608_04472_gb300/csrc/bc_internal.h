@@ -206,9 +206,11 @@ struct bc_ctx {
   // persistent kernel, and its CTAs per SM while the batched engine runs beside
   int32_t deep_levels = 32, multi_cap = 4;
   // graphs of at most solo_n vertices and solo_nnz entries whose state fits
-  // shared memory run one source per CTA at any depth (BCG_SOLO_N, 0: only deep
-  // graphs do; BCG_SOLO_NNZ); solo_threads forces the CTA size (0: by rule)
+  // shared memory can run one source per CTA at any depth (BCG_SOLO_N, BCG_SOLO_NNZ):
+  // where it pays for a call's sources, with BCG_SOLO_N = 0 only deep graphs, with
+  // another value always; solo_threads forces the CTA size (0: by rule)
   int32_t solo_n = 65536, solo_threads = 0;
+  bool solo_always = false;
   int64_t solo_nnz = 1000000;
   // pair lanes of Algorithm 1: 0 = bidirectional search, one pair per CTA
   // (bc_bidir.cu); 2 = the same search one pair per warp with hash-table
@@ -346,15 +348,20 @@ struct SoloRows {
   int32_t *se = nullptr;
   int32_t *tier = nullptr;
 };
-// Whether the graph's sources run one per CTA because their state fits shared
-// memory (deep graphs do as well: one_source_per_cta), and how many run at once.
+// Whether a source's state fits shared memory, whether `count` sources of such a
+// graph are faster one per CTA than 64 to a traversal (adaptive: as Bader's loop
+// draws them; beside: sources of other graphs in the same launch), and how many
+// run at once.
 bool solo_fits(bc_ctx *ctx, const Graph &g);
+bool solo_pays(bc_ctx *ctx, const Graph &g, int64_t count, bool adaptive = false, int64_t beside = 0);
 int solo_slots(bc_ctx *ctx, const Graph &g);
 // The largest finite distance from v by one CTA (any graph without lengths).
 int solo_depth(bc_ctx *ctx, const Graph &g, int32_t v);
-// (lane_major: at any width but 1, weighted graphs apart.)
-bool lane_major(bc_ctx *ctx, const Graph &g);
-bool one_source_per_cta(bc_ctx *ctx, const Graph &g);
+// Whether a call with `count` sources runs one source per persistent CTA: deep
+// graphs, and fitting ones where it pays (lane_major: at any width but 1,
+// weighted graphs apart). Every engine gives the same results.
+bool lane_major(bc_ctx *ctx, const Graph &g, int64_t count, bool adaptive = false, int64_t beside = 0);
+bool one_source_per_cta(bc_ctx *ctx, const Graph &g, int64_t count, bool adaptive = false, int64_t beside = 0);
 void solo_sources(bc_ctx *ctx, const Graph &g, const SoloSources &src, int count, const Sink &sink,
                   const SoloRows &rows);
 void do_uniform_multi(bc_ctx *ctx, const std::vector<bc_graph> &handles, const std::vector<const Graph *> &gs,

@@ -276,14 +276,11 @@ static int solo_tier(const Graph &g) {
   return 2;
 }
 
-// Shallow graphs run one source per CTA up to 65,536 vertices and a million
-// entries. One source per CTA reads every row once per source, the 64-lane
-// engine shares its reads among 64 sources, so density and size favour the
-// latter. us a source, 1024 uniform draws, here / 64-lane engine: ER n = 2000
-// deg 8 0.27 / 6.9, n = 18,000 2.2 / 9.4, n = 50,000 6.6 / 11.0, n = 100,000
-// 29 / 17 (152 CTAs' counts no longer fit L2); BA n = 50,000 7.1 / 24, n =
-// 110,000 34 / 27; R-MAT s14 (nnz 426k) 3.4 / 8.5, s15 (883k) 6.6 / 9.1, s16
-// with 955k entries 7.7 / 8.3, with 1.82M 12.6 / 12.0.
+// Shallow graphs can run one source per CTA up to 65,536 vertices and a million
+// entries (beyond, the 64-lane engine was faster whatever the draws; us a source,
+// 1024 uniform draws, here / there: ER n = 100,000 degree 8 29 / 17, where 152 CTAs'
+// counts no longer fit L2; R-MAT s16 with 1.82M entries 12.6 / 12.0). Whether a call
+// does: solo_pays.
 bool solo_fits(bc_ctx *ctx, const Graph &g) {
   return !g.w && g.n <= ctx->solo_n && g.nnz <= ctx->solo_nnz && solo_tier(g) < 2;
 }
@@ -336,7 +333,64 @@ static SoloCfg solo_cfg(bc_ctx *ctx, int tier, int32_t n, int64_t nnz, int64_t c
   if (tier < 2 && ctx->solo_threads) c.threads = ctx->solo_threads;
   return c;
 }
-//
+
+// Whether `count` sources of a fitting graph that is not deep run one per CTA
+// rather than 64 to a traversal (adaptive: in the windows of Bader's loop;
+// beside: draws of other graphs in the same launch). One source per CTA reads
+// every row once per source at one CTA's speed, so a launch takes as long as a
+// source on a CTA times the rounds over the CTAs, however few the sources; the
+// 64-lane engine takes a batch's time for every 64, mostly per level. Both
+// estimates, in us, follow the times of uniform, adaptive and served calls of 1 to
+// 1024 draws on 40 graphs of 1,500 to 65,536 vertices and 16,000 to a million
+// entries (ER, BA, R-MAT, directed ones among them) with either engine; the 64-lane
+// engine has to be an eighth faster by them (they are off by about that much). The
+// choice costs 1.3 % over the better engine in the geometric mean, at worst it was
+// 1.18 times slower than always here and 5 % than always there. Here / there, us a call
+// of 16 / 64 / 200 / 1024 draws: ER n = 2000 degree 8 133 / 137 / 149 / 291 and 311 / 342
+// / 760 / 2799; ER n = 50,000 934 / 950 / 1978 / 7013 and 528 / 658 / 1737 / 7073; R-MAT
+// s14 (430,000 entries) 770 / 777 / 797 / 3708 and 399 / 469 / 917 / 3385; s15 (890,000)
+// 1617 / 1635 / 1722 / 7246 and 489 / 566 / 1061 / 3995; ER n = 60,000 degree 3 878 / 906 /
+// 1905 / 6825 and 1170 / 1320 / 3580 / 16,700.
+bool solo_pays(bc_ctx *ctx, const Graph &g, int64_t count, bool adaptive, int64_t beside) {
+  if (ctx->solo_always) return true;
+  const int tier = solo_tier(g);
+  const double n = (double)g.n, z = (double)g.nnz, depth = (double)graph_depth_hint(ctx, g);
+  const int64_t sms = solo_sms();
+  auto ctas = [&](int64_t c, bool *small) {
+    *small = solo_cfg(ctx, tier, g.n, g.nnz, c, false).threads == 256;
+    return sms * (*small ? std::min<int64_t>(4, (int64_t)(SOLO_SM_SMEM / solo_cta_smem(tier, g.n))) : 1);
+  };
+  bool small;
+  const int64_t first = adaptive ? std::max<int64_t>(64, ctas((int64_t)1 << 30, &small)) : 0;
+  const double lat[2] = {10e-3 * n + 1.05e-3 * z + 2.5 * depth, 30e-3 * n + 2.6e-3 * z};  // 1024 and 256 threads
+  const double level = 125.0 + 37.0 * depth, rows = n * (3.8e-3 + 0.38e-3 * depth);
+  double solo = 90.0, lane = 50.0;
+  auto window = [](int64_t i, int64_t lo, int64_t hi, int64_t left) {
+    return std::min(left, std::min(hi, std::max(lo, i / 2)));
+  };
+  const int64_t draws = adaptive ? std::min<int64_t>(count, 4096) : count;  // (both are linear beyond)
+  for (int64_t i = 0, w; i < draws; i += w) {
+    w = adaptive ? window(i, first, 4096, draws - i) : draws;
+    const int64_t s = ctas(w, &small), all = w + beside;
+    const double rounds = 0.5 * std::max(1.0, (double)all / (double)s) + 0.5 * (double)((all + s - 1) / s);
+    solo += lat[small] * rounds * ((double)w / (double)all);
+  }
+  // a window's batches overlap but for the first
+  auto lanes = [&](int64_t w) {
+    const double share = std::min(1.0, (double)w / 64.0);
+    return (level * (0.8 + 0.2 * share) + rows * (0.5 + 0.5 * share)) * (double)((w + 63) / 64 + 1) / 2.0;
+  };
+  if (adaptive) {
+    for (int64_t i = 0, w; i < draws; i += w) {
+      w = window(i, 64, 1024, draws - i);
+      lane += lanes(w);
+    }
+  } else {
+    lane += (double)(draws / 1024) * lanes(1024) + (draws % 1024 ? lanes(draws % 1024) : 0.0);
+  }
+  return 0.87 * solo <= lane;
+}
+
 // A deep graph's levels keep few of an SM's threads busy, so what counts is how
 // many sources an SM has at once: where four CTAs' counts don't fit its shared
 // memory (n > 4,700) they go to L2 (tier 1), unless there is no more than one
@@ -713,10 +767,14 @@ void do_uniform_multi(bc_ctx *ctx, const std::vector<bc_graph> &handles, const s
   std::vector<int64_t> off(G + 1, 0);
   for (int g = 0; g < G; ++g) off[g + 1] = off[g] + gs[g]->n;
   std::vector<int> deep, shallow;
-  // deep graphs and ones whose state fits shared memory go to the persistent
-  // kernels; weighted graphs run per graph (the weighted engine)
+  // deep graphs and ones whose state fits shared memory (where their share of the
+  // launch pays) go to the persistent kernels; weighted graphs run per graph (the
+  // weighted engine)
+  int64_t fitting = 0;
   for (int g = 0; g < G; ++g)
-    (one_source_per_cta(ctx, *gs[g]) && !gs[g]->w ? deep : shallow).push_back(g);
+    if (solo_fits(ctx, *gs[g])) fitting += k[g];
+  for (int g = 0; g < G; ++g)
+    (one_source_per_cta(ctx, *gs[g], k[g], false, fitting - k[g]) && !gs[g]->w ? deep : shallow).push_back(g);
   std::lock_guard<std::mutex> lk(g_plans_mu);
   MultiPlan &P = g_plans[ctx];
   cudaEvent_t done = nullptr;

@@ -133,3 +133,73 @@ def test_many_deep_graphs_of_every_residency():
             assert np.array_equal(e, ctx.uniform_sources(h, 3, 7, q))
             if g.n < 6000:
                 assert np.array_equal(e, oracle.uniform_sources(g, 3, 7, q))
+
+
+def _every_call(ctx, h, n):
+    """One call of each kind with few draws, and the sampling calls with many."""
+    t, out = [1, n // 3, n - 2], []
+    for k in (3, 64, 200, 700):
+        out.append(ctx.uniform_sources(h, k, 3, 4))
+        r = ctx.adaptive_sources(h, t, 2.0, k, 5, 6)
+        out += [r["S"], r["k"]]
+    out += list(ctx.source_dependencies(h, [0, n // 2, n - 1], want_dist=True, want_sigma=True))
+    r = ctx.adaptive_pairs(h, t, 1.0, 90, 2, 3)
+    out += [r["S"], r["k"], ctx.target_dependencies(h, t, 5, 6, 10, 70)]
+    q = ctx.submit(h, 1, targets=t, c=2.0, cap=150, seed=8, qid=9)  # BC_QUERY_SOURCES
+    ctx.poll(q, -1)
+    out += [q.outputs()["S"], q.outputs()["k"]]
+    return out + list(ctx.uniform_sources_multi([h, h], [5, 90], [1, 2], [3, 4]))
+
+
+@pytest.mark.parametrize("name", ["hubs", "dense", "sparse", "tier 1"])
+def test_both_engines_and_the_choice_by_count_agree(name):
+    g = {"hubs": lambda: gg.rmat(13, 16, 0.57, 0.19, 0.19, 3), "dense": lambda: gg.erdos_renyi(1500, 200, 5),
+         "sparse": lambda: gg.erdos_renyi(6000, 3, 4), "tier 1": lambda: gg.erdos_renyi(30_000, 8, 6, pairwise=False)}[name]()
+    got = []
+    for solo_n in (None, 0, 65536):  # by the number of sources, never, always
+        with _ctx(solo_n) as ctx:
+            got.append(_every_call(ctx, ctx.load_graph(g.row_ptr, g.col), g.n))
+    for a, b, c in zip(*got):
+        assert np.array_equal(a, b) and np.array_equal(a, c)
+    assert np.array_equal(got[0][0], oracle.uniform_sources(g, 3, 3, 4))
+
+
+@pytest.mark.parametrize("name", list(SMALL))
+def test_small_graphs_equal_the_oracle_whatever_the_count(name):
+    """As test_small_graphs_equal_the_oracle, with every call on one source per CTA."""
+    g = SMALL[name]()
+    src = sorted({0, g.n // 2, g.n - 1})
+    with _ctx(65536) as ctx:
+        h = ctx.load_graph(g.row_ptr, g.col)
+        delta, dist = ctx.source_dependencies_ext(h, src)[:2]
+        for i, s in enumerate(src):
+            d_o, dist_o = oracle.dependencies(g, s)[:2]
+            assert np.array_equal(dist[i], dist_o) and np.array_equal(delta[i], d_o)
+        assert np.array_equal(ctx.uniform_sources(h, 40, 3, 4), oracle.uniform_sources(g, 40, 3, 4))
+
+
+# (launches of the 64-lane forward pass: "fwd"; of one source per CTA: "ext_fwd")
+@pytest.mark.parametrize("graph,draws,family", [
+    ("hubs", 16, "fwd"), ("hubs", 64, "fwd"), ("hubs", 1024, "fwd"),       # 1.6 ms a source and CTA
+    ("tier 1", 16, "fwd"), ("tier 1", 64, "fwd"), ("tier 1", 1024, "ext_fwd"),
+    ("small", 1, "ext_fwd"), ("small", 64, "ext_fwd"), ("small", 1024, "ext_fwd"),
+    ("sparse", 16, "ext_fwd"), ("sparse", 1024, "ext_fwd")])               # many levels
+def test_the_engine_follows_the_number_of_sources(graph, draws, family):
+    g = {"hubs": lambda: gg.rmat(15, 16, 0.57, 0.19, 0.19, 3), "tier 1": lambda: gg.erdos_renyi(40_000, 8, 6, pairwise=False),
+         "small": lambda: gg.erdos_renyi(2000, 8, 1), "sparse": lambda: gg.erdos_renyi(60_000, 3, 4, pairwise=False)}[graph]()
+    other = {"fwd": "ext_fwd", "ext_fwd": "fwd"}[family]
+    with _ctx() as ctx:
+        h = ctx.load_graph(g.row_ptr, g.col)
+        ctx.uniform_sources(h, 65, 1, 1)  # depth and key are made
+        for call in ("uniform", "bader", "served"):
+            if call == "served" and draws != 64:
+                continue  # (64 at a time whatever the query's draws)
+            ctx.reset_stats()
+            if call == "uniform":
+                ctx.uniform_sources(h, draws, 3, 4)
+            elif call == "bader":
+                ctx.adaptive_sources(h, [1, 2], 1e9, draws, 3, 4)
+            else:
+                ctx.poll(ctx.submit(h, 3, k=64, seed=3, qid=4), -1)  # BC_QUERY_UNIFORM
+            ran = ctx.stats()["kernels"]
+            assert ran[family]["launches"] > 0 and ran[other]["launches"] == 0, call
