@@ -21,7 +21,11 @@
  *     graph lists every edge in both rows; a directed one (BC_DIRECTED) lists
  *     out-neighbours.
  *   - Errors are returned as negative bc_status codes; bc_last_error() gives a
- *     message. No C++ exception crosses this boundary. A context serialises the
+ *     message. A call refused for its arguments (BC_E_INVALID,
+ *     BC_E_UNKNOWN_HANDLE) leaves its outputs as they were; what the outputs of a
+ *     call that fails later (memory, device) hold is undefined: their pages are
+ *     touched while the device works, and finished parts may have been copied.
+ *     No C++ exception crosses this boundary. A context serialises the
  *     calls made on it (calls on one context from several threads are safe).
  *   - Random draws come from Philox4x64-10 (Salmon et al., SC'11) keyed by
  *     (seed, qid), counter (i, 0, 0, 0) for draw i = 0, 1, ...: a source is

@@ -1423,7 +1423,10 @@ static void do_adaptive_pairs(bc_ctx *ctx, const Graph &g, const int32_t *target
 // A fresh large array has no pages yet, and the copy back would fault them in
 // one by one on one thread: 70 rows of 50,001 vertices (70 MB of delta,
 // distances and counts) took 26-35 ms a call, 2.6 ms with the threads.
-// Outputs below 4 MB are left alone. The bytes written are overwritten by the copy.
+// Outputs below 4 MB are left alone. The bytes written are overwritten by the copy;
+// a call that fails leaves them changed, as bc.h says. (Ways that keep them cost the
+// time they save: a byte read and written back maps the page of zeros first, 46 ms
+// for 128 rows of 60,000 vertices against 3.8; madvise(MADV_POPULATE_WRITE) 6.2.)
 class PageTouch {
  public:
   void add(void *p, size_t bytes) {

@@ -203,3 +203,23 @@ def test_the_engine_follows_the_number_of_sources(graph, draws, family):
                 ctx.poll(ctx.submit(h, 3, k=64, seed=3, qid=4), -1)  # BC_QUERY_UNIFORM
             ran = ctx.stats()["kernels"]
             assert ran[family]["launches"] > 0 and ran[other]["launches"] == 0, call
+
+
+@pytest.mark.parametrize("lengths", [False, True])
+def test_a_refused_call_leaves_its_outputs_as_they_were(lengths):
+    """Outputs large enough to have their pages touched (4 MB)."""
+    import ctypes
+
+    from paper_1608_04472_gb300 import capi
+    g = gg.erdos_renyi(20_000, 6, 3, pairwise=False)
+    src = np.array([0] * 39 + [g.n], np.int32)
+    delta = np.full((40, g.n), -7.0)
+    dist = np.full((40, g.n), -7, np.int32)
+    with _ctx() as ctx:
+        h = ctx.load_graph(g.row_ptr, g.col, lengths=gg.edge_lengths(g, 1, 9, 2) if lengths else None)
+        rc = capi._lib.bc_source_dependencies(ctx.ptr, h, src.ctypes.data_as(ctypes.POINTER(ctypes.c_int32)), 40,
+                                              delta.ctypes.data_as(ctypes.POINTER(ctypes.c_double)),
+                                              dist.ctypes.data_as(ctypes.POINTER(ctypes.c_int32)) if not lengths else None,
+                                              None)
+    assert rc == -1  # BC_E_INVALID
+    assert (delta == -7.0).all() and (dist == -7).all()
