@@ -494,7 +494,8 @@ typedef struct bc_stats {
   int64_t samples;                 /* per-source (or per-pair) BFS lanes processed */
   int64_t batches;                 /* forward/backward launch sequences (batches) */
   int64_t dag_edges;               /* (vertex, successor, lane) triples of the shortest-path DAGs */
-  int64_t reached;                 /* (vertex, lane) pairs reached at distance >= 1 */
+  int64_t reached;                 /* (vertex, lane) pairs reached at distance >= 1 (both not counted on graphs
+                                      with edge lengths or deeper than deep_levels) */
   int32_t n_kernels;               /* entries used in the arrays below */
   int32_t pair_fallbacks;          /* pair lanes the one-pair-per-warp search (BCG_PAIR_ENGINE=2) gave up
                                       on (a ball above half its table) and handed to one pair per CTA */

@@ -44,7 +44,8 @@ __device__ __forceinline__ void prefetch_acc(const Acc *a) {
 template <int TIER, int T>
 __global__ void __launch_bounds__(T, 1024 / T)
 k_solo(MGraph G, SoloSources src, int count, unsigned *__restrict__ next, unsigned char *__restrict__ scratch,
-       size_t stride, Acc *__restrict__ partials, Sink sink, SoloRows rows, unsigned *__restrict__ err) {
+       size_t stride, Acc *__restrict__ partials, Sink sink, SoloRows rows, unsigned *__restrict__ err,
+       unsigned long long *__restrict__ cnt) {
   __shared__ SoloCtl c;
   const SoloMem<TIER> S =
       solo_mem<TIER>(reinterpret_cast<unsigned char *>(solo_shared), scratch + (size_t)blockIdx.x * stride, G.n, G.nnz);
@@ -104,13 +105,15 @@ k_solo(MGraph G, SoloSources src, int count, unsigned *__restrict__ next, unsign
     __syncthreads();
   }
   if (e) atomicOr(err, e);
+  solo_stats(c, cnt);
 }
 
 // Items of many graphs (all within the launch's nmax).
 template <int TIER, int T>
 __global__ void __launch_bounds__(T, 1024 / T)
 k_multi(const MGraph *__restrict__ graphs, const MItem *__restrict__ items, int nitems, unsigned *__restrict__ next,
-        unsigned char *__restrict__ scratch, size_t stride, Acc *__restrict__ partials, unsigned *__restrict__ err) {
+        unsigned char *__restrict__ scratch, size_t stride, Acc *__restrict__ partials, unsigned *__restrict__ err,
+        unsigned long long *__restrict__ cnt) {
   __shared__ SoloCtl c;
   unsigned e = 0u;
   solo_init(c);
@@ -139,6 +142,7 @@ k_multi(const MGraph *__restrict__ graphs, const MItem *__restrict__ items, int 
     __syncthreads();  // c.item is rewritten only after every thread has used it
   }
   if (e) atomicOr(err, e);
+  solo_stats(c, cnt);
 }
 
 // Pair sampling on a deep graph. Targets: the full BFS of each target into the
@@ -151,7 +155,7 @@ __global__ void __launch_bounds__(T, 1024 / T)
 k_solo_targets(MGraph G, const int32_t *__restrict__ targets, int count, int Tp, unsigned *__restrict__ next,
                unsigned char *__restrict__ scratch, size_t stride, int32_t *__restrict__ tdist,
                uint64_t *__restrict__ tsig, int32_t *__restrict__ texp, int32_t *__restrict__ tx,
-               int32_t *__restrict__ depth) {
+               int32_t *__restrict__ depth, unsigned long long *__restrict__ cnt) {
   __shared__ SoloCtl c;
   const SoloMem<TIER> S =
       solo_mem<TIER>(reinterpret_cast<unsigned char *>(solo_shared), scratch + (size_t)blockIdx.x * stride, G.n, G.nnz);
@@ -185,6 +189,7 @@ k_solo_targets(MGraph G, const int32_t *__restrict__ targets, int count, int Tp,
     if (threadIdx.x == 0) tx[j] = ext ? 1 : 0;
     __syncthreads();
   }
+  if (cnt) solo_stats(c, cnt);
 }
 
 template <int TIER, int T>
@@ -192,7 +197,7 @@ __global__ void __launch_bounds__(T, 1024 / T)
 k_solo_pairs(MGraph G, const int32_t *__restrict__ sources, const int32_t *__restrict__ dests, int count,
              unsigned *__restrict__ next, unsigned char *__restrict__ scratch, size_t stride,
              int32_t *__restrict__ pair_d, uint64_t *__restrict__ pair_sig, int32_t *__restrict__ pair_exp,
-             unsigned long long *__restrict__ pxmask) {
+             unsigned long long *__restrict__ pxmask, unsigned long long *__restrict__ cnt) {
   __shared__ SoloCtl c;
   const SoloMem<TIER> S =
       solo_mem<TIER>(reinterpret_cast<unsigned char *>(solo_shared), scratch + (size_t)blockIdx.x * stride, G.n, G.nnz);
@@ -216,6 +221,7 @@ k_solo_pairs(MGraph G, const int32_t *__restrict__ sources, const int32_t *__res
     }
     __syncthreads();
   }
+  solo_stats(c, cnt);
 }
 
 // acc[v] += the CTAs' partial sums (exact): a block takes 32 vertices, its 32
@@ -420,7 +426,13 @@ static MGraph mgraph_of(const Graph &g) {
   G.rp_in = g.rp_in;
   G.col_in = g.col_in;
   G.n = g.n;
+  G.long_rows = g.max_deg > 32;
   G.nnz = g.nnz;
+  return G;
+}
+static MGraph mgraph_of(bc_ctx *ctx, const Graph &g) {  // with run statistics
+  MGraph G = mgraph_of(g);
+  G.stats = graph_depth_hint(ctx, g) <= ctx->deep_levels;
   return G;
 }
 
@@ -492,7 +504,8 @@ static void enqueue_multi(bc_ctx *ctx, MultiPlan &P) {
     solo_form(m.cfg, [&](auto f) {
       k_multi<decltype(f)::tier, decltype(f)::threads><<<m.cfg.ncta, m.cfg.threads, m.cfg.smem, gs>>>(
           P.d_graphs.as<MGraph>(), P.d_items.as<MItem>() + m.item0, m.nitems, P.d_next.as<unsigned>() + 4 * i,
-          P.scratch.as<unsigned char>() + m.scratch, m.cfg.stride, P.partials.as<Acc>(), ctx->ws.err.as<unsigned>());
+          P.scratch.as<unsigned char>() + m.scratch, m.cfg.stride, P.partials.as<Acc>(), ctx->ws.err.as<unsigned>(),
+          ctx->ws.cnt.as<unsigned long long>());
       return 0;
     });
     if (i > 0) {
@@ -585,7 +598,7 @@ static void build_plan(bc_ctx *ctx, MultiPlan &P, const std::vector<const Graph 
   std::vector<int64_t> estoff(G);
   int64_t off = 0;
   for (int g = 0; g < G; ++g) {
-    mg[g] = mgraph_of(*gs[g]);
+    mg[g] = mgraph_of(ctx, *gs[g]);
     mg[g].k = P.k[g];
     mg[g].seed = P.seed[g];
     mg[g].qid = P.qid[g];
@@ -679,10 +692,10 @@ void solo_sources(bc_ctx *ctx, const Graph &g, const SoloSources &src, int count
     L.scratch.ensure(c.stride * c.ncta);
     if (sink.acc) L.partials.ensure(sizeof(Acc) * (size_t)g.n * c.ncta);
     LaunchScope ls(ctx, F_XFWD);
-    kern<<<c.ncta, c.threads, c.smem, st>>>(mgraph_of(g), src, count, L.next.as<unsigned>(),
+    kern<<<c.ncta, c.threads, c.smem, st>>>(mgraph_of(ctx, g), src, count, L.next.as<unsigned>(),
                                             L.scratch.as<unsigned char>(), c.stride,
                                             sink.acc ? L.partials.as<Acc>() : nullptr, sink, rows,
-                                            ctx->ws.err.as<unsigned>());
+                                            ctx->ws.err.as<unsigned>(), ctx->ws.cnt.as<unsigned long long>());
     return 0;
   });
   if (sink.acc) {
@@ -711,7 +724,7 @@ int solo_depth(bc_ctx *ctx, const Graph &g, int32_t v) {
     L.scratch.ensure(c.stride * c.ncta);
     LaunchScope ls(ctx, F_MISC);
     kern<<<1, c.threads, c.smem, st>>>(mgraph_of(g), word, 1, 1, L.next.as<unsigned>(), L.scratch.as<unsigned char>(),
-                                       c.stride, nullptr, nullptr, nullptr, nullptr, word + 1);
+                                       c.stride, nullptr, nullptr, nullptr, nullptr, word + 1, nullptr);
     return 0;
   });
   int32_t *h = static_cast<int32_t *>(ctx->ws.pinned);
@@ -730,8 +743,9 @@ void lane_targets(bc_ctx *ctx, const Graph &g, const int32_t *d_targets, int T, 
     solo_ctas(c, kern, T, c.stride, 0);
     L.scratch.ensure(c.stride * c.ncta);
     LaunchScope ls(ctx, F_XFWD);
-    kern<<<c.ncta, c.threads, c.smem, ctx->stream>>>(mgraph_of(g), d_targets, T, Tp, L.next.as<unsigned>(),
-                                                     L.scratch.as<unsigned char>(), c.stride, tdist, tsig, texp, d_tx, nullptr);
+    kern<<<c.ncta, c.threads, c.smem, ctx->stream>>>(mgraph_of(ctx, g), d_targets, T, Tp, L.next.as<unsigned>(),
+                                                     L.scratch.as<unsigned char>(), c.stride, tdist, tsig, texp, d_tx, nullptr,
+                                                     ctx->ws.cnt.as<unsigned long long>());
     return 0;
   });
 }
@@ -747,10 +761,11 @@ uint64_t lane_pairs(bc_ctx *ctx, const Graph &g, int count) {
     solo_ctas(c, kern, count, c.stride, 0);
     L.scratch.ensure(c.stride * c.ncta);
     LaunchScope ls(ctx, F_PAIR);
-    kern<<<c.ncta, c.threads, c.smem, st>>>(mgraph_of(g), ws.sources.as<int32_t>(), ws.targets.as<int32_t>(), count,
+    kern<<<c.ncta, c.threads, c.smem, st>>>(mgraph_of(ctx, g), ws.sources.as<int32_t>(), ws.targets.as<int32_t>(), count,
                                             L.next.as<unsigned>(), L.scratch.as<unsigned char>(), c.stride,
                                             ws.pair_d.as<int32_t>(), ws.pair_sig.as<uint64_t>(),
-                                            ws.pair_exp.as<int32_t>(), L.next.as<unsigned long long>() + 1);
+                                            ws.pair_exp.as<int32_t>(), L.next.as<unsigned long long>() + 1,
+                                            ws.cnt.as<unsigned long long>());
     return 0;
   });
   uint64_t *h = static_cast<uint64_t *>(ws.pinned);

@@ -39,7 +39,8 @@ struct MGraph {
   const int32_t *rp_in;  // in-neighbours (the same arrays for an undirected graph): counts in
   const int32_t *col_in; // the extended form are summed over them in CSR order
   int32_t n;
-  int32_t pad;
+  uint8_t long_rows;     // a row has more than 32 entries
+  uint8_t stats;         // count run statistics (not on deep graphs: 3 % of a 200x200 grid's calls)
   int64_t nnz;
   int64_t k;
   uint64_t seed, qid;
@@ -63,6 +64,10 @@ struct SoloCtl {
   int near[SOLO_NEAR];
   unsigned long long red[32][3];
   uint8_t own[32][32];          // per warp: the threads that hold non-empty short rows
+  // run statistics: shortest-path edges of the last source and of the ones
+  // before, vertices at distance >= 1
+  unsigned last_edges;
+  unsigned long long edges, reached;
 };
 
 // The state of one source. Distances are codes: the level (tier 2), or the
@@ -187,6 +192,17 @@ template <int TIER> __device__ __forceinline__ int32_t solo_entry(const SoloMem<
 __device__ __forceinline__ void solo_init(SoloCtl &c) {
   if (threadIdx.x < 3) c.nhuge[threadIdx.x] = c.found[threadIdx.x] = c.over[threadIdx.x] = 0;
   if (threadIdx.x < 2) c.grab[threadIdx.x] = 0;
+  if (threadIdx.x == 0) {
+    c.edges = c.reached = 0ull;
+    c.last_edges = 0u;
+  }
+}
+// Adds the CTA's run statistics to the library's, after its last source.
+__device__ __forceinline__ void solo_stats(const SoloCtl &c, unsigned long long *__restrict__ cnt) {
+  if (threadIdx.x == 0 && c.reached) {
+    atomicAdd(cnt, c.edges + c.last_edges);
+    atomicAdd(cnt + 1, c.reached);
+  }
 }
 
 // A pass over list positions [b, e) in runs of 32 from a shared counter (uneven
@@ -767,6 +783,25 @@ __device__ __forceinline__ void solo_xf_back(const MGraph &G, const SoloMem<TIER
   solo_ahead_row(G, p, b - nb <= T, hint);
 }
 
+// The shortest-path edges of queue entries [0, e), from their bits. (A pass of its
+// own: counted where the bits are made, the counter's register cost the passes
+// 3-6 % on ER n = 2000.)
+template <class Q, int T>
+__device__ __forceinline__ void solo_count_edges(const int32_t *rp, const Q *queue, const uint32_t *qmask,
+                                              const uint32_t *lmask, int e, bool long_rows, unsigned *total) {
+  unsigned edges = 0u;
+#pragma unroll 4
+  for (int i = (int)threadIdx.x; i < e; i += T) edges += (unsigned)__popc(qmask[i]);
+  if (long_rows)
+    for (int i = (int)threadIdx.x; i < e; i += T) {
+      const int hb = rp[queue[i]], d = rp[queue[i] + 1] - hb;
+      if (d > 32)
+        for (int q = 0; 32 * q < d; ++q) edges += (unsigned)__popc(lmask[(hb >> 4) + q]);
+    }
+  edges = __reduce_add_sync(FULL, edges);
+  if ((threadIdx.x & 31) == 0 && edges) atomicAdd(total, edges);
+}
+
 // Forward pass of source s: distance codes, counts, level offsets and edge
 // bits; with dest >= 0 it stops once dest's level is settled. Returns the
 // deepest level; *ext: the counts are in the extended form (a count of the
@@ -802,12 +837,15 @@ __device__ int solo_forward(const MGraph &G, int32_t s, int32_t dest, const Solo
     c.near[1] = 1;
     c.l53 = 0x7FFFFFFF;
     c.maxc = 1ull;
+    c.edges += c.last_edges;
+    c.last_edges = 0u;
   }
   __syncthreads();
   int L = 0, b = 0, e = 1;
   bool xf = false;
   const bool fused = G.rp_in == G.rp;  // (extended form) level L's counts come with the push from it
   uint64_t mymax = 1ull;
+  bool pushed = true;  // the last level's edges have been looked at
   for (;;) {
     const int slot = ph % 3;
     if (xf && fused) {
@@ -853,6 +891,7 @@ __device__ int solo_forward(const MGraph &G, int32_t s, int32_t dest, const Solo
     }
     if (dest >= 0 && __syncthreads_or(S.dist[dest] != solo_unset<TIER>())) {  // dest settled at level L
       if (xf && fused) solo_xf_level<TIER, T>(G, S, L, b, e);
+      pushed = false;
       break;
     }
   }
@@ -862,6 +901,11 @@ __device__ int solo_forward(const MGraph &G, int32_t s, int32_t dest, const Solo
       mymax = o > mymax ? o : mymax;
     }
     if ((tid & 31) == 0 && mymax > 1ull) atomicMax(&c.maxc, (unsigned long long)mymax);
+  }
+  if (G.stats) {
+    solo_count_edges<typename SoloMem<TIER>::Q, T>(G.rp, S.queue, S.qmask, S.lmask, pushed ? e : b, G.long_rows != 0,
+                                                   &c.last_edges);
+    if (tid == 0) c.reached += (unsigned long long)(e - 1);
   }
   __syncthreads();
   *ext = xf;

@@ -223,3 +223,22 @@ def test_a_refused_call_leaves_its_outputs_as_they_were(lengths):
                                               None)
     assert rc == -1  # BC_E_INVALID
     assert (delta == -7.0).all() and (dist == -7).all()
+
+
+@pytest.mark.parametrize("name", ["rows of 34", "star, row above 2048", "70 rows of 2100", "layers beyond 2^64",
+                                  "hubs and isolated vertices"])
+@pytest.mark.parametrize("solo_n", [65536, 0])
+def test_run_statistics_count_edges_and_vertices_of_the_searches(name, solo_n):
+    """bc_get_stats: shortest-path edges and reached vertices, as the distances give
+    them, whichever engine ran the sources."""
+    g = _layers(60, 13) if name == "layers beyond 2^64" else SMALL[name]()
+    src = sorted({0, g.n // 2, g.n - 1})
+    row = np.repeat(np.arange(g.n), np.diff(g.row_ptr))
+    with _ctx(solo_n) as ctx:
+        h = ctx.load_graph(g.row_ptr, g.col)
+        ctx.source_dependencies(h, src)  # the depth is known from here on
+        ctx.reset_stats()
+        dist = ctx.source_dependencies(h, src, want_dist=True)[1]
+        st = ctx.stats()
+    assert st["reached"] == sum(int((d > 0).sum()) for d in dist)
+    assert st["dag_edges"] == sum(int(((d[row] >= 0) & (d[g.col] == d[row] + 1)).sum()) for d in dist)
