@@ -710,7 +710,7 @@ static std::vector<double> leading_component(int K, const std::vector<unsigned l
 static void build_depth(bc_ctx *ctx, const Graph &g, KeyMeta &km) {
   cudaStream_t st = ctx->stream;
   const size_t n = (size_t)g.n;
-  DevBuf dist;
+  LocalBuf dist;
   try {
     // dist, then the hub and its eccentricity
     dist.ensure((n + 2) * 4);
@@ -741,13 +741,13 @@ static void build_key(bc_ctx *ctx, const Graph &g, KeyMeta &km, int K) {
   const size_t n = (size_t)g.n;
   const unsigned nb = (unsigned)((n + 255) / 256);
   const int64_t s0 = ctx->samples, b0 = ctx->batches;
-  DevBuf rows, proj, small;
+  LocalBuf rows, proj, small;
   auto release_all = [&] {
     for (DevBuf *b : {&rows, &proj, &small}) b->release();
   };
   try {
     if (!km.hub.p) build_depth(ctx, g, km);
-    std::swap(rows, km.hub);  // row 0
+    std::swap(static_cast<DevBuf &>(rows), km.hub);  // row 0
     // small: [16] lanes that reach the hub (u64), [32] range, [64] w|mu,
     // [320] row of each lane, [384] the caller's sources (64), [1024] moments
     small.ensure(1024 + 8 * KEY_MOM_THREADS);
@@ -841,7 +841,7 @@ static void build_key(bc_ctx *ctx, const Graph &g, KeyMeta &km, int K) {
   }
   ctx->samples = s0;
   ctx->batches = b0;
-  if (K == 1) std::swap(rows, km.hub);  // (a later call may want the landmarks)
+  if (K == 1) std::swap(static_cast<DevBuf &>(rows), km.hub);  // (a later call may want the landmarks)
   km.K = K;
   release_all();
 }
@@ -1176,7 +1176,7 @@ void target_bfs(bc_ctx *ctx, const Graph &g, const int32_t *d_targets, int T, in
   if (T > 0 && lane_major(ctx, g, T)) {
     // one BFS per CTA and target
     if (!texp.p) texp.ensure(n * (size_t)Tp * 4);
-    DevBuf dtx;
+    LocalBuf dtx;
     dtx.ensure((size_t)Tp * 4);
     try {
       lane_targets(ctx, g, d_targets, T, Tp, tdist, tsig, texp.as<int32_t>(), dtx.as<int32_t>());
@@ -1319,7 +1319,7 @@ static void do_pair_block(bc_ctx *ctx, bc_graph gh, const Graph &g, const int32_
   }
   Workspace &ws = ctx->ws;
   ws.tdelta.ensure((size_t)Tp * pwmax * 8);
-  DevBuf wsrc, wdst, wpd, wpsig, wpexp, wpxf;
+  LocalBuf wsrc, wdst, wpd, wpsig, wpexp, wpxf;
   for (DevBuf *b : {&wsrc, &wdst, &wpd, &wpexp, &wpxf}) b->ensure(pwmax * 4);
   wpsig.ensure(pwmax * 8);
   std::vector<double> h((size_t)T * pwmax);
@@ -1357,7 +1357,7 @@ static void do_adaptive_pairs(bc_ctx *ctx, const Graph &g, const int32_t *target
   const int Tp = std::max(T, 1);
   const int pwmax = pair_window_max(T);
   // Per-target BFS (distance and sigma from every target), layout [n][Tp].
-  DevBuf tdist, tsig, texp, dtx, wsrc, wdst, wpd, wpsig, wpexp, wpxf;
+  LocalBuf tdist, tsig, texp, dtx, wsrc, wdst, wpd, wpsig, wpexp, wpxf;
   tdist.ensure(n * Tp * 4);
   tsig.ensure(n * Tp * 8);
   ws.misc.ensure((size_t)Tp * 4 + 64);
@@ -1475,7 +1475,7 @@ static void do_source_rows_weighted(bc_ctx *ctx, const Graph &g, const int32_t *
   for (int32_t i = 0; i < count; ++i)
     if (sources[i] < 0 || sources[i] >= g.n) fail(BC_E_INVALID, "source out of range");
   const int chunk = std::min<int>(64, std::max(1, count));
-  DevBuf dd, ddist, dsig, dsm, dse, dtier;
+  LocalBuf dd, ddist, dsig, dsm, dse, dtier;
   PageTouch pages;
   pages.add(delta_out, n * count * 8);
   pages.add(dist_out, n * count * 8);
@@ -1590,7 +1590,7 @@ static void do_source_dependencies(bc_ctx *ctx, const Graph &g, const int32_t *s
   for (int32_t i = 0; i < count; ++i)
     if (sources[i] < 0 || sources[i] >= g.n) fail(BC_E_INVALID, "source out of range");
   ws.delta_lm.ensure(n * 64 * 8);
-  DevBuf dd, ddist, dsig, dsm, dse;
+  LocalBuf dd, ddist, dsig, dsm, dse;
   const int width = batch_width(ctx);
   const int chunk = std::min<int>(64, std::max(1, count));
   const bool want_xf = sm_out || se_out;
@@ -1671,15 +1671,18 @@ using namespace bcg;
 
 // ----------------------------------------------------------------- the ABI ---
 
+// A call that runs out of device memory gives back what the context holds for
+// speed and what later calls can make again, and starts over, once.
 #define BC_GUARD_BEGIN                               \
   if (!ctx) return BC_E_INVALID;                     \
   bcg::ApiLock lk(ctx);                              \
-  try {
+  for (bool again = false;; again = true) try {
 #define BC_GUARD_END                                                   \
   ctx->err = "no error";                                               \
   return BC_OK;                                                        \
   }                                                                    \
   catch (const Error &e) {                                             \
+    if (e.code == BC_E_NOMEM && !again && bcg::give_back(ctx)) continue; \
     ctx->err = e.msg;                                                  \
     return e.code;                                                     \
   }                                                                    \
@@ -1693,6 +1696,32 @@ using namespace bcg;
   }
 
 namespace bcg {
+
+bool give_back(bc_ctx *ctx) {
+  size_t before = 0, after = 0, tot = 0;
+  cudaGetLastError();
+  for (cudaStream_t st : {ctx->stream, ctx->side, ctx->stream2, ctx->slot2.stream, ctx->slot2.side})
+    if (st) cudaStreamSynchronize(st);
+  if (cudaMemGetInfo(&before, &tot) != cudaSuccess) return false;
+  Workspace &ws = ctx->ws;
+  for (BatchState *b : {static_cast<BatchState *>(&ws), &ctx->slot2.state}) {
+    // (a batch's draws may be in place already: sources and the lane words stay)
+    b->each([&](DevBuf &x) {
+      if (&x != &b->sources && &x != &b->enable) x.release();
+    });
+    b->lcap = 0;
+  }
+  for (DevBuf *b : {&ws.acc, &ws.tslot, &ws.tdelta, &ws.scan, &ws.misc, &ws.misc2, &ws.delta_lm, &ws.win, &ws.rows,
+                    &ws.x_dist, &ws.x_m, &ws.x_e, &ws.x_vis, &ws.x_nm, &ws.x_list, &ws.x_lmask, &ws.x_ctr, &ws.x_off,
+                    &ws.p_dist, &ws.p_sigma, &ws.p_coef, &ws.p_queue, &ws.p_ctr, &ctx->slot2.acc})
+    b->release();
+  forget_multi_plan(ctx);
+  forget_lane_scratch(ctx);
+  forget_bidir_scratch(ctx);
+  forget_weighted_scratch(ctx);
+  forget_pair_tables(ctx, 0);
+  return cudaMemGetInfo(&after, &tot) == cudaSuccess && after > before;
+}
 
 // BC_NORMALIZE: rows sorted, self-loops and duplicate columns dropped (a
 // duplicate edge with lengths keeps the shortest one); the result is written
@@ -2188,7 +2217,7 @@ bc_status bc_draw_sources(bc_ctx *ctx, uint64_t seed, uint64_t qid, uint64_t i0,
   BC_GUARD_BEGIN
   if (n < 1 || count < 0 || count > (1 << 28) || (count > 0 && !out)) fail(BC_E_INVALID, "bad argument");
   if (count == 0) { ctx->err = "no error"; return BC_OK; }
-  DevBuf b;
+  LocalBuf b;
   b.ensure((size_t)count * 4);
   try {
     launch_draw_sources(ctx, seed, qid, i0, (int)count, n, b.as<int32_t>());
@@ -2207,7 +2236,7 @@ bc_status bc_draw_pairs(bc_ctx *ctx, uint64_t seed, uint64_t qid, uint64_t i0, i
   BC_GUARD_BEGIN
   if (n < 2 || count < 0 || count > (1 << 28) || (count > 0 && (!s_out || !t_out))) fail(BC_E_INVALID, "bad argument");
   if (count == 0) { ctx->err = "no error"; return BC_OK; }
-  DevBuf b;
+  LocalBuf b;
   b.ensure((size_t)count * 8);
   try {
     {
@@ -2229,7 +2258,7 @@ bc_status bc_draw_pairs(bc_ctx *ctx, uint64_t seed, uint64_t qid, uint64_t i0, i
 bc_status bc_exact_sum(bc_ctx *ctx, const double *x, int64_t count, double *out) {
   BC_GUARD_BEGIN
   if (count < 0 || !out || (count > 0 && !x)) fail(BC_E_INVALID, "bad argument");
-  DevBuf b;
+  LocalBuf b;
   b.ensure((size_t)std::max<int64_t>(count, 1) * 8 + 16);
   try {
     if (count) BCG_CUDA(cudaMemcpyAsync(b.p, x, (size_t)count * 8, cudaMemcpyHostToDevice, ctx->stream));

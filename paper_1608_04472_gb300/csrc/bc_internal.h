@@ -41,6 +41,14 @@ struct DevBuf {
   template <class T> T *as() const { return static_cast<T *>(p); }
 };
 
+// One that lives as long as its scope, also when a call fails half way.
+struct LocalBuf : DevBuf {
+  LocalBuf() = default;
+  LocalBuf(const LocalBuf &) = delete;
+  LocalBuf &operator=(const LocalBuf &) = delete;
+  ~LocalBuf() { release(); }
+};
+
 struct Graph {
   int32_t n = 0;
   int64_t nnz = 0;
@@ -265,6 +273,10 @@ struct LaunchScope {
 };
 void resolve_events(bc_ctx *ctx);  // after a stream sync
 
+// Frees what the context holds that any call makes again when it needs it (both
+// batches' state, scratch, kept tables and plans), for a call that found no memory.
+// Returns whether that made room. Only between calls or batches.
+bool give_back(bc_ctx *ctx);
 const Graph &get_graph(bc_ctx *ctx, bc_graph g);
 void sync(bc_ctx *ctx);
 unsigned read_and_clear_err(bc_ctx *ctx);

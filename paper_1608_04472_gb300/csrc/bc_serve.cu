@@ -221,6 +221,17 @@ struct Server {
   void yield_to_api();
   bool prepare(SQuery &q);                    // device state; pairs: per-target BFS
   void run_group(std::vector<std::shared_ptr<SQuery>> &part, std::vector<int> &lanes);
+  // A step that can be done over: once more after the context gave memory back.
+  // (A uniform query's batches add to its sums and are not.)
+  template <class F> void with_room(F step) {
+    try {
+      step();
+      return;
+    } catch (const Error &e) {
+      if (e.code != BC_E_NOMEM || !give_back(ctx)) throw;
+    }
+    step();
+  }
   void finish(SQuery &q);
   void fail_query(SQuery &q, bc_status code, const std::string &msg);
 };
@@ -408,10 +419,11 @@ void Server::run_group(std::vector<std::shared_ptr<SQuery>> &part, std::vector<i
       sink.eq = d_eq.as<int32_t>();
       sink.lane_q = d_laneq.as<int32_t>();
       sink.tdelta = d_tdelta.as<double>();
-      run_source_batch(ctx, g, L, sink);
+      with_room([&] { run_source_batch(ctx, g, L, sink); });
     } else {
       // (the plain pair path handles one lane; batches are of one in that mode)
-      const uint64_t px = pair_batch(ctx, g, L);
+      uint64_t px = 0;
+      with_room([&] { px = pair_batch(ctx, g, L); });
       d_pair.ensure((size_t)std::max(E, 1) * sizeof(PairEntry));
       BCG_CUDA(cudaMemcpyAsync(d_pair.p, pe.data(), (size_t)E * sizeof(PairEntry), cudaMemcpyHostToDevice, st));
       LaunchScope ls(ctx, F_PAIR);
@@ -468,7 +480,7 @@ void Server::loop() {
       yield_to_api();
       std::lock_guard<std::recursive_mutex> g(ctx->mu);
       try {
-        prepare(*q);
+        with_room([&] { prepare(*q); });
         q->prepared = true;
       } catch (const Error &e) {
         std::lock_guard<std::mutex> lk(mu);

@@ -267,3 +267,40 @@ def test_a_call_that_ran_out_of_memory_leaves_nothing_half_built(monkeypatch):
             torch.cuda.empty_cache()
         assert np.array_equal(c.uniform_sources(h, 150, 2, 2), want)
     assert failed
+
+
+@pytest.mark.parametrize("call", ["pairs", "served pairs", "load", "rows"])
+def test_memory_held_for_speed_is_given_back(monkeypatch, call):
+    """A context that holds two batches' state (about 1.2 KB a vertex each) and, beside
+    it, 24 MB of the device's memory: calls that need 100 to 300 MB."""
+    import torch
+    import paper_1608_04472_gb300 as pkg
+    monkeypatch.setenv("BCG_SOLO_N", "0")
+    g, big = gg.erdos_renyi(200_000, 6, 5, pairwise=False), gg.erdos_renyi(1_000_000, 24, 6, pairwise=False)
+    targets, src = np.arange(0, 200_000, 4000, dtype=np.int32), np.arange(64, dtype=np.int32)
+
+    def run(c, h):
+        if call == "pairs":
+            return c.adaptive_pairs(h, targets, 1.0, 40, 2, 3)["S"]
+        if call == "served pairs":
+            t = c.submit(h, pkg.BC_QUERY_PAIRS, targets=targets, c=1.0, cap=40, seed=2, qid=3)
+            c.poll(t, -1)
+            return t.outputs()["S"]
+        if call == "load":
+            c.free_graph(c.load_graph(big.row_ptr, big.col))
+            return np.zeros(1)
+        return c.source_dependencies(h, src)[0]
+
+    with pkg.Context(0, batch_width=64) as c:  # (every kernel loaded, before memory runs short)
+        h = c.load_graph(g.row_ptr, g.col)
+        want, sums = run(c, h), c.uniform_sources(h, 200, 4, 4)
+    with pkg.Context(0, batch_width=64) as c:
+        h = c.load_graph(g.row_ptr, g.col)
+        assert np.array_equal(c.uniform_sources(h, 200, 4, 4), sums)
+        rest = _fill(torch, 24 << 20)
+        try:
+            assert np.array_equal(run(c, h), want)
+        finally:
+            rest.clear()
+            torch.cuda.empty_cache()
+        assert np.array_equal(c.uniform_sources(h, 200, 4, 4), sums)
