@@ -408,14 +408,17 @@ bc_status bc_scan_block(int32_t T, const double *block, int32_t W, int64_t i0, d
  * or coefficients an exact sum rounded once, so only the speed differs.
  */
 typedef struct bc_tuning {
-  int32_t batch_width;        /* 64: 64 sources share one traversal (level masks); 1: plain kernels */
-  int32_t heavy_degree;       /* vertices of larger degree are split into segments (32 ..) */
-  int32_t segment;            /* neighbours per heavy segment (32 ..) */
+  int32_t batch_width;        /* 64: the batched engines, 64 sources to a traversal (level masks) or, on
+                                 deep graphs, graphs with edge lengths and, by the call's number of sources,
+                                 on graphs whose state fits shared memory, one source per persistent CTA;
+                                 1: plain kernels */
+  int32_t heavy_degree;       /* level masks: vertices of larger degree are split into segments (32 ..) */
+  int32_t segment;            /* level masks: neighbours per heavy segment (32 ..) */
   int32_t packed_max_lanes;   /* 0 .. 64, packed_min_preds 1 .. 32, bwd_variant 0 or 1, heavy_lane 0 .. 4: */
   int32_t packed_min_preds;   /* kernel forms of earlier versions. One form is left for each kernel, the */
   int32_t bwd_variant;        /* faster on every graph tried, so these are checked and kept with the */
   int32_t heavy_lane;         /* record but choose nothing. */
-  int32_t push_div;           /* forward level top-down (push from the level's vertices, counts pulled
+  int32_t push_div;           /* level masks: forward level top-down (push from the level's vertices, counts pulled
                                  for the reached ones) when the level's degree sum is <= nnz/push_div;
                                  bottom-up otherwise; 0: always bottom-up (Sec. 3 step 1 either way) */
   int32_t deep_levels;        /* the hub's eccentricity above which the graph runs one source per
@@ -432,8 +435,9 @@ typedef struct bc_tuning {
  * that much). Every trial's estimate must equal the first
  * one bit for bit (else BC_E_DEVICE: a setting changed a result). The result
  * is kept beside the graph (every later call on g uses it, also through the
- * query server) and written to *out. 1 <= k <= 2^20. The plain width (1) is
- * tried only on graphs of at most 2^17 vertices. */
+ * query server) and written to *out. 1 <= k <= 2^20. push_div, heavy_degree and
+ * segment are tried only where k sources run on level masks. The plain width (1)
+ * is tried only on graphs of at most 2^17 vertices. */
 bc_status bc_autotune(bc_ctx *ctx, bc_graph g, int64_t k, uint64_t seed, bc_tuning *out);
 
 /* The tuning in force for graph g (the context's defaults until one is set). */

@@ -2412,11 +2412,18 @@ bc_status bc_autotune(bc_ctx *ctx, bc_graph g, int64_t k, uint64_t seed, bc_tuni
         }
       }
     };
-    // the traversal's direction and the heavy-vertex split first (largest
-    // effects on R-MAT), then the kernel forms
-    sweep(&bc_tuning::push_div, {0, 8, 32, 128});
-    sweep(&bc_tuning::heavy_degree, {32, 64, 128, 256, 512});
-    sweep(&bc_tuning::segment, {128, 256, 512});
+    // the traversal's direction and the heavy-vertex split (largest effects on
+    // R-MAT) where the trials run the engine that has them
+    bool lanes;
+    {
+      KnobScope ks(ctx, gr);
+      lanes = batch_width(ctx) != 1 && !one_source_per_cta(ctx, gr, k);
+    }
+    if (lanes) {
+      sweep(&bc_tuning::push_div, {0, 8, 32, 128});
+      sweep(&bc_tuning::heavy_degree, {32, 64, 128, 256, 512});
+      sweep(&bc_tuning::segment, {128, 256, 512});
+    }
     sweep(&bc_tuning::deep_levels, {16, 32, 64});
     if (gr.n <= (1 << 17)) sweep(&bc_tuning::batch_width, {1, 64});
     best.trial_ms = best_ms;

@@ -44,3 +44,50 @@ def test_autotune_keeps_results_and_the_choice_stays_with_the_graph(tmp_path):
         t2 = at.tune_cached(ctx2, h2, g.row_ptr, g.col, str(tmp_path / "t.json"))
         assert t2["cached"] is True
         assert all(ctx2.get_tuning(h2)[k] == t[k] for k in pkg.capi.TUNING_FIELDS)
+
+
+def _trials(ctx, h, k):
+    """Settings tried: each runs min(k, 64) + k draws (samples of the plain width count too)."""
+    ctx.reset_stats()
+    t = ctx.autotune(h, k, 3)
+    return t, ctx.stats()["samples"] // (64 + k)
+
+
+def test_only_settings_of_the_engine_that_runs_are_tried(monkeypatch):
+    """On a small graph 128 draws run one source per CTA, which has no direction
+    switch and no heavy vertices; with level masks forced they are tried."""
+    import paper_1608_04472_gb300 as pkg
+    g = gg.erdos_renyi(2000, 8, 1)
+    for solo_n, few in ((None, True), ("0", False)):
+        if solo_n is not None:
+            monkeypatch.setenv("BCG_SOLO_N", solo_n)
+        with pkg.Context(0, batch_width=64) as ctx:
+            h = ctx.load_graph(g.row_ptr, g.col)
+            before = ctx.get_tuning(h)
+            t, trials = _trials(ctx, h, 128)
+            # the setting in force, two depths and the plain width; and nine of the others
+            assert trials == (4 if few else 13)
+            if few:
+                assert all(t[x] == before[x] for x in ("push_div", "heavy_degree", "segment"))
+            assert np.array_equal(ctx.uniform_sources(h, 50, 5, 6), oracle.uniform_sources(g, 50, 5, 6))
+
+
+@pytest.mark.parametrize("odd", [dict(heavy_degree=128, segment=128), dict(heavy_degree=32, segment=32, push_div=1000),
+                                 dict(push_div=1), dict(push_div=20, heavy_degree=300)])
+def test_every_knob_of_the_level_masks_gives_the_oracle_s_results(monkeypatch, odd):
+    """Top-down levels and the heavy split on the engine that has them."""
+    import paper_1608_04472_gb300 as pkg
+    monkeypatch.setenv("BCG_SOLO_N", "0")
+    for g in (gg.rmat(12, 16, 0.57, 0.19, 0.19, 91), gg.erdos_renyi(1500, 5, 4)):
+        with pkg.Context(0, batch_width=64) as ctx:
+            h = ctx.load_graph(g.row_ptr, g.col)
+            ctx.set_tuning(h, dict(ctx.get_tuning(h), **odd))
+            for _ in range(2):  # the depth is known the second time
+                assert np.array_equal(ctx.uniform_sources(h, 150, 5, 6), oracle.uniform_sources(g, 150, 5, 6))
+            r, ref = ctx.adaptive_sources(h, [0, 1, 2], 2.0, 300, 7, 8), oracle.adaptive_sources(g, [0, 1, 2], 2.0, 300, 7, 8)
+            assert np.array_equal(r["S"], ref["S"]) and np.array_equal(r["k"], ref["k"])
+    d = gg.directed_rmat(11, 6, 0.57, 0.19, 0.19, 5)
+    with pkg.Context(0, batch_width=64) as ctx:
+        h = ctx.load_graph(d.row_ptr, d.col, directed=True)
+        ctx.set_tuning(h, dict(ctx.get_tuning(h), **odd))
+        assert np.array_equal(ctx.uniform_sources(h, 150, 5, 6), oracle.uniform_sources(d, 150, 5, 6))
