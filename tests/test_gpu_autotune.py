@@ -65,8 +65,9 @@ def test_only_settings_of_the_engine_that_runs_are_tried(monkeypatch):
             h = ctx.load_graph(g.row_ptr, g.col)
             before = ctx.get_tuning(h)
             t, trials = _trials(ctx, h, 128)
-            # the setting in force, two depths and the plain width; and nine of the others
-            assert trials == (4 if few else 13)
+            # the setting in force, two or three depths (one more where one is kept) and one
+            # or two widths; and at least nine of the others
+            assert (trials <= 6) if few else (trials >= 13)
             if few:
                 assert all(t[x] == before[x] for x in ("push_div", "heavy_degree", "segment"))
             assert np.array_equal(ctx.uniform_sources(h, 50, 5, 6), oracle.uniform_sources(g, 50, 5, 6))

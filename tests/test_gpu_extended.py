@@ -123,3 +123,33 @@ def test_pairs_on_overflowing_grid(pkg, width):
         assert np.array_equal(got2[key], ref2[key]), key
         assert np.array_equal(served[key], ref[key]), key
     assert np.sum(ref["S"] > 0) >= 2
+
+
+@pytest.mark.parametrize("side", [40, 70])
+def test_rows_and_estimates_of_overflowed_lanes_on_level_masks(pkg, monkeypatch, side):
+    """The 64-lane engine's own way to the extended form (small and deep graphs run one
+    source per CTA by rule: neither rule here): rows of batches that mix both forms,
+    and lanes recomputed behind the batch's backward pass."""
+    monkeypatch.setenv("BCG_SOLO_N", "0")
+    g = gg.grid(side)
+    c = side // 2
+    sources = [0, side - 1, g.n - 1, c * side + c, c * side, 3 * side + 7, c * side + c, 1]
+    exp = _expected(g, sources)
+    assert any(r[4] for r in exp)
+    with pkg.Context(0, batch_width=64) as ctx:
+        h = ctx.load_graph(g.row_ptr, g.col)
+        ctx.set_tuning(h, dict(ctx.get_tuning(h), deep_levels=100_000))
+        ctx.reset_stats()
+        delta, dist, sm, se, tier = ctx.source_dependencies_ext(h, sources)
+        assert ctx.stats()["kernels"]["fwd"]["launches"] > 0
+        sig = ctx.source_dependencies(h, sources, want_dist=True, want_sigma=True)[2]
+        got_u = ctx.uniform_sources(h, 150, 7, 3)
+        got_b = ctx.adaptive_sources(h, [1, c * side, g.n - 2], 2.0, 200, 9, 4)
+    for i, (ed, edist, esm, ese, eovf) in enumerate(exp):
+        assert tier[i] == eovf and np.array_equal(dist[i], edist) and np.array_equal(delta[i], ed)
+        assert np.array_equal(sm[i], esm) and np.array_equal(se[i].astype(np.int64), ese)
+        if eovf:
+            assert np.all(sig[i][edist >= 0] == np.uint64(2**64 - 1)) and np.all(sig[i][edist < 0] == 0)
+    assert np.array_equal(got_u, oracle.uniform_sources(g, 150, 7, 3))
+    ref = oracle.adaptive_sources(g, [1, c * side, g.n - 2], 2.0, 200, 9, 4)
+    assert np.array_equal(got_b["S"], ref["S"]) and np.array_equal(got_b["k"], ref["k"])

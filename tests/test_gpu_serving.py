@@ -200,3 +200,28 @@ def test_admission_by_device_memory(ctx, graphs, pkg):
         for key in ["est", "k", "S", "status"]:
             _same(tk.outputs()[key], ref[key], key)
     assert any(a1 < d0 for (a0, d0), (a1, d1) in zip(iv, iv[1:])), "with room for all, the queries should overlap"
+
+
+@pytest.mark.parametrize("solo_n", ["0", "65536"])
+def test_queries_that_share_batches_and_targets_on_either_engine(pkg, monkeypatch, solo_n):
+    """Queries with common targets share 64-source batches, on level masks and with one
+    source per CTA: each entry of a target's chain takes its own query's lanes."""
+    monkeypatch.setenv("BCG_SOLO_N", solo_n)
+    g = gg.barabasi_albert(3000, 3, 4)
+    qs = [dict(targets=[0, 1, 2, 7], c=2.0, cap=900, seed=11, qid=1), dict(targets=[2, 0, 9], c=4.0, cap=700, seed=12, qid=2),
+          dict(targets=[2], c=1e9, cap=333, seed=13, qid=3), dict(targets=[1, 2, 0], c=3.0, cap=500, seed=14, qid=4)]
+    with pkg.Context(0, batch_width=64) as c:
+        h = c.load_graph(g.row_ptr, g.col)
+        c.uniform_sources(h, 70, 1, 1)  # the depth is known
+        c.reset_stats()
+        tks = [c.submit(h, pkg.BC_QUERY_SOURCES, **kw) for kw in qs]
+        uni = c.submit(h, pkg.BC_QUERY_UNIFORM, k=100, seed=5, qid=6)
+        for tk in tks + [uni]:
+            assert c.poll(tk, -1) == pkg.BC_OK
+        ran = c.stats()["kernels"]
+    assert (ran["fwd"]["launches"] > 0) == (solo_n == "0") and (ran["ext_fwd"]["launches"] > 0) == (solo_n != "0")
+    for kw, tk in zip(qs, tks):
+        ref = oracle.adaptive_sources(g, kw["targets"], kw["c"], kw["cap"], kw["seed"], kw["qid"])
+        for key in ["est", "k", "S", "status"]:
+            _same(tk.outputs()[key], ref[key], key)
+    _same(uni.outputs()["est"], oracle.uniform_sources(g, 100, 5, 6), "uniform")
