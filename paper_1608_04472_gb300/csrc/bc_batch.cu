@@ -37,7 +37,6 @@ namespace bcg {
 
 constexpr int HEAVY_DEFAULT = 64;    // vertices above this degree are split into segments
 constexpr int SEG_DEFAULT = 256;     // neighbours per heavy segment
-constexpr int GRAB = 16;             // list positions taken per grab by default
 constexpr int UNR = 3;               // neighbours gathered per unrolled step of a top-down level's pull
 constexpr int FWD_THREADS = 256;
 // Resident blocks per SM of the backward kernels (48 registers a thread); the
@@ -76,8 +75,8 @@ __device__ __forceinline__ void block_or_to(uint64_t x, uint64_t *dst) {
 
 
 // Dynamic work distribution: a warp takes `step` consecutive items per atomic
-// (GRAB light vertices; one heavy segment or heavy vertex, whose work is large).
-__device__ __forceinline__ int grab(unsigned *wq, int step = GRAB) {
+// (several light vertices; one heavy segment or heavy vertex, whose work is large).
+__device__ __forceinline__ int grab(unsigned *wq, int step) {
   int base = 0;
   if ((threadIdx.x & 31) == 0) base = (int)atomicAdd(wq, (unsigned)step);
   return __shfl_sync(FULL, base, 0);
@@ -123,7 +122,7 @@ __global__ void k_batch_init(int count, const int32_t *__restrict__ sources,
     atomicOr((unsigned long long *)&visited[s], (unsigned long long)bit);
     sigma[(size_t)s * 64 + t] = 1ull;
     atomicOr((unsigned long long *)active0, (unsigned long long)bit);
-    if (old == 0ull && list0) {  // first lane with this source: it joins the level-0 list
+    if (old == 0ull) {  // first lane with this source: it joins the level-0 list
       list0[atomicAdd(vcnt0, 1u)] = s;
       atomicAdd(vedges0, (unsigned long long)(rp[s + 1] - rp[s]));
     }
@@ -134,7 +133,6 @@ __global__ void k_batch_init(int count, const int32_t *__restrict__ sources,
 // atomic per warp) and adds their degrees to the level's edge count.
 __device__ __forceinline__ void list_append(bool first, int32_t v, int deg, int32_t *__restrict__ list,
                                             unsigned *__restrict__ vcnt, unsigned long long *__restrict__ vedges) {
-  if (!list) return;  // level lists off (bottom-up only): nothing to record
   const int lane = threadIdx.x & 31;
   const unsigned fb = __ballot_sync(FULL, first);
   if (!fb) return;
@@ -949,7 +947,7 @@ __device__ __forceinline__ double delta_of(double sum, uint64_t sg) {
 }
 
 // One warp-wide round over `count` (<= 32) records from ring position head. The
-// coefficient's double bits overwrite sigma[v][t].
+// coefficient goes to its own 96-bit row, or in the wide form over sigma[v][t].
 template <class P>
 __device__ __forceinline__ void ring_round(Ring<P> &R, int head, int count, uint64_t *__restrict__ coef,
                                            const Sink &sink, int unit, unsigned &e) {
@@ -1296,7 +1294,7 @@ struct HeavyMeta {
     for (DevBuf *b : {&heavy, &hseg0, &seg_v, &seg_b, &seg_e, &light}) f(*b);
   }
 };
-static std::map<const int32_t *, HeavyMeta> g_heavy;  // keyed by the graph's device col pointer
+static std::map<const int32_t *, HeavyMeta> g_heavy;  // keyed by the CSR's device row pointers
 static std::mutex g_heavy_mu;
 
 // The heavy-vertex split of the CSR the forward pulls over (in_csr: the

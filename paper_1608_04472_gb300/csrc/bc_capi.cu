@@ -9,9 +9,11 @@
 //   bc_adaptive_pairs    Algorithm 1: one BFS per target, then windows of pair
 //                        draws whose d(s,t), sigma_st come from the bidirectional
 //                        search (bc_bidir.cu), pair values, scan
-// Directed graphs run on the plain and lane-major engines (counts pulled over
-// the in-neighbour CSR); graphs with edge lengths on the weighted engine
-// (bc_weighted.cu).
+// Engines: 64 sources to a traversal (bc_batch.cu), one source per CTA
+// (bc_multi.cu; deep graphs, and small ones where that is faster for the call's
+// sources), the plain kernels (bc_plain.cu, at width 1) and, for edge lengths,
+// the weighted engine (bc_weighted.cu). On directed graphs counts are pulled over
+// the in-neighbour CSR, or pushed along the out-edges.
 #include <algorithm>
 #include <cstdlib>
 #include <cstring>
@@ -2323,10 +2325,10 @@ static bc_tuning current_tuning(bc_ctx *ctx, const Graph &g) {
   t.batch_width = batch_width(ctx);
   t.heavy_degree = ctx->heavy_deg > 0 ? ctx->heavy_deg : 64;
   t.segment = ctx->seg_len > 0 ? ctx->seg_len : 256;
-  t.packed_max_lanes = ctx->pk_maxl;
-  t.packed_min_preds = ctx->pk_mincnt;
-  t.bwd_variant = ctx->bwd_variant;
-  t.heavy_lane = ctx->heavy_lane;
+  t.packed_max_lanes = 16;  // (this and the next three: kernel forms of earlier versions, bc.h)
+  t.packed_min_preds = 6;
+  t.bwd_variant = 1;
+  t.heavy_lane = 4;
   t.push_div = ctx->push_div;
   t.deep_levels = ctx->deep_levels;
   t.trial_ms = 0.0;

@@ -104,7 +104,7 @@ struct Sink {
   int32_t tstride = 64;            // row length of tdelta
   const int32_t *lane_col = nullptr;  // [64] column of each lane (null: column = lane)
   Acc *acc = nullptr;              // [n] exact all-vertex sum of delta over lanes (may be null)
-  double *delta_lm = nullptr;      // [n][64] full per-lane delta (may be null)
+  double *delta_lm = nullptr;      // [n][64] full per-lane delta (may be null; 64-lane and plain engines)
 };
 
 __device__ __forceinline__ void sink_targets(const Sink &sink, int32_t v, int t, double d) {
@@ -202,8 +202,6 @@ struct bc_ctx {
   // batched-engine tuning: degree above which a vertex is split into segments,
   // and the segment length (0 = library defaults)
   int32_t heavy_deg = 0, seg_len = 0;
-  // kernel forms of earlier versions, kept with a graph's tuning record (bc.h)
-  int32_t bwd_variant = 1, pk_maxl = 16, pk_mincnt = 6, heavy_lane = 4;
   // direction of a forward level: top-down (push from the level's vertex list,
   // then counts pulled for the discovered vertices only) when the level's
   // vertices have at most nnz / push_div edges; bottom-up (every vertex with
@@ -376,6 +374,8 @@ bool lane_major(bc_ctx *ctx, const Graph &g, int64_t count, bool adaptive = fals
 bool one_source_per_cta(bc_ctx *ctx, const Graph &g, int64_t count, bool adaptive = false, int64_t beside = 0);
 void solo_sources(bc_ctx *ctx, const Graph &g, const SoloSources &src, int count, const Sink &sink,
                   const SoloRows &rows);
+// acc[v] += the CTAs' exact partial sums partials[p][v].
+void add_partials(bc_ctx *ctx, const Graph &g, int nparts, const Acc *partials, Acc *acc);
 void do_uniform_multi(bc_ctx *ctx, const std::vector<bc_graph> &handles, const std::vector<const Graph *> &gs,
                       const int64_t *k, const uint64_t *seed, const uint64_t *qid, double *est_out);
 void forget_multi_plan(bc_ctx *ctx);
@@ -449,20 +449,17 @@ struct ApiLock {
 // settings restored afterwards.
 struct KnobScope {
   bc_ctx *ctx;
-  int32_t bw, hd, sl, pm, pc, bv, hl, pd, dl;
+  int32_t bw, hd, sl, pd, dl;
   KnobScope(bc_ctx *c, const Graph &g) : ctx(c) {
-    bw = c->batch_width; hd = c->heavy_deg; sl = c->seg_len; pm = c->pk_maxl; pc = c->pk_mincnt;
-    bv = c->bwd_variant; hl = c->heavy_lane; pd = c->push_div; dl = c->deep_levels;
+    bw = c->batch_width; hd = c->heavy_deg; sl = c->seg_len; pd = c->push_div; dl = c->deep_levels;
     if (g.tuned) {
       const bc_tuning &t = g.tune;
       c->batch_width = t.batch_width; c->heavy_deg = t.heavy_degree; c->seg_len = t.segment;
-      c->pk_maxl = t.packed_max_lanes; c->pk_mincnt = t.packed_min_preds; c->bwd_variant = t.bwd_variant;
-      c->heavy_lane = t.heavy_lane; c->push_div = t.push_div; c->deep_levels = t.deep_levels;
+      c->push_div = t.push_div; c->deep_levels = t.deep_levels;
     }
   }
   ~KnobScope() {
-    ctx->batch_width = bw; ctx->heavy_deg = hd; ctx->seg_len = sl; ctx->pk_maxl = pm; ctx->pk_mincnt = pc;
-    ctx->bwd_variant = bv; ctx->heavy_lane = hl; ctx->push_div = pd; ctx->deep_levels = dl;
+    ctx->batch_width = bw; ctx->heavy_deg = hd; ctx->seg_len = sl; ctx->push_div = pd; ctx->deep_levels = dl;
   }
   KnobScope(const KnobScope &) = delete;
   KnobScope &operator=(const KnobScope &) = delete;

@@ -91,7 +91,6 @@ k_solo(MGraph G, SoloSources src, int count, unsigned *__restrict__ next, unsign
     }
     solo_backward<TIER, T>(G, L, ext, maxc, S, c, ph, e, [&](int32_t v, double delta) {
       if (rows.delta) rows.delta[(size_t)t * G.n + v] = delta;
-      if (sink.delta_lm) sink.delta_lm[(size_t)v * 64 + t] = delta;
       if (sink.tslot) sink_targets(sink, v, t, delta);
       if (part) {
         Acc cur = part[v];
@@ -679,6 +678,11 @@ int solo_slots(bc_ctx *ctx, const Graph &g) {
   return c.ncta;
 }
 
+void add_partials(bc_ctx *ctx, const Graph &g, int nparts, const Acc *partials, Acc *acc) {
+  LaunchScope ls(ctx, F_XBWD);
+  k_solo_acc<<<(g.n + 31) / 32, 1024, 0, ctx->stream>>>(g.n, nparts, partials, acc);
+}
+
 void solo_sources(bc_ctx *ctx, const Graph &g, const SoloSources &src, int count, const Sink &sink,
                   const SoloRows &rows) {
   if (count < 1) return;
@@ -698,10 +702,7 @@ void solo_sources(bc_ctx *ctx, const Graph &g, const SoloSources &src, int count
                                             ctx->ws.err.as<unsigned>(), ctx->ws.cnt.as<unsigned long long>());
     return 0;
   });
-  if (sink.acc) {
-    LaunchScope ls(ctx, F_XBWD);
-    k_solo_acc<<<(g.n + 31) / 32, 1024, 0, st>>>(g.n, c.ncta, L.partials.as<Acc>(), sink.acc);
-  }
+  if (sink.acc) add_partials(ctx, g, c.ncta, L.partials.as<Acc>(), sink.acc);
   ctx->samples += count;
   ctx->batches += 1;
 }

@@ -567,7 +567,6 @@ k_w_sink(WGraph W, const int32_t *__restrict__ sources, int count, unsigned *__r
     w_source<TIER, T>(
         W, sources[t], M, sh, ph, e,
         [&](int32_t v, double delta) {
-          if (sink.delta_lm) sink.delta_lm[(size_t)v * 64 + t] = delta;
           if (sink.tslot) sink_targets(sink, v, t, delta);
           if (part) {
             Acc cur = part[v];
@@ -617,24 +616,6 @@ k_w_rows(WGraph W, const int32_t *__restrict__ sources, int count, unsigned *__r
         });
   }
   if (e) atomicOr(err, e);
-}
-
-__global__ void __launch_bounds__(1024) k_w_acc(int32_t n, int nparts, const Acc *__restrict__ partials,
-                                                Acc *__restrict__ acc) {
-  __shared__ Acc sh[32][33];  // (as k_solo_acc)
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int32_t v = blockIdx.x * 32 + lane;
-  Acc a = acc_zero();
-  if (v < n)
-    for (int p = warp; p < nparts; p += 32) acc_add_acc(a, partials[(size_t)p * n + v]);
-  sh[warp][lane] = a;
-  __syncthreads();
-  a = acc_warp_sum(sh[lane][warp]);
-  const int32_t vw = blockIdx.x * 32 + warp;
-  if (lane == 0 && vw < n) {
-    acc_add_acc(a, acc[vw]);
-    acc[vw] = a;
-  }
 }
 
 // ------------------------------------------------------------------ host --
@@ -739,10 +720,7 @@ void wlane_sink(bc_ctx *ctx, const Graph &g, const int32_t *d_sources, int count
                                             sink.acc ? W.partials.as<Acc>() : nullptr, sink, ctx->ws.err.as<unsigned>());
     return 0;
   });
-  if (sink.acc) {
-    LaunchScope ls(ctx, F_XBWD);
-    k_w_acc<<<(g.n + 31) / 32, 1024, 0, st>>>(g.n, c.ncta, W.partials.as<Acc>(), sink.acc);
-  }
+  if (sink.acc) add_partials(ctx, g, c.ncta, W.partials.as<Acc>(), sink.acc);
   ctx->samples += count;
   ctx->batches += 1;
 }
