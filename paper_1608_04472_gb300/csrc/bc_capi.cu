@@ -879,17 +879,17 @@ static KeyMeta &key_meta(bc_ctx *ctx, const Graph &g, bool need_order, int64_t c
 constexpr int WMAX = 1024;       // draws per window of the 64-lane engine
 constexpr int WMAX_SOLO = 4096;  // ... of the engines that run one source per CTA
 
-bool lane_major(bc_ctx *ctx, const Graph &g, int64_t count, bool adaptive, int64_t beside) {
+bool lane_major(bc_ctx *ctx, const Graph &g, int64_t count, SoloCall call, int64_t beside) {
   if (graph_depth_hint(ctx, g) > ctx->deep_levels) return true;
-  return solo_fits(ctx, g) && solo_pays(ctx, g, count, adaptive, beside);
+  return solo_fits(ctx, g) && solo_pays(ctx, g, count, call, beside);
 }
 
 // Engines that run one source per persistent CTA (edge lengths; deep graphs;
 // graphs whose state fits shared memory) take a whole window in one launch, so
 // every resident CTA has a source; the 64-lane engine and the plain width take
 // 64 or 1 at a time.
-bool one_source_per_cta(bc_ctx *ctx, const Graph &g, int64_t count, bool adaptive, int64_t beside) {
-  return batch_width(ctx) != 1 && (g.w || lane_major(ctx, g, count, adaptive, beside));
+bool one_source_per_cta(bc_ctx *ctx, const Graph &g, int64_t count, SoloCall call, int64_t beside) {
+  return batch_width(ctx) != 1 && (g.w || lane_major(ctx, g, count, call, beside));
 }
 
 // A window that the 64-lane engine takes as one batch, in draw order.
@@ -1062,7 +1062,7 @@ static void do_adaptive_sources(bc_ctx *ctx, const Graph &g, const int32_t *targ
   const size_t n = (size_t)g.n;
   cudaStream_t st = ctx->stream;
   ws.tslot.ensure(n * 4);
-  const bool per_cta = one_source_per_cta(ctx, g, cap, true);
+  const bool per_cta = one_source_per_cta(ctx, g, cap, CALL_ADAPTIVE);
   const int wmax = window_max(per_cta, T);
   ws.tdelta.ensure((size_t)std::max(T, 1) * wmax * 8);
   {
@@ -1582,7 +1582,7 @@ static void do_source_dependencies(bc_ctx *ctx, const Graph &g, const int32_t *s
     do_source_rows_weighted(ctx, g, sources, count, delta_out, nullptr, sigma_out, sm_out, se_out, tier_out);
     return;
   }
-  if (batch_width(ctx) != 1 && solo_fits(ctx, g) && lane_major(ctx, g, count)) {
+  if (batch_width(ctx) != 1 && solo_fits(ctx, g) && lane_major(ctx, g, count, CALL_ROWS)) {
     do_source_rows_solo(ctx, g, sources, count, delta_out, dist_out, sigma_out, sm_out, se_out, tier_out);
     return;
   }

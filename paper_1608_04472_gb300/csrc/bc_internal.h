@@ -358,20 +358,22 @@ struct SoloRows {
   int32_t *se = nullptr;
   int32_t *tier = nullptr;
 };
+// What a call does with its sources: their sums (or targets' values) in windows
+// of a size, the growing windows of Bader's loop, or per-source rows.
+enum SoloCall { CALL_SUMS, CALL_ADAPTIVE, CALL_ROWS };
 // Whether a source's state fits shared memory, whether `count` sources of such a
-// graph are faster one per CTA than 64 to a traversal (adaptive: as Bader's loop
-// draws them; beside: sources of other graphs in the same launch), and how many
-// run at once.
+// graph are faster one per CTA than 64 to a traversal (beside: sources of other
+// graphs in the same launch), and how many run at once.
 bool solo_fits(bc_ctx *ctx, const Graph &g);
-bool solo_pays(bc_ctx *ctx, const Graph &g, int64_t count, bool adaptive = false, int64_t beside = 0);
+bool solo_pays(bc_ctx *ctx, const Graph &g, int64_t count, SoloCall call = CALL_SUMS, int64_t beside = 0);
 int solo_slots(bc_ctx *ctx, const Graph &g);
 // The largest finite distance from v by one CTA (any graph without lengths).
 int solo_depth(bc_ctx *ctx, const Graph &g, int32_t v);
 // Whether a call with `count` sources runs one source per persistent CTA: deep
 // graphs, and fitting ones where it pays (lane_major: at any width but 1,
 // weighted graphs apart). Every engine gives the same results.
-bool lane_major(bc_ctx *ctx, const Graph &g, int64_t count, bool adaptive = false, int64_t beside = 0);
-bool one_source_per_cta(bc_ctx *ctx, const Graph &g, int64_t count, bool adaptive = false, int64_t beside = 0);
+bool lane_major(bc_ctx *ctx, const Graph &g, int64_t count, SoloCall call = CALL_SUMS, int64_t beside = 0);
+bool one_source_per_cta(bc_ctx *ctx, const Graph &g, int64_t count, SoloCall call = CALL_SUMS, int64_t beside = 0);
 void solo_sources(bc_ctx *ctx, const Graph &g, const SoloSources &src, int count, const Sink &sink,
                   const SoloRows &rows);
 // acc[v] += the CTAs' exact partial sums partials[p][v].

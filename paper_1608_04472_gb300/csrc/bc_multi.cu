@@ -340,8 +340,8 @@ static SoloCfg solo_cfg(bc_ctx *ctx, int tier, int32_t n, int64_t nnz, int64_t c
 }
 
 // Whether `count` sources of a fitting graph that is not deep run one per CTA
-// rather than 64 to a traversal (adaptive: in the windows of Bader's loop;
-// beside: draws of other graphs in the same launch). One source per CTA reads
+// rather than 64 to a traversal (beside: draws of other graphs in the same
+// launch). One source per CTA reads
 // every row once per source at one CTA's speed, so a launch takes as long as a
 // source on a CTA times the rounds over the CTAs, however few the sources; the
 // 64-lane engine takes a batch's time for every 64, mostly per level. Both
@@ -356,9 +356,10 @@ static SoloCfg solo_cfg(bc_ctx *ctx, int tier, int32_t n, int64_t nnz, int64_t c
 // s14 (430,000 entries) 770 / 777 / 797 / 3708 and 399 / 469 / 917 / 3385; s15 (890,000)
 // 1617 / 1635 / 1722 / 7246 and 489 / 566 / 1061 / 3995; ER n = 60,000 degree 3 878 / 906 /
 // 1905 / 6825 and 1170 / 1320 / 3580 / 16,700.
-bool solo_pays(bc_ctx *ctx, const Graph &g, int64_t count, bool adaptive, int64_t beside) {
+bool solo_pays(bc_ctx *ctx, const Graph &g, int64_t count, SoloCall call, int64_t beside) {
   if (ctx->solo_always) return true;
   const int tier = solo_tier(g);
+  const bool adaptive = call == CALL_ADAPTIVE;
   const double n = (double)g.n, z = (double)g.nnz, depth = (double)graph_depth_hint(ctx, g);
   const int64_t sms = solo_sms();
   auto ctas = [&](int64_t c, bool *small) {
@@ -393,6 +394,9 @@ bool solo_pays(bc_ctx *ctx, const Graph &g, int64_t count, bool adaptive, int64_
   } else {
     lane += (double)(draws / 1024) * lanes(1024) + (draws % 1024 ? lanes(draws % 1024) : 0.0);
   }
+  // per-source rows are extracted and transposed there, through buffers of the call
+  // (BA n = 50,001, 70 rows: 2.7 ms here, 3.4 there)
+  if (call == CALL_ROWS) lane += n * (5e-3 + 0.1e-3 * (double)count);
   return 0.87 * solo <= lane;
 }
 
@@ -790,7 +794,7 @@ void do_uniform_multi(bc_ctx *ctx, const std::vector<bc_graph> &handles, const s
   for (int g = 0; g < G; ++g)
     if (solo_fits(ctx, *gs[g])) fitting += k[g];
   for (int g = 0; g < G; ++g)
-    (one_source_per_cta(ctx, *gs[g], k[g], false, fitting - k[g]) && !gs[g]->w ? deep : shallow).push_back(g);
+    (one_source_per_cta(ctx, *gs[g], k[g], CALL_SUMS, fitting - k[g]) && !gs[g]->w ? deep : shallow).push_back(g);
   std::lock_guard<std::mutex> lk(g_plans_mu);
   MultiPlan &P = g_plans[ctx];
   cudaEvent_t done = nullptr;
