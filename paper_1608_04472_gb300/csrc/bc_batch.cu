@@ -1839,9 +1839,9 @@ static bool second_slot(bc_ctx *ctx, const Graph &g, bool acc) {
 // and the host reads a batch's depth and largest count without the GPU waiting
 // for it. The batches write different columns; all-vertex sums are kept per
 // slot and added at the end (exact sums: any order).
-// ms with one batch at a time and with two: ER n = 100,003 k = 333 5.73 / 4.90,
-// R-MAT s16 Bader 1500 draws 15.0 / 12.2, directed s17 k = 512 6.58 / 5.15, s20 k =
-// 1024 40.4 / 37.1 (a host read per level, one batch: 5.70, 14.0, 6.39, 38.1).
+// ms with one batch at a time and with two: ER n = 100,003 k = 333 5.02 / 3.96,
+// R-MAT s16 Bader 1500 draws 13.8 / 11.1, directed s17 k = 512 6.46 / 4.93, s20 k =
+// 1024 37.3 / 33.8.
 void run_lane_batches(bc_ctx *ctx, const Graph &g, const int32_t *src, const int32_t *pos, int count,
                       const Sink &sink) {
   if (count < 1) return;

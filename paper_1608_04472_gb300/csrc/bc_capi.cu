@@ -892,8 +892,13 @@ bool one_source_per_cta(bc_ctx *ctx, const Graph &g, int64_t count, SoloCall cal
   return batch_width(ctx) != 1 && (g.w || lane_major(ctx, g, count, call, beside));
 }
 
-// A window that the 64-lane engine takes as one batch, in draw order.
-static bool one_batch(bc_ctx *ctx, const Graph &g, int W) { return W <= 64 && batch_width(ctx) != 1 && !g.w; }
+// A call of one batch on a graph small enough that a source key would not pay: its
+// draws run in draw order. (Elsewhere windows of one batch are sorted too: sources
+// alike in neighbouring lanes share sectors of a row, 4 % of Bader's loop with 161
+// draws on R-MAT n = 528,806.)
+static bool one_batch(bc_ctx *ctx, const Graph &g, int64_t total) {
+  return total <= 64 && g.n <= 65536 && batch_width(ctx) != 1 && !g.w;
+}
 
 // The draws a window can hold and the size of the first one, where sources have
 // a CTA each (per_cta) or not; a call keeps to one of the two. Where a source has a CTA
@@ -908,7 +913,8 @@ static int window_first(bc_ctx *ctx, const Graph &g, bool per_cta) {
 // Draws [i0, i0+W) of (seed, qid): ws.win = draws[W] and, for the 64-lane
 // engine, grouped by source key, sorted sources[W] at WMAX and sorted draw
 // positions[W] at 2 WMAX (where a source has a CTA of its own, which sources
-// run together does not matter, nor in a window of one batch: no key is built).
+// run together does not matter, nor in a small graph's single batch: no key is
+// built).
 // total: the call's draws.
 static void draw_window(bc_ctx *ctx, const Graph &g, bool per_cta, int64_t total, uint64_t seed, uint64_t qid,
                         int64_t i0, int W) {
@@ -917,7 +923,7 @@ static void draw_window(bc_ctx *ctx, const Graph &g, bool per_cta, int64_t total
   static_assert(WMAX_SOLO >= 3 * WMAX, "the window buffer holds the draws and their sorted form");
   int32_t *draws = ws.win.as<int32_t>();
   launch_draw_sources(ctx, seed, qid, (uint64_t)i0, W, g.n, draws);
-  if (per_cta || one_batch(ctx, g, W)) return;
+  if (per_cta || one_batch(ctx, g, total)) return;
   const KeyMeta &km = key_meta(ctx, g, false, total);
   LaunchScope ls(ctx, F_DRAW);
   k_sort_window<<<1, 1024, 0, ctx->stream>>>(W, draws, km.key.as<uint8_t>(), draws + WMAX, draws + 2 * WMAX);
@@ -933,14 +939,14 @@ static void run_sources_per_cta(bc_ctx *ctx, const Graph &g, const int32_t *d_so
 // Runs the window's sources: one launch where a source has a CTA, else batches
 // of the context's width (lane t of the batch starting at position b is the
 // window's sorted entry b + t).
-static void run_window(bc_ctx *ctx, const Graph &g, bool per_cta, int W, Sink sink) {
+static void run_window(bc_ctx *ctx, const Graph &g, bool per_cta, int64_t total, int W, Sink sink) {
   Workspace &ws = ctx->ws;
   const int width = batch_width(ctx);
   if (per_cta) {  // column = draw position
     run_sources_per_cta(ctx, g, ws.win.as<int32_t>(), W, sink);
     return;
   }
-  if (one_batch(ctx, g, W)) {
+  if (one_batch(ctx, g, total)) {
     run_lane_batches(ctx, g, ws.win.as<int32_t>(), nullptr, W, sink);
     return;
   }
@@ -977,7 +983,7 @@ static void run_draws(bc_ctx *ctx, const Graph &g, uint64_t seed, uint64_t qid, 
       solo_sources(ctx, g, src, W, sink, SoloRows{});
     } else {
       draw_window(ctx, g, per_cta, count, seed, qid, i0 + a, W);
-      run_window(ctx, g, per_cta, W, sink);
+      run_window(ctx, g, per_cta, count, W, sink);
     }
   }
 }
@@ -1088,7 +1094,7 @@ static void do_adaptive_sources(bc_ctx *ctx, const Graph &g, const int32_t *targ
     sink.tslot = ws.tslot.as<int32_t>();
     sink.tdelta = ws.tdelta.as<double>();
     sink.tstride = W;
-    run_window(ctx, g, per_cta, W, sink);
+    run_window(ctx, g, per_cta, cap, W, sink);
     {
       LaunchScope ls(ctx, F_SCAN);
       k_stop_scan<<<(T + 3) / 4, 128, 0, st>>>(T, W, ws.tdelta.as<double>(), ss, i0, cn, 1.0, W);
@@ -1133,7 +1139,7 @@ static void do_target_block(bc_ctx *ctx, const Graph &g, const int32_t *targets,
     sink.tslot = ws.tslot.as<int32_t>();
     sink.tdelta = ws.tdelta.as<double>();
     sink.tstride = W;
-    run_window(ctx, g, per_cta, W, sink);
+    run_window(ctx, g, per_cta, count, W, sink);
     BCG_CUDA(cudaMemcpyAsync(h.data(), ws.tdelta.p, (size_t)T * W * 8, cudaMemcpyDeviceToHost, st));
     sync(ctx);
     for (int32_t j = 0; j < T; ++j)

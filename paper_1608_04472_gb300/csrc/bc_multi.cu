@@ -15,6 +15,7 @@
 // successor sums (order-free); a source whose counts exceed 2^64-1 continues
 // in the extended form (bc_xf.cuh; sums in CSR order of the vertex).
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <map>
 #include <tuple>
@@ -349,8 +350,8 @@ static SoloCfg solo_cfg(bc_ctx *ctx, int tier, int32_t n, int64_t nnz, int64_t c
 // 1024 draws on 40 graphs of 1,500 to 65,536 vertices and 16,000 to a million
 // entries (ER, BA, R-MAT, directed ones among them) with either engine; the 64-lane
 // engine has to be an eighth faster by them (they are off by about that much). The
-// choice costs 1.3 % over the better engine in the geometric mean, at worst it was
-// 1.18 times slower than always here and 5 % than always there. Here / there, us a call
+// choice costs 1.4 % over the better engine in the geometric mean, for sums at worst
+// 1.21 times what always here and 1.05 what the engine before this one took. Here / there, us a call
 // of 16 / 64 / 200 / 1024 draws: ER n = 2000 degree 8 133 / 137 / 149 / 291 and 311 / 342
 // / 760 / 2799; ER n = 50,000 934 / 950 / 1978 / 7013 and 528 / 658 / 1737 / 7073; R-MAT
 // s14 (430,000 entries) 770 / 777 / 797 / 3708 and 399 / 469 / 917 / 3385; s15 (890,000)
@@ -368,7 +369,8 @@ bool solo_pays(bc_ctx *ctx, const Graph &g, int64_t count, SoloCall call, int64_
   };
   bool small;
   const int64_t first = adaptive ? std::max<int64_t>(64, ctas((int64_t)1 << 30, &small)) : 0;
-  const double lat[2] = {10e-3 * n + 1.05e-3 * z + 2.5 * depth, 30e-3 * n + 2.6e-3 * z};  // 1024 and 256 threads
+  // a source on a CTA of 1024 and of 256 threads (rows above 64 entries: uneven work)
+  const double lat[2] = {10e-3 * n + (g.max_deg > 64 ? 1.2e-3 : 0.85e-3) * z + 2.5 * depth, 30e-3 * n + 2.6e-3 * z};
   const double level = 125.0 + 37.0 * depth, rows = n * (3.8e-3 + 0.38e-3 * depth);
   double solo = 90.0, lane = 50.0;
   auto window = [](int64_t i, int64_t lo, int64_t hi, int64_t left) {
@@ -395,8 +397,11 @@ bool solo_pays(bc_ctx *ctx, const Graph &g, int64_t count, SoloCall call, int64_
     lane += (double)(draws / 1024) * lanes(1024) + (draws % 1024 ? lanes(draws % 1024) : 0.0);
   }
   // per-source rows are extracted and transposed there, through buffers of the call
-  // (BA n = 50,001, 70 rows: 2.7 ms here, 3.4 there)
-  if (call == CALL_ROWS) lane += n * (5e-3 + 0.1e-3 * (double)count);
+  // (BA n = 50,001, 70 rows: 2.7 ms here, 3.4 there; n = 2389, 12 rows: 0.27 and 0.35)
+  if (call == CALL_ROWS) {
+    const double q = std::sqrt(1e-3 * n * (double)count);
+    lane += 40.0 + std::min(14.0 * q, 100.0 + 8.0 * q);
+  }
   return 0.87 * solo <= lane;
 }
 

@@ -23,7 +23,7 @@
 //   tier 1  distances (2 B) in shared memory, queue and counts in global
 //           memory, where 152 CTAs' arrays mostly fit L2 (n up to ~111,000);
 //   tier 2  everything in global memory (any n).
-// Where each is taken, with the times: solo_fits (bc_multi.cu).
+// Where each is taken, with the times: solo_pays, solo_cfg (bc_multi.cu).
 #pragma once
 
 #include <type_traits>

@@ -185,7 +185,7 @@ def test_small_graphs_equal_the_oracle_whatever_the_count(name):
     ("small", 1, "ext_fwd"), ("small", 64, "ext_fwd"), ("small", 1024, "ext_fwd"),
     ("sparse", 16, "ext_fwd"), ("sparse", 1024, "ext_fwd")])               # many levels
 def test_the_engine_follows_the_number_of_sources(graph, draws, family):
-    g = {"hubs": lambda: gg.rmat(15, 16, 0.57, 0.19, 0.19, 3), "tier 1": lambda: gg.erdos_renyi(40_000, 8, 6, pairwise=False),
+    g = {"hubs": lambda: gg.rmat(15, 16, 0.57, 0.19, 0.19, 3), "tier 1": lambda: gg.erdos_renyi(60_000, 8, 6, pairwise=False),
          "small": lambda: gg.erdos_renyi(2000, 8, 1), "sparse": lambda: gg.erdos_renyi(60_000, 3, 4, pairwise=False)}[graph]()
     other = {"fwd": "ext_fwd", "ext_fwd": "fwd"}[family]
     with _ctx() as ctx:
