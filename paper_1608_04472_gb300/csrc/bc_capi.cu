@@ -20,6 +20,9 @@
 #include <thread>
 #include <vector>
 
+#include <sys/mman.h>
+#include <unistd.h>
+
 #include "bc_internal.h"
 #include "bc_xf.cuh"
 
@@ -1438,11 +1441,19 @@ static void do_adaptive_pairs(bc_ctx *ctx, const Graph &g, const int32_t *target
 class PageTouch {
  public:
   void add(void *p, size_t bytes) {
-    if (p) parts_.push_back({static_cast<volatile char *>(p), bytes});
+    if (p && bytes) parts_.push_back({static_cast<volatile char *>(p), bytes});
   }
   void start() {
-    size_t total = 0;
-    for (const auto &x : parts_) total += x.second;
+    auto bytes = [&] {
+      size_t total = 0;
+      for (const auto &x : parts_) total += x.second;
+      return total;
+    };
+    if (bytes() < ((size_t)4 << 20)) return;
+    // (arrays that an allocator hands out again have their pages: 16 rows of ER
+    // n = 50,000 took 1.54 ms with the threads, 1.19 without)
+    parts_.erase(std::remove_if(parts_.begin(), parts_.end(), present), parts_.end());
+    const size_t total = bytes();
     if (total < ((size_t)4 << 20)) return;
     const size_t most = std::max<size_t>(1, std::min<size_t>(8, std::thread::hardware_concurrency() / 2));
     const size_t nt = std::min(most, total >> 21);
@@ -1465,7 +1476,20 @@ class PageTouch {
   ~PageTouch() { wait(); }
 
  private:
-  std::vector<std::pair<volatile char *, size_t>> parts_;
+  using Part = std::pair<volatile char *, size_t>;
+  // Whether 16 pages spread over the array are all there.
+  static bool present(const Part &x) {
+    const long size = sysconf(_SC_PAGESIZE);
+    const uintptr_t page = size > 0 ? (uintptr_t)size : 4096, first = reinterpret_cast<uintptr_t>(x.first) / page;
+    const uintptr_t n = (reinterpret_cast<uintptr_t>(x.first) + x.second + page - 1) / page - first;
+    for (uintptr_t i = 0; i < 16; ++i) {
+      unsigned char there = 0;
+      if (mincore(reinterpret_cast<void *>((first + (n - 1) * i / 15) * page), page, &there) != 0 || !(there & 1))
+        return false;
+    }
+    return true;
+  }
+  std::vector<Part> parts_;
   std::vector<std::thread> threads_;
 };
 
