@@ -1035,14 +1035,15 @@ static void do_exact_or_uniform(bc_ctx *ctx, const Graph &g, bool exact, int64_t
 // The depth that decides between the level-mask engine and one source per
 // persistent CTA: the largest finite distance from the hub (along out-edges on
 // a directed graph; the level-mask engine pulls counts over the in-neighbour CSR).
-// Small graphs get it from one CTA's BFS (about 5 ns a vertex and 0.5 an entry;
-// the plain engine's takes 20 us a level, in all of 6 to 15 here).
+// Small graphs get it from one CTA's BFS (about 5 ns a vertex, 0.5 an entry and 3 us
+// a level); larger ones of them with more than six entries a vertex, which have few
+// levels, from the plain engine's (20 us a level: a 200x200 grid took 8 ms).
 int graph_depth_hint(bc_ctx *ctx, const Graph &g) {
   {
     std::lock_guard<std::mutex> lk(g_keys_mu);
     KeyMeta &km = g_keys[g.rp];
     if (km.ecc >= 0) return km.ecc;
-    if (!solo_fits(ctx, g) || g.n + g.nnz / 10 > 40000) {
+    if (!solo_fits(ctx, g) || (g.n + g.nnz / 10 > 40000 && g.nnz > 6 * (int64_t)g.n)) {
       const int64_t s0 = ctx->samples, b0 = ctx->batches;
       build_depth(ctx, g, km);
       ctx->samples = s0;
