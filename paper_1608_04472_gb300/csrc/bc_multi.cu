@@ -396,11 +396,13 @@ bool solo_pays(bc_ctx *ctx, const Graph &g, int64_t count, SoloCall call, int64_
   } else {
     lane += (double)(draws / 1024) * lanes(1024) + (draws % 1024 ? lanes(draws % 1024) : 0.0);
   }
-  // per-source rows are extracted and transposed there, through buffers of the call
-  // (BA n = 50,001, 70 rows: 2.7 ms here, 3.4 there; n = 2389, 12 rows: 0.27 and 0.35)
+  // per-source rows are extracted and transposed there, through buffers of the call,
+  // which starts to cost with a few of them (here / there, us, 1 / 3 / 20 rows: ER n =
+  // 43,309 degree 6 663 / 704 / 1071 and 544 / 732 / 1373; R-MAT n = 20,000 degree 6
+  // 620 / 750 / 936 and 408 / 443 / 967)
   if (call == CALL_ROWS) {
     const double q = std::sqrt(1e-3 * n * (double)count);
-    lane += 40.0 + std::min(14.0 * q, 100.0 + 8.0 * q);
+    lane += std::min(14.0 * q, 250.0 + 8.0 * q) - 70.0;
   }
   return 0.87 * solo <= lane;
 }

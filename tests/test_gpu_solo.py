@@ -205,6 +205,19 @@ def test_the_engine_follows_the_number_of_sources(graph, draws, family):
             assert ran[family]["launches"] > 0 and ran[other]["launches"] == 0, call
 
 
+@pytest.mark.parametrize("n,rows,family", [(43_309, 1, "fwd"), (43_309, 20, "ext_fwd"), (5000, 1, "ext_fwd")])
+def test_the_engine_of_per_source_rows_follows_their_number(n, rows, family):
+    g = gg.erdos_renyi(n, 6, 5, pairwise=False)
+    other = {"fwd": "ext_fwd", "ext_fwd": "fwd"}[family]
+    with _ctx() as ctx:
+        h = ctx.load_graph(g.row_ptr, g.col)
+        ctx.source_dependencies(h, np.arange(rows, dtype=np.int32))  # the depth is known from here on
+        ctx.reset_stats()
+        ctx.source_dependencies(h, np.arange(rows, dtype=np.int32))
+        ran = ctx.stats()["kernels"]
+        assert ran[family]["launches"] > 0 and ran[other]["launches"] == 0
+
+
 @pytest.mark.parametrize("lengths", [False, True])
 def test_a_refused_call_leaves_its_outputs_as_they_were(lengths):
     """Outputs large enough to have their pages touched (4 MB)."""
